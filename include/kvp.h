@@ -88,7 +88,8 @@ int kvp_timing_events_used(int kernel);
 /* Measurement switch of the GEMM's tile shape.  1 (the default): the forward GEMMs (kvp_proj_fwd,
  * kvp_out_proj_fwd, kvp_gemm) run on CTA pairs (256 x 256 tiles, one per pair of SMs) when every problem of the
  * launch has more than 128 rows, the gradient GEMMs on single-CTA 128 x 256 tiles; 0: single-CTA tiles
- * everywhere; 2: CTA pairs everywhere.  The results are the same in every mode (same products, same summation
+ * everywhere; 2: CTA pairs everywhere.  (K-major problems of at most 128 rows have a kernel of their own in every
+ * mode.)  The results are the same in every mode (same products, same summation
  * order along K).  Not thread-safe. */
 void kvp_set_gemm_pair_mode(int mode);
 

@@ -11,6 +11,8 @@
 // One launch walks the tiles of a whole list of problems (different shapes, operands, operand modes and output
 // types): the Q, K and V projections of every layer are one launch, so are all weight and input gradients of a
 // backward pass, and the SMs idle only behind the last tile of the list instead of behind each GEMM's last wave.
+#include <algorithm>
+
 #include "kvp_host.h"
 #include "kvp_sm100.cuh"
 
@@ -473,6 +475,174 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
   }
 }
 
+// ------------------------------------------------------------------------------------------------------------
+// Few rows of A (the tokens of a decode step): C^T = B A^T, K split over a cluster.
+//
+// With at most 128 rows of A the product is bound by reading B once, and the 128 x 256 tiles above put it on N / 256
+// CTAs: 16 of 148 SMs at N = 4096, 29 us for 33.5 MB.  Here B supplies the M = 128 side of the MMA and the tokens its
+// N side (a multiple of 16, so 16 tokens cost 16 columns and not 128 rows), and the k-blocks of a tile are dealt to
+// the CTAs of a cluster, each with its own ring.  The partials meet in shared memory: every CTA moves its accumulator
+// from TMEM to shared memory as [token][128 columns] fp32 and sums its share of the tokens over the cluster's CTAs
+// through distributed shared memory, in rank order, so results do not depend on timing.
+// Measured (us, K x N at M tokens; 128 x 256 tiles -> this kernel; reading B at the copy rate): 4096 x 4096 at 16
+// tokens 28.7 -> 11.6 (5.2), 4096 x 11008 at 16 30.8 -> 20.6 (13.9), 11008 x 4096 at 16 65.5 -> 20.6 (13.9), 4096 x
+// 4096 at 128 28.9 -> 14.5 (5.5); a launch that does almost nothing takes 6.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int SROWS = 128;                       // rows of B (output columns) per tile: the M of the MMA
+constexpr int SB_BYTES = SROWS * BK * 2;         // 16 KB
+constexpr int SPLIT_THREADS = 192;
+constexpr int SPLIT_MAX_STAGES = 8;
+
+struct SplitProblem {
+  int M, N;
+  int tok_tiles;           // token tiles of `nt` rows
+  int tile_end;
+  int kblocks;
+  int out_f32;
+  long long ldc;
+  void* c;
+};
+template <int NP>
+struct SplitParams {
+  CUtensorMap map_a[NP], map_b[NP];
+  SplitProblem prob[NP];
+  int nt;                  // tokens per tile: the N of the MMA, a multiple of 16
+  int stages;
+  int tmem_cols;
+  uint32_t idesc;
+};
+
+template <int NP>
+__global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ uint64_t full[SPLIT_MAX_STAGES], empty[SPLIT_MAX_STAGES], acc_full;
+  __shared__ uint32_t tmem_slot;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  int* err = &g_gemm_status;
+  const uint32_t split = cluster_nctarank(), rank = cluster_ctarank();
+  const int t = blockIdx.x / split;
+  const int stages = p.stages, nt = p.nt;
+  const int stage_bytes = SB_BYTES + nt * (BK * 2);
+
+  int pi = 0;
+  if constexpr (NP > 1)
+    while (t >= p.prob[pi].tile_end) ++pi;
+  const SplitProblem& pr = p.prob[pi];
+  const int within = t - (pi ? p.prob[pi - 1].tile_end : 0);
+  const int n0 = (within / pr.tok_tiles) * SROWS;   // first output column (row of B)
+  const int m0 = (within % pr.tok_tiles) * nt;      // first token
+  const int kb0 = int(rank) * pr.kblocks / int(split), kb1 = (int(rank) + 1) * pr.kblocks / int(split);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&acc_full, 1);
+    mbar_fence_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(&tmem_slot, p.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = tmem_slot;
+
+  if (warp == 0) {
+    const uint32_t leader = elect_one();
+    int s = 0;
+    uint32_t ph = 1;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait(&empty[s], ph, err)) break;
+      uint8_t* sb = smem + s * stage_bytes;
+      mbar_expect_tx_e(&full[s], stage_bytes, leader);
+      tma_load_2d_e(sb, &p.map_b[pi], &full[s], kb * BK, n0, leader);
+      tma_load_2d_e(sb + SB_BYTES, &p.map_a[pi], &full[s], kb * BK, m0, leader);
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+  } else if (warp == 1) {
+    const uint32_t leader = elect_one();
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait(&full[s], ph, err)) { ok = false; break; }
+      tc_fence_after_sync();
+      const uint32_t b_lo = desc_lo_sw128(smem_u32(smem + s * stage_bytes), 0);
+      const uint32_t a_lo = desc_lo_sw128(smem_u32(smem + s * stage_bytes + SB_BYTES), 0);
+#pragma unroll
+      for (int k = 0; k < BK / 16; ++k)
+        umma_ss_w(tmem_base, desc_lo_add(b_lo, k * 32), desc_lo_add(a_lo, k * 32), desc_hi_sw128(1024), p.idesc,
+                  kb != kb0 || k != 0, leader);
+      umma_commit(&empty[s], leader);
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    if (ok) umma_commit(&acc_full, leader);
+  }
+  // every warp waits for the accumulator; the four warps that own its lanes move it to shared memory as [token][128]
+  // fp32 (the ring is idle now)
+  __syncwarp();
+  float* part = reinterpret_cast<float*>(smem);
+  bool ok = mbar_wait(&acc_full, 0, err);
+  ok = __all_sync(0xffffffffu, ok);
+  if (ok && warp >= 2) {
+    tc_fence_after_sync();
+    const int quarter = warp & 3;
+    const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16);
+    for (int c0 = 0; c0 < nt; c0 += 16) {
+      uint32_t r[16];
+      tmem_ld_x16(taddr + c0, r);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) part[(c0 + i) * SROWS + quarter * 32 + lane] = __uint_as_float(r[i]);
+    }
+    tc_fence_before_sync();
+  }
+  __syncthreads();
+  if (split > 1) cluster_sync_all();
+  // each CTA of the cluster sums its share of the tokens over all partials, always in rank order
+  if (ok) {
+    const int col = n0 + lane * 4;
+    const uint32_t mine = smem_u32(part) + lane * 16;
+    const int n_tok = min(nt, pr.M - m0);
+    for (int tk = rank + warp * split; tk < n_tok; tk += split * (SPLIT_THREADS / 32)) {
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (uint32_t j = 0; j < split; ++j) {
+        const float4 v = ld_cluster_f4(cluster_map_addr(mine + tk * (SROWS * 4), j));
+        acc.x += v.x;
+        acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
+      }
+      if (col < pr.N) {
+        const size_t at = size_t(m0 + tk) * pr.ldc + col;
+        if (pr.out_f32)
+          *reinterpret_cast<float4*>(reinterpret_cast<float*>(pr.c) + at) = acc;
+        else
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(pr.c) + at) =
+              make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+      }
+    }
+  }
+  __syncthreads();
+  if (split > 1) cluster_sync_all();   // no CTA leaves while a peer may still read its partial
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem_base, p.tmem_cols);
+  }
+}
+
 }  // namespace
 
 int gemm_read_status() {
@@ -584,6 +754,99 @@ int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withh
   return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
+struct SplitConfig {
+  int nt;       // tokens per tile
+  int split;    // CTAs of a cluster along K
+  int stages;
+};
+
+constexpr int SPLIT_MAX_ROWS = 128;
+constexpr int SPLIT_MAX_PROB = 32;
+
+// Both operands K-major, one segment: the shape of every forward projection.
+bool split_applies(const GemmProblem* probs, int n) {
+  for (int i = 0; i < n; ++i)
+    if (probs[i].M > SPLIT_MAX_ROWS || probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
+  return n > 0;
+}
+
+// The smallest split that gives 128 CTAs: enough of them to draw the full memory bandwidth, and no partial more than
+// that needs (at N = K = 4096 and 16 tokens a split of 2 / 4 / 8 measured 12.3 / 11.6 / 10.8 us, at 64 tokens and 4 / 8
+// it measured 12.5 / 14.3).  One CTA per SM takes a ring as deep as fits; more CTAs than SMs share them in twos.
+SplitConfig split_config(const GemmProblem* probs, int n) {
+  int rows = 0, tiles = 0, kblocks = 1 << 30;
+  for (int i = 0; i < n; ++i) {
+    rows = std::max(rows, probs[i].M);
+    tiles += (probs[i].N + SROWS - 1) / SROWS;
+    kblocks = std::min(kblocks, (probs[i].segs[0].K + BK - 1) / BK);
+  }
+  SplitConfig c;
+  c.nt = (rows + 15) / 16 * 16;
+  c.split = 1;
+  while (c.split < 8 && 2 * c.split <= kblocks && tiles * c.split < 128) c.split *= 2;
+  const int ring_bytes = (tiles * c.split <= sm_count() ? 220 : 110) * 1024;
+  c.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SB_BYTES + c.nt * BK * 2));
+  return c;
+}
+
+template <int NP>
+int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaStream_t stream) {
+  SplitParams<NP> p;
+  int tiles = 0;
+  for (int i = 0; i < n; ++i) {
+    const GemmProblem& g = probs[i];
+    SplitProblem& q = p.prob[i];
+    q.M = g.M;
+    q.N = g.N;
+    q.tok_tiles = (g.M + cfg.nt - 1) / cfg.nt;
+    tiles += q.tok_tiles * ((g.N + SROWS - 1) / SROWS);
+    q.tile_end = tiles;
+    q.kblocks = (g.segs[0].K + BK - 1) / BK;
+    q.out_f32 = g.out_f32;
+    q.ldc = g.ldc;
+    q.c = g.c;
+    const GemmSeg& e = g.segs[0];
+    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.M)}, strides[1] = {uint64_t(e.lda) * 2};
+    uint32_t box[2] = {BK, uint32_t(cfg.nt)};
+    int rc = make_tensor_map(&p.map_a[i], e.a, 2, 2, dims, strides, box, true);
+    if (rc != KVP_OK) return rc;
+    dims[1] = uint64_t(g.N);
+    strides[0] = uint64_t(e.ldb) * 2;
+    box[1] = SROWS;
+    rc = make_tensor_map(&p.map_b[i], e.b, 2, 2, dims, strides, box, true);
+    if (rc != KVP_OK) return rc;
+  }
+  p.nt = cfg.nt;
+  p.stages = cfg.stages;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < cfg.nt) p.tmem_cols *= 2;
+  p.idesc = umma_idesc_bf16(SROWS, cfg.nt, 0, 0);
+  // Tensor memory is shared out in proportion to shared memory, so that the CTAs that fit on an SM by the latter never
+  // wait for the former (a CTA of a cluster that waited could hold up a peer that another kernel's CTA waits for); 40 KB
+  // keep it off the SMs of the kernels that take all 512 columns.
+  const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
+  const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 456));
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(gemm_split_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  if (attr != cudaSuccess) return KVP_ERR_CUDA;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cfg.split;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(tiles * cfg.split);
+  lc.blockDim = dim3(SPLIT_THREADS);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  timing_before(KVP_KERNEL_GEMM, stream);
+  const cudaError_t e = cudaLaunchKernelEx(&lc, gemm_split_kernel<NP>, p);
+  timing_after(KVP_KERNEL_GEMM, stream);
+  note_launch();
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+}
+
 // 0: single-CTA tiles only; 1: CTA pairs where the caller prefers them (forward GEMMs); 2: CTA pairs everywhere.
 // Pairs are never used for a group with a problem of at most 128 rows (half of every pair tile would be padding).
 int g_pair_mode = 1;
@@ -600,12 +863,25 @@ bool use_pair(const GemmProblem* probs, int n, bool prefer_pair) {
 void gemm_set_pair_mode(int mode) { g_pair_mode = mode; }
 int gemm_pair_mode() { return g_pair_mode; }
 
+static int gemm_split(const GemmProblem* probs, int n, cudaStream_t stream) {
+  for (int begin = 0; begin < n; begin += SPLIT_MAX_PROB) {
+    const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
+    const SplitConfig cfg = split_config(probs + begin, cnt);
+    const int rc = cnt == 1   ? launch_split<1>(probs + begin, cnt, cfg, stream)
+                   : cnt <= 4 ? launch_split<4>(probs + begin, cnt, cfg, stream)
+                              : launch_split<SPLIT_MAX_PROB>(probs + begin, cnt, cfg, stream);
+    if (rc != KVP_OK) return rc;
+  }
+  return KVP_OK;
+}
+
 int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool prefer_pair) {
   if (n < 0 || (n > 0 && probs == nullptr)) return KVP_ERR_INVALID_ARG;
   for (int i = 0; i < n; ++i) {
     const int rc = check_problem(probs[i]);
     if (rc != KVP_OK) return rc;
   }
+  if (split_applies(probs, n)) return gemm_split(probs, n, stream);
   // as many problems per launch as the parameter block holds
   int begin = 0;
   while (begin < n) {
@@ -633,6 +909,7 @@ int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, v
   g.out_f32 = out_f32;
   const int rc = check_problem(g);
   if (rc != KVP_OK) return rc;
+  if (withhold_at == 0 && split_applies(&g, 1)) return gemm_split(&g, 1, stream);
   return launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1, prefer_pair));
 }
 

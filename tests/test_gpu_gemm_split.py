@@ -1,0 +1,54 @@
+"""GEMMs with at most 128 rows of A (decode-step projections): operands swapped, K split over a cluster of CTAs."""
+import pytest
+import torch
+
+from guard import Guarded
+from paper_2608_15943_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (1, 8, 8),            # less than one tile and one k-block: split 1
+    (16, 128, 64), (17, 136, 72),          # edges of the token tile, the column tile and the k-block
+    (31, 264, 1032),      # split 8, 17 k-blocks dealt unevenly
+    (128, 4096, 520),     # widest token tile; 32 column tiles: split 4
+    (40, 19208, 200),     # more CTAs than SMs: two per SM, shallow ring, split 1
+])
+def test_few_rows(M, N, K):
+    from paper_2608_15943_b200 import kvp
+    a = synth.normal((M, K), 31, 1, 1.0, "cuda")
+    b = synth.normal((N, K), 31, 2, 1.0, "cuda")
+    ref = a.double() @ b.double().T
+    gd = Guarded()
+    c32 = gd.empty((M, N), torch.float32, float("nan"))
+    c16 = gd.empty((M, N), torch.bfloat16, float("nan"))
+    kvp.gemm(a, b, c32)
+    kvp.gemm(a, b, c16)
+    gd.check()
+    assert kvp.device_status() == kvp.OK
+    # fp32 accumulation of K products of bf16 values (each product exact): |error| <= K 2^-24 sum|a b|, of which the
+    # average case is far below; bf16 storage (8 significant bits) adds half an ulp, at most 2^-8 of the value
+    bound = K * 2.0 ** -24 * (a.double().abs() @ b.double().abs().T) + 1e-30
+    assert ((c32.double() - ref).abs() <= bound).all()
+    assert ((c16.double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all()
+
+
+def test_few_rows_grouped_projections():
+    """Q, K and V projections of twelve layers with one token per sequence: 20 problems in one launch, two widths."""
+    from paper_2608_15943_b200 import kvp
+    L, B, D, Hq, Hkv, dh = 12, 5, 256, 4, 2, 64
+    donor = [0, 1, 2, 3, 3, 3, 3, 3, 3, 3, 3, 3]
+    sh = kvp.Shape(L, B, 1, D, Hq, Hkv, dh)
+    x = [synth.normal((B, D), 32, synth.tid(0, l), 1.0, "cuda") for l in range(L)]
+    w = {n: [synth.normal((h * dh, D), 32, synth.tid(i, l), 0.02, "cuda") for l in range(L)]
+         for i, (n, h) in enumerate((("q", Hq), ("k", Hkv), ("v", Hkv)), 1)}
+    gd = Guarded()
+    out = {n: [gd.empty((B, 1, h, dh), torch.bfloat16, float("nan")) for _ in range(L)] for n, h in (("q", Hq), ("k", Hkv), ("v", Hkv))}
+    kvp.proj_fwd(sh, donor, x, w["q"], w["k"], w["v"], out["q"], out["k"], out["v"])
+    gd.check()
+    for l in range(L):
+        for n in ("q", "k", "v") if donor[l] == l else ("q",):
+            ref = x[l].double() @ w[n][l].double().T
+            got = out[n][l].view(B, -1).double()
+            assert ((got - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4).all(), (n, l)   # bf16 storage; 256 terms of size 0.02
