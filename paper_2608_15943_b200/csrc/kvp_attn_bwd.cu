@@ -219,6 +219,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dep_launch();
+  grid_dep_wait();
   const uint32_t tm_dp = tmem_base + 128;
   const uint32_t tm_dq = tmem_base + 192;
   const uint32_t tm_dk = tmem_base + 256;
@@ -578,6 +580,8 @@ template <int DH>
 __global__ void dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int B, int S, int Hq,
                                   float scale) {
   constexpr int TPR = DH / 8;  // threads per query row
+  grid_dep_launch();
+  grid_dep_wait();
   const int n_qt = (S + BQ2 - 1) / BQ2;
   const size_t rows = size_t(B) * Hq * n_qt * BQ2;
   const size_t stride = size_t(gridDim.x) * blockDim.x / TPR;
@@ -612,6 +616,8 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfl
                              float* __restrict__ delta, int B, int S, int Hq) {
   constexpr int LANES = DH / 8;          // lanes per row
   constexpr int ROWS = 32 / LANES;       // rows per warp and load
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t rows = size_t(B) * S * Hq;
   const int lane = threadIdx.x & 31;
   const int sub = lane / LANES, piece = lane % LANES;
@@ -715,18 +721,12 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     float* dl = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
     const size_t rows = size_t(s->B) * s->S * s->Hq;
     const int blocks = int(min(size_t(sm_count()) * 16, (rows + 7) / 8));
-    if (dh == 128)
-      delta_kernel<128><<<blocks, 256, 0, stream>>>(reinterpret_cast<const __nv_bfloat16*>(o[l]),
-                                                    reinterpret_cast<const __nv_bfloat16*>(d_o[l]), dl, s->B, s->S,
-                                                    s->Hq);
-    else
-      delta_kernel<64><<<blocks, 256, 0, stream>>>(reinterpret_cast<const __nv_bfloat16*>(o[l]),
-                                                   reinterpret_cast<const __nv_bfloat16*>(d_o[l]), dl, s->B, s->S,
-                                                   s->Hq);
-    note_launch();
+    const cudaError_t e = launch_kernel(dh == 128 ? delta_kernel<128> : delta_kernel<64>, blocks, 256, 0, stream, 1,
+                                        reinterpret_cast<const __nv_bfloat16*>(o[l]),
+                                        reinterpret_cast<const __nv_bfloat16*>(d_o[l]), dl, s->B, s->S, s->Hq);
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
-  if (cudaGetLastError() != cudaSuccess) return KVP_ERR_CUDA;
 
   // Donor groups, largest first; a launch takes groups until it holds MAX_GROUP member layers.  A launch writes
   // dK / dV of its donors through reductions into cleared buffers, so a donor shared by more than MAX_GROUP
@@ -820,27 +820,20 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     dim3 grid(p.cta_begin[ng]);
     timing_before(KVP_KERNEL_ATTN_BWD, stream);
-    if (dh == 128)
-      bwd_kernel<128><<<grid, BWD_THREADS, BwdSmem<128>::TOTAL, stream>>>(p);
-    else
-      bwd_kernel<64><<<grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream>>>(p);
+    const cudaError_t e = dh == 128 ? launch_kernel(bwd_kernel<128>, grid, BWD_THREADS, BwdSmem<128>::TOTAL, stream, 1, p)
+                                    : launch_kernel(bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream, 1, p);
     timing_after(KVP_KERNEL_ATTN_BWD, stream);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return KVP_ERR_CUDA;
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
     for (int i = 0; i < slots; ++i) {
       const size_t threads = dq_acc_floats(s->B, s->S, s->Hq, dh) / 8;
       const int blocks = int(min(size_t(sm_count()) * 16, (threads + 255) / 256));
-      if (dh == 128)
-        dq_convert_kernel<128><<<blocks, 256, 0, stream>>>(p.dq_acc[i], reinterpret_cast<__nv_bfloat16*>(dq[slot_layer[i]]),
-                                                           s->B, s->S, s->Hq, sc);
-      else
-        dq_convert_kernel<64><<<blocks, 256, 0, stream>>>(p.dq_acc[i], reinterpret_cast<__nv_bfloat16*>(dq[slot_layer[i]]),
-                                                          s->B, s->S, s->Hq, sc);
-      note_launch();
+      const cudaError_t ec = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, blocks, 256, 0, stream, 1,
+                                           p.dq_acc[i], reinterpret_cast<__nv_bfloat16*>(dq[slot_layer[i]]), s->B, s->S,
+                                           s->Hq, sc);
+      if (ec != cudaSuccess) return KVP_ERR_CUDA;
     }
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    if (cudaGetLastError() != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;
 }

@@ -159,6 +159,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dep_launch();
+  grid_dep_wait();
   // tile X: score buffer u at [X*128 + u*64, +64) with P over its first 32 columns; output accumulator at
   // [256 + X*128, +128)
   //
@@ -496,16 +498,11 @@ int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* con
       cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::TOTAL);
   if (attr128 != cudaSuccess || attr64 != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_ATTN_FWD, stream);
-  if (s->dh == 128) {
-    attn_fwd_kernel<128><<<grid, FWD_THREADS, FwdSmem<128>::TOTAL, stream>>>(p);
-  } else if (s->dh == 64) {
-    attn_fwd_kernel<64><<<grid, FWD_THREADS, FwdSmem<64>::TOTAL, stream>>>(p);
-  } else {
-    return KVP_ERR_UNSUPPORTED;
-  }
+  const cudaError_t e =
+      s->dh == 128 ? launch_kernel(attn_fwd_kernel<128>, grid, FWD_THREADS, FwdSmem<128>::TOTAL, stream, 1, p)
+                   : launch_kernel(attn_fwd_kernel<64>, grid, FWD_THREADS, FwdSmem<64>::TOTAL, stream, 1, p);
   timing_after(KVP_KERNEL_ATTN_FWD, stream);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
 int attn_fwd_max_layers() { return FWD_MAX_LAYERS; }

@@ -111,6 +111,8 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) decode_kernel(const __grid_con
   const DecGroup& grp = p.grp[gi];
   const int G = p.Hq / p.Hkv;
   const int R = grp.n_members * G;  // valid query rows (<= 16)
+  grid_dep_launch();
+  grid_dep_wait();
 
   int len = p.lengths[b];
   const int cap = p.max_pages * p.page_size;
@@ -338,6 +340,8 @@ __global__ void decode_combine_kernel(const __grid_constant__ DecParams p) {
   const DecGroup& grp = p.grp[gi];
   const int G = p.Hq / p.Hkv;
   const int R = grp.n_members * G;
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t unit0 = ((size_t(gi) * p.B + b) * p.Hkv + hk) * p.num_splits;
   for (int idx = threadIdx.x; idx < R * DH; idx += blockDim.x) {
     const int row = idx / DH, col = idx % DH;
@@ -374,6 +378,8 @@ struct AppendParams {
 __global__ void append_kernel(const __grid_constant__ AppendParams p) {
   const int layer = blockIdx.y;
   const int b = blockIdx.x;
+  grid_dep_launch();
+  grid_dep_wait();
   int len = p.lengths[b];
   const int cap = p.max_pages * p.page_size;
   if (len < 1 || len > cap) return;  // nothing sensible to write; decode flags the bad length
@@ -520,9 +526,7 @@ extern "C" int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, 
       ++n;
     }
     if (n == MAX_DEC_GROUPS || (l == d->L && n > 0)) {
-      append_kernel<<<dim3(d->B, n), 128, 0, stream>>>(p);
-      note_launch();
-      if (cudaGetLastError() != cudaSuccess) return KVP_ERR_CUDA;
+      if (launch_kernel(append_kernel, dim3(d->B, n), 128, 0, stream, 1, p) != cudaSuccess) return KVP_ERR_CUDA;
       n = 0;
     }
   }
@@ -596,17 +600,11 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
     dim3 grid(ns, d->B * d->Hkv, n);
     dim3 cgrid(1, d->B * d->Hkv, n);
     timing_before(KVP_KERNEL_DECODE, stream);
-    if (d->dh == 128)
-      decode_kernel<128><<<grid, DEC_THREADS, smem, stream>>>(p);
-    else
-      decode_kernel<64><<<grid, DEC_THREADS, smem, stream>>>(p);
+    cudaError_t e = launch_kernel(d->dh == 128 ? decode_kernel<128> : decode_kernel<64>, grid, DEC_THREADS, smem, stream, 1, p);
     timing_after(KVP_KERNEL_DECODE, stream);
-    if (d->dh == 128)
-      decode_combine_kernel<128><<<cgrid, 128, 0, stream>>>(p);
-    else
-      decode_combine_kernel<64><<<cgrid, 128, 0, stream>>>(p);
-    note_launch(2);
-    if (cudaGetLastError() != cudaSuccess) return KVP_ERR_CUDA;
+    if (e == cudaSuccess)
+      e = launch_kernel(d->dh == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, cgrid, 128, 0, stream, 1, p);
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;
 }

@@ -74,6 +74,37 @@ enum {
   KVP_KERNEL_COUNT = 5
 };
 void note_launch(int n = 1);
+
+template <typename T>
+struct SameType { using type = T; };   // keeps the argument types of launch_kernel out of template deduction
+
+// Every kernel of the library is launched through this: programmatic stream serialisation lets its CTAs come up (barriers,
+// tensor-memory allocation, descriptor fetches) while the kernel before it on the stream drains.  The kernel must
+// execute grid_dep_wait() before it touches global memory, and grid_dep_launch() once its own CTAs hold what they
+// need, so that the next kernel may do the same.  cluster > 1 sets a runtime cluster size.  Device time of a pass
+// (graph replay), plain launches -> these: tiny fp32 training step 155 -> 125 us (79 kernels), token step of a
+// four-layer stage 631 -> 595 us (56 kernels), decode step of the tiny stack 11.3 -> 10.3 us (3 kernels).
+template <typename... KP>
+cudaError_t launch_kernel(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,
+                          const typename SameType<KP>::type&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = unsigned(cluster);
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = block;
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  lc.attrs = at;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
+  void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  note_launch();
+  return cudaLaunchKernelExC(&lc, reinterpret_cast<const void*>(kernel), ptrs);
+}
+
 void timing_before(int kernel, cudaStream_t stream);
 void timing_after(int kernel, cudaStream_t stream);
 

@@ -7,6 +7,8 @@ namespace kvp {
 namespace {
 
 __global__ void cast_f32_bf16_kernel(const float4* __restrict__ src, uint2* __restrict__ dst, size_t n4) {
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride) {
     const float4 v = src[i];
@@ -15,6 +17,8 @@ __global__ void cast_f32_bf16_kernel(const float4* __restrict__ src, uint2* __re
 }
 
 __global__ void cast_bf16_f32_kernel(const uint2* __restrict__ src, float4* __restrict__ dst, size_t n4) {
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride) {
     const uint2 v = src[i];
@@ -30,9 +34,8 @@ int cast_bf16_to_f32(const void* src, float* dst, size_t n, cudaStream_t stream)
   const size_t n4 = n / 4;
   const int threads = 256;
   const int blocks = int(min(size_t(sm_count()) * 8, (n4 + threads - 1) / threads));
-  cast_bf16_f32_kernel<<<blocks, threads, 0, stream>>>(reinterpret_cast<const uint2*>(src), reinterpret_cast<float4*>(dst), n4);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  const cudaError_t e = launch_kernel(cast_bf16_f32_kernel, blocks, threads, 0, stream, 1, reinterpret_cast<const uint2*>(src), reinterpret_cast<float4*>(dst), n4);
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
 // n must be a multiple of 4 (it is a multiple of the head dimension).
@@ -41,10 +44,9 @@ int cast_f32_to_bf16(const float* src, void* dst, size_t n, cudaStream_t stream)
   const size_t n4 = n / 4;
   const int threads = 256;
   const int blocks = int(min(size_t(sm_count()) * 8, (n4 + threads - 1) / threads));
-  cast_f32_bf16_kernel<<<blocks, threads, 0, stream>>>(reinterpret_cast<const float4*>(src),
+  const cudaError_t e = launch_kernel(cast_f32_bf16_kernel, blocks, threads, 0, stream, 1, reinterpret_cast<const float4*>(src),
                                                        reinterpret_cast<uint2*>(dst), n4);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
 }  // namespace kvp

@@ -24,6 +24,13 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
+// Programmatic dependent launch.  Between the two calls a kernel may only set up its own CTA (shared memory, barriers,
+// tensor memory, kernel parameters, prefetches): after grid_dep_wait() everything the kernels before it on the stream
+// wrote is visible, and everything they read may be overwritten.  EVERY thread block executes grid_dep_wait(), so that
+// the completion of a kernel implies the completion of all kernels before it.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ----------------------------------------------------------------------------------------
 // mbarrier
 // ----------------------------------------------------------------------------------------
@@ -122,6 +129,17 @@ __device__ __forceinline__ void tma_load_2d_e(void* dst, const CUtensorMap* map,
       " @q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n"
       "}\n" ::"r"(smem_u32(dst)),
       "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(leader)
+      : "memory");
+}
+// the tile of a later tma_load_2d_e, requested into L2 only
+__device__ __forceinline__ void tma_prefetch_2d_e(const CUtensorMap* map, int x, int y, uint32_t leader) {
+  asm volatile(
+      "{\n"
+      " .reg .pred q;\n"
+      " setp.ne.b32 q, %3, 0;\n"
+      " @q cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];\n"
+      "}\n" ::"l"(map),
+      "r"(x), "r"(y), "r"(leader)
       : "memory");
 }
 __device__ __forceinline__ void tma_load_4d_e(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z, int w,

@@ -32,6 +32,8 @@ constexpr int kMaxChunks = 4;  // D <= 8192
 __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
                                                                uint4* __restrict__ y, int T, int D8, float inv_d, float eps) {
   __shared__ float part[kNormThreads / 32];
+  grid_dep_launch();
+  grid_dep_wait();
   auto load_row = [&](int row, uint4 (&v)[kMaxChunks]) {
     const uint4* xr = x + size_t(row) * D8;
 #pragma unroll
@@ -100,8 +102,10 @@ __global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, 
   // lanes of a warp need different table entries: shared memory serves them in one pass, the constant bank
   // that holds kernel parameters would replay once per distinct address
   __shared__ float2 freq[kMaxRopePairs];
+  grid_dep_launch();
   for (int k = threadIdx.x; k < kMaxRopePairs; k += blockDim.x) freq[k] = fr.f[k];
   __syncthreads();
+  grid_dep_wait();
   const uint32_t stride = gridDim.x * blockDim.x;
   const uint32_t per_tok = H * dh8;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_work; i += stride) {  // 32-bit index arithmetic only
@@ -152,6 +156,8 @@ __global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, 
 
 // out = silu(gate) * up
 __global__ void swiglu_kernel(const uint4* __restrict__ gate, const uint4* __restrict__ up, uint4* __restrict__ out, size_t n8) {
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n8; i += stride) {
     float g[8], u[8];
@@ -164,6 +170,8 @@ __global__ void swiglu_kernel(const uint4* __restrict__ gate, const uint4* __res
 }
 
 __global__ void add_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b, uint4* __restrict__ out, size_t n8) {
+  grid_dep_launch();
+  grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n8; i += stride) {
     float f[8], g[8];
@@ -188,10 +196,9 @@ extern "C" int kvp_rmsnorm(int32_t T, int32_t D, const void* x, const void* w, f
   if (D % 8 != 0 || D > 8 * kNormThreads * kMaxChunks || !is_aligned16(x) || !is_aligned16(w) || !is_aligned16(y)) return KVP_ERR_UNSUPPORTED;
   if (T == 0) return KVP_OK;
   const int blocks = min(T, sm_count() * 8);
-  rmsnorm_kernel<<<blocks, kNormThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+  const cudaError_t e = launch_kernel(rmsnorm_kernel, blocks, kNormThreads, 0, reinterpret_cast<cudaStream_t>(stream), 1,
       reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), reinterpret_cast<uint4*>(y), T, D / 8, 1.f / float(D), eps);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
 extern "C" int kvp_rope(int32_t B, int32_t S, int32_t H, int32_t dh, float theta, int32_t pos0, void* x, kvp_stream_t stream) {
@@ -211,29 +218,27 @@ extern "C" int kvp_rope(int32_t B, int32_t S, int32_t H, int32_t dh, float theta
   const int seqs_per_launch = int(std::max<size_t>(1, ((size_t(1) << 31) - 1) / per_seq));
   for (int b0 = 0; b0 < B; b0 += seqs_per_launch) {
     const uint32_t n_work = uint32_t(size_t(std::min(seqs_per_launch, B - b0)) * S * (dh / 8));   // (token, 8-element slice)
-    rope_kernel<<<streaming_blocks(n_work, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+    const cudaError_t e = launch_kernel(rope_kernel, streaming_blocks(n_work, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream), 1,
         reinterpret_cast<uint4*>(x) + size_t(b0) * per_seq, n_work, uint32_t(S), uint32_t(H), uint32_t(dh / 8), pos0, fr);
-    note_launch();
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return KVP_OK;
 }
 
 extern "C" int kvp_swiglu(int64_t n, const void* gate, const void* up, void* out, kvp_stream_t stream) {
   if (n < 0 || gate == nullptr || up == nullptr || out == nullptr) return KVP_ERR_INVALID_ARG;
   if (n % 8 != 0 || !is_aligned16(gate) || !is_aligned16(up) || !is_aligned16(out)) return KVP_ERR_UNSUPPORTED;
   if (n == 0) return KVP_OK;
-  swiglu_kernel<<<streaming_blocks(size_t(n / 8), 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+  const cudaError_t e = launch_kernel(swiglu_kernel, streaming_blocks(size_t(n / 8), 256), 256, 0, reinterpret_cast<cudaStream_t>(stream), 1,
       reinterpret_cast<const uint4*>(gate), reinterpret_cast<const uint4*>(up), reinterpret_cast<uint4*>(out), size_t(n / 8));
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
 extern "C" int kvp_add(int64_t n, const void* a, const void* b, void* out, kvp_stream_t stream) {
   if (n < 0 || a == nullptr || b == nullptr || out == nullptr) return KVP_ERR_INVALID_ARG;
   if (n % 8 != 0 || !is_aligned16(a) || !is_aligned16(b) || !is_aligned16(out)) return KVP_ERR_UNSUPPORTED;
   if (n == 0) return KVP_OK;
-  add_kernel<<<streaming_blocks(size_t(n / 8), 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+  const cudaError_t e = launch_kernel(add_kernel, streaming_blocks(size_t(n / 8), 256), 256, 0, reinterpret_cast<cudaStream_t>(stream), 1,
       reinterpret_cast<const uint4*>(a), reinterpret_cast<const uint4*>(b), reinterpret_cast<uint4*>(out), size_t(n / 8));
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
