@@ -708,12 +708,8 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   const size_t acc_bytes = align256(dq_acc_floats(s->B, s->S, s->Hq, dh) * 4);
   uint8_t* wsb = reinterpret_cast<uint8_t*>(ws);
   uint8_t* acc_base = wsb + size_t(s->L) * delta_bytes;
-  static const cudaError_t attr = [] {
-    cudaError_t e = cudaFuncSetAttribute(bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<128>::TOTAL);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<64>::TOTAL);
-  }();
-  if (attr != cudaSuccess) return KVP_ERR_CUDA;
+  if ((dh == 128 ? allow_smem<bwd_kernel<128>>(BwdSmem<128>::TOTAL) : allow_smem<bwd_kernel<64>>(BwdSmem<64>::TOTAL)) != cudaSuccess)
+    return KVP_ERR_CUDA;
 
   // Delta for every layer
   timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);

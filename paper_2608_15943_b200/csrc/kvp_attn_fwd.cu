@@ -492,11 +492,9 @@ int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* con
   if (n_items > 0x7fffffffLL) return KVP_ERR_UNSUPPORTED;
   // persistent: one CTA per SM walks a list of (layer, b, hq, tile pair) items
   const int grid = int(n_items < (long long)sm_count() ? n_items : (long long)sm_count());
-  static const cudaError_t attr128 =
-      cudaFuncSetAttribute(attn_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::TOTAL);
-  static const cudaError_t attr64 =
-      cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::TOTAL);
-  if (attr128 != cudaSuccess || attr64 != cudaSuccess) return KVP_ERR_CUDA;
+  if ((s->dh == 128 ? allow_smem<attn_fwd_kernel<128>>(FwdSmem<128>::TOTAL)
+                    : allow_smem<attn_fwd_kernel<64>>(FwdSmem<64>::TOTAL)) != cudaSuccess)
+    return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_ATTN_FWD, stream);
   const cudaError_t e =
       s->dh == 128 ? launch_kernel(attn_fwd_kernel<128>, grid, FWD_THREADS, FwdSmem<128>::TOTAL, stream, 1, p)

@@ -572,12 +572,7 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
   p.scale_log2 = sc * 1.4426950408889634f;
 
   const int smem = DEC_WARPS * DEC_STAGES * 2 * GRAN * d->dh * 2;
-  cudaError_t e;
-  if (d->dh == 128)
-    e = cudaFuncSetAttribute(decode_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  else
-    e = cudaFuncSetAttribute(decode_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return KVP_ERR_CUDA;
+  if ((d->dh == 128 ? allow_smem<decode_kernel<128>>(smem) : allow_smem<decode_kernel<64>>(smem)) != cudaSuccess) return KVP_ERR_CUDA;
 
   for (int s0 = 0; s0 < n_sub; s0 += MAX_DEC_GROUPS) {
     const int n = n_sub - s0 < MAX_DEC_GROUPS ? n_sub - s0 : MAX_DEC_GROUPS;

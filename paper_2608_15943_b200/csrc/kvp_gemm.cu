@@ -753,11 +753,7 @@ int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withh
   }
   for (int i = n; i < MAX_PROB; ++i) p.prob[i] = p.prob[n - 1];
   p.total_tiles = tiles;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GEMM_SMEM));
-  static const cudaError_t attr_pair =
-      cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PAIR_SMEM));
-  if (attr != cudaSuccess || attr_pair != cudaSuccess) return KVP_ERR_CUDA;
+  if ((pair ? allow_smem<gemm_pair_kernel>(int(PAIR_SMEM)) : allow_smem<gemm_kernel>(int(GEMM_SMEM))) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e =
       pair ? launch_kernel(gemm_pair_kernel, 2 * min(tiles, sm_count() / 2), GEMM_THREADS, PAIR_SMEM, stream, 1, p)
@@ -838,9 +834,7 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // keep it off the SMs of the kernels that take all 512 columns.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 456));
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(gemm_split_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-  if (attr != cudaSuccess) return KVP_ERR_CUDA;
+  if (allow_smem<gemm_split_kernel<NP>>(226 * 1024) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e = launch_kernel(gemm_split_kernel<NP>, tiles * cfg.split, SPLIT_THREADS, smem, stream, cfg.split, p);
   timing_after(KVP_KERNEL_GEMM, stream);

@@ -57,26 +57,33 @@ def device_status() -> int:
     return int(lib.kvp_device_status())
 
 
-def _stream() -> C.c_void_p:
+# torch's stream object is built anew for every look at it (4.4 us a call, half of what a small operator's whole call
+# took); its handle alone takes 0.3 us where this torch offers it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream() -> int:
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
     # Without a device the entry points still validate their arguments (and fail before any launch).
     if not torch.cuda.is_available():
-        return C.c_void_p(0)
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return 0
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: Optional[torch.Tensor]) -> int:
     return 0 if t is None else t.data_ptr()
 
 
+_void_p, _int32 = C.c_void_p, C.c_int32
+
+
 def _ptr_array(ts: Sequence[Optional[torch.Tensor]]):
-    arr = (C.c_void_p * len(ts))()
-    for i, t in enumerate(ts):
-        arr[i] = _ptr(t)
-    return arr
+    return (_void_p * len(ts))(*[None if t is None else t.data_ptr() for t in ts])
 
 
 def _i32_array(xs: Sequence[int]):
-    return (C.c_int32 * len(xs))(*[int(x) for x in xs])
+    return (_int32 * len(xs))(*map(int, xs))
 
 
 def _u64_array(xs: Sequence[int]):
