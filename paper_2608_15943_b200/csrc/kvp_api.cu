@@ -14,8 +14,6 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
                  const float* const* lse, void* const* dq, float* const* dk_sum, float* const* dv_sum, void* ws,
                  size_t ws_bytes, cudaStream_t stream);
-int cast_f32_to_bf16(const float* src, void* dst, size_t n, cudaStream_t stream);
-int cast_bf16_to_f32(const void* src, float* dst, size_t n, cudaStream_t stream);
 
 namespace {
 
@@ -69,33 +67,24 @@ class Shadows {
  public:
   Shadows(const kvp_shape* s, const int32_t* donor, void* ws, size_t offset, cudaStream_t stream)
       : s_(s), donor_(donor), cur_(reinterpret_cast<uint8_t*>(ws) + offset), stream_(stream) {}
-  // bf16 copies of an fp32 input array
+  // bf16 copies of an fp32 input array, filled by round_inputs()
   const void* const* in(const void* const* src, const TensorSet& t) {
     std::vector<void*>& arr = reserve(t);
     for (int l = 0; l < s_->L; ++l)
-      if (arr[l] != nullptr && rc_ == KVP_OK) rc_ = cast_f32_to_bf16(reinterpret_cast<const float*>(src[l]), arr[l], t.elems, stream_);
+      if (arr[l] != nullptr) inputs_.push_back(CastItem{src[l], arr[l], t.elems});
     return reinterpret_cast<const void* const*>(arr.data());
   }
   // bf16 buffers standing in for an fp32 output array; finish() widens them into the caller's tensors
   void* const* out(void* const* dst, const TensorSet& t) {
     std::vector<void*>& arr = reserve(t);
     for (int l = 0; l < s_->L; ++l)
-      if (arr[l] != nullptr) pending_.push_back(Pending{arr[l], reinterpret_cast<float*>(dst[l]), t.elems});
+      if (arr[l] != nullptr) outputs_.push_back(CastItem{arr[l], dst[l], t.elems});
     return arr.data();
   }
-  int status() const { return rc_; }
-  int finish() {
-    for (const Pending& p : pending_)
-      if (rc_ == KVP_OK) rc_ = cast_bf16_to_f32(p.src, p.dst, p.elems, stream_);
-    return rc_;
-  }
+  int round_inputs() { return cast_tensors(inputs_.data(), int(inputs_.size()), false, stream_); }
+  int finish() { return cast_tensors(outputs_.data(), int(outputs_.size()), true, stream_); }
 
  private:
-  struct Pending {
-    const void* src;
-    float* dst;
-    size_t elems;
-  };
   std::vector<void*>& reserve(const TensorSet& t) {
     arrays_.emplace_back(size_t(s_->L), nullptr);
     std::vector<void*>& arr = arrays_.back();
@@ -110,9 +99,8 @@ class Shadows {
   const int32_t* donor_;
   uint8_t* cur_;
   cudaStream_t stream_;
-  int rc_ = KVP_OK;
   std::vector<std::vector<void*>> arrays_;
-  std::vector<Pending> pending_;
+  std::vector<CastItem> inputs_, outputs_;
 };
 
 struct Sizes {
@@ -213,7 +201,8 @@ extern "C" int kvp_proj_fwd(const kvp_shape* s, const int32_t* donor, const void
     void* const* q16 = sh.out(q, z.q);
     void* const* k16 = sh.out(k, z.kv);
     void* const* v16 = sh.out(v, z.kv);
-    if (sh.status() != KVP_OK) return sh.status();
+    rc = sh.round_inputs();
+    if (rc != KVP_OK) return rc;
     kvp_shape s16 = *s;
     s16.dtype = KVP_BF16;
     rc = kvp_proj_fwd(&s16, donor, x16, wq16, wk16, wv16, q16, k16, v16, ws, ws_bytes, stream_);
@@ -270,7 +259,8 @@ extern "C" int kvp_proj_bwd_range(const kvp_shape* s, const int32_t* donor, cons
     const void* const* wv16 = sh.in(wv, z.wkv);
     const void* const* dq16 = sh.in(dq, z.q);
     void* const* dx16 = sh.out(dx, z.x);
-    if (sh.status() != KVP_OK) return sh.status();
+    rc = sh.round_inputs();
+    if (rc != KVP_OK) return rc;
     kvp_shape s16 = *s;
     s16.dtype = KVP_BF16;
     if (layer_begin != 0 || layer_end != s->L) return KVP_ERR_UNSUPPORTED;   // the fp32 interface converts whole arrays
@@ -290,16 +280,18 @@ extern "C" int kvp_proj_bwd_range(const kvp_shape* s, const int32_t* donor, cons
     const int c1 = std::min(layer_end, c0 + kProjBwdChunk);
     probs.clear();
     std::vector<uint8_t*> dk_bf(size_t(c1 - c0), nullptr), dv_bf(size_t(c1 - c0), nullptr);
+    std::vector<CastItem> sums;
     int owners = 0;
     for (int l = c0; l < c1; ++l) {
       if (donor[l] != l) continue;
       dk_bf[l - c0] = bf + size_t(2 * owners) * slot;
       dv_bf[l - c0] = bf + size_t(2 * owners + 1) * slot;
       ++owners;
-      rc = cast_f32_to_bf16(dk_sum[l], dk_bf[l - c0], n_kv, stream);
-      if (rc == KVP_OK) rc = cast_f32_to_bf16(dv_sum[l], dv_bf[l - c0], n_kv, stream);
-      if (rc != KVP_OK) return rc;
+      sums.push_back(CastItem{dk_sum[l], dk_bf[l - c0], n_kv});
+      sums.push_back(CastItem{dv_sum[l], dv_bf[l - c0], n_kv});
     }
+    rc = cast_tensors(sums.data(), int(sums.size()), false, stream);
+    if (rc != KVP_OK) return rc;
     // dWq = dQ^T X : A = dQ stored [T, Nq] (MN-major for M = Nq), B = X stored [T, D] (MN-major for N = D)
     for (int l = c0; l < c1; ++l) probs.push_back(problem(Nq, D, {dq[l], x[l], Nq, D, T}, 1, 1, dwq[l], D, 1));
     for (int l = c0; l < c1; ++l) {
@@ -377,7 +369,8 @@ extern "C" int kvp_attn_fwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* k16 = sh.in(k, z.kv);
     const void* const* v16 = sh.in(v, z.kv);
     void* const* o16 = sh.out(o, z.q);
-    if (sh.status() != KVP_OK) return sh.status();
+    rc = sh.round_inputs();
+    if (rc != KVP_OK) return rc;
     kvp_shape s16 = *s;
     s16.dtype = KVP_BF16;
     rc = kvp_attn_fwd(&s16, donor, causal, scale, q16, k16, v16, o16, lse, ws, ws_bytes, stream_);
@@ -423,7 +416,8 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* o16 = sh.in(o, z.q);
     const void* const* do16 = sh.in(d_o, z.q);
     void* const* dq16 = sh.out(dq, z.q);
-    if (sh.status() != KVP_OK) return sh.status();
+    rc = sh.round_inputs();
+    if (rc != KVP_OK) return rc;
     kvp_shape s16 = *s;
     s16.dtype = KVP_BF16;
     rc = kvp_attn_bwd(&s16, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq16, dk_sum, dv_sum, ws, ws_bytes, stream_);

@@ -56,6 +56,15 @@ struct GemmProblem {
 // board's power limit the attention backward sharing the step with them slowed by more than the pairs gained.
 int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool prefer_pair);
 
+// Conversion of a list of tensors in as few launches as the parameter block allows.  widen: bf16 -> fp32, else
+// fp32 -> bf16 (round-to-nearest-even).  elems: multiples of 4.
+struct CastItem {
+  const void* src;
+  void* dst;
+  size_t elems;
+};
+int cast_tensors(const CastItem* items, int n, bool widen, cudaStream_t stream);
+
 void gemm_set_pair_mode(int mode);   // 0: single-CTA tiles only, 1: pairs where the caller prefers them, 2: pairs everywhere
 int gemm_pair_mode();
 int gemm_read_status();

@@ -1,52 +1,88 @@
-// Small memory-bound helpers: fp32 -> bf16 rounding (the donor-group gradient sums before they enter the
-// projection GEMMs; fp32 inputs of the KVP_F32 interface) and bf16 -> fp32 widening (its outputs).
+// Conversions between the caller's fp32 tensors and the library's bf16 ones: fp32 -> bf16 rounding (the donor-group
+// gradient sums before they enter the projection GEMMs; fp32 inputs of the KVP_F32 interface) and bf16 -> fp32 widening
+// (its outputs).
+//
+// One launch converts a whole list of tensors: a call of the fp32 interface has 3 to 8 of them per layer, each of a few
+// hundred KB at the sizes that interface is for, where a launch costs more than the copy.  A four-layer training step of
+// 2 x 128 tokens had 64 such launches of 1.6 us each; it has 8 (device time of the step 124 -> 78 us).  Bound: HBM for
+// large tensors, launch latency for small.
+#include <algorithm>
+
 #include "kvp_host.h"
 #include "kvp_sm100.cuh"
 
 namespace kvp {
 namespace {
 
-__global__ void cast_f32_bf16_kernel(const float4* __restrict__ src, uint2* __restrict__ dst, size_t n4) {
-  grid_dep_launch();
-  grid_dep_wait();
-  const size_t stride = size_t(gridDim.x) * blockDim.x;
-  for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const float4 v = src[i];
-    dst[i] = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
-  }
+constexpr int MAX_CAST = 64;             // tensors per launch
+constexpr int CAST_THREADS = 256;
+constexpr int CAST_UNROLL = 4;           // 4-element pieces in flight per thread
+constexpr uint32_t CAST_CHUNK = CAST_THREADS * CAST_UNROLL;   // pieces per block and turn
+
+struct CastParams {
+  const void* src[MAX_CAST];
+  void* dst[MAX_CAST];
+  size_t n4[MAX_CAST];                   // 4-element pieces
+  uint32_t chunk_end[MAX_CAST];          // one past the tensor's last chunk in the launch's chunk order
+  uint32_t chunks;
+};
+
+__device__ __forceinline__ uint2 convert(const float4& v) { return make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w)); }
+__device__ __forceinline__ float4 convert(const uint2& v) {
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
 }
 
-__global__ void cast_bf16_f32_kernel(const uint2* __restrict__ src, float4* __restrict__ dst, size_t n4) {
+template <typename Src, typename Dst>
+__global__ void __launch_bounds__(CAST_THREADS) cast_kernel(const __grid_constant__ CastParams p) {
   grid_dep_launch();
   grid_dep_wait();
-  const size_t stride = size_t(gridDim.x) * blockDim.x;
-  for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const uint2 v = src[i];
-    dst[i] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
-                         __uint_as_float(v.y & 0xffff0000u));
+  int t = 0;
+  for (uint32_t c = blockIdx.x; c < p.chunks; c += gridDim.x) {
+    while (c >= p.chunk_end[t]) ++t;
+    const size_t first = size_t(c - (t ? p.chunk_end[t - 1] : 0)) * CAST_CHUNK + threadIdx.x;
+    const Src* src = reinterpret_cast<const Src*>(p.src[t]);
+    Dst* dst = reinterpret_cast<Dst*>(p.dst[t]);
+    const size_t n4 = p.n4[t];
+    Src v[CAST_UNROLL];
+#pragma unroll
+    for (int u = 0; u < CAST_UNROLL; ++u)
+      if (first + u * CAST_THREADS < n4) v[u] = src[first + u * CAST_THREADS];
+#pragma unroll
+    for (int u = 0; u < CAST_UNROLL; ++u)
+      if (first + u * CAST_THREADS < n4) dst[first + u * CAST_THREADS] = convert(v[u]);
   }
 }
 
 }  // namespace
 
-int cast_bf16_to_f32(const void* src, float* dst, size_t n, cudaStream_t stream) {
-  if ((n & 3) != 0) return KVP_ERR_UNSUPPORTED;
-  const size_t n4 = n / 4;
-  const int threads = 256;
-  const int blocks = int(min(size_t(sm_count()) * 8, (n4 + threads - 1) / threads));
-  const cudaError_t e = launch_kernel(cast_bf16_f32_kernel, blocks, threads, 0, stream, 1, reinterpret_cast<const uint2*>(src), reinterpret_cast<float4*>(dst), n4);
-  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
-}
-
-// n must be a multiple of 4 (it is a multiple of the head dimension).
-int cast_f32_to_bf16(const float* src, void* dst, size_t n, cudaStream_t stream) {
-  if ((n & 3) != 0) return KVP_ERR_UNSUPPORTED;
-  const size_t n4 = n / 4;
-  const int threads = 256;
-  const int blocks = int(min(size_t(sm_count()) * 8, (n4 + threads - 1) / threads));
-  const cudaError_t e = launch_kernel(cast_f32_bf16_kernel, blocks, threads, 0, stream, 1, reinterpret_cast<const float4*>(src),
-                                                       reinterpret_cast<uint2*>(dst), n4);
-  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+int cast_tensors(const CastItem* items, int n, bool widen, cudaStream_t stream) {
+  for (int i = 0; i < n; ++i)
+    if ((items[i].elems & 3) != 0) return KVP_ERR_UNSUPPORTED;
+  CastParams p;
+  int begin = 0;
+  while (begin < n) {
+    uint64_t chunks = 0;
+    int cnt = 0;
+    for (; cnt < MAX_CAST && begin + cnt < n; ++cnt) {
+      const CastItem& it = items[begin + cnt];
+      const uint64_t more = (it.elems / 4 + CAST_CHUNK - 1) / CAST_CHUNK;
+      if (more > 0xffffffffu) return KVP_ERR_UNSUPPORTED;
+      if (chunks + more > 0xffffffffu) break;
+      chunks += more;
+      p.src[cnt] = it.src;
+      p.dst[cnt] = it.dst;
+      p.n4[cnt] = it.elems / 4;
+      p.chunk_end[cnt] = uint32_t(chunks);
+    }
+    p.chunks = uint32_t(chunks);
+    begin += cnt;
+    if (chunks == 0) continue;
+    const int blocks = int(std::min<uint64_t>(uint64_t(sm_count()) * 8, chunks));
+    const cudaError_t e = launch_kernel(widen ? cast_kernel<uint2, float4> : cast_kernel<float4, uint2>, blocks, CAST_THREADS, 0, stream, 1, p);
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
+  }
+  return KVP_OK;
 }
 
 }  // namespace kvp
