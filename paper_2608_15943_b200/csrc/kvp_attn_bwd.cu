@@ -574,16 +574,37 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   }
 }
 
-// dq[b,s,hq,:] = bf16(scale * accumulator), from the blocked fp32 layout [b][hq][tile][quarter][64][32].
-// One thread per 8 consecutive columns of one query row: two 16-byte loads, one 16-byte store.
+// The passes before and after bwd_kernel, each ONE launch for all member layers of a bwd_kernel launch (blockIdx.y is
+// the layer's slot): a layer's share is a few microseconds at small sizes, where every launch cost as much again
+// (Delta, clears and conversion of three layers of 3 x 776 tokens: 11 launches, 39 us -> 2 launches, 20 us).
+struct AuxParams {
+  const __nv_bfloat16* o[MAX_GROUP];
+  const __nv_bfloat16* d_o[MAX_GROUP];
+  __nv_bfloat16* dq[MAX_GROUP];
+  float* delta[MAX_GROUP];
+  float* dq_acc[MAX_GROUP];
+  float* dk_sum[MAX_GROUP];   // per group
+  float* dv_sum[MAX_GROUP];
+  int n_groups;
+  int B, S, Hq;
+  size_t acc_v4;              // 16-byte pieces of one dQ accumulator
+  size_t kv_v4;               // 16-byte pieces of one dK (dV) sum
+  float scale;
+};
+
+// After: dq[b,s,hq,:] = bf16(scale * accumulator), from the blocked fp32 layout [b][hq][tile][quarter][64][32].
+// One thread per 8 consecutive columns of one query row: two 16-byte loads, one 16-byte store.  Bound: HBM.
 template <int DH>
-__global__ void dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int B, int S, int Hq,
-                                  float scale) {
+__global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   constexpr int TPR = DH / 8;  // threads per query row
   grid_dep_launch();
   grid_dep_wait();
+  const float* __restrict__ acc = p.dq_acc[blockIdx.y];
+  __nv_bfloat16* __restrict__ dq = p.dq[blockIdx.y];
+  const int S = p.S, Hq = p.Hq;
+  const float scale = p.scale;
   const int n_qt = (S + BQ2 - 1) / BQ2;
-  const size_t rows = size_t(B) * Hq * n_qt * BQ2;
+  const size_t rows = size_t(p.B) * Hq * n_qt * BQ2;
   const size_t stride = size_t(gridDim.x) * blockDim.x / TPR;
   const int j = threadIdx.x % TPR;
   const int quarter = j / 4, d0 = (j % 4) * 8;
@@ -608,21 +629,36 @@ __global__ void dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* 
   }
 }
 
-// Delta[b,hq,s] = sum_c dO[b,s,hq,c] * O[b,s,hq,c].  A row of DH bf16 is DH/8 16-byte pieces: each warp takes
+// Before: clears the slot's dQ accumulator and the slot's share of the dK / dV sums (stores, nothing waits for them),
+// and forms Delta[b,hq,s] = sum_c dO[b,s,hq,c] * O[b,s,hq,c].  A row of DH bf16 is DH/8 16-byte pieces: each warp takes
 // 256/DH rows at a time (one piece per lane, every lane busy), two such groups per iteration so that four
-// loads per lane are in flight, and reduces inside the DH/8-lane segments.
+// loads per lane are in flight, and reduces inside the DH/8-lane segments.  Bound: HBM.
 template <int DH>
-__global__ void delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                             float* __restrict__ delta, int B, int S, int Hq) {
+__global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
   constexpr int LANES = DH / 8;          // lanes per row
   constexpr int ROWS = 32 / LANES;       // rows per warp and load
   grid_dep_launch();
   grid_dep_wait();
-  const size_t rows = size_t(B) * S * Hq;
+  const int slot = blockIdx.y;
+  const size_t first = size_t(blockIdx.x) * blockDim.x + threadIdx.x, stride = size_t(gridDim.x) * blockDim.x;
+  auto clear = [&](float* dst, size_t n) {
+    float4* d = reinterpret_cast<float4*>(dst);
+    for (size_t i = first; i < n; i += stride) d[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  clear(p.dq_acc[slot], p.acc_v4);
+  if (slot < p.n_groups) {
+    clear(p.dk_sum[slot], p.kv_v4);
+    clear(p.dv_sum[slot], p.kv_v4);
+  }
+  const __nv_bfloat16* __restrict__ o = p.o[slot];
+  const __nv_bfloat16* __restrict__ d_o = p.d_o[slot];
+  float* __restrict__ delta = p.delta[slot];
+  const int S = p.S, Hq = p.Hq;
+  const size_t rows = size_t(p.B) * S * Hq;
   const int lane = threadIdx.x & 31;
   const int sub = lane / LANES, piece = lane % LANES;
-  const size_t warp_global = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const size_t n_warps = (size_t(gridDim.x) * blockDim.x) >> 5;
+  const size_t warp_global = first >> 5;
+  const size_t n_warps = stride >> 5;
   auto dot8 = [](const uint4& a, const uint4& g) {
     const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
     const __nv_bfloat162* pg = reinterpret_cast<const __nv_bfloat162*>(&g);
@@ -662,7 +698,6 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfl
     }
   }
 }
-
 
 int make_map_bshd(CUtensorMap* m, const void* base, int B, int S, int H, int dh, int rows) {
   uint64_t dims[4] = {uint64_t(dh), uint64_t(H), uint64_t(S), uint64_t(B)};
@@ -711,19 +746,6 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   if ((dh == 128 ? allow_smem<bwd_kernel<128>>(BwdSmem<128>::TOTAL) : allow_smem<bwd_kernel<64>>(BwdSmem<64>::TOTAL)) != cudaSuccess)
     return KVP_ERR_CUDA;
 
-  // Delta for every layer
-  timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-  for (int l = 0; l < s->L; ++l) {
-    float* dl = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
-    const size_t rows = size_t(s->B) * s->S * s->Hq;
-    const int blocks = int(min(size_t(sm_count()) * 16, (rows + 7) / 8));
-    const cudaError_t e = launch_kernel(dh == 128 ? delta_kernel<128> : delta_kernel<64>, blocks, 256, 0, stream, 1,
-                                        reinterpret_cast<const __nv_bfloat16*>(o[l]),
-                                        reinterpret_cast<const __nv_bfloat16*>(d_o[l]), dl, s->B, s->S, s->Hq);
-    if (e != cudaSuccess) return KVP_ERR_CUDA;
-  }
-  timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
-
   // Donor groups, largest first; a launch takes groups until it holds MAX_GROUP member layers.  A launch writes
   // dK / dV of its donors through reductions into cleared buffers, so a donor shared by more than MAX_GROUP
   // layers is not supported.
@@ -747,12 +769,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.n > b.n; });
   const int n_jt = (s->S + BT - 1) / BT, n_qt = (s->S + BQ2 - 1) / BQ2, n_pairs = s->Hkv * s->B;
   const int G = s->Hq / s->Hkv;
-  const size_t kv_bytes = size_t(s->B) * s->S * s->Hkv * dh * 4;
   size_t gi = 0;
   while (gi < groups.size()) {
     BwdParams p;
+    AuxParams ax = {};
     int slots = 0, ng = 0;
-    int slot_layer[MAX_GROUP];
     p.cta_begin[0] = 0;
     p.first_slot[0] = 0;
     while (gi < groups.size() && slots + groups[gi].n <= MAX_GROUP) {
@@ -768,11 +789,15 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         p.lse[slots] = lse[l];
         p.delta[slots] = reinterpret_cast<const float*>(wsb + size_t(l) * delta_bytes);
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
-        slot_layer[slots] = l;
+        ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
+        ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
+        ax.dq[slots] = reinterpret_cast<__nv_bfloat16*>(dq[l]);
+        ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
+        ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
       }
-      p.dk_sum[ng] = dk_sum[g.owner];
-      p.dv_sum[ng] = dv_sum[g.owner];
+      p.dk_sum[ng] = ax.dk_sum[ng] = dk_sum[g.owner];
+      p.dv_sum[ng] = ax.dv_sum[ng] = dv_sum[g.owner];
       p.window[ng] = std::min(n_qt, std::max(kMinWindow, (kStepsPerCta + g.n * G - 1) / (g.n * G)));
       p.ctas_per_pair[ng] = 0;
       for (int w = 0; w * p.window[ng] < n_qt; ++w)
@@ -807,29 +832,30 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     p.causal = causal;
     p.scale = sc;
     p.scale_log2 = sc * 1.4426950408889634f;
+    ax.n_groups = ng;
+    ax.B = s->B;
+    ax.S = s->S;
+    ax.Hq = s->Hq;
+    ax.acc_v4 = dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;
+    ax.kv_v4 = size_t(s->B) * s->S * s->Hkv * dh / 4;
+    ax.scale = sc;
+    // enough blocks for every slot to fill the device, no more than its 8-element pieces (convert) give work to
+    const int aux_blocks = int(min(size_t(sm_count()) * 16, (dq_acc_floats(s->B, s->S, s->Hq, dh) / 8 + 255) / 256));
+    const dim3 aux_grid(aux_blocks, slots);
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    if (cudaMemsetAsync(acc_base, 0, size_t(slots) * acc_bytes, stream) != cudaSuccess) return KVP_ERR_CUDA;
-    for (int i = 0; i < ng; ++i)
-      if (cudaMemsetAsync(p.dk_sum[i], 0, kv_bytes, stream) != cudaSuccess ||
-          cudaMemsetAsync(p.dv_sum[i], 0, kv_bytes, stream) != cudaSuccess)
-        return KVP_ERR_CUDA;
+    cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128> : bwd_prepare_kernel<64>, aux_grid, 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
     dim3 grid(p.cta_begin[ng]);
     timing_before(KVP_KERNEL_ATTN_BWD, stream);
-    const cudaError_t e = dh == 128 ? launch_kernel(bwd_kernel<128>, grid, BWD_THREADS, BwdSmem<128>::TOTAL, stream, 1, p)
-                                    : launch_kernel(bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream, 1, p);
+    e = dh == 128 ? launch_kernel(bwd_kernel<128>, grid, BWD_THREADS, BwdSmem<128>::TOTAL, stream, 1, p)
+                  : launch_kernel(bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream, 1, p);
     timing_after(KVP_KERNEL_ATTN_BWD, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    for (int i = 0; i < slots; ++i) {
-      const size_t threads = dq_acc_floats(s->B, s->S, s->Hq, dh) / 8;
-      const int blocks = int(min(size_t(sm_count()) * 16, (threads + 255) / 256));
-      const cudaError_t ec = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, blocks, 256, 0, stream, 1,
-                                           p.dq_acc[i], reinterpret_cast<__nv_bfloat16*>(dq[slot_layer[i]]), s->B, s->S,
-                                           s->Hq, sc);
-      if (ec != cudaSuccess) return KVP_ERR_CUDA;
-    }
+    e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid, 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
+    if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;
 }
