@@ -57,6 +57,12 @@ constexpr int DQ_STAGE_BYTES = BQ2 * 32 * 4;  // one drain warp's share of a ste
 // to amortise its prologue and its dK / dV reduction, short enough that a wave's footprint stays in L2.
 constexpr int kStepsPerCta = 256;
 constexpr int kMinWindow = 16;
+// A CTA costs about seven steps besides its steps (prologue, dK / dV reduction, gap between two CTAs), and the last CTAs of
+// a launch leave the device idle for half of their length: with n steps per SM in all, n * 7 / t + t / 2 is least at
+// t = sqrt(14 n).  Measured (us; always 256 steps -> this): B3 S776 H16/4 dh64, 3 layers 119 -> 95; B4 S632 H8/2 dh128,
+// 8 layers 201 -> 119; B1 S4096 H32/8 dh128, 1 layer 445 -> 337.  From about 4700 steps per SM on the 256 stand.
+constexpr float kTailFactor = 14.f;
+constexpr int kMinSteps = 2;
 
 template <int DH>
 struct BwdSmem {
@@ -91,7 +97,8 @@ struct BwdParams {
   int first_slot[MAX_GROUP + 1];
   int cta_begin[MAX_GROUP + 1];
   int window[MAX_GROUP];          // query tiles per CTA
-  int ctas_per_pair[MAX_GROUP];   // CTAs of one (batch, KV head): sum over windows of the key tiles that see the window
+  int parts[MAX_GROUP];           // parts the query streams of a (window, key tile) are dealt out in
+  int ctas_per_pair[MAX_GROUP];   // CTAs of one (batch, KV head): parts x sum over windows of the key tiles that see the window
   int n_groups;
   int B, S, Hq, Hkv;
   int causal;
@@ -174,7 +181,9 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   const int window = p.window[grp];
   const int in_group = blockIdx.x - p.cta_begin[grp];
   const int pair = in_group / p.ctas_per_pair[grp];
-  int jt = in_group - pair * p.ctas_per_pair[grp];
+  const int parts = p.parts[grp];
+  const int part = (in_group - pair * p.ctas_per_pair[grp]) % parts;
+  int jt = (in_group - pair * p.ctas_per_pair[grp]) / parts;
   int win = 0;
   for (;; ++win) {
     const int vis = p.causal ? min(n_jt, ((win + 1) * window * BQ2 + BT - 1) / BT) : n_jt;
@@ -187,7 +196,9 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   const int kv0 = jt * BT;
   const int qt_first = max(p.causal ? (kv0 / BQ2) : 0, win * window);
   const int per_stream = min(n_qt, (win + 1) * window) - qt_first;
-  const int n_iter = n_layers * G * per_stream;
+  const int n_streams = n_layers * G;
+  const int stream0 = part * n_streams / parts;
+  const int n_iter = ((part + 1) * n_streams / parts - stream0) * per_stream;
 
   if (threadIdx.x == 0) {
     mbar_init(kv_full, 1);
@@ -229,8 +240,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   auto decode_iter = [&](int it, int& li, int& hq, int& q0) {
     const int stream = it / per_stream;
     const int qi = it - stream * per_stream;
-    li = stream / G;
-    hq = hk * G + (stream - li * G);
+    li = (stream0 + stream) / G;
+    hq = hk * G + (stream0 + stream - li * G);
     q0 = (qt_first + qi) * BQ2;
   };
 
@@ -486,7 +497,9 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       return c.row + (valid ? qc : p.S - 1);
     };
     Cursor cf, cp;
-    cf.row = cp.row = row_of(0, 0);
+    cf.li = cp.li = stream0 / G;
+    cf.g = cp.g = stream0 % G;
+    cf.row = cp.row = row_of(cf.li, cf.g);
     for (int i = 0; i < kStatAhead; ++i) advance(cp);
     auto request = [&]() -> bool {  // cp.async of the next step's value into its ring slot; returns its validity
       bool ahead_valid, valid;
@@ -516,7 +529,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     }
     fence_proxy_async_smem();
     mbar_arrive(stat0);
-    int li = 0, g = 0, qi = 0;
+    int li = stream0 / G, g = stream0 % G, qi = 0;
     bool ok = true;
     for (int it = 0; it < n_iter; ++it) {
       ok = mbar_wait(dq_full, it & 1, err);
@@ -769,6 +782,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.n > b.n; });
   const int n_jt = (s->S + BT - 1) / BT, n_qt = (s->S + BQ2 - 1) / BQ2, n_pairs = s->Hkv * s->B;
   const int G = s->Hq / s->Hkv;
+  // steps of one query stream of one (batch, KV head), and the steps one CTA should run
+  long long stream_steps = 0;
+  for (int j = 0; j < n_jt; ++j) stream_steps += causal ? n_qt - j * (BT / BQ2) : n_qt;
+  const float steps_per_sm = float(stream_steps) * n_pairs * s->L * G / sm_count();
+  const int target = std::max(kMinSteps, int(sqrtf(std::min(float(kStepsPerCta) * kStepsPerCta, kTailFactor * steps_per_sm))));
   size_t gi = 0;
   while (gi < groups.size()) {
     BwdParams p;
@@ -798,10 +816,20 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       }
       p.dk_sum[ng] = ax.dk_sum[ng] = dk_sum[g.owner];
       p.dv_sum[ng] = ax.dv_sum[ng] = dv_sum[g.owner];
-      p.window[ng] = std::min(n_qt, std::max(kMinWindow, (kStepsPerCta + g.n * G - 1) / (g.n * G)));
+      // Windows first (a CTA that serves all streams of its window loads K and V once for them), then parts of the streams
+      // where even the smallest window holds more steps than a CTA should run.
+      const int streams = g.n * G;
+      int window = std::max(std::max(1, target / (kStepsPerCta / kMinWindow)), (target + streams - 1) / streams);
+      if (window > 1) window += window & 1;   // whole key tiles of two query tiles: no CTA for half of a diagonal tile
+      p.window[ng] = std::min(n_qt, window);
+      p.parts[ng] = target < kStepsPerCta ? std::max(1, std::min(streams, (streams * p.window[ng] + target / 2) / target)) : 1;
+      // Up to 128 tokens dQ has one term, and two CTAs' terms of dK / dV add up to the same value in either order: such
+      // short sequences keep results that do not differ from run to run.
+      if (n_jt == 1) p.parts[ng] = std::min(p.parts[ng], p.window[ng] < n_qt ? 1 : 2);
       p.ctas_per_pair[ng] = 0;
       for (int w = 0; w * p.window[ng] < n_qt; ++w)
         p.ctas_per_pair[ng] += causal ? std::min(n_jt, ((w + 1) * p.window[ng] * BQ2 + BT - 1) / BT) : n_jt;
+      p.ctas_per_pair[ng] *= p.parts[ng];
       p.first_slot[ng + 1] = slots;
       p.cta_begin[ng + 1] = p.cta_begin[ng] + n_pairs * p.ctas_per_pair[ng];
       ++ng;
@@ -820,6 +848,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       p.dk_sum[i] = p.dk_sum[0];
       p.dv_sum[i] = p.dv_sum[0];
       p.window[i] = p.window[0];
+      p.parts[i] = p.parts[0];
       p.ctas_per_pair[i] = p.ctas_per_pair[0];
       p.first_slot[i + 1] = slots;
       p.cta_begin[i + 1] = p.cta_begin[ng];
