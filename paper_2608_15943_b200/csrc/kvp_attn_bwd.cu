@@ -92,8 +92,7 @@ struct BwdParams {
   const float* lse[MAX_GROUP];    // [B,Hq,S]
   const float* delta[MAX_GROUP];  // [B,Hq,S]
   float* dq_acc[MAX_GROUP];       // blocked fp32 accumulators, see dq_acc_floats()
-  float* dk_sum[MAX_GROUP];       // per group: fp32 [B,S,Hkv,dh]
-  float* dv_sum[MAX_GROUP];
+  CUtensorMap map_dk[MAX_GROUP], map_dv[MAX_GROUP]; // per group: the fp32 sums [B,S,Hkv,dh], box 32 rows x 32 columns
   int first_slot[MAX_GROUP + 1];
   int cta_begin[MAX_GROUP + 1];
   int window[MAX_GROUP];          // query tiles per CTA
@@ -200,20 +199,126 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   const int stream0 = part * n_streams / parts;
   const int n_iter = ((part + 1) * n_streams / parts - stream0) * per_stream;
 
-  if (threadIdx.x == 0) {
-    mbar_init(kv_full, 1);
-    for (int s = 0; s < BWD_STAGES; ++s) {
-      mbar_init(&q_full[s], 1);
-      mbar_init(&q_empty[s], 1);
+  auto decode_iter = [&](int it, int& li, int& hq, int& q0) {
+    const int stream = it / per_stream;
+    const int qi = it - stream * per_stream;
+    li = (stream0 + stream) / G;
+    hq = hk * G + (stream0 + stream - li * G);
+    q0 = (qt_first + qi) * BQ2;
+  };
+  auto load_step = [&](int it, uint32_t leader) {
+    int li, hq, q0;
+    decode_iter(it, li, hq, q0);
+    const int s = it % BWD_STAGES;
+    mbar_expect_tx_e(&q_full[s], L::STAGE, leader);
+    uint8_t* dst = smem + L::OFF_RING + s * L::STAGE;
+#pragma unroll
+    for (int h = 0; h < HALVES; ++h) {
+      tma_load_4d_e(dst + h * QHALF_BYTES, &p.map_q[slot0 + li], &q_full[s], h * 64, hq, q0, b, leader);
+      tma_load_4d_e(dst + L::Q_TILE + h * QHALF_BYTES, &p.map_do[slot0 + li], &q_full[s], h * 64, hq, q0, b, leader);
     }
-    mbar_init(st_full, 1);
-    mbar_init(dp_free, 256);
-    for (int i = 0; i < 2; ++i) mbar_init(&pds_ready[i], 256);
-    mbar_init(dq_full, 1);
-    mbar_init(dq_free, 128);
-    mbar_init(stat0, 128);
-    mbar_init(acc_done, 1);
-    mbar_fence_init();
+  };
+
+  // Statistics.  The drain warpgroup also prepares the per-query operand tiles the tensor core adds to the scores:
+  // thread t < 64 handles -LSE/scale of query column t, thread 64 + t handles -Delta of column t, as the
+  // three-term bf16 split.  The raw fp32 values come in through cp.async into a small ring in shared memory,
+  // requested eight steps before the step that uses them and staged as an operand tile three steps before: no
+  // register ever waits on global memory, and the compute warpgroups never touch the statistics.
+  const int stat_tid = int(threadIdx.x) - 10 * 32;   // (used by the drain warpgroup only)
+  const int stat_kind = stat_tid >> 6;   // 0 lse, 1 delta
+  const int stat_col = stat_tid & 63;
+  uint8_t* stat_row = smem + L::OFF_STAT + stat_kind * 1024 + stat_col * 16;
+  float* raw = reinterpret_cast<float*>(smem + L::OFF_RAW) + stat_tid;   // ring slot s at raw[s * 128]
+  const float stat_mul = stat_kind == 0 ? -1.f / p.scale : -1.f;
+  const float stat_pad = stat_kind == 0 ? -30000.f : 0.f;  // a query beyond the sequence: exp2 underflows to zero
+  // Two cursors walk the steps in order (incremental decode of step -> layer, head, query tile): one for the
+  // step whose statistics are requested next, one kStatAhead steps further that only pulls the line into L2.
+  // `row` is the statistic row of the cursor's (layer, head): it is looked up (an indexed read of the kernel
+  // parameters) only when the stream changes, never on the per-step path.
+  constexpr int kStatAhead = 12;
+  struct Cursor {
+    int it = 0, qi = 0, g = 0, li = 0;
+    const float* row = nullptr;
+  };
+  auto row_of = [&](int li, int g) {
+    const int slot = slot0 + (li < n_layers ? li : 0);
+    const float* src = stat_kind == 0 ? p.lse[slot] : p.delta[slot];
+    return src + (size_t(b) * p.Hq + hk * G + g) * p.S;
+  };
+  auto advance = [&](Cursor& c) {
+    ++c.it;
+    if (++c.qi == per_stream) {
+      c.qi = 0;
+      if (++c.g == G) {
+        c.g = 0;
+        ++c.li;
+      }
+      c.row = row_of(c.li, c.g);
+    }
+  };
+  auto locate = [&](const Cursor& c, bool& valid) {  // address of this thread's statistic of step c (clamped, always valid)
+    const int qc = (qt_first + c.qi) * BQ2 + stat_col;
+    valid = c.it < n_iter && qc < p.S;
+    return c.row + (valid ? qc : p.S - 1);
+  };
+  Cursor cf, cp;
+  auto request = [&]() -> bool {  // cp.async of the next step's value into its ring slot; returns its validity
+    bool valid;
+    const float* ptr = locate(cf, valid);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(raw + (cf.it & 7) * 128)), "l"(ptr) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    advance(cf);
+    return valid;
+  };
+  auto look_ahead = [&]() {  // the line of the step kStatAhead further on, into L2
+    bool valid;
+    const float* ahead = locate(cp, valid);
+    if ((stat_col & 31) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead));
+    advance(cp);
+  };
+  auto stage = [&](int step, bool valid) {  // the value of `step` has landed: split it into the step's operand tile
+    *reinterpret_cast<uint4*>(stat_row + (step & 3) * 2048) = split3_bf16(valid ? raw[(step & 7) * 128] * stat_mul : stat_pad);
+  };
+  uint32_t vbits = 0;
+
+  // The loads that everything waits for go out before the block has set itself up: the TMA warp initialises the barriers
+  // and fills the ring, the drain warpgroup requests the first statistics, then the block meets.
+  if (warp == 0) {
+    const uint32_t leader = elect_one();
+    if (leader) {
+      mbar_init(kv_full, 1);
+      for (int s = 0; s < BWD_STAGES; ++s) {
+        mbar_init(&q_full[s], 1);
+        mbar_init(&q_empty[s], 1);
+      }
+      mbar_init(st_full, 1);
+      mbar_init(dp_free, 256);
+      for (int i = 0; i < 2; ++i) mbar_init(&pds_ready[i], 256);
+      mbar_init(dq_full, 1);
+      mbar_init(dq_free, 128);
+      mbar_init(stat0, 128);
+      mbar_init(acc_done, 1);
+      mbar_fence_init();
+      fence_proxy_async_smem();
+    }
+    __syncwarp();
+    grid_dep_wait();
+    mbar_expect_tx_e(kv_full, 2 * L::KV_TILE, leader);
+#pragma unroll
+    for (int h = 0; h < HALVES; ++h) {
+      tma_load_4d_e(smem + L::OFF_K + h * HALF_BYTES, &p.map_k[grp], kv_full, h * 64, hk, kv0, b, leader);
+      tma_load_4d_e(smem + L::OFF_V + h * HALF_BYTES, &p.map_v[grp], kv_full, h * 64, hk, kv0, b, leader);
+    }
+    for (int it = 0; it < min(n_iter, BWD_STAGES); ++it) load_step(it, leader);
+  }
+  if (warp >= 10) {
+    grid_dep_wait();
+    cf.li = stream0 / G;
+    cf.g = stream0 % G;
+    cf.row = row_of(cf.li, cf.g);
+    cp = cf;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) vbits |= uint32_t(request()) << i;
   }
   // constant operand tiles: ones in the first three columns; statistics tiles and the shared zero half start as zeros
   for (int i = threadIdx.x; i < (L::OFF_RAW - L::OFF_ONES) / 16; i += blockDim.x) {
@@ -237,40 +342,12 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   const uint32_t tm_dk = tmem_base + 256;
   const uint32_t tm_dv = tmem_base + 256 + DH;
 
-  auto decode_iter = [&](int it, int& li, int& hq, int& q0) {
-    const int stream = it / per_stream;
-    const int qi = it - stream * per_stream;
-    li = (stream0 + stream) / G;
-    hq = hk * G + (stream0 + stream - li * G);
-    q0 = (qt_first + qi) * BQ2;
-  };
-
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
-    {
-      const uint32_t leader = elect_one();  // the whole warp runs the loop; one lane issues
-      if (leader) tma_prefetch_desc(&p.map_k[grp]);
-      if (leader) tma_prefetch_desc(&p.map_v[grp]);
-      mbar_expect_tx_e(kv_full, 2 * L::KV_TILE, leader);
-#pragma unroll
-      for (int h = 0; h < HALVES; ++h) {
-        tma_load_4d_e(smem + L::OFF_K + h * HALF_BYTES, &p.map_k[grp], kv_full, h * 64, hk, kv0, b, leader);
-        tma_load_4d_e(smem + L::OFF_V + h * HALF_BYTES, &p.map_v[grp], kv_full, h * 64, hk, kv0, b, leader);
-      }
-      for (int it = 0; it < n_iter; ++it) {
-        int li, hq, q0;
-        decode_iter(it, li, hq, q0);
-        const int s = it % BWD_STAGES;
-        const uint32_t ph = (it / BWD_STAGES) & 1;
-        if (!mbar_wait(&q_empty[s], ph ^ 1, err)) break;
-        mbar_expect_tx_e(&q_full[s], L::STAGE, leader);
-        uint8_t* dst = smem + L::OFF_RING + s * L::STAGE;
-#pragma unroll
-        for (int h = 0; h < HALVES; ++h) {
-          tma_load_4d_e(dst + h * QHALF_BYTES, &p.map_q[slot0 + li], &q_full[s], h * 64, hq, q0, b, leader);
-          tma_load_4d_e(dst + L::Q_TILE + h * QHALF_BYTES, &p.map_do[slot0 + li], &q_full[s], h * 64, hq, q0, b, leader);
-        }
-      }
+    const uint32_t leader = elect_one();  // the whole warp runs the loop; one lane issues
+    for (int it = BWD_STAGES; it < n_iter; ++it) {
+      if (!mbar_wait(&q_empty[it % BWD_STAGES], ((it / BWD_STAGES) & 1) ^ 1, err)) break;
+      load_step(it, leader);
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
@@ -423,25 +500,36 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     }
     if (ok) {
       tc_fence_after_sync();
-      // warpgroup 0 adds dK (scaled), warpgroup 1 adds dV; every lane loads, valid rows reduce
-      const bool valid = kv_row < p.S;
-      const size_t row_off = ((size_t(b) * p.S + (valid ? kv_row : 0)) * p.Hkv + hk) * DH;
-      float* dst = (wg == 0 ? p.dk_sum[grp] : p.dv_sum[grp]) + row_off;
+      // Warpgroup 0 adds dK (scaled), warpgroup 1 adds dV: each warp moves its 32 rows, 32 columns at a time, into
+      // shared memory that the finished MMAs have left (dK over the ring, dV over K and V) and adds them with one TMA
+      // reduction each, which clips rows beyond the sequence.  (Adding straight from registers, one 16-byte piece of
+      // 32 different rows per instruction, moves one line per cycle: with the early loads above, a CTA of dh 128 spends
+      // 7 us besides its steps instead of 12, at 1.25 us a step.)
       const uint32_t src = (wg == 0 ? tm_dk : tm_dv) + lane_sel;
       const float mul = wg == 0 ? p.scale : 1.f;
+      uint8_t* area = smem + (wg == 0 ? L::OFF_RING : L::OFF_K) + quarter * 4096;
+      const CUtensorMap* map = wg == 0 ? &p.map_dk[grp] : &p.map_dv[grp];
+      if (kv0 + quarter * 32 < p.S) {
 #pragma unroll 1
-      for (int c = 0; c < DH / 32; ++c) {
-        uint32_t a[32];
-        tmem_ld_x32(src + c * 32, a);
-        tmem_ld_wait();
-        if (valid) {
+        for (int c = 0; c < DH / 32; ++c) {
+          uint32_t a[32];
+          tmem_ld_x32(src + c * 32, a);
+          tmem_ld_wait();
+          uint8_t* tile = area + c * HALF_BYTES;
 #pragma unroll
           for (int v4 = 0; v4 < 8; ++v4)
-            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + c * 32 + v4 * 4),
-                         "f"(__uint_as_float(a[4 * v4]) * mul), "f"(__uint_as_float(a[4 * v4 + 1]) * mul),
-                         "f"(__uint_as_float(a[4 * v4 + 2]) * mul), "f"(__uint_as_float(a[4 * v4 + 3]) * mul)
-                         : "memory");
+            *reinterpret_cast<float4*>(tile + sw128_offset(lane, v4)) =
+                make_float4(__uint_as_float(a[4 * v4]) * mul, __uint_as_float(a[4 * v4 + 1]) * mul,
+                            __uint_as_float(a[4 * v4 + 2]) * mul, __uint_as_float(a[4 * v4 + 3]) * mul);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_reduce_add_4d(map, tile, c * 32, hk, kv0 + quarter * 32, b);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
       }
     }
   } else {
@@ -454,81 +542,18 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     const bool active = quarter * 32 < DH;  // with DH == 64 the upper lanes hold nothing
     float* stg = reinterpret_cast<float*>(smem + L::OFF_DQ + (warp - 10) * DQ_STAGE_BYTES);
     const uint32_t stg_s = smem_u32(stg);
-    // Statistics.  This warpgroup also prepares the per-query operand tiles the tensor core adds to the scores:
-    // thread t < 64 handles -LSE/scale of query column t, thread 64 + t handles -Delta of column t, as the
-    // three-term bf16 split.  The raw fp32 values come in through cp.async into a small ring in shared memory,
-    // requested eight steps before the step that uses them and staged as an operand tile three steps before: no
-    // register ever waits on global memory, and the compute warpgroups never touch the statistics.
-    const int stat_tid = threadIdx.x - 10 * 32;
-    const int stat_kind = stat_tid >> 6;   // 0 lse, 1 delta
-    const int stat_col = stat_tid & 63;
-    uint8_t* stat_row = smem + L::OFF_STAT + stat_kind * 1024 + stat_col * 16;
-    float* raw = reinterpret_cast<float*>(smem + L::OFF_RAW) + stat_tid;   // ring slot s at raw[s * 128]
-    const float stat_mul = stat_kind == 0 ? -1.f / p.scale : -1.f;
-    const float stat_pad = stat_kind == 0 ? -30000.f : 0.f;  // a query beyond the sequence: exp2 underflows to zero
-    // Two cursors walk the steps in order (incremental decode of step -> layer, head, query tile): one for the
-    // step whose statistics are requested next, one kStatAhead steps further that only pulls the line into L2.
-    // `row` is the statistic row of the cursor's (layer, head): it is looked up (an indexed read of the kernel
-    // parameters) only when the stream changes, never on the per-step path.
-    constexpr int kStatAhead = 12;
-    struct Cursor {
-      int it = 0, qi = 0, g = 0, li = 0;
-      const float* row = nullptr;
-    };
-    auto row_of = [&](int li, int g) {
-      const int slot = slot0 + (li < n_layers ? li : 0);
-      const float* src = stat_kind == 0 ? p.lse[slot] : p.delta[slot];
-      return src + (size_t(b) * p.Hq + hk * G + g) * p.S;
-    };
-    auto advance = [&](Cursor& c) {
-      ++c.it;
-      if (++c.qi == per_stream) {
-        c.qi = 0;
-        if (++c.g == G) {
-          c.g = 0;
-          ++c.li;
-        }
-        c.row = row_of(c.li, c.g);
-      }
-    };
-    auto locate = [&](const Cursor& c, bool& valid) {  // address of this thread's statistic of step c (clamped, always valid)
-      const int qc = (qt_first + c.qi) * BQ2 + stat_col;
-      valid = c.it < n_iter && qc < p.S;
-      return c.row + (valid ? qc : p.S - 1);
-    };
-    Cursor cf, cp;
-    cf.li = cp.li = stream0 / G;
-    cf.g = cp.g = stream0 % G;
-    cf.row = cp.row = row_of(cf.li, cf.g);
-    for (int i = 0; i < kStatAhead; ++i) advance(cp);
-    auto request = [&]() -> bool {  // cp.async of the next step's value into its ring slot; returns its validity
-      bool ahead_valid, valid;
-      const float* ahead = locate(cp, ahead_valid);
-      if ((stat_col & 31) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead));
-      advance(cp);
-      const float* ptr = locate(cf, valid);
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(raw + (cf.it & 7) * 128)), "l"(ptr) : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      advance(cf);
-      return valid;
-    };
-    auto stage = [&](int step, bool valid) {  // the value of `step` has landed: split it into the step's operand tile
-      *reinterpret_cast<uint4*>(stat_row + (step & 3) * 2048) = split3_bf16(valid ? raw[(step & 7) * 128] * stat_mul : stat_pad);
-    };
-    // validity flags of the requests in flight, oldest (step it+3) in bit 0
-    uint32_t vbits = 0;
-    {
-      const bool a0 = request(), a1 = request(), a2 = request();
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      stage(0, a0);
-      stage(1, a1);
-      stage(2, a2);
-      // steps 3..7; from here on a ring slot is requested again only after its previous value has been staged
-#pragma unroll
-      for (int i = 0; i < 5; ++i) vbits |= uint32_t(request()) << i;
-    }
+    // the statistics of steps 0, 1, 2 were requested above
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    stage(0, vbits & 1u);
+    stage(1, vbits & 2u);
+    stage(2, vbits & 4u);
     fence_proxy_async_smem();
     mbar_arrive(stat0);
+    // Five more requests stay in flight (vbits: their validity, oldest in bit 0); from here on a ring slot is requested
+    // again only after its value has been staged.
+    vbits = 0;
+    for (int i = 0; i < 5; ++i) vbits |= uint32_t(request()) << i;
+    for (int i = 0; i < kStatAhead + 8; ++i) look_ahead();
     int li = stream0 / G, g = stream0 % G, qi = 0;
     bool ok = true;
     for (int it = 0; it < n_iter; ++it) {
@@ -542,6 +567,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       // The operand tile of step it+3 (last read by the scores of step it-1, which completed before this step's
       // dQ^T did) and the request for step it+8.  The arrival below publishes the tile: the issuing warp waits for
       // it before the next step's dQ^T, a whole step before the scores of step it+3 are issued.
+      look_ahead();
       vbits |= uint32_t(request()) << 5;
       asm volatile("cp.async.wait_group 5;" ::: "memory");
       stage(it + 3, vbits & 1u);
@@ -574,8 +600,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
         }
       }
     }
-    // the reductions must have completed before the block's shared memory goes away and the grid ends
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // the reductions must have read the block's shared memory before it goes away (their writes complete with the grid)
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     __syncwarp();
   }
 
@@ -719,6 +745,14 @@ int make_map_bshd(CUtensorMap* m, const void* base, int B, int S, int H, int dh,
   return make_tensor_map(m, base, 2, 4, dims, strides, box, true);
 }
 
+// fp32 [B,S,H,dh], boxes of 32 rows x 32 columns
+int make_map_sum(CUtensorMap* m, const void* base, int B, int S, int H, int dh) {
+  uint64_t dims[4] = {uint64_t(dh), uint64_t(H), uint64_t(S), uint64_t(B)};
+  uint64_t strides[3] = {uint64_t(dh) * 4, uint64_t(H) * dh * 4, uint64_t(S) * H * dh * 4};
+  uint32_t box[4] = {32, 1, 32, 1};
+  return make_tensor_map(m, base, 4, 4, dims, strides, box, true);
+}
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Member layers of the launches' accumulators that are live at once: a launch takes whole donor groups until it
@@ -814,8 +848,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
       }
-      p.dk_sum[ng] = ax.dk_sum[ng] = dk_sum[g.owner];
-      p.dv_sum[ng] = ax.dv_sum[ng] = dv_sum[g.owner];
+      ax.dk_sum[ng] = dk_sum[g.owner];
+      ax.dv_sum[ng] = dv_sum[g.owner];
+      rc = make_map_sum(&p.map_dk[ng], dk_sum[g.owner], s->B, s->S, s->Hkv, dh);
+      if (rc == KVP_OK) rc = make_map_sum(&p.map_dv[ng], dv_sum[g.owner], s->B, s->S, s->Hkv, dh);
+      if (rc != KVP_OK) return rc;
       // Windows first (a CTA that serves all streams of its window loads K and V once for them), then parts of the streams
       // where even the smallest window holds more steps than a CTA should run.
       const int streams = g.n * G;
@@ -845,8 +882,8 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     for (int i = ng; i < MAX_GROUP; ++i) {
       p.map_k[i] = p.map_k[0];
       p.map_v[i] = p.map_v[0];
-      p.dk_sum[i] = p.dk_sum[0];
-      p.dv_sum[i] = p.dv_sum[0];
+      p.map_dk[i] = p.map_dk[0];
+      p.map_dv[i] = p.map_dv[0];
       p.window[i] = p.window[0];
       p.parts[i] = p.parts[0];
       p.ctas_per_pair[i] = p.ctas_per_pair[0];
