@@ -335,7 +335,6 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  grid_dep_launch();
   grid_dep_wait();
   const uint32_t tm_dp = tmem_base + 128;
   const uint32_t tm_dq = tmem_base + 192;
@@ -349,6 +348,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       if (!mbar_wait(&q_empty[it % BWD_STAGES], ((it / BWD_STAGES) & 1) ^ 1, err)) break;
       load_step(it, leader);
     }
+    grid_dep_launch();   // all loads are out
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     {
@@ -636,7 +636,6 @@ struct AuxParams {
 template <int DH>
 __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   constexpr int TPR = DH / 8;  // threads per query row
-  grid_dep_launch();
   grid_dep_wait();
   const float* __restrict__ acc = p.dq_acc[blockIdx.y];
   __nv_bfloat16* __restrict__ dq = p.dq[blockIdx.y];
@@ -648,6 +647,7 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   const int j = threadIdx.x % TPR;
   const int quarter = j / 4, d0 = (j % 4) * 8;
   for (size_t row = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) / TPR; row < rows; row += stride) {
+    if (row + stride >= rows) grid_dep_launch();
     const int q = int(row % BQ2);
     const size_t tile = row / BQ2;  // (b * Hq + hq) * n_qt + qt
     const int qt = int(tile % n_qt);
@@ -676,7 +676,6 @@ template <int DH>
 __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
   constexpr int LANES = DH / 8;          // lanes per row
   constexpr int ROWS = 32 / LANES;       // rows per warp and load
-  grid_dep_launch();
   grid_dep_wait();
   const int slot = blockIdx.y;
   const size_t first = size_t(blockIdx.x) * blockDim.x + threadIdx.x, stride = size_t(gridDim.x) * blockDim.x;
@@ -710,6 +709,7 @@ __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
     return acc;
   };
   for (size_t base = warp_global * (2 * ROWS); base < rows; base += n_warps * (2 * ROWS)) {
+    if (base + n_warps * (2 * ROWS) >= rows) grid_dep_launch();
     const size_t r0 = base + sub, r1 = base + ROWS + sub;
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     const uint4 a0 = r0 < rows ? *reinterpret_cast<const uint4*>(o + r0 * DH + piece * 8) : z;

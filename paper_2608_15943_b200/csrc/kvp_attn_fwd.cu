@@ -159,7 +159,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  grid_dep_launch();
   grid_dep_wait();
   // tile X: score buffer u at [X*128 + u*64, +64) with P over its first 32 columns; output accumulator at
   // [256 + X*128, +128)
@@ -214,6 +213,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
         }
         ++it;
       }
+      grid_dep_launch();   // all loads are out
     }
   } else if (warp == 1 || warp == 2) {
     // ------------------------------ MMA issuer of query tile x ------------------------------

@@ -111,7 +111,6 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) decode_kernel(const __grid_con
   const DecGroup& grp = p.grp[gi];
   const int G = p.Hq / p.Hkv;
   const int R = grp.n_members * G;  // valid query rows (<= 16)
-  grid_dep_launch();
   grid_dep_wait();
 
   int len = p.lengths[b];
@@ -281,6 +280,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) decode_kernel(const __grid_con
     }
     __syncwarp();  // every lane is done with this stage before it is refilled
   }
+  grid_dep_launch();   // every load of this CTA is out
   cp_async_wait<0>();
 
   // ---- merge the four warps of the CTA, then write this split's partial ----

@@ -104,7 +104,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  grid_dep_launch();
   grid_dep_wait();
 
   if (warp == 0) {
@@ -148,6 +147,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_cons
           }
         }
       }
+      grid_dep_launch();   // all loads are out: the next kernel may come up while the last tiles are finished
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
@@ -315,7 +315,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
   cluster_sync_all();  // the partner's barriers exist before anything of this CTA can signal them
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  grid_dep_launch();
   grid_dep_wait();
 
   if (warp == 0) {
@@ -360,6 +359,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
           }
         }
       }
+      grid_dep_launch();   // all loads are out: the next kernel may come up while the last tiles are finished
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (even CTA only) ------------------------------

@@ -105,10 +105,12 @@ struct SameType { using type = T; };   // keeps the argument types of launch_ker
 
 // Every kernel of the library is launched through this: programmatic stream serialisation lets its CTAs come up (barriers,
 // tensor-memory allocation, descriptor fetches) while the kernel before it on the stream drains.  The kernel must
-// execute grid_dep_wait() before it touches global memory, and grid_dep_launch() once its own CTAs hold what they
-// need, so that the next kernel may do the same.  cluster > 1 sets a runtime cluster size.  Device time of a pass
-// (graph replay), plain launches -> these: tiny fp32 training step 155 -> 125 us (79 kernels), token step of a
-// four-layer stage 631 -> 595 us (56 kernels), decode step of the tiny stack 11.3 -> 10.3 us (3 kernels).
+// execute grid_dep_wait() before it touches global memory, and grid_dep_launch() when its last loads are out, so that the
+// next kernel may do the same.  (Any thread's grid_dep_launch() counts for its CTA.  Given as soon as a CTA was set up,
+// it parked the next kernel's CTAs on the SMs for the whole of a long kernel, and the 46 ms training step of 2 x 8192
+// tokens took 1.2 ms longer.)  cluster > 1 sets a runtime cluster size.  Device time of a pass (graph replay), plain
+// launches -> these: tiny fp32 training step 59.4 -> 54.4 us, token step of a four-layer stage 635 -> 588 us (56
+// kernels), prompt of 347 tokens through it 1064 -> 1031 us.
 template <typename... KP>
 cudaError_t launch_kernel(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,
                           const typename SameType<KP>::type&... args) {

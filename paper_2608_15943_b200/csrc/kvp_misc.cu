@@ -35,10 +35,10 @@ __device__ __forceinline__ float4 convert(const uint2& v) {
 
 template <typename Src, typename Dst>
 __global__ void __launch_bounds__(CAST_THREADS) cast_kernel(const __grid_constant__ CastParams p) {
-  grid_dep_launch();
   grid_dep_wait();
   int t = 0;
   for (uint32_t c = blockIdx.x; c < p.chunks; c += gridDim.x) {
+    if (c + gridDim.x >= p.chunks) grid_dep_launch();
     while (c >= p.chunk_end[t]) ++t;
     const size_t first = size_t(c - (t ? p.chunk_end[t - 1] : 0)) * CAST_CHUNK + threadIdx.x;
     const Src* src = reinterpret_cast<const Src*>(p.src[t]);

@@ -32,7 +32,6 @@ constexpr int kMaxChunks = 4;  // D <= 8192
 __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
                                                                uint4* __restrict__ y, int T, int D8, float inv_d, float eps) {
   __shared__ float part[kNormThreads / 32];
-  grid_dep_launch();
   grid_dep_wait();
   auto load_row = [&](int row, uint4 (&v)[kMaxChunks]) {
     const uint4* xr = x + size_t(row) * D8;
@@ -49,6 +48,7 @@ __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __re
     // block barriers and the stores of this row
     const int next = row + gridDim.x;
     if (next < T) load_row(next, vn);
+    else grid_dep_launch();
     float ss = 0.f;
 #pragma unroll
     for (int c = 0; c < kMaxChunks; ++c) {
@@ -102,13 +102,13 @@ __global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, 
   // lanes of a warp need different table entries: shared memory serves them in one pass, the constant bank
   // that holds kernel parameters would replay once per distinct address
   __shared__ float2 freq[kMaxRopePairs];
-  grid_dep_launch();
   for (int k = threadIdx.x; k < int(dh8) * 4; k += blockDim.x) freq[k] = fr.f[k];
   __syncthreads();
   grid_dep_wait();
   const uint32_t stride = gridDim.x * blockDim.x;
   const uint32_t per_tok = H * dh8;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_work; i += stride) {  // 32-bit index arithmetic only
+    if (n_work - i <= stride) grid_dep_launch();
     const uint32_t c = i % dh8;                       // which group of 4 pairs inside the head
     const uint32_t tok = i / dh8;                     // b * S + s
     const float pos = float(pos0 + int(tok % S));     // exact
@@ -156,10 +156,10 @@ __global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, 
 
 // out = silu(gate) * up
 __global__ void swiglu_kernel(const uint4* __restrict__ gate, const uint4* __restrict__ up, uint4* __restrict__ out, size_t n8) {
-  grid_dep_launch();
   grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n8; i += stride) {
+    if (i + stride >= n8) grid_dep_launch();
     float g[8], u[8];
     unpack8(gate[i], g);
     unpack8(up[i], u);
@@ -170,10 +170,10 @@ __global__ void swiglu_kernel(const uint4* __restrict__ gate, const uint4* __res
 }
 
 __global__ void add_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b, uint4* __restrict__ out, size_t n8) {
-  grid_dep_launch();
   grid_dep_wait();
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n8; i += stride) {
+    if (i + stride >= n8) grid_dep_launch();
     float f[8], g[8];
     unpack8(a[i], f);
     unpack8(b[i], g);
