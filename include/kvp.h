@@ -273,7 +273,7 @@ typedef struct {
   int32_t page_size;  /* tokens per page: a multiple of 16 */
   int32_t max_pages;  /* columns of block_table */
   int32_t n_pages;    /* pages in each owner layer's pool */
-  int32_t num_splits; /* KV splits per (sequence, KV head); 0 lets the library choose */
+  int32_t num_splits; /* KV splits per (sequence, KV head); 0: the library deals the step's K/V rows out evenly */
   int32_t dtype;      /* KVP_BF16, or KVP_F32: q, k_new, v_new, o are fp32; the cache is bf16 either way */
 } kvp_decode_desc;
 
@@ -309,11 +309,12 @@ int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float scale, cons
  * of KVP_DECODE_STATIC_SCRATCH_BYTES that is part of the library image: every GPU that loads the
  * library holds those bytes until the process exits.
  *
- *  - A request whose partials need more than that (they grow with the number of donor groups that
- *    [layer_begin, layer_end) touches, up to 64 per launch, and with B, Hkv and the split count;
+ *  - With num_splits > 0, a request whose partials need more than that (they grow with the number of donor groups
+ *    that [layer_begin, layer_end) touches, up to 64 per launch, and with B, Hkv and num_splits;
  *    kvp_decode_workspace_bytes(d, donor) is the figure for all layers) is refused with
- *    KVP_ERR_STATIC_SCRATCH and nothing is launched; lower num_splits, decode a narrower layer
- *    range per call, or use kvp_decode with your own workspace.
+ *    KVP_ERR_STATIC_SCRATCH and nothing is launched; lower num_splits, set it to 0, decode a narrower layer
+ *    range per call, or use kvp_decode with your own workspace.  With num_splits == 0 every request fits (where the
+ *    partials would need more, the rows are dealt out in fewer shares: the same results up to fp32 summation order).
  *  - No cudaMalloc / cudaFree / allocating library call is made, on any call.
  *  - The first call on each device looks up the array's device address (with that device current);
  *    make that first call outside any stream capture.

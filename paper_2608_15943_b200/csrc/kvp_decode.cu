@@ -1,17 +1,31 @@
 // Split-KV decode attention over the shared paged cache, and the cache append.
 //
-// A work unit is (donor group, sequence, KV head, split).  The CTA streams its share of the DONOR's
-// K/V pages from HBM exactly once and applies them to every query row that reads them: the Hq/Hkv
-// query heads of the KV head's group for the donor layer AND for each consumer layer of the group
-// (Eq. 3 of the paper: consumers reuse the donor's K/V), up to 16 rows, as the M dimension of
-// mma.sync m16n8k16 (bf16 in, fp32 accumulate).  The kernel is bound by HBM bandwidth, so the
-// design is about bytes in flight: every warp owns a three-stage ring of 16-token granules (8 KB:
-// 4 KB of K, 4 KB of V) filled by 16-byte cp.async copies that are fully coalesced (a page block
-// of one KV head is contiguous), two CTAs per SM, and no transposes in HBM -- V fragments come from
-// ldmatrix.trans on the swizzled ring.  Partial (max, sum, output) triples per split are merged by
-// a second small kernel.
+// A unit is (donor group, sequence, KV head): its K/V rows are streamed from HBM exactly once and applied to every
+// query row that reads them: the Hq/Hkv query heads of the KV head's group for the donor layer AND for each consumer
+// layer of the group (Eq. 3 of the paper: consumers reuse the donor's K/V), up to 16 rows, as the M dimension of
+// mma.sync m16n8k16 (bf16 in, fp32 accumulate).  The kernel is bound by HBM bandwidth, so the design is about bytes in
+// flight and about every warp having the same share of them:
+//  - The rows of a group's units form one list of 16-token granules (8 KB at dh 128: 4 KB of K, 4 KB of V; both
+//    contiguous, a page block of one KV head is), in order of (sequence, KV head, position).  The lengths are in device
+//    memory, so every block sums them up itself and takes an equal share of each group's list, wherever its ends fall:
+//    no part-filled last wave, whatever the batch and the lengths.  Long lists are cut into more shares than blocks
+//    that fit, so that the block scheduler evens out SMs that draw memory at different rates.  The shares of a group do
+//    not depend on the other groups of the call: any layer range gives a layer the same bits.
+//  - Short units are not cut: a list whose units hold 32 granules or fewer on average (64, where there are enough units)
+//    is dealt out by units, since every piece costs a block a merge of its warps (30 sequences of 500 tokens, 8 groups
+//    at dh 64: 49 us by units, 96 us by equal shares).
+//  - The four warps of a block take the granules of a share in turn, each with a ring of its own filled by 16-byte
+//    cp.async copies that are fully coalesced and continue across the ends of units; two blocks per SM.  (A contiguous
+//    share for every warp instead read memory 3 % slower.)  No transposes in HBM -- V fragments come from ldmatrix.trans
+//    on the swizzled ring.
+//  - A unit that lies inside one share is finished there.  The pieces of the others, (max, sum, output) triples, at most
+//    two per share, are merged by a second small kernel that finds them by the same arithmetic.
+// Measured with the merge, against a grid of (unit, 2048-token split) blocks with a merge of one thread per output
+// element: 16 sequences of 4096 tokens 61 -> 50 us (the copy rate takes 41), 8 of 8K-16K in two groups 141 -> 129 (113),
+// one of 65536 74 -> 49 (41), 4 of 128K at 32 KV heads 1187 -> 1172 (1313), 32 of 16K-32K in six groups 2768 -> 2740.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "kvp_host.h"
@@ -23,7 +37,12 @@ namespace {
 constexpr int DEC_WARPS = 4;
 constexpr int DEC_THREADS = DEC_WARPS * 32;
 constexpr int GRAN = 16;           // tokens per ring stage
-constexpr int DEC_STAGES = 3;
+constexpr int DEC_STAGES = 3;      // granules per warp in the ring
+template <int DH>
+constexpr int DEC_CTAS_PER_SM = DH == 128 ? 2 : 4;   // as many as shared memory holds
+constexpr int MIN_SHARE = 8;       // granules of a share at least: a piece costs about as much again
+constexpr int LONG_SHARE = 128;    // granules of a share at least where there are more shares than blocks that fit
+constexpr int MAX_ROUNDS = 16;     // shares per block that fits, at most
 constexpr int MAX_DEC_GROUPS = 64;
 constexpr int MAX_MEMBERS = 4;     // layers of a donor group served by one pass (rows = members * G <= 16)
 
@@ -43,11 +62,66 @@ struct DecParams {
   DecGroup grp[MAX_DEC_GROUPS];
   const int32_t* block_table;  // [B, max_pages]
   const int32_t* lengths;      // [B]
-  float* part_o;               // [n_groups][B][Hkv][NS][16][DH]
-  float* part_ml;              // [n_groups][B][Hkv][NS][16][2]
-  int B, Hq, Hkv, page_size, max_pages, n_pages, num_splits;
+  float* part_o;               // [pieces][rows][DH]
+  float* part_ml;              // [pieces][rows][2]
+  int rows;                    // query rows of the largest group
+  int n_groups, B, Hq, Hkv, page_size, max_pages, n_pages;
+  int blocks;                  // MAX_ROUNDS times the blocks that fit on the device
+  int max_shares;              // most shares of one group's list (divides blocks)
+  int by_units;                // the lists are short at any length: whole units are dealt out, no sums are formed
+  int num_splits;              // > 0: the caller's split count instead; a block is one (unit, split)
   int io_f32;                  // queries are read and outputs written as fp32 (rounded to bf16 on load / widened on store)
   float scale_log2;
+};
+
+__device__ __forceinline__ int clamped_length(const DecParams& p, int b) {
+  return min(max(p.lengths[b], 1), p.max_pages * p.page_size);
+}
+__device__ __forceinline__ int granules_of(int len) { return (len + GRAN - 1) / GRAN; }
+
+// Sums over the batch, formed by one warp: granules (of one KV head) of the sequences before b_before, and of all.
+__device__ __forceinline__ void sum_granules(const DecParams& p, int b_before, int& before, int& all) {
+  before = all = 0;
+  for (int b = threadIdx.x & 31; b < p.B; b += 32) {
+    const int n = granules_of(clamped_length(p, b));
+    all += n;
+    before += b < b_before ? n : 0;
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    before += __shfl_xor_sync(0xffffffffu, before, s);
+    all += __shfl_xor_sync(0xffffffffu, all, s);
+  }
+}
+// Shares a list of `total` granules is dealt out in: always a divisor of `blocks`, so that a block's shares of different
+// groups start at the same place of their lists.  The divisors tried are blocks / 2^k, then powers of two.
+__host__ __device__ inline int fewer_shares(int blocks, int n) {
+  if (n % 2 == 0) return n / 2;
+  int pow2 = blocks & -blocks;
+  while (pow2 >= n) pow2 /= 2;
+  return pow2 > 0 ? pow2 : 1;
+}
+__host__ __device__ inline bool dealt_by_units(long long total, int units) {
+  return total < 32ll * units || (total < 64ll * units && units >= 64);
+}
+__host__ __device__ inline int shares_for(int blocks, int max_shares, long long total) {
+  int n = max_shares;
+  while (n > 1 && n * (long long)(n > blocks / MAX_ROUNDS ? LONG_SHARE : MIN_SHARE) > total) n = fewer_shares(blocks, n);
+  return n;
+}
+// The first T mod n of n shares of a list of T granules hold one more than the others.
+__device__ __forceinline__ uint32_t div_long(long long a, uint32_t b) {   // quotients here fit 32 bits; so do nearly all dividends
+  return a <= 0xffffffffll ? uint32_t(a) / b : uint32_t(a / b);
+}
+struct Dealt {
+  uint32_t q, r;
+  __device__ __forceinline__ Dealt(long long total, uint32_t n) : q(div_long(total, n)), r(uint32_t(total - (long long)q * n)) {}
+  __device__ __forceinline__ long long begin(uint32_t i) const { return (long long)i * q + min(i, r); }
+  __device__ __forceinline__ uint32_t size(uint32_t i) const { return q + (i < r ? 1u : 0u); }
+  __device__ __forceinline__ int share_of(long long g) const {
+    const long long longer = (long long)r * (q + 1);
+    return g < longer ? int(div_long(g, q + 1)) : int(r + div_long(g - longer, q));
+  }
 };
 
 // 16-byte asynchronous copy; with src_bytes == 0 nothing is read and the destination is filled with zeros
@@ -90,11 +164,12 @@ __device__ __forceinline__ uint32_t ring_off(int row, int chunk) {
 }
 
 template <int DH>
-__global__ void __launch_bounds__(DEC_THREADS, 2) decode_kernel(const __grid_constant__ DecParams p) {
+__global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kernel(const __grid_constant__ DecParams p) {
   constexpr int ROW_BYTES = DH * 2;
   constexpr int CHUNKS = ROW_BYTES / 16;           // 16-byte chunks per row
   constexpr int TILE_BYTES = GRAN * ROW_BYTES;     // K (or V) part of a stage
   constexpr int STAGE_BYTES = 2 * TILE_BYTES;
+  constexpr int STAGES = DEC_STAGES;
   constexpr int CP_PER_LANE = TILE_BYTES / 16 / 32;
   constexpr int KSTEPS = DH / 16;
   constexpr int NBLK = DH / 8;
@@ -103,263 +178,502 @@ __global__ void __launch_bounds__(DEC_THREADS, 2) decode_kernel(const __grid_con
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-
-  const int split = blockIdx.x;
-  const int b = blockIdx.y / p.Hkv;
-  const int hk = blockIdx.y % p.Hkv;
-  const int gi = blockIdx.z;
-  const DecGroup& grp = p.grp[gi];
   const int G = p.Hq / p.Hkv;
-  const int R = grp.n_members * G;  // valid query rows (<= 16)
+  __shared__ float2 s_o[2][NBLK * 32];             // eight rows of two warps' results while a block merges its four
+  __shared__ float2 s_ml[2][32];
   grid_dep_wait();
-
-  int len = p.lengths[b];
-  const int cap = p.max_pages * p.page_size;
-  if (len < 1 || len > cap) {
-    if (threadIdx.x == 0) atomicOr(&g_dec_status, 2);  // clamped length
-    len = len < 1 ? 1 : cap;
+  if (blockIdx.x == 0 && warp == 0) {
+    for (int b = lane; b < p.B; b += 32)
+      if (p.lengths[b] < 1 || p.lengths[b] > p.max_pages * p.page_size) atomicOr(&g_dec_status, 2);  // clamped length
   }
-  // this split's token range, in whole granules
-  const int n_gran = (len + GRAN - 1) / GRAN;
-  const int gran_per_split = (n_gran + p.num_splits - 1) / p.num_splits;
-  const int gran_begin = split * gran_per_split;
-  const int gran_end = min(n_gran, gran_begin + gran_per_split);
 
-  // ---- query fragments (A operand, rows = members x heads of the group, zero beyond R) ----
-  uint32_t qa[KSTEPS][4];
-  {
-    const int r0 = g, r1 = g + 8;
-    const size_t off0 = r0 < R ? (size_t(b) * p.Hq + hk * G + r0 % G) * DH : 0;
-    const size_t off1 = r1 < R ? (size_t(b) * p.Hq + hk * G + r1 % G) * DH : 0;
-    auto pair_at = [&](const void* base, size_t off, int c) -> uint32_t {   // elements c, c+1 of a query row as bf16
-      if (p.io_f32) {
-        const float2 f = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + off + c);
-        return pack_bf16(f.x, f.y);
+  // A position in the list of granules: unit (grp, b, hk), granule `gran` of its `ng`.
+  struct Cursor {
+    int grp, b, hk, gran, ng, len;
+    int id;                                        // the unit's number, where units are dealt out
+  };
+  Cursor c;                                        // start of the block's next piece
+  int todo;                                        // granules of the block's share of a group's list still to do
+  int n_shares = 1, group_step = p.n_groups;       // the block's groups: c.grp, c.grp + group_step, ...
+  const bool caller_splits = p.num_splits > 0;
+  auto go_to_unit = [&](Cursor& x, int id) {       // (past the last unit: grp >= n_groups)
+    x.id = id;
+    x.hk = id % p.Hkv;
+    x.b = id / p.Hkv % p.B;
+    x.grp = id / p.Hkv / p.B;
+    x.gran = 0;
+    x.len = clamped_length(p, x.b);
+    x.ng = granules_of(x.len);
+  };
+  long long total = 0;
+  bool by_units = p.by_units != 0;
+  if (!caller_splits && !by_units) {
+    int before, all;
+    sum_granules(p, 0, before, all);
+    total = (long long)all * p.Hkv;
+    by_units = dealt_by_units(total, p.B * p.Hkv);
+  }
+  if (caller_splits) {
+    const int split = blockIdx.x % p.num_splits;
+    go_to_unit(c, blockIdx.x / p.num_splits);
+    const int per = (c.ng + p.num_splits - 1) / p.num_splits;
+    c.gran = min(c.ng, split * per);
+    todo = min(c.ng - c.gran, per);
+  } else if (by_units) {
+    go_to_unit(c, blockIdx.x);
+    if (c.grp >= p.n_groups) return;
+    todo = c.ng;
+  } else {
+    n_shares = shares_for(p.blocks, p.max_shares, total);
+    group_step = p.blocks / n_shares;
+    c.id = 0;
+    c.grp = blockIdx.x / n_shares;
+    if (c.grp >= p.n_groups) return;
+    const int share = blockIdx.x % n_shares;
+    const Dealt dealt(total, n_shares);
+    long long at = dealt.begin(share);             // find its sequence, 32 lengths at a time
+    todo = int(dealt.size(share));
+    for (int b0 = 0;; b0 += 32) {
+      const int mine = b0 + lane < p.B ? granules_of(clamped_length(p, b0 + lane)) : 0;
+      int upto = mine;
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, upto, s);
+        if (lane >= s) upto += v;
       }
-      return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(base) + off + c);
-    };
-    const void* q0 = r0 < R ? grp.q[r0 / G] : nullptr;
-    const void* q1 = r1 < R ? grp.q[r1 / G] : nullptr;
-#pragma unroll
-    for (int ks = 0; ks < KSTEPS; ++ks) {
-      const int c = ks * 16 + t * 2;
-      qa[ks][0] = q0 ? pair_at(q0, off0, c) : 0u;
-      qa[ks][1] = q1 ? pair_at(q1, off1, c) : 0u;
-      qa[ks][2] = q0 ? pair_at(q0, off0, c + 8) : 0u;
-      qa[ks][3] = q1 ? pair_at(q1, off1, c + 8) : 0u;
+      const uint32_t hit = __ballot_sync(0xffffffffu, at < (long long)upto * p.Hkv);
+      if (hit != 0u) {
+        const int src = __ffs(hit) - 1;
+        at -= (long long)__shfl_sync(0xffffffffu, upto - mine, src) * p.Hkv;
+        c.b = b0 + src;
+        break;
+      }
+      at -= (long long)__shfl_sync(0xffffffffu, upto, 31) * p.Hkv;
     }
+    c.len = clamped_length(p, c.b);
+    c.ng = granules_of(c.len);
+    c.hk = int(at) / c.ng;                         // (a sequence's granules of all KV heads fit 32 bits)
+    c.gran = int(at) % c.ng;
   }
 
-  float oacc[NBLK][4];
-#pragma unroll
-  for (int n = 0; n < NBLK; ++n) oacc[n][0] = oacc[n][1] = oacc[n][2] = oacc[n][3] = 0.f;
-  float m_run[2] = {-INFINITY, -INFINITY};  // rows g, g+8 (log2 domain)
-  float l_run[2] = {0.f, 0.f};              // per-lane partial sums
-
-  uint8_t* ring = dsmem + size_t(warp) * DEC_STAGES * STAGE_BYTES;
+  uint8_t* ring = dsmem + size_t(warp) * STAGES * STAGE_BYTES;
   const uint32_t ring_u32 = smem_u32(ring);
-  const int32_t* bt = p.block_table + size_t(b) * p.max_pages;
 
-  auto issue = [&](int gran, int stage) {
-    const int tok = gran * GRAN;
-    int page = bt[tok / p.page_size];
-    page = min(max(page, 0), p.n_pages - 1);
-    const size_t elem = ((size_t(page) * p.Hkv + hk) * p.page_size + tok % p.page_size) * DH;
-    const uint8_t* ksrc = reinterpret_cast<const uint8_t*>(grp.k_cache + elem);
-    const uint8_t* vsrc = reinterpret_cast<const uint8_t*>(grp.v_cache + elem);
-    const uint32_t dst = ring_u32 + stage * STAGE_BYTES;
-#pragma unroll
-    for (int i = 0; i < CP_PER_LANE; ++i) {
-      const int idx = i * 32 + lane;          // 16-byte chunk index inside the contiguous granule
-      const int row = idx / CHUNKS, chunk = idx % CHUNKS;
-      const uint32_t off = ring_off<DH>(row, chunk);
-      // Slots at or past the sequence length were never appended and may hold anything (a NaN there would
-      // survive the zero probability in P V): they are filled with zeros instead of being read.
-      const uint32_t nbytes = tok + row < len ? 16u : 0u;
-      cp_async16(dst + off, ksrc + size_t(idx) * 16, nbytes);
-      cp_async16(dst + TILE_BYTES + off, vsrc + size_t(idx) * 16, nbytes);
+  const Cursor start = c;
+  const int share_len = todo;
+  auto next_unit = [&](Cursor& x) {                // (wraps at the end of the list, where a share ends too)
+    x.gran = 0;
+    if (++x.hk == p.Hkv) {
+      x.hk = 0;
+      if (++x.b == p.B) x.b = 0;
+      x.len = clamped_length(p, x.b);
+      x.ng = granules_of(x.len);
+    }
+  };
+  // The piece behind the one at x, of the `left` granules of the block's share from x on; past the end: grp >= n_groups.
+  auto next_piece = [&](Cursor& x, int& left) {
+    left -= min(left, x.ng - x.gran);
+    if (left > 0) {
+      next_unit(x);
+    } else if (caller_splits) {
+      x.grp = p.n_groups;
+    } else if (by_units) {
+      go_to_unit(x, x.id + gridDim.x);
+      left = x.ng;
+    } else {
+      const int grp = x.grp + group_step;
+      x = start;
+      x.grp = grp;
+      left = share_len;
     }
   };
 
-  // granules of the split are dealt round-robin to the warps
-  const int first = gran_begin + warp;
-  int n_mine = first < gran_end ? (gran_end - first + DEC_WARPS - 1) / DEC_WARPS : 0;
-#pragma unroll
-  for (int s = 0; s < DEC_STAGES - 1; ++s) {
-    if (s < n_mine) issue(first + s * DEC_WARPS, s);
-    cp_async_commit();
-  }
-  for (int i = 0; i < n_mine; ++i) {
-    cp_async_wait<DEC_STAGES - 2>();
-    __syncwarp();
-    // prefetch granule i + STAGES-1 into the stage freed by iteration i-1
-    {
-      const int nx = i + DEC_STAGES - 1;
-      if (nx < n_mine) issue(first + nx * DEC_WARPS, nx % DEC_STAGES);
-      cp_async_commit();
+  // ---- copies: a cursor of their own, STAGES - 1 of this warp's granules ahead of the arithmetic ----
+  Cursor f = c;                                    // start of the piece the copies are in
+  int f_todo = todo;                               // granules of the share from there on
+  int f_left;                                      // granules of the piece from this warp's next one on (<= 0: none)
+  const int gran_per_page = p.page_size / GRAN;
+  const uint8_t *kbase = nullptr, *vbase = nullptr;   // the group's pools
+  const int32_t* bt = nullptr;                     // block-table entry of the page the next granule is in,
+  int in_page = 0, f_tok = 0;                      // its place there, and its first token
+  size_t page_elem = 0;                            // offset of this KV head's block of that page
+  int stage_in = 0;
+  auto enter_page = [&]() {
+    const int page = min(max(*bt, 0), p.n_pages - 1);
+    page_elem = (size_t(page) * p.Hkv + f.hk) * p.page_size;
+  };
+  auto enter_piece = [&]() {
+    f_left = min(f_todo, f.ng - f.gran) - warp;
+    if (f_left <= 0) return;
+    const int gran = f.gran + warp, col = gran / gran_per_page;
+    kbase = reinterpret_cast<const uint8_t*>(p.grp[f.grp].k_cache);
+    vbase = reinterpret_cast<const uint8_t*>(p.grp[f.grp].v_cache);
+    bt = p.block_table + size_t(f.b) * p.max_pages + col;
+    in_page = gran - col * gran_per_page;
+    f_tok = gran * GRAN;
+    enter_page();
+  };
+  auto issue_next = [&]() {
+    // find the piece that holds the next granule of this warp (pieces may be shorter than the block has warps)
+    while (f_left <= 0 && f.grp < p.n_groups) {
+      next_piece(f, f_todo);
+      if (f.grp < p.n_groups) enter_piece();
     }
-    const int gran = first + i * DEC_WARPS;
-    const uint32_t sK = ring_u32 + (i % DEC_STAGES) * STAGE_BYTES;
-    const uint32_t sV = sK + TILE_BYTES;
-
-    // ---- S[16 rows, 16 tokens] = Q K^T ----
-    float sacc[2][4];
+    if (f_left > 0) {
+      const size_t at = (page_elem + size_t(in_page) * GRAN) * ROW_BYTES;
+      const uint8_t* ksrc = kbase + at;
+      const uint8_t* vsrc = vbase + at;
+      const uint32_t dst = ring_u32 + stage_in * STAGE_BYTES;
 #pragma unroll
-    for (int nb = 0; nb < 2; ++nb) sacc[nb][0] = sacc[nb][1] = sacc[nb][2] = sacc[nb][3] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < KSTEPS; ++ks) {
-      // four 8x8 matrices: (tokens 0-7, dh ks*16..+7), (tokens 0-7, +8..15), (tokens 8-15, ...), (tokens 8-15, +8)
-      const int mat = lane >> 3, rr = lane & 7;
-      const int row = (mat >> 1) * 8 + rr;
-      const int chunk = ks * 2 + (mat & 1);
-      uint32_t b00, b01, b10, b11;
-      ldsm_x4(sK + ring_off<DH>(row, chunk), b00, b01, b10, b11);
-      mma_bf16(sacc[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b00, b01);
-      mma_bf16(sacc[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b10, b11);
-    }
-    // ---- online softmax over the 16 tokens ----
-    const int tok0 = gran * GRAN;
-    float mt[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-    for (int nb = 0; nb < 2; ++nb) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int tk = tok0 + nb * 8 + t * 2 + (u & 1);
-        float x = sacc[nb][u] * p.scale_log2;
-        if (tk >= len) x = -INFINITY;
-        sacc[nb][u] = x;
-        mt[u >> 1] = fmaxf(mt[u >> 1], x);
+      for (int i = 0; i < CP_PER_LANE; ++i) {
+        const int idx = i * 32 + lane;          // 16-byte chunk index inside the contiguous granule
+        const int row = idx / CHUNKS, chunk = idx % CHUNKS;
+        const uint32_t off = ring_off<DH>(row, chunk);
+        // Slots at or past the sequence length were never appended and may hold anything (a NaN there would
+        // survive the zero probability in P V): they are filled with zeros instead of being read.
+        const uint32_t nbytes = f_tok + row < f.len ? 16u : 0u;
+        cp_async16(dst + off, ksrc + size_t(idx) * 16, nbytes);
+        cp_async16(dst + TILE_BYTES + off, vsrc + size_t(idx) * 16, nbytes);
+      }
+      if (++stage_in == STAGES) stage_in = 0;
+      f_left -= DEC_WARPS;
+      f_tok += DEC_WARPS * GRAN;
+      in_page += DEC_WARPS;
+      if (in_page >= gran_per_page && f_left > 0) {
+        const int pages = in_page / gran_per_page;
+        bt += pages;
+        in_page -= pages * gran_per_page;
+        enter_page();
       }
     }
-    float alpha[2];
+    cp_async_commit();
+  };
+  enter_piece();
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      mt[h] = fmaxf(mt[h], __shfl_xor_sync(0xffffffffu, mt[h], 1));
-      mt[h] = fmaxf(mt[h], __shfl_xor_sync(0xffffffffu, mt[h], 2));
-      const float m_new = fmaxf(m_run[h], mt[h]);
-      alpha[h] = m_run[h] == -INFINITY ? 0.f : fast_exp2(m_run[h] - m_new);
-      m_run[h] = m_new;
-      l_run[h] *= alpha[h];
-    }
-    uint32_t pa[4];
+  for (int s = 0; s < STAGES - 1; ++s) issue_next();
+
+  int stage_out = 0;
+  do {
+    // ---- one unit, or this block's piece of it ----
+    const DecGroup& grp = p.grp[c.grp];
+    const int R = grp.n_members * G;               // valid query rows (<= 16)
+    const int n_here = min(todo, c.ng - c.gran);
+    const bool from_start = c.gran == 0, to_end = c.gran + n_here == c.ng;
+
+    // query fragments (A operand, rows = members x heads of the group, zero beyond R)
+    uint32_t qa[KSTEPS][4];
     {
-      float pr[2][4];
+      const int r0 = g, r1 = g + 8;
+      const size_t off0 = r0 < R ? (size_t(c.b) * p.Hq + c.hk * G + r0 % G) * DH : 0;
+      const size_t off1 = r1 < R ? (size_t(c.b) * p.Hq + c.hk * G + r1 % G) * DH : 0;
+      auto pair_at = [&](const void* base, size_t off, int col) -> uint32_t {   // two elements of a query row as bf16
+        if (p.io_f32) {
+          const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + off + col);
+          return pack_bf16(v.x, v.y);
+        }
+        return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(base) + off + col);
+      };
+      const void* q0 = r0 < R ? grp.q[r0 / G] : nullptr;
+      const void* q1 = r1 < R ? grp.q[r1 / G] : nullptr;
 #pragma unroll
-      for (int nb = 0; nb < 2; ++nb)
+      for (int ks = 0; ks < KSTEPS; ++ks) {
+        const int col = ks * 16 + t * 2;
+        qa[ks][0] = q0 ? pair_at(q0, off0, col) : 0u;
+        qa[ks][1] = q1 ? pair_at(q1, off1, col) : 0u;
+        qa[ks][2] = q0 ? pair_at(q0, off0, col + 8) : 0u;
+        qa[ks][3] = q1 ? pair_at(q1, off1, col + 8) : 0u;
+      }
+    }
+
+    float oacc[NBLK][4];
+#pragma unroll
+    for (int n = 0; n < NBLK; ++n) oacc[n][0] = oacc[n][1] = oacc[n][2] = oacc[n][3] = 0.f;
+    float m_run[2] = {-INFINITY, -INFINITY};  // rows g, g+8 (log2 domain)
+    float l_run[2] = {0.f, 0.f};              // per-lane partial sums
+
+    for (int i = warp; i < n_here; i += DEC_WARPS) {
+      cp_async_wait<STAGES - 2>();
+      __syncwarp();
+      issue_next();   // into the stage freed by the previous granule
+      const int gran = c.gran + i;
+      const uint32_t sK = ring_u32 + stage_out * STAGE_BYTES;
+      const uint32_t sV = sK + TILE_BYTES;
+      if (++stage_out == STAGES) stage_out = 0;
+
+      // ---- S[16 rows, 16 tokens] = Q K^T ----
+      float sacc[2][4];
+#pragma unroll
+      for (int nb = 0; nb < 2; ++nb) sacc[nb][0] = sacc[nb][1] = sacc[nb][2] = sacc[nb][3] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < KSTEPS; ++ks) {
+        // four 8x8 matrices: (tokens 0-7, dh ks*16..+7), (tokens 0-7, +8..15), (tokens 8-15, ...), (tokens 8-15, +8)
+        const int mat = lane >> 3, rr = lane & 7;
+        const int row = (mat >> 1) * 8 + rr;
+        const int chunk = ks * 2 + (mat & 1);
+        uint32_t b00, b01, b10, b11;
+        ldsm_x4(sK + ring_off<DH>(row, chunk), b00, b01, b10, b11);
+        mma_bf16(sacc[0], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b00, b01);
+        mma_bf16(sacc[1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b10, b11);
+      }
+      // ---- online softmax over the 16 tokens ----
+      const int tok0 = gran * GRAN;
+      float mt[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+      for (int nb = 0; nb < 2; ++nb) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          pr[nb][u] = fast_exp2(sacc[nb][u] - m_run[u >> 1]);
-          l_run[u >> 1] += pr[nb][u];
+          const int tk = tok0 + nb * 8 + t * 2 + (u & 1);
+          float x = sacc[nb][u] * p.scale_log2;
+          if (tk >= c.len) x = -INFINITY;
+          sacc[nb][u] = x;
+          mt[u >> 1] = fmaxf(mt[u >> 1], x);
         }
-      pa[0] = pack_bf16(pr[0][0], pr[0][1]);
-      pa[1] = pack_bf16(pr[0][2], pr[0][3]);
-      pa[2] = pack_bf16(pr[1][0], pr[1][1]);
-      pa[3] = pack_bf16(pr[1][2], pr[1][3]);
-    }
-    if (!__all_sync(0xffffffffu, alpha[0] == 1.f && alpha[1] == 1.f)) {
+      }
+      float alpha[2];
 #pragma unroll
-      for (int n = 0; n < NBLK; ++n) {
-        oacc[n][0] *= alpha[0];
-        oacc[n][1] *= alpha[0];
-        oacc[n][2] *= alpha[1];
-        oacc[n][3] *= alpha[1];
+      for (int h = 0; h < 2; ++h) {
+        mt[h] = fmaxf(mt[h], __shfl_xor_sync(0xffffffffu, mt[h], 1));
+        mt[h] = fmaxf(mt[h], __shfl_xor_sync(0xffffffffu, mt[h], 2));
+        const float m_new = fmaxf(m_run[h], mt[h]);
+        alpha[h] = m_run[h] == -INFINITY ? 0.f : fast_exp2(m_run[h] - m_new);
+        m_run[h] = m_new;
+        l_run[h] *= alpha[h];
+      }
+      uint32_t pa[4];
+      {
+        float pr[2][4];
+#pragma unroll
+        for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            pr[nb][u] = fast_exp2(sacc[nb][u] - m_run[u >> 1]);
+            l_run[u >> 1] += pr[nb][u];
+          }
+        pa[0] = pack_bf16(pr[0][0], pr[0][1]);
+        pa[1] = pack_bf16(pr[0][2], pr[0][3]);
+        pa[2] = pack_bf16(pr[1][0], pr[1][1]);
+        pa[3] = pack_bf16(pr[1][2], pr[1][3]);
+      }
+      if (!__all_sync(0xffffffffu, alpha[0] == 1.f && alpha[1] == 1.f)) {
+#pragma unroll
+        for (int n = 0; n < NBLK; ++n) {
+          oacc[n][0] *= alpha[0];
+          oacc[n][1] *= alpha[0];
+          oacc[n][2] *= alpha[1];
+          oacc[n][3] *= alpha[1];
+        }
+      }
+      // ---- O[16 rows, DH] += P[16 rows, 16 tokens] V[16 tokens, DH] ----
+#pragma unroll
+      for (int n2 = 0; n2 < NBLK / 2; ++n2) {
+        // four 8x8 matrices (transposed on load): (tokens 0-7, dh n2*16..+7), (tokens 8-15, same dh),
+        // (tokens 0-7, dh +8..15), (tokens 8-15, dh +8..15)
+        const int mat = lane >> 3, rr = lane & 7;
+        const int row = (mat & 1) * 8 + rr;
+        const int chunk = n2 * 2 + (mat >> 1);
+        uint32_t v00, v01, v10, v11;
+        ldsm_x4_t(sV + ring_off<DH>(row, chunk), v00, v01, v10, v11);
+        mma_bf16(oacc[2 * n2], pa[0], pa[1], pa[2], pa[3], v00, v01);
+        mma_bf16(oacc[2 * n2 + 1], pa[0], pa[1], pa[2], pa[3], v10, v11);
+      }
+      __syncwarp();  // every lane is done with this stage before it is refilled
+    }
+    const Cursor here = c;
+    next_piece(c, todo);
+    const bool last = c.grp >= p.n_groups;
+    if (last) grid_dep_launch();   // this warp's loads are out, the others' within a granule
+
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
+      l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
+    }
+    // ---- merge the four warps of the block, eight rows at a time: 2 into 0 and 3 into 1, then 1 into 0 ----
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (8 * h >= R) break;
+      auto put = [&](int slot) {
+#pragma unroll
+        for (int n = 0; n < NBLK; ++n) s_o[slot][n * 32 + lane] = make_float2(oacc[n][2 * h], oacc[n][2 * h + 1]);
+        s_ml[slot][lane] = make_float2(m_run[h], l_run[h]);
+      };
+      auto take = [&](int slot) {
+        const float2 om = s_ml[slot][lane];
+        const float mn = fmaxf(m_run[h], om.x);
+        const float fa = m_run[h] == -INFINITY ? 0.f : fast_exp2(m_run[h] - mn);
+        const float fb = om.x == -INFINITY ? 0.f : fast_exp2(om.x - mn);
+        m_run[h] = mn;
+        l_run[h] = l_run[h] * fa + om.y * fb;
+#pragma unroll
+        for (int n = 0; n < NBLK; ++n) {
+          const float2 v = s_o[slot][n * 32 + lane];
+          oacc[n][2 * h] = oacc[n][2 * h] * fa + v.x * fb;
+          oacc[n][2 * h + 1] = oacc[n][2 * h + 1] * fa + v.y * fb;
+        }
+      };
+      if (warp >= 2) put(warp - 2);
+      __syncthreads();
+      if (warp < 2) take(warp);
+      __syncthreads();
+      if (warp == 1) put(1);
+      __syncthreads();
+      if (warp == 0) take(1);
+      __syncthreads();
+    }
+    if (warp != 0) {
+      // (warp 0 alone goes on to store)
+    } else if (!caller_splits && from_start && to_end) {
+      // ---- the whole unit: normalise and store ----
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = g + 8 * h;
+        if (row < R) {
+          const int mem = row / G;
+          const size_t head = size_t(here.b) * p.Hq + here.hk * G + row % G;
+          const float inv = 1.f / l_run[h];
+#pragma unroll
+          for (int n = 0; n < NBLK; ++n) {
+            const uint32_t v = pack_bf16(oacc[n][2 * h] * inv, oacc[n][2 * h + 1] * inv);   // rounded to bf16 either way: one set of results
+            const size_t at = head * DH + n * 8 + t * 2;
+            if (p.io_f32)
+              *reinterpret_cast<float2*>(reinterpret_cast<float*>(grp.o[mem]) + at) = make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+            else
+              *reinterpret_cast<uint32_t*>(reinterpret_cast<__nv_bfloat16*>(grp.o[mem]) + at) = v;
+          }
+          if (t == 0) grp.lse[mem][head] = (m_run[h] + log2f(l_run[h])) * 0.6931471805599453f;
+        }
+      }
+    } else {
+      // ---- a piece: the first of a share, or the last one if that starts a unit ----
+      const size_t piece = caller_splits ? size_t(blockIdx.x) : (size_t(here.grp) * n_shares + blockIdx.x % n_shares) * 2 + (from_start ? 1 : 0);
+      float* po = p.part_o + piece * p.rows * DH;
+      float* pml = p.part_ml + piece * p.rows * 2;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = g + 8 * h;
+        if (row < R) {
+#pragma unroll
+          for (int n = 0; n < NBLK; ++n)
+            *reinterpret_cast<float2*>(po + row * DH + n * 8 + t * 2) = make_float2(oacc[n][2 * h], oacc[n][2 * h + 1]);
+          if (t == 0) *reinterpret_cast<float2*>(pml + row * 2) = make_float2(m_run[h], l_run[h]);
+        }
       }
     }
-    // ---- O[16 rows, DH] += P[16 rows, 16 tokens] V[16 tokens, DH] ----
-#pragma unroll
-    for (int n2 = 0; n2 < NBLK / 2; ++n2) {
-      // four 8x8 matrices (transposed on load): (tokens 0-7, dh n2*16..+7), (tokens 8-15, same dh),
-      // (tokens 0-7, dh +8..15), (tokens 8-15, dh +8..15)
-      const int mat = lane >> 3, rr = lane & 7;
-      const int row = (mat & 1) * 8 + rr;
-      const int chunk = n2 * 2 + (mat >> 1);
-      uint32_t v00, v01, v10, v11;
-      ldsm_x4_t(sV + ring_off<DH>(row, chunk), v00, v01, v10, v11);
-      mma_bf16(oacc[2 * n2], pa[0], pa[1], pa[2], pa[3], v00, v01);
-      mma_bf16(oacc[2 * n2 + 1], pa[0], pa[1], pa[2], pa[3], v10, v11);
-    }
-    __syncwarp();  // every lane is done with this stage before it is refilled
-  }
-  grid_dep_launch();   // every load of this CTA is out
+    if (last) break;
+  } while (true);
   cp_async_wait<0>();
-
-  // ---- merge the four warps of the CTA, then write this split's partial ----
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
-    l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
-  }
-  __syncthreads();  // all rings are idle: reuse the memory
-  float* s_o = reinterpret_cast<float*>(dsmem);                   // [DEC_WARPS][16][DH]
-  float* s_ml = s_o + DEC_WARPS * 16 * DH;                        // [DEC_WARPS][16][2]
-#pragma unroll
-  for (int n = 0; n < NBLK; ++n) {
-    float* base = s_o + (size_t(warp) * 16) * DH + n * 8 + t * 2;
-    base[size_t(g) * DH] = oacc[n][0];
-    base[size_t(g) * DH + 1] = oacc[n][1];
-    base[size_t(g + 8) * DH] = oacc[n][2];
-    base[size_t(g + 8) * DH + 1] = oacc[n][3];
-  }
-  if (t == 0) {
-    s_ml[(warp * 16 + g) * 2] = m_run[0];
-    s_ml[(warp * 16 + g) * 2 + 1] = l_run[0];
-    s_ml[(warp * 16 + g + 8) * 2] = m_run[1];
-    s_ml[(warp * 16 + g + 8) * 2 + 1] = l_run[1];
-  }
-  __syncthreads();
-  const size_t unit = ((size_t(gi) * p.B + b) * p.Hkv + hk) * p.num_splits + split;
-  float* po = p.part_o + unit * 16 * DH;
-  float* pml = p.part_ml + unit * 16 * 2;
-  for (int idx = threadIdx.x; idx < R * DH; idx += DEC_THREADS) {
-    const int row = idx / DH, col = idx % DH;
-    float mm = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < DEC_WARPS; ++w) mm = fmaxf(mm, s_ml[(w * 16 + row) * 2]);
-    float acc = 0.f, ll = 0.f;
-#pragma unroll
-    for (int w = 0; w < DEC_WARPS; ++w) {
-      const float mw = s_ml[(w * 16 + row) * 2];
-      const float f = mw == -INFINITY ? 0.f : fast_exp2(mw - mm);
-      acc += f * s_o[(size_t(w) * 16 + row) * DH + col];
-      ll += f * s_ml[(w * 16 + row) * 2 + 1];
-    }
-    po[size_t(row) * DH + col] = acc;
-    if (col == 0) {
-      pml[row * 2] = mm;
-      pml[row * 2 + 1] = ll;
-    }
-  }
 }
 
-// One CTA per (group, sequence, KV head): merge the splits and write bf16 outputs and LSE.
+// Merges the pieces of the units that more than one share holds and writes bf16 outputs and LSE.  Eight warps per block;
+// `wpr` of them share a row of a unit (one where a unit has few pieces, eight where it has many), each lane four
+// columns.  Bound: latency; the pieces are in L2.
+constexpr int COMBINE_THREADS = 256;
 template <int DH>
-__global__ void decode_combine_kernel(const __grid_constant__ DecParams p) {
-  const int b = blockIdx.y / p.Hkv;
-  const int hk = blockIdx.y % p.Hkv;
-  const int gi = blockIdx.z;
-  const DecGroup& grp = p.grp[gi];
+__global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const __grid_constant__ DecParams p, int wpr) {
+  constexpr int LANES = DH / 4;               // lanes per piece and row
+  constexpr int PER_WARP = 32 / LANES;        // pieces a warp takes at a time
+  __shared__ float s_m[COMBINE_THREADS / 32], s_l[COMBINE_THREADS / 32];
+  __shared__ float4 s_o[COMBINE_THREADS / 32][LANES];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rows_per_block = (COMBINE_THREADS / 32) / wpr;
   const int G = p.Hq / p.Hkv;
+  const int unit = blockIdx.x;
+  const int hk = unit % p.Hkv, b = unit / p.Hkv % p.B, gi = unit / p.Hkv / p.B;
+  const DecGroup& grp = p.grp[gi];
   const int R = grp.n_members * G;
+  const int row = blockIdx.y * rows_per_block + warp / wpr;
   grid_dep_launch();
   grid_dep_wait();
-  const size_t unit0 = ((size_t(gi) * p.B + b) * p.Hkv + hk) * p.num_splits;
-  for (int idx = threadIdx.x; idx < R * DH; idx += blockDim.x) {
-    const int row = idx / DH, col = idx % DH;
-    float mm = -INFINITY;
-    for (int s = 0; s < p.num_splits; ++s) mm = fmaxf(mm, p.part_ml[((unit0 + s) * 16 + row) * 2]);
-    float acc = 0.f, ll = 0.f;
-    for (int s = 0; s < p.num_splits; ++s) {
-      const float ms = p.part_ml[((unit0 + s) * 16 + row) * 2];
-      const float f = ms == -INFINITY ? 0.f : fast_exp2(ms - mm);
-      acc += f * p.part_o[((unit0 + s) * 16 + row) * DH + col];
-      ll += f * p.part_ml[((unit0 + s) * 16 + row) * 2 + 1];
+  if (blockIdx.y * rows_per_block >= R) return;
+  int w0, w1;                                 // shares (or splits) that hold the unit
+  size_t piece0 = 0;
+  if (p.num_splits > 0) {
+    w0 = unit * p.num_splits;
+    w1 = w0 + p.num_splits - 1;
+  } else {
+    int before, all;
+    sum_granules(p, b, before, all);
+    const long long total = (long long)all * p.Hkv;
+    if (dealt_by_units(total, p.B * p.Hkv)) return;   // finished by the blocks that held them
+    const int n = shares_for(p.blocks, p.max_shares, total), ng = granules_of(clamped_length(p, b));
+    const long long first = (long long)before * p.Hkv + (long long)hk * ng;
+    const Dealt dealt(total, n);
+    w0 = dealt.share_of(first);
+    w1 = dealt.share_of(first + ng - 1);
+    piece0 = size_t(gi) * n;
+    if (w0 == w1) return;                     // finished by the block that had the share
+  }
+  const int sub = lane / LANES, col = (lane % LANES) * 4;
+  float m = -INFINITY, l = 0.f;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (row < R) {
+    constexpr int UNROLL = 4;                 // pieces in flight per lane
+    const int step = wpr * PER_WARP;
+    for (int w = w0 + (warp % wpr) * PER_WARP + sub; w <= w1; w += step * UNROLL) {
+      float2 ml[UNROLL];
+      float4 o[UNROLL];
+#pragma unroll
+      for (int u = 0; u < UNROLL; ++u) {
+        const int wu = w + u * step;
+        ml[u] = make_float2(-INFINITY, 0.f);
+        if (wu <= w1) {
+          const size_t piece = p.num_splits > 0 ? size_t(wu) : (piece0 + wu) * 2 + (wu == w0 ? 1 : 0);
+          ml[u] = *reinterpret_cast<const float2*>(p.part_ml + (piece * p.rows + row) * 2);
+          o[u] = *reinterpret_cast<const float4*>(p.part_o + (piece * p.rows + row) * DH + col);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UNROLL; ++u) {
+        if (ml[u].x == -INFINITY) continue;   // an empty split
+        const float mn = fmaxf(m, ml[u].x);
+        const float fa = m == -INFINITY ? 0.f : fast_exp2(m - mn), fb = fast_exp2(ml[u].x - mn);
+        acc.x = acc.x * fa + o[u].x * fb;
+        acc.y = acc.y * fa + o[u].y * fb;
+        acc.z = acc.z * fa + o[u].z * fb;
+        acc.w = acc.w * fa + o[u].w * fb;
+        l = l * fa + ml[u].y * fb;
+        m = mn;
+      }
     }
-    const int mem = row / G, hq = hk * G + row % G;
-    const __nv_bfloat16 val = __float2bfloat16_rn(acc / ll);   // rounded to bf16 either way: one set of results
-    const size_t at = (size_t(b) * p.Hq + hq) * DH + col;
-    if (p.io_f32) reinterpret_cast<float*>(grp.o[mem])[at] = __bfloat162float(val);
-    else reinterpret_cast<__nv_bfloat16*>(grp.o[mem])[at] = val;
-    if (col == 0) grp.lse[mem][size_t(b) * p.Hq + hq] = (mm + log2f(ll)) * 0.6931471805599453f;
+  }
+  auto merge = [&](float om, float ol, const float4& oo) {
+    if (om == -INFINITY) return;
+    const float mn = fmaxf(m, om);
+    const float fa = m == -INFINITY ? 0.f : fast_exp2(m - mn), fb = fast_exp2(om - mn);
+    acc.x = acc.x * fa + oo.x * fb;
+    acc.y = acc.y * fa + oo.y * fb;
+    acc.z = acc.z * fa + oo.z * fb;
+    acc.w = acc.w * fa + oo.w * fb;
+    l = l * fa + ol * fb;
+    m = mn;
+  };
+  if (PER_WARP == 2) {                        // the two halves of the warp hold different pieces
+    const float om = __shfl_xor_sync(0xffffffffu, m, 16), ol = __shfl_xor_sync(0xffffffffu, l, 16);
+    const float4 oo = make_float4(__shfl_xor_sync(0xffffffffu, acc.x, 16), __shfl_xor_sync(0xffffffffu, acc.y, 16),
+                                  __shfl_xor_sync(0xffffffffu, acc.z, 16), __shfl_xor_sync(0xffffffffu, acc.w, 16));
+    merge(om, ol, oo);
+  }
+  if (wpr > 1) {                              // the block's warps hold pieces of one row (uniform: every thread arrives)
+    if (lane < LANES) s_o[warp][lane] = acc;
+    if (lane == 0) {
+      s_m[warp] = m;
+      s_l[warp] = l;
+    }
+    __syncthreads();
+    if (warp % wpr != 0) return;
+    for (int k = 1; k < wpr; ++k) merge(s_m[warp + k], s_l[warp + k], s_o[warp + k][lane % LANES]);
+  }
+  if (row < R && lane < LANES) {
+    const int mem = row / G;
+    const size_t head = size_t(b) * p.Hq + hk * G + row % G;
+    const float inv = 1.f / l;
+    const uint2 v = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));   // rounded to bf16 either way
+    if (p.io_f32)
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(grp.o[mem]) + head * DH + col) =
+          make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+    else
+      *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(grp.o[mem]) + head * DH + col) = v;
+    if (lane == 0) grp.lse[mem][head] = (m + log2f(l)) * 0.6931471805599453f;
   }
 }
 
@@ -415,15 +729,6 @@ int check_desc(const kvp_decode_desc* d) {
   return KVP_OK;
 }
 
-int pick_splits(const kvp_decode_desc* d) {
-  if (d->num_splits > 0) return d->num_splits;
-  const long long cap = (long long)d->max_pages * d->page_size;
-  long long ns = (cap + 2047) / 2048;
-  if (ns < 1) ns = 1;
-  if (ns > 32) ns = 32;
-  return int(ns);
-}
-
 // Sub-groups of at most min(MAX_MEMBERS, 16 / G) layers that share a donor inside [begin, end).
 struct SubGroup {
   int owner;
@@ -460,16 +765,45 @@ int build_groups(const kvp_decode_desc* d, const int32_t* donor, int begin, int 
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Bytes of per-split partials that decoding layers [begin, end) needs: one launch holds at most MAX_DEC_GROUPS
-// sub-groups and launches reuse the space.  0 when the request cannot be served at all.
+// Pieces and their bytes.  When the library chooses: two for each share of each group's list at its longest; with the
+// caller's split count: one for every (unit, split).  One launch holds at most MAX_DEC_GROUPS sub-groups and launches
+// reuse the space.
+int decode_blocks(int dh) { return sm_count() * (dh == 128 ? DEC_CTAS_PER_SM<128> : DEC_CTAS_PER_SM<64>) * MAX_ROUNDS; }
+size_t piece_bytes(const kvp_decode_desc* d, size_t pieces, int rows) {
+  return align256(pieces * rows * d->dh * 4) + align256(pieces * rows * 2 * 4);
+}
+long long longest_list(const kvp_decode_desc* d) {
+  return (long long)d->B * d->Hkv * ((long long)d->max_pages * d->page_size / GRAN);
+}
+struct Scratch {
+  int max_shares = 0, rows = 0;
+  size_t pieces = 0, bytes = 0;
+};
+// limit > 0: fewer shares until the pieces fit into that many bytes
+Scratch plan_scratch(const kvp_decode_desc* d, const SubGroup* subs, int n_sub, size_t limit) {
+  Scratch s;
+  const size_t per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
+  for (int i = 0; i < n_sub; ++i) s.rows = std::max(s.rows, subs[i].n * (d->Hq / d->Hkv));
+  const int blocks = decode_blocks(d->dh);
+  s.max_shares = shares_for(blocks, blocks, longest_list(d));
+  for (;;) {
+    s.pieces = d->num_splits > 0 ? per_launch * d->B * d->Hkv * d->num_splits : per_launch * s.max_shares * 2;
+    s.bytes = piece_bytes(d, s.pieces, s.rows);
+    if (limit == 0 || s.bytes <= limit || d->num_splits > 0 || s.max_shares == 1) return s;
+    s.max_shares = fewer_shares(blocks, s.max_shares);
+  }
+}
+// bytes for decoding layers [begin, end); 0 when the request cannot be served at all
 size_t decode_scratch_bytes(const kvp_decode_desc* d, const int32_t* donor, int begin, int end) {
   static thread_local SubGroup tmp[4096];
   const int n_sub = build_groups(d, donor, begin, end, tmp, 4096);
-  if (n_sub <= 0) return 0;
-  const int per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
-  const size_t units = size_t(per_launch) * d->B * d->Hkv * pick_splits(d);
-  return align256(units * 16 * d->dh * 4) + align256(units * 16 * 2 * 4);
+  return n_sub <= 0 ? 0 : plan_scratch(d, tmp, n_sub, 0).bytes;
 }
+
+int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q, const void* const* k_cache,
+                const void* const* v_cache, const int32_t* block_table, const int32_t* lengths, void* const* o,
+                float* const* lse, int layer_begin, int layer_end, void* ws, size_t ws_bytes, size_t limit,
+                cudaStream_t stream);
 
 }  // namespace
 
@@ -533,10 +867,13 @@ extern "C" int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, 
   return KVP_OK;
 }
 
-extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q,
-                          const void* const* k_cache, const void* const* v_cache, const int32_t* block_table,
-                          const int32_t* lengths, void* const* o, float* const* lse, int layer_begin, int layer_end,
-                          void* ws, size_t ws_bytes, kvp_stream_t stream_) {
+namespace kvp {
+namespace {
+
+int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q, const void* const* k_cache,
+                const void* const* v_cache, const int32_t* block_table, const int32_t* lengths, void* const* o,
+                float* const* lse, int layer_begin, int layer_end, void* ws, size_t ws_bytes, size_t limit,
+                cudaStream_t stream) {
   int rc = check_desc(d);
   if (rc != KVP_OK) return rc;
   if (donor == nullptr || q == nullptr || k_cache == nullptr || v_cache == nullptr || block_table == nullptr ||
@@ -548,12 +885,9 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
   static thread_local SubGroup subs[4096];
   const int n_sub = build_groups(d, donor, layer_begin, layer_end, subs, 4096);
   if (n_sub < 0) return KVP_ERR_UNSUPPORTED;
-  const int ns = pick_splits(d);
-  const int per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
-  const size_t units = size_t(per_launch) * d->B * d->Hkv * ns;
-  const size_t po_bytes = align256(units * 16 * d->dh * 4), pml_bytes = align256(units * 16 * 2 * 4);
-  if (ws == nullptr || ws_bytes < po_bytes + pml_bytes || !aligned16(ws)) return KVP_ERR_WORKSPACE;
-  cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
+  const Scratch sc_plan = plan_scratch(d, subs, n_sub, limit);
+  if (ws == nullptr || ws_bytes < sc_plan.bytes || !aligned16(ws)) return KVP_ERR_WORKSPACE;
+  const size_t po_bytes = align256(sc_plan.pieces * sc_plan.rows * d->dh * 4);
 
   DecParams p;
   p.block_table = block_table;
@@ -566,7 +900,10 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
   p.page_size = d->page_size;
   p.max_pages = d->max_pages;
   p.n_pages = d->n_pages;
-  p.num_splits = ns;
+  p.rows = sc_plan.rows;
+  p.blocks = decode_blocks(d->dh);
+  p.max_shares = sc_plan.max_shares;
+  p.num_splits = d->num_splits;
   p.io_f32 = d->dtype == KVP_F32;
   const float sc = scale == 0.f ? 1.f / sqrtf(float(d->dh)) : scale;
   p.scale_log2 = sc * 1.4426950408889634f;
@@ -576,6 +913,7 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
 
   for (int s0 = 0; s0 < n_sub; s0 += MAX_DEC_GROUPS) {
     const int n = n_sub - s0 < MAX_DEC_GROUPS ? n_sub - s0 : MAX_DEC_GROUPS;
+    int rows = 0;
     for (int i = 0; i < n; ++i) {
       const SubGroup& sg = subs[s0 + i];
       DecGroup& g = p.grp[i];
@@ -584,6 +922,7 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
       g.v_cache = reinterpret_cast<const __nv_bfloat16*>(v_cache[sg.owner]);
       g.n_members = sg.n;
       g.pad = 0;
+      rows = std::max(rows, sg.n * (d->Hq / d->Hkv));
       for (int m = 0; m < MAX_MEMBERS; ++m) {
         const int l = sg.members[m < sg.n ? m : 0];
         if (q[l] == nullptr || o[l] == nullptr || lse[l] == nullptr) return KVP_ERR_INVALID_ARG;
@@ -592,16 +931,38 @@ extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float 
         g.lse[m] = lse[l];
       }
     }
-    dim3 grid(ns, d->B * d->Hkv, n);
-    dim3 cgrid(1, d->B * d->Hkv, n);
+    const long long units = (long long)n * d->B * d->Hkv;
+    // No more blocks than the longest lists could give work to; shares go by the lengths on the device, and so does
+    // whether whole units are dealt out instead.
+    const long long blocks = d->num_splits > 0 ? units * d->num_splits
+                                               : std::min((long long)p.blocks, std::max((long long)n * sc_plan.max_shares, units));
+    if (units > 0x7fffffffLL || blocks > 0x7fffffffLL) return KVP_ERR_UNSUPPORTED;
+    p.n_groups = n;
+    p.by_units = dealt_by_units(longest_list(d), d->B * d->Hkv);
+    const long long unit_pieces = d->num_splits > 0 ? d->num_splits : sc_plan.max_shares / ((long long)d->B * d->Hkv);
+    const int wpr = unit_pieces > 8 ? 8 : 1;   // many pieces a unit: eight warps share those of a row
+    const int rows_per_block = COMBINE_THREADS / 32 / wpr;
+    const dim3 grid(static_cast<unsigned>(blocks));
+    const dim3 cgrid(unsigned(units), (rows + rows_per_block - 1) / rows_per_block);
     timing_before(KVP_KERNEL_DECODE, stream);
     cudaError_t e = launch_kernel(d->dh == 128 ? decode_kernel<128> : decode_kernel<64>, grid, DEC_THREADS, smem, stream, 1, p);
     timing_after(KVP_KERNEL_DECODE, stream);
-    if (e == cudaSuccess)
-      e = launch_kernel(d->dh == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, cgrid, 128, 0, stream, 1, p);
+    if (e == cudaSuccess && (d->num_splits > 0 || p.by_units == 0))   // whole units leave no pieces
+      e = launch_kernel(d->dh == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, cgrid, COMBINE_THREADS, 0, stream, 1, p, wpr);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;
+}
+
+}  // namespace
+}  // namespace kvp
+
+extern "C" int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q,
+                          const void* const* k_cache, const void* const* v_cache, const int32_t* block_table,
+                          const int32_t* lengths, void* const* o, float* const* lse, int layer_begin, int layer_end,
+                          void* ws, size_t ws_bytes, kvp_stream_t stream) {
+  return decode_impl(d, donor, scale, q, k_cache, v_cache, block_table, lengths, o, lse, layer_begin, layer_end, ws,
+                     ws_bytes, 0, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -651,12 +1012,14 @@ extern "C" int kvp_decode_static(const kvp_decode_desc* d, const int32_t* donor,
     if (donor[l] < 0 || donor[l] > l || donor[donor[l]] != donor[l]) return KVP_ERR_BAD_DONOR;
   if (layer_begin < 0 || layer_end > d->L || layer_begin >= layer_end) return KVP_ERR_INVALID_ARG;
   // only the donor groups that the layer range touches need room, so a narrower range can fit where all layers do not
+  // (when the library deals the rows out, it does so in fewer shares until their pieces fit)
   const size_t need = decode_scratch_bytes(d, donor, layer_begin, layer_end);
   if (need == 0) return KVP_ERR_UNSUPPORTED;
-  if (need > size_t(KVP_DECODE_STATIC_SCRATCH_BYTES)) return KVP_ERR_STATIC_SCRATCH;
+  if (d->num_splits > 0 && need > size_t(KVP_DECODE_STATIC_SCRATCH_BYTES)) return KVP_ERR_STATIC_SCRATCH;
   void* scratch = nullptr;
   rc = static_scratch_address(&scratch);
   if (rc != KVP_OK) return rc;
-  return kvp_decode(d, donor, scale, q, k_cache, v_cache, block_table, lengths, o, lse, layer_begin, layer_end,
-                    scratch, size_t(KVP_DECODE_STATIC_SCRATCH_BYTES), stream);
+  return decode_impl(d, donor, scale, q, k_cache, v_cache, block_table, lengths, o, lse, layer_begin, layer_end, scratch,
+                     size_t(KVP_DECODE_STATIC_SCRATCH_BYTES), size_t(KVP_DECODE_STATIC_SCRATCH_BYTES),
+                     reinterpret_cast<cudaStream_t>(stream));
 }
