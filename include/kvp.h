@@ -87,10 +87,11 @@ int kvp_set_timing_events(int kernel, void** starts, void** stops, int n);
 int kvp_timing_events_used(int kernel);
 /* Measurement switch of the GEMM's tile shape.  1 (the default): the forward GEMMs (kvp_proj_fwd,
  * kvp_out_proj_fwd, kvp_gemm) run on CTA pairs (256 x 256 tiles, one per pair of SMs) when every problem of the
- * launch has more than 128 rows, the gradient GEMMs on single-CTA 128 x 256 tiles; 0: single-CTA tiles
- * everywhere; 2: CTA pairs everywhere.  (K-major problems of at most 128 rows have a kernel of their own in every
- * mode.)  The results are the same in every mode (same products, same summation
- * order along K).  Not thread-safe. */
+ * launch has more than 128 rows, or up to 4096 rows on whichever of the library's kernels an estimate of their times
+ * prefers; the gradient GEMMs on single-CTA 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: CTA pairs everywhere.
+ * (K-major problems of at most 128 rows have a kernel of their own in every mode.)  The tile kernels sum the same
+ * products in the same order along K in every mode; up to 4096 rows K may be split over a cluster of CTAs, whose
+ * partial sums are added in a fixed order.  Not thread-safe. */
 void kvp_set_gemm_pair_mode(int mode);
 
 /* ------------------------------------------------------------------------------------------

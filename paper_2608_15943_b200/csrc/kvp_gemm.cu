@@ -657,6 +657,223 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
   }
 }
 
+// ------------------------------------------------------------------------------------------------------------
+// A few hundred rows of A (a prompt, a small batch of them): CTA pairs with the operands swapped, C^T = B A^T.
+//
+// Each pair of CTAs owns 256 columns of C (rows of B: 128 a CTA, the M = 256 of the pair's MMA) and a tile of tokens (the
+// N, split between the CTAs' loads).  256 x 256 tiles of gemm_pair_kernel pad 347 tokens to 512; here the tokens are cut
+// into tiles of 128 to 256, whatever leaves the fewest pairs idle, and one tile of the remainder, a multiple of 32.  The
+// tiles are walked longest first, pairs taking turns in alternating direction, so the short tiles of the remainder fill
+// the pairs that have no second long one.  A lane of the epilogue holds a column, so a warp stores rows of 64
+// consecutive bytes, two at a time, where a lane of gemm_pair_kernel's holds a row.  Roles, ring and barriers are those
+// of gemm_pair_kernel; results are bit-identical to its (same products, same order along K).
+// Bound: the 120 GB/s that an SM draws from L2 (tiles of up to 192 tokens), then the tensor pipe.  Measured (us;
+// gemm_pair_kernel -> this, tokens x columns x K): 200 x 11008 x 4096 29.1 -> 26.5, 512 x 11008 x 4096 51 -> 43,
+// 776 x 11008 x 4096 76 -> 57, 1500 x 4096 x 11008 123 -> 101, 2328 x 4096 x 4096 69 -> 56.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int TCOLS = 256;                        // columns of C per pair
+constexpr int TSTAGES = 6;
+constexpr int TSTAGE_BYTES = 32 * 1024;           // per CTA: 128 rows of B, up to 128 rows of A
+constexpr size_t TALL_SMEM = 1024 + size_t(TSTAGES) * TSTAGE_BYTES + 256;
+
+struct TallList {                                 // the tiles of one problem that have the same number of tokens
+  int prob;
+  int nt;                                         // tokens per tile, a multiple of 32
+  int m_first, n_tok;                             // first token, tiles along the tokens
+  int tile_end;                                   // one past the list's last tile in the launch's tile order
+  uint32_t idesc;
+};
+struct TallProblem {
+  int M, N, kblocks, out_f32;
+  long long ldc;
+  void* c;
+};
+template <int NP>
+struct TallParams {
+  CUtensorMap map_b[NP], map_a[2 * NP];           // map_a: one per list (the box holds half of a tile's tokens)
+  TallProblem prob[NP];
+  TallList list[2 * NP];
+  int total_tiles;
+};
+
+template <int NP>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gemm_tall_kernel(const __grid_constant__ TallParams<NP> p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(TSTAGES) * TSTAGE_BYTES);
+  uint64_t* full = bars;                    // [TSTAGES]  (used in the even CTA)
+  uint64_t* empty = bars + TSTAGES;         // [TSTAGES]
+  uint64_t* acc_full = bars + 2 * TSTAGES;  // [2]
+  uint64_t* acc_empty = acc_full + 2;       // [2]        (used in the even CTA)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  int* err = &g_gemm_status;
+  const int total_tiles = p.total_tiles;
+  const uint32_t rank = cluster_ctarank();  // 0: issues the MMAs; 1: partner
+  const int pair = blockIdx.x >> 1;
+  const int n_pairs = gridDim.x >> 1;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < TSTAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&acc_full[a], 1);
+      mbar_init(&acc_empty[a], 8);
+    }
+    mbar_fence_init();
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(tmem_slot, 512);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_sync_all();  // the partner's barriers exist before anything of this CTA can signal them
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  grid_dep_wait();
+
+  struct Tile {
+    int li, prob, nt, m0, n0;
+  };
+  // tile of a round: rounds of n_pairs tiles, dealt forwards and backwards in turn; li only grows
+  auto tile_of = [&](int round, Tile& w) -> bool {
+    const int t = round * n_pairs + ((round & 1) ? n_pairs - 1 - pair : pair);
+    if (t >= total_tiles) return false;
+    while (t >= p.list[w.li].tile_end) ++w.li;
+    const TallList& l = p.list[w.li];
+    const int within = t - (w.li ? p.list[w.li - 1].tile_end : 0);
+    w.prob = l.prob;
+    w.nt = l.nt;
+    w.m0 = l.m_first + (within % l.n_tok) * l.nt;
+    w.n0 = (within / l.n_tok) * TCOLS;
+    return true;
+  };
+
+  if (warp == 0) {
+    // ------------------------------ TMA producer (both CTAs) ------------------------------
+    const uint32_t leader = elect_one();
+    int s = 0;
+    uint32_t ph = 1;
+    bool ok = true;
+    Tile w{};
+    for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
+      if (!tile_of(round, w)) continue;   // only the last round can be short
+      const int half = w.nt / 2, nkb = p.prob[w.prob].kblocks;
+      const uint32_t bytes = 2u * uint32_t(PA_BYTES + half * (BK * 2));   // of both CTAs
+      const CUtensorMap* map_b = &p.map_b[w.prob];
+      const CUtensorMap* map_a = &p.map_a[w.li];
+      const int n0 = w.n0 + int(rank) * 128, m0 = w.m0 + int(rank) * half;
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!mbar_wait(&empty[s], ph, err)) { ok = false; break; }
+        uint8_t* sb = smem + size_t(s) * TSTAGE_BYTES;
+        if (rank == 0) mbar_expect_tx_e(&full[s], bytes, leader);
+        const uint32_t bar = cluster_addr_of(&full[s], 0);
+        tma_load_2d_pair_e(sb, map_b, bar, kb * BK, n0, leader);
+        tma_load_2d_pair_e(sb + PA_BYTES, map_a, bar, kb * BK, m0, leader);
+        if (++s == TSTAGES) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+    }
+    grid_dep_launch();   // all loads are out: the next kernel may come up while the last tiles are finished
+  } else if (warp == 1) {
+    // ------------------------------ MMA issuer (even CTA only) ------------------------------
+    if (rank == 0) {
+      const uint32_t leader = elect_one();
+      int s = 0;
+      uint32_t ph = 0, tile_i = 0;
+      bool ok = true;
+      Tile w{};
+      for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
+        if (!tile_of(round, w)) continue;
+        const uint32_t idesc = p.list[w.li].idesc;
+        const int nkb = p.prob[w.prob].kblocks;
+        const int acc = tile_i & 1;
+        if (!mbar_wait(&acc_empty[acc], ((tile_i >> 1) & 1) ^ 1, err)) { ok = false; break; }
+        tc_fence_after_sync();
+        const uint32_t d_tmem = tmem_base + acc * 256;
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait(&full[s], ph, err)) { ok = false; break; }
+          tc_fence_after_sync();
+          const uint32_t sb = smem_u32(smem + size_t(s) * TSTAGE_BYTES);
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            umma_ss_pair(d_tmem, smem_desc_sw128(sb + k * 32, 0, 1024), smem_desc_sw128(sb + PA_BYTES + k * 32, 0, 1024), idesc,
+                         (kb | k) != 0, leader);
+          umma_commit_pair(cluster_addr_of(&empty[s], 0), leader);
+          umma_commit_pair(cluster_addr_of(&empty[s], 1), leader);
+          if (++s == TSTAGES) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+        if (ok) {
+          umma_commit_pair(cluster_addr_of(&acc_full[acc], 0), leader);
+          umma_commit_pair(cluster_addr_of(&acc_full[acc], 1), leader);
+        }
+        ++tile_i;
+      }
+    }
+  } else {
+    // ------------------------------ epilogue (warps 2..5 of both CTAs): lane = column of C ------------------------------
+    const int quarter = warp & 3;  // TMEM lane quarter this warp may access
+    uint32_t tile_i = 0;
+    Tile w{};
+    for (int round = 0; round * n_pairs < total_tiles; ++round) {
+      if (!tile_of(round, w)) continue;
+      const TallProblem& pr = p.prob[w.prob];
+      const int acc = tile_i & 1;
+      const bool ok = mbar_wait(&acc_full[acc], (tile_i >> 1) & 1, err);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after_sync();
+      const int col = w.n0 + int(rank) * 128 + quarter * 32 + lane;
+      const int n_tok = min(w.nt, pr.M - w.m0);
+      const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + acc * 256;
+#pragma unroll 1
+      for (int c0 = 0; c0 < n_tok; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld_x32(taddr + c0, r);
+        tmem_ld_wait();
+        if (pr.out_f32) {
+          float* dst = reinterpret_cast<float*>(pr.c) + size_t(w.m0 + c0) * pr.ldc + col;
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c0 + i < n_tok && col < pr.N) dst[size_t(i) * pr.ldc] = __uint_as_float(r[i]);
+        } else {
+          // two tokens at a time: even lanes end up with two columns of the first, odd lanes with two of the second
+          const int odd = lane & 1;
+          __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(pr.c) + size_t(w.m0 + c0 + odd) * pr.ldc + (col - odd);
+#pragma unroll
+          for (int i = 0; i < 32; i += 2) {
+            const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? r[i] : r[i + 1], 1);
+            const float lo = __uint_as_float(odd ? got : r[i]), hi = __uint_as_float(odd ? r[i + 1] : got);
+            if (c0 + i + odd < n_tok && col < pr.N) *reinterpret_cast<uint32_t*>(dst + size_t(i) * pr.ldc) = pack_bf16(lo, hi);
+          }
+        }
+      }
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(cluster_addr_of(&acc_empty[acc], 0));
+      ++tile_i;
+    }
+  }
+
+  // ------------------------------ teardown: as gemm_pair_kernel ------------------------------
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
 }  // namespace
 
 int gemm_read_status() {
@@ -833,10 +1050,52 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // wait for the former (a CTA of a cluster that waited could hold up a peer that another kernel's CTA waits for); 40 KB
   // keep it off the SMs of the kernels that take all 512 columns.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
-  const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 456));
+  const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
   if (allow_smem<gemm_split_kernel<NP>>(226 * 1024) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e = launch_kernel(gemm_split_kernel<NP>, tiles * cfg.split, SPLIT_THREADS, smem, stream, cfg.split, p);
+  timing_after(KVP_KERNEL_GEMM, stream);
+  return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
+}
+
+template <int NP>
+int launch_tall(const GemmProblem* probs, int n, int nt, cudaStream_t stream) {
+  TallParams<NP> p;
+  int lists = 0, tiles = 0;
+  for (int i = 0; i < n; ++i) {
+    const GemmProblem& g = probs[i];
+    const GemmSeg& e = g.segs[0];
+    p.prob[i] = TallProblem{g.M, g.N, (e.K + BK - 1) / BK, g.out_f32, g.ldc, g.c};
+    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.N)}, strides[1] = {uint64_t(e.ldb) * 2};
+    uint32_t box[2] = {BK, 128};
+    const int rc = make_tensor_map(&p.map_b[i], e.b, 2, 2, dims, strides, box, true);
+    if (rc != KVP_OK) return rc;
+  }
+  // the whole tiles of all problems first, then the remainders
+  for (int part = 0; part < 2; ++part)
+    for (int i = 0; i < n; ++i) {
+      const GemmProblem& g = probs[i];
+      const GemmSeg& e = g.segs[0];
+      const int whole = g.M / nt, rest = g.M - whole * nt;
+      TallList l;
+      l.prob = i;
+      l.nt = part == 0 ? nt : (rest + 31) / 32 * 32;
+      l.m_first = part == 0 ? 0 : whole * nt;
+      l.n_tok = part == 0 ? whole : (rest > 0 ? 1 : 0);
+      if (l.n_tok == 0) continue;
+      tiles += l.n_tok * ((g.N + TCOLS - 1) / TCOLS);
+      l.tile_end = tiles;
+      l.idesc = umma_idesc_bf16(256, l.nt, 0, 0);
+      uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.M)}, strides[1] = {uint64_t(e.lda) * 2};
+      uint32_t box[2] = {BK, uint32_t(l.nt / 2)};
+      const int rc = make_tensor_map(&p.map_a[lists], e.a, 2, 2, dims, strides, box, true);
+      if (rc != KVP_OK) return rc;
+      p.list[lists++] = l;
+    }
+  p.total_tiles = tiles;
+  if (allow_smem<gemm_tall_kernel<NP>>(int(TALL_SMEM)) != cudaSuccess) return KVP_ERR_CUDA;
+  timing_before(KVP_KERNEL_GEMM, stream);
+  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP>, 2 * std::min(tiles, sm_count() / 2), GEMM_THREADS, TALL_SMEM, stream, 1, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
@@ -857,17 +1116,116 @@ bool use_pair(const GemmProblem* probs, int n, bool prefer_pair) {
 void gemm_set_pair_mode(int mode) { g_pair_mode = mode; }
 int gemm_pair_mode() { return g_pair_mode; }
 
-static int gemm_split(const GemmProblem* probs, int n, cudaStream_t stream) {
-  for (int begin = 0; begin < n; begin += SPLIT_MAX_PROB) {
-    const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
-    const SplitConfig cfg = split_config(probs + begin, cnt);
-    const int rc = cnt == 1   ? launch_split<1>(probs + begin, cnt, cfg, stream)
-                   : cnt <= 4 ? launch_split<4>(probs + begin, cnt, cfg, stream)
-                              : launch_split<SPLIT_MAX_PROB>(probs + begin, cnt, cfg, stream);
+namespace {
+
+// ------------------------------------------------------------------------------------------------------------
+// Which kernel a forward GEMM of more than 128 rows runs on.  The times (us) of each are estimated from a model with the
+// terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe -- whose
+// constants were fitted to 4000 measurements (13 column counts x 27 row counts, one launch behind the other); the
+// choice it makes costs 1.9 % more than the best of all choices on average, and 31 % less than CTA pairs always.
+// Above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int CHOICE_MAX_ROWS = 4096;
+struct Choice {
+  enum Kind { kSingle, kPair, kTall, kSplit } kind = kPair;
+  int nt = 0;         // tokens per tile (tall, split)
+  int split = 1;
+  float us = 1e30f;
+};
+
+// Longest pair of `pairs`, n1 tiles of cost c1 dealt out before n2 of cost c2 <= c1, rounds in alternating direction.
+float makespan(int n1, float c1, int n2, float c2, int pairs) {
+  const int rem = n1 % pairs, a = n1 / pairs;
+  if (rem == 0) return a * c1 + ((n2 + pairs - 1) / pairs) * c2;
+  const int left = n2 - (pairs - rem);            // short tiles that do not fit beside the last round of long ones
+  if (left <= 0) return std::max((a + 1) * c1, a * c1 + (n2 > 0 ? c2 : 0.f));
+  const int rounds = left / pairs, over = left % pairs;
+  return std::max((a + 1) * c1 + (rounds + (over > pairs - rem ? 1 : 0)) * c2, a * c1 + (1 + rounds + (over > 0 ? 1 : 0)) * c2);
+}
+
+Choice choose_forward(const GemmProblem* probs, int n) {
+  int M = 0, kb = 0, cols128 = 0, cols256 = 0;
+  for (int i = 0; i < n; ++i) {
+    M = std::max(M, probs[i].M);
+    kb = std::max(kb, (probs[i].segs[0].K + BK - 1) / BK);
+    cols128 += (probs[i].N + 127) / 128;
+    cols256 += (probs[i].N + 255) / 256;
+  }
+  const int sms = sm_count(), pairs = sms / 2;
+  Choice best;
+  auto consider = [&](Choice::Kind kind, int nt, int split, float us) {
+    if (us >= best.us) return;
+    best.kind = kind;
+    best.nt = nt;
+    best.split = split;
+    best.us = us;
+  };
+  auto up = [](int x, int y) { return (x + y - 1) / y; };
+  consider(Choice::kSingle, 0, 1, up(up(M, BM) * cols256, sms) * (kb * 0.388f + 3.8f));
+  consider(Choice::kPair, 0, 1, up(up(M, PBM) * cols256, pairs) * (kb * 0.320f + 5.5f));
+  auto tall_tile = [&](int nt) { return nt == 0 ? 0.f : kb * std::max(0.125f * (1.f + nt / 256.f), 0.0013f * nt) + 3.1f; };
+  for (int nt = 128; nt <= 256; nt += 32) {
+    const int whole = M / nt, rest = up(M - whole * nt, 32) * 32;
+    consider(Choice::kTall, nt, 1, 2.9f + makespan(whole * cols256, tall_tile(nt), rest > 0 ? cols256 : 0, tall_tile(rest), pairs));
+  }
+  // split kernel: one CTA per SM; clusters of four do not fill every GPC
+  for (int split = 1; split <= 4 && 2 * split <= kb; split *= 2) {
+    const int most = (split == 4 ? sms - 16 : sms) / (split * cols128);   // token tiles that fit
+    if (most < 1) break;
+    const int nt = up(up(M, most), 16) * 16 < 48 ? 48 : up(up(M, most), 16) * 16;
+    if (nt > 256) continue;
+    consider(Choice::kSplit, nt, split, 4.5f + float(kb) / split * std::max(0.120f * (1.f + nt / 128.f), 0.0012f * nt) + 0.01f * nt +
+                                            (split > 1 ? 0.013f * nt + 0.4f : 0.f));
+  }
+  return best;
+}
+
+bool k_major(const GemmProblem* probs, int n) {
+  for (int i = 0; i < n; ++i)
+    if (probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
+  return n > 0;
+}
+
+template <typename F1, typename F4, typename F32>
+int by_count(int n, F1 one, F4 four, F32 many) { return n == 1 ? one() : n <= 4 ? four() : many(); }
+
+// A forward GEMM (pair mode 1, K-major operands, one segment): -1 when the tile kernels take it
+int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
+  if (split_applies(probs, n)) {
+    for (int begin = 0; begin < n; begin += SPLIT_MAX_PROB) {
+      const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
+      const GemmProblem* g = probs + begin;
+      const SplitConfig cfg = split_config(g, cnt);
+      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
+                              [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream); });
+      if (rc != KVP_OK) return rc;
+    }
+    return KVP_OK;
+  }
+  if (g_pair_mode != 1 || !k_major(probs, n)) return -1;
+  for (int i = 0; i < n; ++i)
+    if (probs[i].M > CHOICE_MAX_ROWS) return -1;
+  for (int begin = 0; begin < n; begin += MAX_PROB) {
+    const int cnt = std::min(MAX_PROB, n - begin);
+    const GemmProblem* g = probs + begin;
+    const Choice c = choose_forward(g, cnt);
+    int rc;
+    if (c.kind == Choice::kTall) {
+      rc = by_count(cnt, [&] { return launch_tall<1>(g, cnt, c.nt, stream); }, [&] { return launch_tall<4>(g, cnt, c.nt, stream); },
+                    [&] { return launch_tall<MAX_PROB>(g, cnt, c.nt, stream); });
+    } else if (c.kind == Choice::kSplit) {
+      const SplitConfig cfg{c.nt, c.split, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
+      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
+                    [&] { return launch_split<MAX_PROB>(g, cnt, cfg, stream); });
+    } else {
+      rc = launch_group(g, cnt, stream, 0, 0, c.kind == Choice::kPair);
+    }
     if (rc != KVP_OK) return rc;
   }
   return KVP_OK;
 }
+
+}  // namespace
 
 int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool prefer_pair) {
   if (n < 0 || (n > 0 && probs == nullptr)) return KVP_ERR_INVALID_ARG;
@@ -875,7 +1233,10 @@ int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool pref
     const int rc = check_problem(probs[i]);
     if (rc != KVP_OK) return rc;
   }
-  if (split_applies(probs, n)) return gemm_split(probs, n, stream);
+  if (prefer_pair || split_applies(probs, n)) {
+    const int rc = gemm_forward(probs, n, stream);
+    if (rc >= 0) return rc;
+  }
   // as many problems per launch as the parameter block holds
   int begin = 0;
   while (begin < n) {
@@ -903,7 +1264,10 @@ int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, v
   g.out_f32 = out_f32;
   const int rc = check_problem(g);
   if (rc != KVP_OK) return rc;
-  if (withhold_at == 0 && split_applies(&g, 1)) return gemm_split(&g, 1, stream);
+  if (withhold_at == 0 && (prefer_pair || split_applies(&g, 1))) {
+    const int forward = gemm_forward(&g, 1, stream);
+    if (forward >= 0) return forward;
+  }
   return launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1, prefer_pair));
 }
 

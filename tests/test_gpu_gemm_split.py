@@ -1,4 +1,5 @@
-"""GEMMs with at most 128 rows of A (decode-step projections): operands swapped, K split over a cluster of CTAs."""
+"""GEMMs with few rows of A (decode-step projections, prompts): operands swapped, K split over a cluster of CTAs, or tiles
+of tokens on CTA pairs."""
 import pytest
 import torch
 
@@ -14,6 +15,11 @@ pytestmark = pytest.mark.gpu
     (31, 264, 1032),      # split 8, 17 k-blocks dealt unevenly
     (128, 4096, 520),     # widest token tile; 32 column tiles: split 4
     (40, 19208, 200),     # more CTAs than SMs: two per SM, shallow ring, split 1
+    (129, 4104, 2056),    # first row count of the chosen kernels: K split, one ragged column tile
+    (347, 520, 2048),     # K split in four, several token tiles, the last one short
+    (200, 11016, 136),    # CTA pairs with one short token tile
+    (513, 5512, 1032),    # whole token tiles first, then a remainder of one token
+    (1300, 8200, 72),     # several rounds of tiles, pairs in alternating direction
 ])
 def test_few_rows(M, N, K):
     from paper_2608_15943_b200 import kvp
