@@ -5,24 +5,24 @@
 // layer of the group (Eq. 3 of the paper: consumers reuse the donor's K/V), up to 16 rows, as the M dimension of
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate).  The kernel is bound by HBM bandwidth, so the design is about bytes in
 // flight and about every warp having the same share of them:
-//  - The rows of a group's units form one list of 16-token granules (8 KB at dh 128: 4 KB of K, 4 KB of V; both
-//    contiguous, a page block of one KV head is), in order of (sequence, KV head, position).  The lengths are in device
-//    memory, so every block sums them up itself and takes an equal share of each group's list, wherever its ends fall:
-//    no part-filled last wave, whatever the batch and the lengths.  Long lists are cut into more shares than blocks
-//    that fit, so that the block scheduler evens out SMs that draw memory at different rates.  The shares of a group do
-//    not depend on the other groups of the call: any layer range gives a layer the same bits.
-//  - Short units are not cut: a list whose units hold 32 granules or fewer on average (64, where there are enough units)
-//    is dealt out by units, since every piece costs a block a merge of its warps (30 sequences of 500 tokens, 8 groups
-//    at dh 64: 49 us by units, 96 us by equal shares).
+//  - The rows of all units form one list of 16-token granules (8 KB at dh 128: 4 KB of K, 4 KB of V; both contiguous,
+//    a page block of one KV head is), in order of (group, sequence, KV head, position).  The lengths are in device
+//    memory, so every block sums them up itself and takes an equal share of the list, wherever its ends fall: no
+//    part-filled last wave, whatever the batch and the lengths.  Long lists are cut into more shares than blocks that
+//    fit, so that the block scheduler evens out SMs that draw memory at different rates.
+//  - Short units are not cut: units of 32 granules or fewer on average (64, where there are enough of them) are dealt
+//    out whole, since every piece costs a block a merge of its warps (30 sequences of 500 tokens, 8 groups at dh 64:
+//    46 us by units, 96 us when each was cut in two).
 //  - The four warps of a block take the granules of a share in turn, each with a ring of its own filled by 16-byte
 //    cp.async copies that are fully coalesced and continue across the ends of units; two blocks per SM.  (A contiguous
 //    share for every warp instead read memory 3 % slower.)  No transposes in HBM -- V fragments come from ldmatrix.trans
 //    on the swizzled ring.
 //  - A unit that lies inside one share is finished there.  The pieces of the others, (max, sum, output) triples, at most
 //    two per share, are merged by a second small kernel that finds them by the same arithmetic.
-// Measured with the merge, against a grid of (unit, 2048-token split) blocks with a merge of one thread per output
-// element: 16 sequences of 4096 tokens 61 -> 50 us (the copy rate takes 41), 8 of 8K-16K in two groups 141 -> 129 (113),
-// one of 65536 74 -> 49 (41), 4 of 128K at 32 KV heads 1187 -> 1172 (1313), 32 of 16K-32K in six groups 2768 -> 2740.
+// Measured with the merge (us), against a grid of (unit, 2048-token split) blocks with a merge of one thread per output
+// element: 16 sequences of 4096 tokens 61 -> 50 (the copy rate takes 41), 8 of 8K-16K in two groups 141 -> 128 (113), one
+// of 65536 74 -> 49 (41), 2 of 16K in eight groups 172 -> 170, 3 of 3000 in six groups at dh 64 26.8 -> 27.1, 4 of 128K
+// at 32 KV heads 1192 -> 1177 (1313), 32 of 16K-32K in six groups 2767 -> 2687.
 #include <math.h>
 
 #include <algorithm>
@@ -40,8 +40,8 @@ constexpr int GRAN = 16;           // tokens per ring stage
 constexpr int DEC_STAGES = 3;      // granules per warp in the ring
 template <int DH>
 constexpr int DEC_CTAS_PER_SM = DH == 128 ? 2 : 4;   // as many as shared memory holds
-constexpr int MIN_SHARE = 8;       // granules of a share at least: a piece costs about as much again
-constexpr int LONG_SHARE = 128;    // granules of a share at least where there are more shares than blocks that fit
+constexpr int MIN_SHARE = 8;       // granules of a share at least: a piece costs a block about as much again
+constexpr int LONG_SHARE = 160;    // granules of a share at least where there are more shares than blocks that fit
 constexpr int MAX_ROUNDS = 16;     // shares per block that fits, at most
 constexpr int MAX_DEC_GROUPS = 64;
 constexpr int MAX_MEMBERS = 4;     // layers of a donor group served by one pass (rows = members * G <= 16)
@@ -66,8 +66,8 @@ struct DecParams {
   float* part_ml;              // [pieces][rows][2]
   int rows;                    // query rows of the largest group
   int n_groups, B, Hq, Hkv, page_size, max_pages, n_pages;
-  int blocks;                  // MAX_ROUNDS times the blocks that fit on the device
-  int max_shares;              // most shares of one group's list (divides blocks)
+  int fit;                     // blocks that fit on the device
+  int max_shares;              // most shares of the list
   int by_units;                // the lists are short at any length: whole units are dealt out, no sums are formed
   int num_splits;              // > 0: the caller's split count instead; a block is one (unit, split)
   int io_f32;                  // queries are read and outputs written as fp32 (rounded to bf16 on load / widened on store)
@@ -93,21 +93,17 @@ __device__ __forceinline__ void sum_granules(const DecParams& p, int b_before, i
     all += __shfl_xor_sync(0xffffffffu, all, s);
   }
 }
-// Shares a list of `total` granules is dealt out in: always a divisor of `blocks`, so that a block's shares of different
-// groups start at the same place of their lists.  The divisors tried are blocks / 2^k, then powers of two.
-__host__ __device__ inline int fewer_shares(int blocks, int n) {
-  if (n % 2 == 0) return n / 2;
-  int pow2 = blocks & -blocks;
-  while (pow2 >= n) pow2 /= 2;
-  return pow2 > 0 ? pow2 : 1;
+__host__ __device__ inline bool dealt_by_units(long long total, long long units, int fit) {
+  return total < 32 * units || (total < 64 * units && units >= fit);
 }
-__host__ __device__ inline bool dealt_by_units(long long total, int units) {
-  return total < 32ll * units || (total < 64ll * units && units >= 64);
-}
-__host__ __device__ inline int shares_for(int blocks, int max_shares, long long total) {
-  int n = max_shares;
-  while (n > 1 && n * (long long)(n > blocks / MAX_ROUNDS ? LONG_SHARE : MIN_SHARE) > total) n = fewer_shares(blocks, n);
-  return n;
+// Shares a list of `total` granules is dealt out in.
+__host__ __device__ inline int shares_for(int fit, int max_shares, long long total) {
+  long long n = total / MIN_SHARE;
+  if (n > fit) {
+    const long long rounds = total / ((long long)fit * LONG_SHARE);
+    n = (long long)fit * (rounds < 1 ? 1 : rounds > MAX_ROUNDS ? MAX_ROUNDS : rounds);
+  }
+  return int(n < 1 ? 1 : n > max_shares ? max_shares : n);
 }
 // The first T mod n of n shares of a list of T granules hold one more than the others.
 __device__ __forceinline__ uint32_t div_long(long long a, uint32_t b) {   // quotients here fit 32 bits; so do nearly all dividends
@@ -179,8 +175,8 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int G = p.Hq / p.Hkv;
-  __shared__ float2 s_o[2][NBLK * 32];             // eight rows of two warps' results while a block merges its four
-  __shared__ float2 s_ml[2][32];
+  __shared__ float2 s_o[DEC_WARPS - 1][NBLK * 32]; // eight rows of the results that warp 0 merges into its own
+  __shared__ float2 s_ml[DEC_WARPS - 1][32];
   grid_dep_wait();
   if (blockIdx.x == 0 && warp == 0) {
     for (int b = lane; b < p.B; b += 32)
@@ -194,7 +190,6 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
   };
   Cursor c;                                        // start of the block's next piece
   int todo;                                        // granules of the block's share of a group's list still to do
-  int n_shares = 1, group_step = p.n_groups;       // the block's groups: c.grp, c.grp + group_step, ...
   const bool caller_splits = p.num_splits > 0;
   auto go_to_unit = [&](Cursor& x, int id) {       // (past the last unit: grp >= n_groups)
     x.id = id;
@@ -205,13 +200,13 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     x.len = clamped_length(p, x.b);
     x.ng = granules_of(x.len);
   };
-  long long total = 0;
+  long long per_group = 0;
   bool by_units = p.by_units != 0;
   if (!caller_splits && !by_units) {
     int before, all;
     sum_granules(p, 0, before, all);
-    total = (long long)all * p.Hkv;
-    by_units = dealt_by_units(total, p.B * p.Hkv);
+    per_group = (long long)all * p.Hkv;
+    by_units = dealt_by_units(per_group * p.n_groups, (long long)p.n_groups * p.B * p.Hkv, p.fit);
   }
   if (caller_splits) {
     const int split = blockIdx.x % p.num_splits;
@@ -224,15 +219,15 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     if (c.grp >= p.n_groups) return;
     todo = c.ng;
   } else {
-    n_shares = shares_for(p.blocks, p.max_shares, total);
-    group_step = p.blocks / n_shares;
-    c.id = 0;
-    c.grp = blockIdx.x / n_shares;
-    if (c.grp >= p.n_groups) return;
-    const int share = blockIdx.x % n_shares;
+    const long long total = per_group * p.n_groups;
+    const int n_shares = shares_for(p.fit, p.max_shares, total);
+    if (blockIdx.x >= n_shares) return;
     const Dealt dealt(total, n_shares);
-    long long at = dealt.begin(share);             // find its sequence, 32 lengths at a time
-    todo = int(dealt.size(share));
+    long long at = dealt.begin(blockIdx.x);
+    todo = int(dealt.size(blockIdx.x));
+    c.id = 0;
+    c.grp = int(div_long(at, uint32_t(per_group)));
+    at -= c.grp * per_group;                       // inside the group: find the sequence, 32 lengths at a time
     for (int b0 = 0;; b0 += 32) {
       const int mine = b0 + lane < p.B ? granules_of(clamped_length(p, b0 + lane)) : 0;
       int upto = mine;
@@ -259,13 +254,14 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
   uint8_t* ring = dsmem + size_t(warp) * STAGES * STAGE_BYTES;
   const uint32_t ring_u32 = smem_u32(ring);
 
-  const Cursor start = c;
-  const int share_len = todo;
-  auto next_unit = [&](Cursor& x) {                // (wraps at the end of the list, where a share ends too)
+  auto next_unit = [&](Cursor& x) {
     x.gran = 0;
     if (++x.hk == p.Hkv) {
       x.hk = 0;
-      if (++x.b == p.B) x.b = 0;
+      if (++x.b == p.B) {
+        x.b = 0;
+        ++x.grp;
+      }
       x.len = clamped_length(p, x.b);
       x.ng = granules_of(x.len);
     }
@@ -275,16 +271,11 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     left -= min(left, x.ng - x.gran);
     if (left > 0) {
       next_unit(x);
-    } else if (caller_splits) {
-      x.grp = p.n_groups;
-    } else if (by_units) {
+    } else if (by_units && !caller_splits) {
       go_to_unit(x, x.id + gridDim.x);
       left = x.ng;
     } else {
-      const int grp = x.grp + group_step;
-      x = start;
-      x.grp = grp;
-      left = share_len;
+      x.grp = p.n_groups;
     }
   };
 
@@ -349,8 +340,37 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     cp_async_commit();
   };
   enter_piece();
+  // query fragments (A operand, rows = members x heads of the group, zero beyond its rows); those of the next piece are
+  // requested before the merge at the end of a piece
+  uint32_t qa[KSTEPS][4];
+  auto load_queries = [&]() {
+    const DecGroup& grp = p.grp[c.grp];
+    const int R = grp.n_members * G;
+    const int r0 = g, r1 = g + 8;
+    const size_t off0 = r0 < R ? (size_t(c.b) * p.Hq + c.hk * G + r0 % G) * DH : 0;
+    const size_t off1 = r1 < R ? (size_t(c.b) * p.Hq + c.hk * G + r1 % G) * DH : 0;
+    auto pair_at = [&](const void* base, size_t off, int col) -> uint32_t {   // two elements of a query row as bf16
+      if (p.io_f32) {
+        const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + off + col);
+        return pack_bf16(v.x, v.y);
+      }
+      return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(base) + off + col);
+    };
+    const void* q0 = r0 < R ? grp.q[r0 / G] : nullptr;
+    const void* q1 = r1 < R ? grp.q[r1 / G] : nullptr;
+#pragma unroll
+    for (int ks = 0; ks < KSTEPS; ++ks) {
+      const int col = ks * 16 + t * 2;
+      qa[ks][0] = q0 ? pair_at(q0, off0, col) : 0u;
+      qa[ks][1] = q1 ? pair_at(q1, off1, col) : 0u;
+      qa[ks][2] = q0 ? pair_at(q0, off0, col + 8) : 0u;
+      qa[ks][3] = q1 ? pair_at(q1, off1, col + 8) : 0u;
+    }
+  };
+
 #pragma unroll
   for (int s = 0; s < STAGES - 1; ++s) issue_next();
+  load_queries();
 
   int stage_out = 0;
   do {
@@ -359,31 +379,6 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     const int R = grp.n_members * G;               // valid query rows (<= 16)
     const int n_here = min(todo, c.ng - c.gran);
     const bool from_start = c.gran == 0, to_end = c.gran + n_here == c.ng;
-
-    // query fragments (A operand, rows = members x heads of the group, zero beyond R)
-    uint32_t qa[KSTEPS][4];
-    {
-      const int r0 = g, r1 = g + 8;
-      const size_t off0 = r0 < R ? (size_t(c.b) * p.Hq + c.hk * G + r0 % G) * DH : 0;
-      const size_t off1 = r1 < R ? (size_t(c.b) * p.Hq + c.hk * G + r1 % G) * DH : 0;
-      auto pair_at = [&](const void* base, size_t off, int col) -> uint32_t {   // two elements of a query row as bf16
-        if (p.io_f32) {
-          const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(base) + off + col);
-          return pack_bf16(v.x, v.y);
-        }
-        return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(base) + off + col);
-      };
-      const void* q0 = r0 < R ? grp.q[r0 / G] : nullptr;
-      const void* q1 = r1 < R ? grp.q[r1 / G] : nullptr;
-#pragma unroll
-      for (int ks = 0; ks < KSTEPS; ++ks) {
-        const int col = ks * 16 + t * 2;
-        qa[ks][0] = q0 ? pair_at(q0, off0, col) : 0u;
-        qa[ks][1] = q1 ? pair_at(q1, off1, col) : 0u;
-        qa[ks][2] = q0 ? pair_at(q0, off0, col + 8) : 0u;
-        qa[ks][3] = q1 ? pair_at(q1, off1, col + 8) : 0u;
-      }
-    }
 
     float oacc[NBLK][4];
 #pragma unroll
@@ -482,43 +477,52 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     next_piece(c, todo);
     const bool last = c.grp >= p.n_groups;
     if (last) grid_dep_launch();   // this warp's loads are out, the others' within a granule
+    else load_queries();
 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
       l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
     }
-    // ---- merge the four warps of the block, eight rows at a time: 2 into 0 and 3 into 1, then 1 into 0 ----
+    // ---- warp 0 merges the results of the others into its own, eight rows at a time ----
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (8 * h >= R) break;
-      auto put = [&](int slot) {
+      __syncthreads();   // warp 0 is done with the previous ones
+      if (warp > 0) {
 #pragma unroll
-        for (int n = 0; n < NBLK; ++n) s_o[slot][n * 32 + lane] = make_float2(oacc[n][2 * h], oacc[n][2 * h + 1]);
-        s_ml[slot][lane] = make_float2(m_run[h], l_run[h]);
-      };
-      auto take = [&](int slot) {
-        const float2 om = s_ml[slot][lane];
-        const float mn = fmaxf(m_run[h], om.x);
+        for (int n = 0; n < NBLK; ++n) s_o[warp - 1][n * 32 + lane] = make_float2(oacc[n][2 * h], oacc[n][2 * h + 1]);
+        s_ml[warp - 1][lane] = make_float2(m_run[h], l_run[h]);
+      }
+      __syncthreads();
+      if (warp == 0) {
+        float2 om[DEC_WARPS - 1];
+        float mn = m_run[h];
+#pragma unroll
+        for (int w = 0; w < DEC_WARPS - 1; ++w) {
+          om[w] = s_ml[w][lane];
+          mn = fmaxf(mn, om[w].x);
+        }
         const float fa = m_run[h] == -INFINITY ? 0.f : fast_exp2(m_run[h] - mn);
-        const float fb = om.x == -INFINITY ? 0.f : fast_exp2(om.x - mn);
         m_run[h] = mn;
-        l_run[h] = l_run[h] * fa + om.y * fb;
+        l_run[h] *= fa;
 #pragma unroll
         for (int n = 0; n < NBLK; ++n) {
-          const float2 v = s_o[slot][n * 32 + lane];
-          oacc[n][2 * h] = oacc[n][2 * h] * fa + v.x * fb;
-          oacc[n][2 * h + 1] = oacc[n][2 * h + 1] * fa + v.y * fb;
+          oacc[n][2 * h] *= fa;
+          oacc[n][2 * h + 1] *= fa;
         }
-      };
-      if (warp >= 2) put(warp - 2);
-      __syncthreads();
-      if (warp < 2) take(warp);
-      __syncthreads();
-      if (warp == 1) put(1);
-      __syncthreads();
-      if (warp == 0) take(1);
-      __syncthreads();
+#pragma unroll
+        for (int w = 0; w < DEC_WARPS - 1; ++w) {
+          const float fb = om[w].x == -INFINITY ? 0.f : fast_exp2(om[w].x - mn);
+          l_run[h] += om[w].y * fb;
+#pragma unroll
+          for (int n = 0; n < NBLK; ++n) {
+            const float2 v = s_o[w][n * 32 + lane];
+            oacc[n][2 * h] += v.x * fb;
+            oacc[n][2 * h + 1] += v.y * fb;
+          }
+        }
+      }
     }
     if (warp != 0) {
       // (warp 0 alone goes on to store)
@@ -545,7 +549,7 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
       }
     } else {
       // ---- a piece: the first of a share, or the last one if that starts a unit ----
-      const size_t piece = caller_splits ? size_t(blockIdx.x) : (size_t(here.grp) * n_shares + blockIdx.x % n_shares) * 2 + (from_start ? 1 : 0);
+      const size_t piece = caller_splits ? size_t(blockIdx.x) : size_t(blockIdx.x) * 2 + (from_start ? 1 : 0);
       float* po = p.part_o + piece * p.rows * DH;
       float* pml = p.part_ml + piece * p.rows * 2;
 #pragma unroll
@@ -586,21 +590,19 @@ __global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const _
   grid_dep_wait();
   if (blockIdx.y * rows_per_block >= R) return;
   int w0, w1;                                 // shares (or splits) that hold the unit
-  size_t piece0 = 0;
   if (p.num_splits > 0) {
     w0 = unit * p.num_splits;
     w1 = w0 + p.num_splits - 1;
   } else {
     int before, all;
     sum_granules(p, b, before, all);
-    const long long total = (long long)all * p.Hkv;
-    if (dealt_by_units(total, p.B * p.Hkv)) return;   // finished by the blocks that held them
-    const int n = shares_for(p.blocks, p.max_shares, total), ng = granules_of(clamped_length(p, b));
-    const long long first = (long long)before * p.Hkv + (long long)hk * ng;
+    const long long per_group = (long long)all * p.Hkv, total = per_group * p.n_groups;
+    if (dealt_by_units(total, (long long)p.n_groups * p.B * p.Hkv, p.fit)) return;   // finished by the blocks that held them
+    const int n = shares_for(p.fit, p.max_shares, total), ng = granules_of(clamped_length(p, b));
+    const long long first = gi * per_group + (long long)before * p.Hkv + (long long)hk * ng;
     const Dealt dealt(total, n);
     w0 = dealt.share_of(first);
     w1 = dealt.share_of(first + ng - 1);
-    piece0 = size_t(gi) * n;
     if (w0 == w1) return;                     // finished by the block that had the share
   }
   const int sub = lane / LANES, col = (lane % LANES) * 4;
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const _
         const int wu = w + u * step;
         ml[u] = make_float2(-INFINITY, 0.f);
         if (wu <= w1) {
-          const size_t piece = p.num_splits > 0 ? size_t(wu) : (piece0 + wu) * 2 + (wu == w0 ? 1 : 0);
+          const size_t piece = p.num_splits > 0 ? size_t(wu) : size_t(wu) * 2 + (wu == w0 ? 1 : 0);
           ml[u] = *reinterpret_cast<const float2*>(p.part_ml + (piece * p.rows + row) * 2);
           o[u] = *reinterpret_cast<const float4*>(p.part_o + (piece * p.rows + row) * DH + col);
         }
@@ -765,15 +767,15 @@ int build_groups(const kvp_decode_desc* d, const int32_t* donor, int begin, int 
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Pieces and their bytes.  When the library chooses: two for each share of each group's list at its longest; with the
+// Pieces and their bytes.  When the library chooses: two for each share of the list at its longest; with the
 // caller's split count: one for every (unit, split).  One launch holds at most MAX_DEC_GROUPS sub-groups and launches
 // reuse the space.
-int decode_blocks(int dh) { return sm_count() * (dh == 128 ? DEC_CTAS_PER_SM<128> : DEC_CTAS_PER_SM<64>) * MAX_ROUNDS; }
+int blocks_that_fit(int dh) { return sm_count() * (dh == 128 ? DEC_CTAS_PER_SM<128> : DEC_CTAS_PER_SM<64>); }
 size_t piece_bytes(const kvp_decode_desc* d, size_t pieces, int rows) {
   return align256(pieces * rows * d->dh * 4) + align256(pieces * rows * 2 * 4);
 }
-long long longest_list(const kvp_decode_desc* d) {
-  return (long long)d->B * d->Hkv * ((long long)d->max_pages * d->page_size / GRAN);
+long long longest_list(const kvp_decode_desc* d, int n_groups) {
+  return (long long)n_groups * d->B * d->Hkv * ((long long)d->max_pages * d->page_size / GRAN);
 }
 struct Scratch {
   int max_shares = 0, rows = 0;
@@ -782,15 +784,15 @@ struct Scratch {
 // limit > 0: fewer shares until the pieces fit into that many bytes
 Scratch plan_scratch(const kvp_decode_desc* d, const SubGroup* subs, int n_sub, size_t limit) {
   Scratch s;
-  const size_t per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
+  const int per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
   for (int i = 0; i < n_sub; ++i) s.rows = std::max(s.rows, subs[i].n * (d->Hq / d->Hkv));
-  const int blocks = decode_blocks(d->dh);
-  s.max_shares = shares_for(blocks, blocks, longest_list(d));
+  const int fit = blocks_that_fit(d->dh);
+  s.max_shares = shares_for(fit, fit * MAX_ROUNDS, longest_list(d, per_launch));
   for (;;) {
-    s.pieces = d->num_splits > 0 ? per_launch * d->B * d->Hkv * d->num_splits : per_launch * s.max_shares * 2;
+    s.pieces = d->num_splits > 0 ? size_t(per_launch) * d->B * d->Hkv * d->num_splits : size_t(s.max_shares) * 2;
     s.bytes = piece_bytes(d, s.pieces, s.rows);
     if (limit == 0 || s.bytes <= limit || d->num_splits > 0 || s.max_shares == 1) return s;
-    s.max_shares = fewer_shares(blocks, s.max_shares);
+    s.max_shares = (s.max_shares + 1) / 2;
   }
 }
 // bytes for decoding layers [begin, end); 0 when the request cannot be served at all
@@ -901,7 +903,7 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
   p.max_pages = d->max_pages;
   p.n_pages = d->n_pages;
   p.rows = sc_plan.rows;
-  p.blocks = decode_blocks(d->dh);
+  p.fit = blocks_that_fit(d->dh);
   p.max_shares = sc_plan.max_shares;
   p.num_splits = d->num_splits;
   p.io_f32 = d->dtype == KVP_F32;
@@ -932,14 +934,14 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
       }
     }
     const long long units = (long long)n * d->B * d->Hkv;
-    // No more blocks than the longest lists could give work to; shares go by the lengths on the device, and so does
-    // whether whole units are dealt out instead.
+    // a block for every share of the longest list; shares go by the lengths on the device, and so does whether whole units
+    // are dealt out instead
     const long long blocks = d->num_splits > 0 ? units * d->num_splits
-                                               : std::min((long long)p.blocks, std::max((long long)n * sc_plan.max_shares, units));
+                                               : std::max((long long)sc_plan.max_shares, std::min(units, (long long)p.fit * MAX_ROUNDS));
     if (units > 0x7fffffffLL || blocks > 0x7fffffffLL) return KVP_ERR_UNSUPPORTED;
     p.n_groups = n;
-    p.by_units = dealt_by_units(longest_list(d), d->B * d->Hkv);
-    const long long unit_pieces = d->num_splits > 0 ? d->num_splits : sc_plan.max_shares / ((long long)d->B * d->Hkv);
+    p.by_units = dealt_by_units(longest_list(d, n), units, p.fit);
+    const long long unit_pieces = d->num_splits > 0 ? d->num_splits : sc_plan.max_shares / units;
     const int wpr = unit_pieces > 8 ? 8 : 1;   // many pieces a unit: eight warps share those of a row
     const int rows_per_block = COMBINE_THREADS / 32 / wpr;
     const dim3 grid(static_cast<unsigned>(blocks));

@@ -25,7 +25,7 @@ def dense(pool, bt, lens, page):
     (1, [0], 1, 16, 1, 64, 64, [9001], False),                           # the same at dh 64, all 16 rows
     (2, [0, 0], 40, 8, 2, 128, 16, [17 + 13 * b for b in range(40)], False),   # more than 32 lengths; units of 2 to 34 granules
     (3, [0, 1, 2], 33, 2, 2, 64, 32, [16] * 33, False),                  # units of one granule, dealt out whole
-    (2, [0, 1], 3, 4, 4, 128, 16, [1100, 3, 900], False),                # units of 1 to 69 granules in equal shares, two groups
+    (2, [0, 1], 3, 4, 4, 128, 16, [1100, 3, 900], False),                # units of 1 to 69 granules, two groups
     (4, [0, 0, 0, 0], 3, 12, 2, 128, 32, [640, 1, 333], True),           # 16-row passes of uneven groups; built-in scratch
 ])
 def test_decode_shares(L, donor, B, Hq, Hkv, dh, page, lens, static):
