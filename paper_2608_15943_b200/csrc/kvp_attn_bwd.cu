@@ -37,6 +37,7 @@ namespace {
 
 constexpr int BT = 128;    // key rows per tile
 constexpr int BQ2 = 64;    // query rows per step
+constexpr int MAX_CLASSES = 128;
 constexpr int MAX_GROUP = 8;  // layers of one donor group per launch
 constexpr uint32_t HALF_BYTES = 128 * 128;  // [128 rows x 128 B] block
 constexpr uint32_t QHALF_BYTES = 64 * 128;  // [ 64 rows x 128 B] block
@@ -58,11 +59,15 @@ constexpr int DQ_STAGE_BYTES = BQ2 * 32 * 4;  // one drain warp's share of a ste
 constexpr int kStepsPerCta = 256;
 constexpr int kMinWindow = 16;
 // A CTA costs about seven steps besides its steps (prologue, dK / dV reduction, gap between two CTAs), and the last CTAs of
-// a launch leave the device idle for half of their length: with n steps per SM in all, n * 7 / t + t / 2 is least at
-// t = sqrt(14 n).  Measured (us; always 256 steps -> this): B3 S776 H16/4 dh64, 3 layers 119 -> 95; B4 S632 H8/2 dh128,
-// 8 layers 201 -> 119; B1 S4096 H32/8 dh128, 1 layer 445 -> 337.  From about 4700 steps per SM on the 256 stand.
-constexpr float kTailFactor = 14.f;
+// a launch leave the device idle for some part of their length: with n steps per SM in all, n * 7 / t + 0.3 t is least at
+// t = sqrt(24 n), and there is nothing to gain from fewer CTAs than one for every SM (1.5 n).  Up to kLongestFirst steps per SM the CTAs are dispatched longest first; beyond, in an order that keeps
+// what a wave touches in L2 (2 layers of 4 x 4096 tokens, dh 64: 1970 us in that order, 2010 longest first).
+// Measured (us; always 256 steps, index order -> this): B3 S776 H16/4 dh64, 3 layers 119 -> 80; B4 S632 H8/2 dh128, 8
+// layers 201 -> 107; B1 S2048 H8/8 dh128, 1 layer 50 -> 44; B1 S4096 H32/8 dh128, 1 layer 445 -> 345.  From about 2700
+// steps per SM on the 256 stand.
+constexpr float kTailFactor = 24.f;
 constexpr int kMinSteps = 2;
+constexpr float kLongestFirst = 512.f;
 
 template <int DH>
 struct BwdSmem {
@@ -98,6 +103,11 @@ struct BwdParams {
   int window[MAX_GROUP];          // query tiles per CTA
   int parts[MAX_GROUP];           // parts the query streams of a (window, key tile) are dealt out in
   int ctas_per_pair[MAX_GROUP];   // CTAs of one (batch, KV head): parts x sum over windows of the key tiles that see the window
+  // Longest CTAs first (small launches): classes of CTAs with the same (group, window, key tile), hence the same number of
+  // steps; class c holds blocks [class_end[c - 1], class_end[c]), (batch, KV head) and part inside.  0: in index order.
+  int n_classes;
+  uint16_t class_end[MAX_CLASSES];
+  uint32_t class_id[MAX_CLASSES];   // group << 24 | window << 12 | key tile
   int n_groups;
   int B, S, Hq, Hkv;
   int causal;
@@ -173,22 +183,37 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   // dK / dV partials to the (cleared) output with reductions.
   const int n_jt = (p.S + BT - 1) / BT;
   const int n_qt = (p.S + BQ2 - 1) / BQ2;
-  int grp = 0;
-  while (grp + 1 < p.n_groups && int(blockIdx.x) >= p.cta_begin[grp + 1]) ++grp;
+  int grp = 0, jt = 0, win = 0, pair = 0, part = 0;
+  if (p.n_classes > 0) {
+    int lo = 0, hi = p.n_classes - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if (int(blockIdx.x) < p.class_end[mid]) hi = mid;
+      else lo = mid + 1;
+    }
+    const uint32_t id = p.class_id[lo];
+    grp = id >> 24;
+    win = (id >> 12) & 0xfff;
+    jt = id & 0xfff;
+    const int in_class = int(blockIdx.x) - (lo ? p.class_end[lo - 1] : 0);
+    pair = in_class / p.parts[grp];
+    part = in_class - pair * p.parts[grp];
+  } else {
+    while (grp + 1 < p.n_groups && int(blockIdx.x) >= p.cta_begin[grp + 1]) ++grp;
+    const int in_group = blockIdx.x - p.cta_begin[grp];
+    pair = in_group / p.ctas_per_pair[grp];
+    part = (in_group - pair * p.ctas_per_pair[grp]) % p.parts[grp];
+    jt = (in_group - pair * p.ctas_per_pair[grp]) / p.parts[grp];
+    for (;; ++win) {
+      const int vis = p.causal ? min(n_jt, ((win + 1) * p.window[grp] * BQ2 + BT - 1) / BT) : n_jt;
+      if (jt < vis) break;
+      jt -= vis;
+    }
+  }
+  const int parts = p.parts[grp];
+  const int window = p.window[grp];
   const int slot0 = p.first_slot[grp];
   const int n_layers = p.first_slot[grp + 1] - slot0;
-  const int window = p.window[grp];
-  const int in_group = blockIdx.x - p.cta_begin[grp];
-  const int pair = in_group / p.ctas_per_pair[grp];
-  const int parts = p.parts[grp];
-  const int part = (in_group - pair * p.ctas_per_pair[grp]) % parts;
-  int jt = (in_group - pair * p.ctas_per_pair[grp]) / parts;
-  int win = 0;
-  for (;; ++win) {
-    const int vis = p.causal ? min(n_jt, ((win + 1) * window * BQ2 + BT - 1) / BT) : n_jt;
-    if (jt < vis) break;
-    jt -= vis;
-  }
   const int hk = pair % p.Hkv;
   const int b = pair / p.Hkv;
   const int G = p.Hq / p.Hkv;
@@ -755,6 +780,39 @@ int make_map_sum(CUtensorMap* m, const void* base, int B, int S, int H, int dh) 
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Orders the CTAs of a launch by their number of steps, longest first, so that the short ones (diagonal key tiles, last
+// windows) fill in at the end; 0 when there are more classes than the parameter block holds.  Only for launches that do
+// not run long enough for the order to cost L2 locality.  Three layers of 3 x 776 tokens, dh 64: 95 us in index
+// order, 79 longest first.
+int longest_first(BwdParams& p, int n_groups, int n_pairs, int n_jt, int n_qt, int G, int causal) {
+  struct Class {
+    int steps, ctas;
+    uint32_t id;
+  } cls[MAX_CLASSES];
+  int n = 0, total = 0;
+  for (int g = 0; g < n_groups; ++g) {
+    const int streams = (p.first_slot[g + 1] - p.first_slot[g]) * G, w = p.window[g];
+    for (int win = 0; win * w < n_qt; ++win) {
+      const int vis = causal ? std::min(n_jt, ((win + 1) * w * BQ2 + BT - 1) / BT) : n_jt;
+      for (int j = 0; j < vis; ++j) {
+        if (n == MAX_CLASSES || win > 0xfff || j > 0xfff) return 0;
+        const int tiles = std::min(n_qt, (win + 1) * w) - std::max(causal ? j * (BT / BQ2) : 0, win * w);
+        cls[n++] = Class{tiles * streams / p.parts[g], n_pairs * p.parts[g], uint32_t(g) << 24 | uint32_t(win) << 12 | uint32_t(j)};
+        total += n_pairs * p.parts[g];
+      }
+    }
+  }
+  if (total > 0xffff) return 0;
+  std::stable_sort(cls, cls + n, [](const Class& a, const Class& b) { return a.steps > b.steps; });
+  int end = 0;
+  for (int c = 0; c < n; ++c) {
+    end += cls[c].ctas;
+    p.class_end[c] = uint16_t(end);
+    p.class_id[c] = cls[c].id;
+  }
+  return n;
+}
+
 // Member layers of the launches' accumulators that are live at once: a launch takes whole donor groups until it
 // holds MAX_GROUP member layers.
 int max_layers_per_launch(const kvp_shape* s) { return s->L < MAX_GROUP ? s->L : MAX_GROUP; }
@@ -820,7 +878,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   long long stream_steps = 0;
   for (int j = 0; j < n_jt; ++j) stream_steps += causal ? n_qt - j * (BT / BQ2) : n_qt;
   const float steps_per_sm = float(stream_steps) * n_pairs * s->L * G / sm_count();
-  const int target = std::max(kMinSteps, int(sqrtf(std::min(float(kStepsPerCta) * kStepsPerCta, kTailFactor * steps_per_sm))));
+  const int target = std::max(kMinSteps, int(std::min(std::min(float(kStepsPerCta), 1.5f * steps_per_sm), sqrtf(kTailFactor * steps_per_sm))));
   size_t gi = 0;
   while (gi < groups.size()) {
     BwdParams p;
@@ -843,7 +901,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
         ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
         ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
-        ax.dq[slots] = reinterpret_cast<__nv_bfloat16*>(dq[l]);
+        ax.dq[slots] = dq[l];
         ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
         ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
@@ -859,7 +917,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       int window = std::max(std::max(1, target / (kStepsPerCta / kMinWindow)), (target + streams - 1) / streams);
       if (window > 1) window += window & 1;   // whole key tiles of two query tiles: no CTA for half of a diagonal tile
       p.window[ng] = std::min(n_qt, window);
-      p.parts[ng] = target < kStepsPerCta ? std::max(1, std::min(streams, (streams * p.window[ng] + target / 2) / target)) : 1;
+      p.parts[ng] = target < kStepsPerCta ? std::max(1, std::min(streams, (streams * p.window[ng] + (p.window[ng] == 1 ? target - 1 : target / 2)) / target)) : 1;
       // Up to 128 tokens dQ has one term, and two CTAs' terms of dK / dV add up to the same value in either order: such
       // short sequences keep results that do not differ from run to run.
       if (n_jt == 1) p.parts[ng] = std::min(p.parts[ng], p.window[ng] < n_qt ? 1 : 2);
@@ -890,6 +948,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       p.first_slot[i + 1] = slots;
       p.cta_begin[i + 1] = p.cta_begin[ng];
     }
+    p.n_classes = steps_per_sm <= kLongestFirst ? longest_first(p, ng, n_pairs, n_jt, n_qt, G, causal) : 0;
     p.n_groups = ng;
     p.B = s->B;
     p.S = s->S;
