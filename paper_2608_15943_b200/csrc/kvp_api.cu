@@ -7,13 +7,13 @@
 
 namespace kvp {
 int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* const* q, const void* const* k,
-                    const void* const* v, void* const* o, float* const* lse, int n, cudaStream_t stream);
+                    const void* const* v, void* const* o, bool o_f32, float* const* lse, int n, cudaStream_t stream);
 int attn_fwd_max_layers();
 size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor);
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, float* const* dk_sum, float* const* dv_sum, void* ws,
-                 size_t ws_bytes, cudaStream_t stream);
+                 const float* const* lse, void* const* dq, bool dq_f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 cudaStream_t stream);
 
 namespace {
 
@@ -47,8 +47,8 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // ---------------------------------------------------------------------------------------------
 // KVP_F32 interface: bf16 shadow copies of the caller's fp32 tensors, carved from the workspace behind the
-// operation's own scratch.  Inputs are rounded on the way in, outputs widened on the way out; in between the
-// bf16 entry point runs unchanged.
+// operation's own scratch.  Inputs are rounded on the way in by one launch; the kernels of the bf16 entry point then
+// store their bf16 results as fp32.
 // ---------------------------------------------------------------------------------------------
 struct TensorSet {   // one per-layer tensor array of an entry point
   size_t elems;      // elements per layer
@@ -74,15 +74,8 @@ class Shadows {
       if (arr[l] != nullptr) inputs_.push_back(CastItem{src[l], arr[l], t.elems});
     return reinterpret_cast<const void* const*>(arr.data());
   }
-  // bf16 buffers standing in for an fp32 output array; finish() widens them into the caller's tensors
-  void* const* out(void* const* dst, const TensorSet& t) {
-    std::vector<void*>& arr = reserve(t);
-    for (int l = 0; l < s_->L; ++l)
-      if (arr[l] != nullptr) outputs_.push_back(CastItem{arr[l], dst[l], t.elems});
-    return arr.data();
-  }
-  int round_inputs() { return cast_tensors(inputs_.data(), int(inputs_.size()), false, stream_); }
-  int finish() { return cast_tensors(outputs_.data(), int(outputs_.size()), true, stream_); }
+  const std::vector<CastItem>& inputs() const { return inputs_; }
+  int round_inputs() { return cast_tensors(inputs_.data(), int(inputs_.size()), stream_); }
 
  private:
   std::vector<void*>& reserve(const TensorSet& t) {
@@ -100,7 +93,7 @@ class Shadows {
   uint8_t* cur_;
   cudaStream_t stream_;
   std::vector<std::vector<void*>> arrays_;
-  std::vector<CastItem> inputs_, outputs_;
+  std::vector<CastItem> inputs_;
 };
 
 struct Sizes {
@@ -149,24 +142,117 @@ size_t op_shadow_bytes(int op, const kvp_shape* s, const int32_t* donor) {
   const Sizes z = sizes_of(s);
   switch (op) {
     case KVP_OP_PROJ_FWD: {
-      const TensorSet sets[] = {z.x, z.wq, z.wkv, z.wkv, z.q, z.kv, z.kv};
-      return shadow_bytes(s, donor, sets, 7);
-    }
-    case KVP_OP_PROJ_BWD: {
-      const TensorSet sets[] = {z.x, z.wq, z.wkv, z.wkv, z.q, z.x};   // x, wq, wk, wv, dq in; dx out
-      return shadow_bytes(s, donor, sets, 6);
-    }
-    case KVP_OP_ATTN_FWD: {
-      const TensorSet sets[] = {z.q, z.kv, z.kv, z.q};                // q, k, v in; o out
+      const TensorSet sets[] = {z.x, z.wq, z.wkv, z.wkv};
       return shadow_bytes(s, donor, sets, 4);
     }
+    case KVP_OP_PROJ_BWD: {
+      const TensorSet sets[] = {z.x, z.wq, z.wkv, z.wkv, z.q};   // x, wq, wk, wv, dq
+      return shadow_bytes(s, donor, sets, 5);
+    }
+    case KVP_OP_ATTN_FWD: {
+      const TensorSet sets[] = {z.q, z.kv, z.kv};
+      return shadow_bytes(s, donor, sets, 3);
+    }
     case KVP_OP_ATTN_BWD: {
-      const TensorSet sets[] = {z.q, z.kv, z.kv, z.q, z.q, z.q};      // q, k, v, o, dO in; dq out
-      return shadow_bytes(s, donor, sets, 6);
+      const TensorSet sets[] = {z.q, z.kv, z.kv, z.q, z.q};      // q, k, v, o, dO
+      return shadow_bytes(s, donor, sets, 5);
     }
     default:
       return 0;
   }
+}
+
+}  // namespace
+}  // namespace kvp
+
+namespace kvp {
+namespace {
+
+// The bf16 forms of the entry points; out_f32: bf16 results stored as fp32.
+int proj_fwd_bf16(const kvp_shape* s, const int32_t* donor, const void* const* x, const void* const* wq, const void* const* wk,
+                  const void* const* wv, void* const* q, void* const* k, void* const* v, bool out_f32, cudaStream_t stream) {
+  const int T = s->B * s->S, D = s->D, Nq = s->Hq * s->dh, Nkv = s->Hkv * s->dh;
+  const int out = out_f32 ? OUT_F32_OF_BF16 : OUT_BF16;
+  // Every projection of every layer in one grouped launch; consumers have no K/V projections (Eq. 3).
+  std::vector<GemmProblem> probs;
+  probs.reserve(size_t(3) * s->L);
+  for (int l = 0; l < s->L; ++l) probs.push_back(problem(T, Nq, {x[l], wq[l], D, D, D}, 0, 0, q[l], Nq, out));
+  for (int l = 0; l < s->L; ++l) {
+    if (donor[l] != l) continue;
+    probs.push_back(problem(T, Nkv, {x[l], wk[l], D, D, D}, 0, 0, k[l], Nkv, out));
+    probs.push_back(problem(T, Nkv, {x[l], wv[l], D, D, D}, 0, 0, v[l], Nkv, out));
+  }
+  return gemm_grouped(probs.data(), int(probs.size()), stream, true);
+}
+
+// before: conversions that the same launch as those of the first chunk's sums performs
+int proj_bwd_bf16(const kvp_shape* s, const int32_t* donor, const void* const* x, const void* const* wq, const void* const* wk,
+                  const void* const* wv, const void* const* dq, const float* const* dk_sum, const float* const* dv_sum,
+                  float* const* dwq, float* const* dwk, float* const* dwv, void* const* dx, bool dx_f32, int layer_begin,
+                  int layer_end, void* ws, const std::vector<CastItem>& before, cudaStream_t stream) {
+  const int T = s->B * s->S, D = s->D, Nq = s->Hq * s->dh, Nkv = s->Hkv * s->dh;
+  const size_t n_kv = size_t(T) * Nkv;
+  const size_t slot = align256(n_kv * 2);
+  uint8_t* bf = reinterpret_cast<uint8_t*>(ws);
+  // Chunks of up to kProjBwdChunk layers: the fp32 donor-group sums of the chunk's owners are rounded to bf16 into
+  // the workspace, then ONE grouped launch produces every gradient of the chunk.  The weight gradients come first
+  // in the list (their tiles run over all T tokens, the longest), then dX = dQ Wq + dK Wk + dV Wv of the owners
+  // (three K segments into one accumulator), then the consumers' dX = dQ Wq.
+  std::vector<GemmProblem> probs;
+  for (int c0 = layer_begin; c0 < layer_end; c0 += kProjBwdChunk) {
+    const int c1 = std::min(layer_end, c0 + kProjBwdChunk);
+    probs.clear();
+    std::vector<uint8_t*> dk_bf(size_t(c1 - c0), nullptr), dv_bf(size_t(c1 - c0), nullptr);
+    std::vector<CastItem> sums = c0 == layer_begin ? before : std::vector<CastItem>();
+    int owners = 0;
+    for (int l = c0; l < c1; ++l) {
+      if (donor[l] != l) continue;
+      dk_bf[l - c0] = bf + size_t(2 * owners) * slot;
+      dv_bf[l - c0] = bf + size_t(2 * owners + 1) * slot;
+      ++owners;
+      sums.push_back(CastItem{dk_sum[l], dk_bf[l - c0], n_kv});
+      sums.push_back(CastItem{dv_sum[l], dv_bf[l - c0], n_kv});
+    }
+    int rc = cast_tensors(sums.data(), int(sums.size()), stream);
+    if (rc != KVP_OK) return rc;
+    // dWq = dQ^T X : A = dQ stored [T, Nq] (MN-major for M = Nq), B = X stored [T, D] (MN-major for N = D)
+    for (int l = c0; l < c1; ++l) probs.push_back(problem(Nq, D, {dq[l], x[l], Nq, D, T}, 1, 1, dwq[l], D, 1));
+    for (int l = c0; l < c1; ++l) {
+      if (donor[l] != l) continue;
+      probs.push_back(problem(Nkv, D, {dk_bf[l - c0], x[l], Nkv, D, T}, 1, 1, dwk[l], D, 1));
+      probs.push_back(problem(Nkv, D, {dv_bf[l - c0], x[l], Nkv, D, T}, 1, 1, dwv[l], D, 1));
+    }
+    for (int l = c0; l < c1; ++l) {
+      if (donor[l] != l) continue;
+      GemmProblem g = problem(T, D, {dq[l], wq[l], Nq, D, Nq}, 0, 1, dx[l], D, dx_f32 ? OUT_F32_OF_BF16 : OUT_BF16);
+      g.segs[1] = {dk_bf[l - c0], wk[l], Nkv, D, Nkv};
+      g.segs[2] = {dv_bf[l - c0], wv[l], Nkv, D, Nkv};
+      g.nseg = 3;
+      probs.push_back(g);
+    }
+    for (int l = c0; l < c1; ++l)
+      if (donor[l] != l) probs.push_back(problem(T, D, {dq[l], wq[l], Nq, D, Nq}, 0, 1, dx[l], D, dx_f32 ? OUT_F32_OF_BF16 : OUT_BF16));
+    rc = gemm_grouped(probs.data(), int(probs.size()), stream, false);
+    if (rc != KVP_OK) return rc;
+  }
+  return KVP_OK;
+}
+
+int attn_fwd_bf16(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q, const void* const* k,
+                  const void* const* v, void* const* o, bool o_f32, float* const* lse, cudaStream_t stream) {
+  // up to eight layers per launch, each with the K / V of its donor
+  std::vector<const void*> kd(size_t(s->L)), vd(size_t(s->L));
+  for (int l = 0; l < s->L; ++l) {
+    kd[l] = k[donor[l]];
+    vd[l] = v[donor[l]];
+  }
+  const int chunk = attn_fwd_max_layers();
+  for (int l0 = 0; l0 < s->L; l0 += chunk) {
+    const int n = std::min(chunk, s->L - l0);
+    const int rc = attn_fwd_layers(s, causal, scale, q + l0, kd.data() + l0, vd.data() + l0, o + l0, o_f32, lse + l0, n, stream);
+    if (rc != KVP_OK) return rc;
+  }
+  return KVP_OK;
 }
 
 }  // namespace
@@ -198,27 +284,11 @@ extern "C" int kvp_proj_fwd(const kvp_shape* s, const int32_t* donor, const void
     const void* const* wq16 = sh.in(wq, z.wq);
     const void* const* wk16 = sh.in(wk, z.wkv);
     const void* const* wv16 = sh.in(wv, z.wkv);
-    void* const* q16 = sh.out(q, z.q);
-    void* const* k16 = sh.out(k, z.kv);
-    void* const* v16 = sh.out(v, z.kv);
     rc = sh.round_inputs();
     if (rc != KVP_OK) return rc;
-    kvp_shape s16 = *s;
-    s16.dtype = KVP_BF16;
-    rc = kvp_proj_fwd(&s16, donor, x16, wq16, wk16, wv16, q16, k16, v16, ws, ws_bytes, stream_);
-    return rc != KVP_OK ? rc : sh.finish();
+    return proj_fwd_bf16(s, donor, x16, wq16, wk16, wv16, q, k, v, true, stream);
   }
-  const int T = s->B * s->S, D = s->D, Nq = s->Hq * s->dh, Nkv = s->Hkv * s->dh;
-  // Every projection of every layer in one grouped launch; consumers have no K/V projections (Eq. 3).
-  std::vector<GemmProblem> probs;
-  probs.reserve(size_t(3) * s->L);
-  for (int l = 0; l < s->L; ++l) probs.push_back(problem(T, Nq, {x[l], wq[l], D, D, D}, 0, 0, q[l], Nq, 0));
-  for (int l = 0; l < s->L; ++l) {
-    if (donor[l] != l) continue;
-    probs.push_back(problem(T, Nkv, {x[l], wk[l], D, D, D}, 0, 0, k[l], Nkv, 0));
-    probs.push_back(problem(T, Nkv, {x[l], wv[l], D, D, D}, 0, 0, v[l], Nkv, 0));
-  }
-  return gemm_grouped(probs.data(), int(probs.size()), stream, true);
+  return proj_fwd_bf16(s, donor, x, wq, wk, wv, q, k, v, false, stream);
 }
 
 extern "C" int kvp_proj_bwd(const kvp_shape* s, const int32_t* donor, const void* const* x, const void* const* wq,
@@ -251,6 +321,7 @@ extern "C" int kvp_proj_bwd_range(const kvp_shape* s, const int32_t* donor, cons
   if (ws == nullptr || ws_bytes < need || !aligned16(ws)) return KVP_ERR_WORKSPACE;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   if (s->dtype == KVP_F32) {
+    if (layer_begin != 0 || layer_end != s->L) return KVP_ERR_UNSUPPORTED;   // the fp32 interface converts whole arrays
     const Sizes z = sizes_of(s);
     Shadows sh(s, donor, ws, align256(op_scratch_bytes(KVP_OP_PROJ_BWD, s, donor)), stream);
     const void* const* x16 = sh.in(x, z.x);
@@ -258,61 +329,10 @@ extern "C" int kvp_proj_bwd_range(const kvp_shape* s, const int32_t* donor, cons
     const void* const* wk16 = sh.in(wk, z.wkv);
     const void* const* wv16 = sh.in(wv, z.wkv);
     const void* const* dq16 = sh.in(dq, z.q);
-    void* const* dx16 = sh.out(dx, z.x);
-    rc = sh.round_inputs();
-    if (rc != KVP_OK) return rc;
-    kvp_shape s16 = *s;
-    s16.dtype = KVP_BF16;
-    if (layer_begin != 0 || layer_end != s->L) return KVP_ERR_UNSUPPORTED;   // the fp32 interface converts whole arrays
-    rc = kvp_proj_bwd(&s16, donor, x16, wq16, wk16, wv16, dq16, dk_sum, dv_sum, dwq, dwk, dwv, dx16, ws, ws_bytes, stream_);
-    return rc != KVP_OK ? rc : sh.finish();
+    return proj_bwd_bf16(s, donor, x16, wq16, wk16, wv16, dq16, dk_sum, dv_sum, dwq, dwk, dwv, dx, true, 0, s->L, ws, sh.inputs(),
+                         stream);
   }
-  const int T = s->B * s->S, D = s->D, Nq = s->Hq * s->dh, Nkv = s->Hkv * s->dh;
-  const size_t n_kv = size_t(T) * Nkv;
-  const size_t slot = align256(n_kv * 2);
-  uint8_t* bf = reinterpret_cast<uint8_t*>(ws);
-  // Chunks of up to kProjBwdChunk layers: the fp32 donor-group sums of the chunk's owners are rounded to bf16 into
-  // the workspace, then ONE grouped launch produces every gradient of the chunk.  The weight gradients come first
-  // in the list (their tiles run over all T tokens, the longest), then dX = dQ Wq + dK Wk + dV Wv of the owners
-  // (three K segments into one accumulator), then the consumers' dX = dQ Wq.
-  std::vector<GemmProblem> probs;
-  for (int c0 = layer_begin; c0 < layer_end; c0 += kProjBwdChunk) {
-    const int c1 = std::min(layer_end, c0 + kProjBwdChunk);
-    probs.clear();
-    std::vector<uint8_t*> dk_bf(size_t(c1 - c0), nullptr), dv_bf(size_t(c1 - c0), nullptr);
-    std::vector<CastItem> sums;
-    int owners = 0;
-    for (int l = c0; l < c1; ++l) {
-      if (donor[l] != l) continue;
-      dk_bf[l - c0] = bf + size_t(2 * owners) * slot;
-      dv_bf[l - c0] = bf + size_t(2 * owners + 1) * slot;
-      ++owners;
-      sums.push_back(CastItem{dk_sum[l], dk_bf[l - c0], n_kv});
-      sums.push_back(CastItem{dv_sum[l], dv_bf[l - c0], n_kv});
-    }
-    rc = cast_tensors(sums.data(), int(sums.size()), false, stream);
-    if (rc != KVP_OK) return rc;
-    // dWq = dQ^T X : A = dQ stored [T, Nq] (MN-major for M = Nq), B = X stored [T, D] (MN-major for N = D)
-    for (int l = c0; l < c1; ++l) probs.push_back(problem(Nq, D, {dq[l], x[l], Nq, D, T}, 1, 1, dwq[l], D, 1));
-    for (int l = c0; l < c1; ++l) {
-      if (donor[l] != l) continue;
-      probs.push_back(problem(Nkv, D, {dk_bf[l - c0], x[l], Nkv, D, T}, 1, 1, dwk[l], D, 1));
-      probs.push_back(problem(Nkv, D, {dv_bf[l - c0], x[l], Nkv, D, T}, 1, 1, dwv[l], D, 1));
-    }
-    for (int l = c0; l < c1; ++l) {
-      if (donor[l] != l) continue;
-      GemmProblem g = problem(T, D, {dq[l], wq[l], Nq, D, Nq}, 0, 1, dx[l], D, 0);
-      g.segs[1] = {dk_bf[l - c0], wk[l], Nkv, D, Nkv};
-      g.segs[2] = {dv_bf[l - c0], wv[l], Nkv, D, Nkv};
-      g.nseg = 3;
-      probs.push_back(g);
-    }
-    for (int l = c0; l < c1; ++l)
-      if (donor[l] != l) probs.push_back(problem(T, D, {dq[l], wq[l], Nq, D, Nq}, 0, 1, dx[l], D, 0));
-    rc = gemm_grouped(probs.data(), int(probs.size()), stream, false);
-    if (rc != KVP_OK) return rc;
-  }
-  return KVP_OK;
+  return proj_bwd_bf16(s, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx, false, layer_begin, layer_end, ws, {}, stream);
 }
 
 extern "C" int kvp_out_proj_fwd(const kvp_shape* s, const void* const* o, const void* const* wo, void* const* y,
@@ -368,27 +388,11 @@ extern "C" int kvp_attn_fwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* q16 = sh.in(q, z.q);
     const void* const* k16 = sh.in(k, z.kv);
     const void* const* v16 = sh.in(v, z.kv);
-    void* const* o16 = sh.out(o, z.q);
     rc = sh.round_inputs();
     if (rc != KVP_OK) return rc;
-    kvp_shape s16 = *s;
-    s16.dtype = KVP_BF16;
-    rc = kvp_attn_fwd(&s16, donor, causal, scale, q16, k16, v16, o16, lse, ws, ws_bytes, stream_);
-    return rc != KVP_OK ? rc : sh.finish();
+    return attn_fwd_bf16(s, donor, causal, scale, q16, k16, v16, o, true, lse, stream);
   }
-  // up to eight layers per launch, each with the K / V of its donor
-  std::vector<const void*> kd(size_t(s->L)), vd(size_t(s->L));
-  for (int l = 0; l < s->L; ++l) {
-    kd[l] = k[donor[l]];
-    vd[l] = v[donor[l]];
-  }
-  const int chunk = attn_fwd_max_layers();
-  for (int l0 = 0; l0 < s->L; l0 += chunk) {
-    const int n = std::min(chunk, s->L - l0);
-    rc = attn_fwd_layers(s, causal, scale, q + l0, kd.data() + l0, vd.data() + l0, o + l0, lse + l0, n, stream);
-    if (rc != KVP_OK) return rc;
-  }
-  return KVP_OK;
+  return attn_fwd_bf16(s, donor, causal, scale, q, k, v, o, false, lse, stream);
 }
 
 extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
@@ -415,14 +419,11 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* v16 = sh.in(v, z.kv);
     const void* const* o16 = sh.in(o, z.q);
     const void* const* do16 = sh.in(d_o, z.q);
-    void* const* dq16 = sh.out(dq, z.q);
     rc = sh.round_inputs();
     if (rc != KVP_OK) return rc;
-    kvp_shape s16 = *s;
-    s16.dtype = KVP_BF16;
-    rc = kvp_attn_bwd(&s16, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq16, dk_sum, dv_sum, ws, ws_bytes, stream_);
-    return rc != KVP_OK ? rc : sh.finish();
+    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, true, dk_sum, dv_sum, ws,
+                        reinterpret_cast<cudaStream_t>(stream_));
   }
-  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, dk_sum, dv_sum, ws, ws_bytes,
+  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, false, dk_sum, dv_sum, ws,
                       reinterpret_cast<cudaStream_t>(stream_));
 }

@@ -644,12 +644,13 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
 struct AuxParams {
   const __nv_bfloat16* o[MAX_GROUP];
   const __nv_bfloat16* d_o[MAX_GROUP];
-  __nv_bfloat16* dq[MAX_GROUP];
+  void* dq[MAX_GROUP];        // bf16 or (dq_f32) the bf16 values as fp32
   float* delta[MAX_GROUP];
   float* dq_acc[MAX_GROUP];
   float* dk_sum[MAX_GROUP];   // per group
   float* dv_sum[MAX_GROUP];
   int n_groups;
+  int dq_f32;
   int B, S, Hq;
   size_t acc_v4;              // 16-byte pieces of one dQ accumulator
   size_t kv_v4;               // 16-byte pieces of one dK (dV) sum
@@ -663,7 +664,6 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   constexpr int TPR = DH / 8;  // threads per query row
   grid_dep_wait();
   const float* __restrict__ acc = p.dq_acc[blockIdx.y];
-  __nv_bfloat16* __restrict__ dq = p.dq[blockIdx.y];
   const int S = p.S, Hq = p.Hq;
   const float scale = p.scale;
   const int n_qt = (S + BQ2 - 1) / BQ2;
@@ -689,7 +689,14 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
     v.w = pack_bf16(hi.z * scale, hi.w * scale);
     const int hq = int(bh % Hq);
     const int bb = int(bh / Hq);
-    *reinterpret_cast<uint4*>(dq + ((size_t(bb) * S + s) * Hq + hq) * DH + quarter * 32 + d0) = v;
+    const size_t at = ((size_t(bb) * S + s) * Hq + hq) * DH + quarter * 32 + d0;
+    if (p.dq_f32) {
+      float* out = reinterpret_cast<float*>(p.dq[blockIdx.y]) + at;
+      *reinterpret_cast<uint4*>(out) = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
+      *reinterpret_cast<uint4*>(out + 4) = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
+    } else {
+      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dq[blockIdx.y]) + at) = v;
+    }
   }
 }
 
@@ -839,9 +846,8 @@ size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor) {
 
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, float* const* dk_sum, float* const* dv_sum, void* ws,
-                 size_t ws_bytes, cudaStream_t stream) {
-  (void)ws_bytes;
+                 const float* const* lse, void* const* dq, bool dq_f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 cudaStream_t stream) {
   const int dh = s->dh;
   const float sc = scale == 0.f ? 1.f / sqrtf(float(dh)) : scale;
   const size_t delta_bytes = align256(size_t(s->B) * s->Hq * s->S * 4);
@@ -958,6 +964,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     p.scale = sc;
     p.scale_log2 = sc * 1.4426950408889634f;
     ax.n_groups = ng;
+    ax.dq_f32 = dq_f32;
     ax.B = s->B;
     ax.S = s->S;
     ax.Hq = s->Hq;

@@ -53,9 +53,10 @@ constexpr int FWD_MAX_LAYERS = 8;   // layers per launch
 struct FwdParams {
   // per layer: 4-D [B, S, H, dh] tensors, box {64, 1, 128, 1}; K and V are those of the layer's donor
   CUtensorMap map_q[FWD_MAX_LAYERS], map_k[FWD_MAX_LAYERS], map_v[FWD_MAX_LAYERS];
-  __nv_bfloat16* o[FWD_MAX_LAYERS];  // [B, S, Hq, dh]
+  void* o[FWD_MAX_LAYERS];           // [B, S, Hq, dh], bf16 or (o_f32) the bf16 values as fp32
   float* lse[FWD_MAX_LAYERS];        // [B, Hq, S]
   int n_layers;
+  int o_f32;
   int B, S, Hq, Hkv;
   int causal;
   float scale_log2;                 // scale * log2(e)
@@ -407,7 +408,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
         const float l_sum = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
         const float inv_l = 1.f / l_sum;
         const bool valid = q_row < p.S;
-        __nv_bfloat16* dst = p.o[w.layer] + ((size_t(w.b) * p.S + (valid ? q_row : 0)) * p.Hq + w.hq) * DH;
+        const size_t o_at = ((size_t(w.b) * p.S + (valid ? q_row : 0)) * p.Hq + w.hq) * DH;
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.o[w.layer]) + o_at;
 #pragma unroll
         for (int g = 0; g < DH / 32; ++g) {
           uint32_t tmp[32];
@@ -417,7 +419,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
             tc_fence_before_sync();
             mbar_arrive(&o_free[x]);
           }
-          if (valid) {
+          if (valid && p.o_f32) {
+            float* dst32 = reinterpret_cast<float*>(p.o[w.layer]) + o_at;
+#pragma unroll
+            for (int v4 = 0; v4 < 8; ++v4)
+              *reinterpret_cast<uint4*>(dst32 + g * 32 + v4 * 4) =
+                  make_uint4(bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 0]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 1]) * inv_l),
+                             bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 2]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 3]) * inv_l));
+          } else if (valid) {
 #pragma unroll
             for (int v4 = 0; v4 < 4; ++v4) {
               uint4 v;
@@ -467,18 +476,25 @@ int attn_fwd_read_status() {
 
 // n layers (at most FWD_MAX_LAYERS) in one launch: q[i] [B,S,Hq,dh], k[i] / v[i] [B,S,Hkv,dh] of layer i's donor.
 int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* const* q, const void* const* k,
-                    const void* const* v, void* const* o, float* const* lse, int n, cudaStream_t stream) {
+                    const void* const* v, void* const* o, bool o_f32, float* const* lse, int n, cudaStream_t stream) {
   if (n < 1 || n > FWD_MAX_LAYERS) return KVP_ERR_INVALID_ARG;
   static thread_local FwdParams p;   // 3 KB of tensor maps: kept off the stack
-  for (int i = 0; i < FWD_MAX_LAYERS; ++i) {
-    const int l = i < n ? i : 0;
-    int rc = make_map_bshd(&p.map_q[i], q[l], s->B, s->S, s->Hq, s->dh, BQ);
-    if (rc == KVP_OK) rc = make_map_bshd(&p.map_k[i], k[l], s->B, s->S, s->Hkv, s->dh, BKV);
-    if (rc == KVP_OK) rc = make_map_bshd(&p.map_v[i], v[l], s->B, s->S, s->Hkv, s->dh, BKV);
+  for (int i = 0; i < n; ++i) {
+    int rc = make_map_bshd(&p.map_q[i], q[i], s->B, s->S, s->Hq, s->dh, BQ);
+    if (rc == KVP_OK) rc = make_map_bshd(&p.map_k[i], k[i], s->B, s->S, s->Hkv, s->dh, BKV);
+    if (rc == KVP_OK) rc = make_map_bshd(&p.map_v[i], v[i], s->B, s->S, s->Hkv, s->dh, BKV);
     if (rc != KVP_OK) return rc;
-    p.o[i] = reinterpret_cast<__nv_bfloat16*>(o[l]);
-    p.lse[i] = lse[l];
+    p.o[i] = o[i];
+    p.lse[i] = lse[i];
   }
+  for (int i = n; i < FWD_MAX_LAYERS; ++i) {   // unused entries repeat layer 0, so that no descriptor is left unset
+    p.map_q[i] = p.map_q[0];
+    p.map_k[i] = p.map_k[0];
+    p.map_v[i] = p.map_v[0];
+    p.o[i] = p.o[0];
+    p.lse[i] = p.lse[0];
+  }
+  p.o_f32 = o_f32;
   p.n_layers = n;
   p.B = s->B;
   p.S = s->S;

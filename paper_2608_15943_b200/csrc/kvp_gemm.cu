@@ -224,6 +224,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_cons
             for (int v = 0; v < 8; ++v) {
               if (n0 + c0 + v * 4 < N) {
                 uint4 val = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+                if (out_f32 == OUT_F32_OF_BF16)
+                  val = make_uint4(bf16_bits_f32(__uint_as_float(val.x)), bf16_bits_f32(__uint_as_float(val.y)),
+                                   bf16_bits_f32(__uint_as_float(val.z)), bf16_bits_f32(__uint_as_float(val.w)));
                 *reinterpret_cast<uint4*>(dst + v * 4) = val;
               }
             }
@@ -442,6 +445,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
             for (int v = 0; v < 8; ++v) {
               if (n0 + c0 + v * 4 < N) {
                 uint4 val = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+                if (out_f32 == OUT_F32_OF_BF16)
+                  val = make_uint4(bf16_bits_f32(__uint_as_float(val.x)), bf16_bits_f32(__uint_as_float(val.y)),
+                                   bf16_bits_f32(__uint_as_float(val.z)), bf16_bits_f32(__uint_as_float(val.w)));
                 *reinterpret_cast<uint4*>(dst + v * 4) = val;
               }
             }
@@ -641,9 +647,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
       }
       if (col < pr.N) {
         const size_t at = size_t(m0 + tk) * pr.ldc + col;
-        if (pr.out_f32)
+        if (pr.out_f32) {
+          if (pr.out_f32 == OUT_F32_OF_BF16)
+            acc = make_float4(__uint_as_float(bf16_bits_f32(acc.x)), __uint_as_float(bf16_bits_f32(acc.y)),
+                              __uint_as_float(bf16_bits_f32(acc.z)), __uint_as_float(bf16_bits_f32(acc.w)));
           *reinterpret_cast<float4*>(reinterpret_cast<float*>(pr.c) + at) = acc;
-        else
+        } else
           *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(pr.c) + at) =
               make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
       }
@@ -844,7 +853,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
           float* dst = reinterpret_cast<float*>(pr.c) + size_t(w.m0 + c0) * pr.ldc + col;
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            if (c0 + i < n_tok && col < pr.N) dst[size_t(i) * pr.ldc] = __uint_as_float(r[i]);
+            if (c0 + i < n_tok && col < pr.N)
+              dst[size_t(i) * pr.ldc] = __uint_as_float(pr.out_f32 == OUT_F32_OF_BF16 ? bf16_bits_f32(__uint_as_float(r[i])) : r[i]);
         } else {
           // two tokens at a time: even lanes end up with two columns of the first, odd lanes with two of the second
           const int odd = lane & 1;

@@ -20,6 +20,9 @@ int make_tensor_map(CUtensorMap* out, const void* base, int elem_bytes, int rank
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Types of C: bf16; the fp32 sums; the sums rounded to bf16 and stored as fp32 (the fp32 interface's outputs).
+enum { OUT_BF16 = 0, OUT_F32 = 1, OUT_F32_OF_BF16 = 2 };
+
 // One GEMM "segment": C += op(A) * op(B) over this segment's K extent.
 struct GemmSeg {
   const void* a;   // bf16
@@ -32,7 +35,7 @@ struct GemmSeg {
 // C[M,N] = sum over segments of A_s * B_s, bf16 inputs, fp32 accumulation in TMEM.
 //   a_mn == 0: A_s stored [M, K] row-major (K-major);  a_mn == 1: stored [K, M] row-major.
 //   b_mn == 0: B_s stored [N, K] row-major (K-major);  b_mn == 1: stored [K, N] row-major.
-//   out_f32: C is fp32 (else bf16); ldc in elements.
+//   out_f32: type of C (OUT_*); ldc in elements.
 // withhold_at / wait_limit_ns serve the self-test of the bounded waits (kvp_selftest_bounded_wait) only.
 // prefer_pair: run on CTA pairs (256 x 256 tiles) when M > 128 and the pair mode allows it.
 int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, void* c, int64_t ldc, int out_f32,
@@ -56,14 +59,14 @@ struct GemmProblem {
 // board's power limit the attention backward sharing the step with them slowed by more than the pairs gained.
 int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool prefer_pair);
 
-// Conversion of a list of tensors in as few launches as the parameter block allows.  widen: bf16 -> fp32, else
-// fp32 -> bf16 (round-to-nearest-even).  elems: multiples of 4.
+// fp32 -> bf16 (round-to-nearest-even) of a list of tensors in as few launches as the parameter block allows.  elems:
+// multiples of 4.
 struct CastItem {
-  const void* src;
-  void* dst;
+  const void* src;   // fp32
+  void* dst;         // bf16
   size_t elems;
 };
-int cast_tensors(const CastItem* items, int n, bool widen, cudaStream_t stream);
+int cast_tensors(const CastItem* items, int n, cudaStream_t stream);
 
 void gemm_set_pair_mode(int mode);   // 0: single-CTA tiles only, 1: pairs where the caller prefers them, 2: pairs everywhere
 int gemm_pair_mode();

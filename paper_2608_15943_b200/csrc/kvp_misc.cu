@@ -1,11 +1,11 @@
-// Conversions between the caller's fp32 tensors and the library's bf16 ones: fp32 -> bf16 rounding (the donor-group
-// gradient sums before they enter the projection GEMMs; fp32 inputs of the KVP_F32 interface) and bf16 -> fp32 widening
-// (its outputs).
+// fp32 -> bf16 rounding of whole tensors: the donor-group gradient sums before they enter the projection GEMMs, and the
+// inputs of the KVP_F32 interface (its outputs are widened by the kernels that produce them).
 //
-// One launch converts a whole list of tensors: a call of the fp32 interface has 3 to 8 of them per layer, each of a few
+// One launch converts a whole list of tensors: a call of the fp32 interface has 3 to 5 of them per layer, each of a few
 // hundred KB at the sizes that interface is for, where a launch costs more than the copy.  A four-layer training step of
-// 2 x 128 tokens had 64 such launches of 1.6 us each; it has 8 (device time of the step 124 -> 78 us).  Bound: HBM for
-// large tensors, launch latency for small.
+// 2 x 128 tokens had 64 conversion launches of 1.6 us each, outputs included; it has 4 (device time of the step 124 -> 78
+// us with a launch per list, 55 -> 52 with the outputs widened where they are produced).  Bound: HBM for large tensors,
+// launch latency for small.
 #include <algorithm>
 
 #include "kvp_host.h"
@@ -27,13 +27,6 @@ struct CastParams {
   uint32_t chunks;
 };
 
-__device__ __forceinline__ uint2 convert(const float4& v) { return make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w)); }
-__device__ __forceinline__ float4 convert(const uint2& v) {
-  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
-                     __uint_as_float(v.y & 0xffff0000u));
-}
-
-template <typename Src, typename Dst>
 __global__ void __launch_bounds__(CAST_THREADS) cast_kernel(const __grid_constant__ CastParams p) {
   grid_dep_wait();
   int t = 0;
@@ -41,22 +34,22 @@ __global__ void __launch_bounds__(CAST_THREADS) cast_kernel(const __grid_constan
     if (c + gridDim.x >= p.chunks) grid_dep_launch();
     while (c >= p.chunk_end[t]) ++t;
     const size_t first = size_t(c - (t ? p.chunk_end[t - 1] : 0)) * CAST_CHUNK + threadIdx.x;
-    const Src* src = reinterpret_cast<const Src*>(p.src[t]);
-    Dst* dst = reinterpret_cast<Dst*>(p.dst[t]);
+    const float4* src = reinterpret_cast<const float4*>(p.src[t]);
+    uint2* dst = reinterpret_cast<uint2*>(p.dst[t]);
     const size_t n4 = p.n4[t];
-    Src v[CAST_UNROLL];
+    float4 v[CAST_UNROLL];
 #pragma unroll
     for (int u = 0; u < CAST_UNROLL; ++u)
       if (first + u * CAST_THREADS < n4) v[u] = src[first + u * CAST_THREADS];
 #pragma unroll
     for (int u = 0; u < CAST_UNROLL; ++u)
-      if (first + u * CAST_THREADS < n4) dst[first + u * CAST_THREADS] = convert(v[u]);
+      if (first + u * CAST_THREADS < n4) dst[first + u * CAST_THREADS] = make_uint2(pack_bf16(v[u].x, v[u].y), pack_bf16(v[u].z, v[u].w));
   }
 }
 
 }  // namespace
 
-int cast_tensors(const CastItem* items, int n, bool widen, cudaStream_t stream) {
+int cast_tensors(const CastItem* items, int n, cudaStream_t stream) {
   for (int i = 0; i < n; ++i)
     if ((items[i].elems & 3) != 0) return KVP_ERR_UNSUPPORTED;
   CastParams p;
@@ -79,7 +72,7 @@ int cast_tensors(const CastItem* items, int n, bool widen, cudaStream_t stream) 
     begin += cnt;
     if (chunks == 0) continue;
     const int blocks = int(std::min<uint64_t>(uint64_t(sm_count()) * 8, chunks));
-    const cudaError_t e = launch_kernel(widen ? cast_kernel<uint2, float4> : cast_kernel<float4, uint2>, blocks, CAST_THREADS, 0, stream, 1, p);
+    const cudaError_t e = launch_kernel(cast_kernel, blocks, CAST_THREADS, 0, stream, 1, p);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;

@@ -446,6 +446,8 @@ __device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t chunk16)
   return row * 128u + ((chunk16 ^ (row & 7u)) << 4);
 }
 
+// an fp32 value rounded to bf16, as the bits of the fp32 number it then is
+__device__ __forceinline__ uint32_t bf16_bits_f32(float v) { return uint32_t(__bfloat16_as_ushort(__float2bfloat16_rn(v))) << 16; }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
