@@ -85,13 +85,13 @@ int kvp_selftest_bounded_wait_pair(void* scratch, size_t scratch_bytes, kvp_stre
 unsigned long long kvp_launch_count(void);
 int kvp_set_timing_events(int kernel, void** starts, void** stops, int n);
 int kvp_timing_events_used(int kernel);
-/* Measurement switch of the GEMM's tile shape.  1 (the default): the forward GEMMs (kvp_proj_fwd,
- * kvp_out_proj_fwd, kvp_gemm) run on CTA pairs (256 x 256 tiles, one per pair of SMs) when every problem of the
- * launch has more than 128 rows, or up to 4096 rows on whichever of the library's kernels an estimate of their times
- * prefers; the gradient GEMMs on single-CTA 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: CTA pairs everywhere.
- * (K-major problems of at most 128 rows have a kernel of their own in every mode.)  The tile kernels sum the same
- * products in the same order along K in every mode; up to 4096 rows K may be split over a cluster of CTAs, whose
- * partial sums are added in a fixed order.  Not thread-safe. */
+/* Measurement switch of the GEMM's tile shape.  1 (the default): forward GEMMs (K-major operands) run on CTA pairs
+ * (256 x 256 tiles, one per pair of SMs), or up to 4096 rows on whichever of the library's kernels an estimate of their
+ * times prefers; the gradient GEMMs on pairs that own 256 columns, large launches (more than 0.5 TFLOP) on single-CTA
+ * 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: 256 x 256 tiles on CTA pairs for every launch whose problems all
+ * have more than 128 rows.  (K-major problems of at most 128 rows have a kernel of their own in every mode.)  The tile
+ * kernels sum the same products in the same order along K in every mode; up to 4096 rows K may be split over a cluster of
+ * CTAs, whose partial sums are added in a fixed order.  Not thread-safe. */
 void kvp_set_gemm_pair_mode(int mode);
 
 /* ------------------------------------------------------------------------------------------

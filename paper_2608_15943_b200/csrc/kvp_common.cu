@@ -169,5 +169,5 @@ extern "C" int kvp_selftest_bounded_wait_pair(void* scratch, size_t scratch_byte
   // both producers' waits for that stage run out after 5 ms
   if (kvp::gemm_pair_mode() == 0) return KVP_ERR_UNSUPPORTED;
   return kvp::gemm_bf16(256, 256, &seg, 1, 0, 0, base + a_bytes + b_bytes, 256, 1, reinterpret_cast<cudaStream_t>(stream), 1,
-                        5000000ull, true);
+                        5000000ull);
 }

@@ -1,5 +1,5 @@
 // bf16 GEMM on tcgen05 tensor cores with TMEM accumulators, operands staged by TMA.
-// Used for the Q / K / V / output projections (Eq. 1 of the paper) and their chain rule.
+// Used for the Q / K / V / output projections (Eq. 1 of the paper) and their chain rule.  Four kernels; gemm_kernel:
 //
 // One persistent CTA per SM walks 128 x 256 output tiles.  Warp 0 issues TMA loads into a
 // 4-stage shared-memory ring, warp 1 issues tcgen05.mma into one of two 256-column TMEM
@@ -667,46 +667,57 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// A few hundred rows of A (a prompt, a small batch of them): CTA pairs with the operands swapped, C^T = B A^T.
+// Up to a few thousand rows of A (prompts, small batches), and the gradients: CTA pairs with the operands swapped,
+// C^T = B A^T.
 //
 // Each pair of CTAs owns 256 columns of C (rows of B: 128 a CTA, the M = 256 of the pair's MMA) and a tile of tokens (the
 // N, split between the CTAs' loads).  256 x 256 tiles of gemm_pair_kernel pad 347 tokens to 512; here the tokens are cut
-// into tiles of 128 to 256, whatever leaves the fewest pairs idle, and one tile of the remainder, a multiple of 32.  The
-// tiles are walked longest first, pairs taking turns in alternating direction, so the short tiles of the remainder fill
-// the pairs that have no second long one.  A lane of the epilogue holds a column, so a warp stores rows of 64
-// consecutive bytes, two at a time, where a lane of gemm_pair_kernel's holds a row.  Roles, ring and barriers are those
-// of gemm_pair_kernel; results are bit-identical to its (same products, same order along K).
+// into tiles of 128 to 256, whatever leaves the fewest pairs idle, and one tile of the remainder, a multiple of 32 (of
+// 128 where A is MN-major: its TMA boxes hold 64 rows and each CTA loads half of the tile).  The tiles are walked longest
+// first, pairs taking turns in alternating direction, so the short tiles of the remainder fill the pairs that have no
+// second long one.  A lane of the epilogue holds a column, so a warp stores rows of 64 consecutive bytes, two at a time
+// (128 in fp32), where a lane of gemm_pair_kernel's holds a row.  Roles, ring, segments and barriers are those of
+// gemm_pair_kernel; results are bit-identical to its (same products, same order along K).
 // Bound: the 120 GB/s that an SM draws from L2 (tiles of up to 192 tokens), then the tensor pipe.  Measured (us;
 // gemm_pair_kernel -> this, tokens x columns x K): 200 x 11008 x 4096 29.1 -> 26.5, 512 x 11008 x 4096 51 -> 43,
-// 776 x 11008 x 4096 76 -> 57, 1500 x 4096 x 11008 123 -> 101, 2328 x 4096 x 4096 69 -> 56.
+// 776 x 11008 x 4096 76 -> 57, 1500 x 4096 x 11008 123 -> 101, 2328 x 4096 x 4096 69 -> 56.  With a short K the stores
+// bound it, and four epilogue warps leave them waiting for one another: sixteen instead of four took fp32 results of
+// 2328 x 1024 x 1024, four problems, from 48 to 24 us and those of 776 tokens, six problems, from 26 to 16 (bf16: 13.8
+// -> 14.6; the same change slowed gemm_kernel and gemm_pair_kernel by 2 to 10 %).
 // ------------------------------------------------------------------------------------------------------------
 constexpr int TCOLS = 256;                        // columns of C per pair
 constexpr int TSTAGES = 6;
 constexpr int TSTAGE_BYTES = 32 * 1024;           // per CTA: 128 rows of B, up to 128 rows of A
+constexpr int TALL_EPI_WARPS = 16;                // four for every quarter of the TMEM lanes, taking 32 tokens each in turn
+constexpr int TALL_THREADS = (2 + TALL_EPI_WARPS) * 32;
 constexpr size_t TALL_SMEM = 1024 + size_t(TSTAGES) * TSTAGE_BYTES + 256;
 
 struct TallList {                                 // the tiles of one problem that have the same number of tokens
   int prob;
-  int nt;                                         // tokens per tile, a multiple of 32
+  int nt;                                         // tokens (rows of C) per tile, a multiple of 32; of 128 if A is MN-major
   int m_first, n_tok;                             // first token, tiles along the tokens
   int tile_end;                                   // one past the list's last tile in the launch's tile order
   uint32_t idesc;
+  short map_a[MAX_SEG];                           // per segment; the box holds half of a tile's tokens
 };
 struct TallProblem {
-  int M, N, kblocks, out_f32;
+  int M, N, nseg, kblocks[MAX_SEG], total_kb;
+  short map_b[MAX_SEG];
+  int a_mn, b_mn, out_f32;
   long long ldc;
   void* c;
 };
-template <int NP>
+template <int NP, int NSEG>                       // problems, and segments of all of them, that the parameter block holds
 struct TallParams {
-  CUtensorMap map_b[NP], map_a[2 * NP];           // map_a: one per list (the box holds half of a tile's tokens)
+  CUtensorMap map_b[NSEG], map_a[2 * NSEG];
   TallProblem prob[NP];
   TallList list[2 * NP];
   int total_tiles;
 };
 
-template <int NP>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gemm_tall_kernel(const __grid_constant__ TallParams<NP> p) {
+template <int NP, int NSEG>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
+    gemm_tall_kernel(const __grid_constant__ TallParams<NP, NSEG> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(TSTAGES) * TSTAGE_BYTES);
@@ -731,7 +742,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 8);
+      mbar_init(&acc_empty[a], 2 * TALL_EPI_WARPS);
     }
     mbar_fence_init();
   }
@@ -772,21 +783,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
     Tile w{};
     for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
       if (!tile_of(round, w)) continue;   // only the last round can be short
-      const int half = w.nt / 2, nkb = p.prob[w.prob].kblocks;
+      const TallProblem& pr = p.prob[w.prob];
+      const int half = w.nt / 2, a_mn = pr.a_mn, b_mn = pr.b_mn;
       const uint32_t bytes = 2u * uint32_t(PA_BYTES + half * (BK * 2));   // of both CTAs
-      const CUtensorMap* map_b = &p.map_b[w.prob];
-      const CUtensorMap* map_a = &p.map_a[w.li];
       const int n0 = w.n0 + int(rank) * 128, m0 = w.m0 + int(rank) * half;
-      for (int kb = 0; kb < nkb; ++kb) {
-        if (!mbar_wait(&empty[s], ph, err)) { ok = false; break; }
-        uint8_t* sb = smem + size_t(s) * TSTAGE_BYTES;
-        if (rank == 0) mbar_expect_tx_e(&full[s], bytes, leader);
-        const uint32_t bar = cluster_addr_of(&full[s], 0);
-        tma_load_2d_pair_e(sb, map_b, bar, kb * BK, n0, leader);
-        tma_load_2d_pair_e(sb + PA_BYTES, map_a, bar, kb * BK, m0, leader);
-        if (++s == TSTAGES) {
-          s = 0;
-          ph ^= 1;
+      for (int seg = 0; seg < pr.nseg && ok; ++seg) {
+        const CUtensorMap* map_b = &p.map_b[pr.map_b[seg]];
+        const CUtensorMap* map_a = &p.map_a[p.list[w.li].map_a[seg]];
+        const int nkb = pr.kblocks[seg];
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait(&empty[s], ph, err)) { ok = false; break; }
+          uint8_t* sb = smem + size_t(s) * TSTAGE_BYTES;
+          uint8_t* sa = sb + PA_BYTES;
+          if (rank == 0) mbar_expect_tx_e(&full[s], bytes, leader);
+          const uint32_t bar = cluster_addr_of(&full[s], 0);
+          if (b_mn == 0) {
+            tma_load_2d_pair_e(sb, map_b, bar, kb * BK, n0, leader);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) tma_load_2d_pair_e(sb + j * 8192, map_b, bar, n0 + 64 * j, kb * BK, leader);
+          }
+          if (a_mn == 0) {
+            tma_load_2d_pair_e(sa, map_a, bar, kb * BK, m0, leader);
+          } else {
+            for (int j = 0; j < half / 64; ++j) tma_load_2d_pair_e(sa + j * 8192, map_a, bar, m0 + 64 * j, kb * BK, leader);
+          }
+          if (++s == TSTAGES) {
+            s = 0;
+            ph ^= 1;
+          }
         }
       }
     }
@@ -802,7 +827,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
       for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
         if (!tile_of(round, w)) continue;
         const uint32_t idesc = p.list[w.li].idesc;
-        const int nkb = p.prob[w.prob].kblocks;
+        const TallProblem& pr = p.prob[w.prob];
+        const int nkb = pr.total_kb;
+        const uint32_t a_step = pr.a_mn ? 2048u : 32u, b_step = pr.b_mn ? 2048u : 32u;   // bytes per 16-deep K step
+        const uint32_t a_lbo = pr.a_mn ? 8192u : 0u, b_lbo = pr.b_mn ? 8192u : 0u;
         const int acc = tile_i & 1;
         if (!mbar_wait(&acc_empty[acc], ((tile_i >> 1) & 1) ^ 1, err)) { ok = false; break; }
         tc_fence_after_sync();
@@ -813,8 +841,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
           const uint32_t sb = smem_u32(smem + size_t(s) * TSTAGE_BYTES);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
-            umma_ss_pair(d_tmem, smem_desc_sw128(sb + k * 32, 0, 1024), smem_desc_sw128(sb + PA_BYTES + k * 32, 0, 1024), idesc,
-                         (kb | k) != 0, leader);
+            umma_ss_pair(d_tmem, smem_desc_sw128(sb + k * b_step, b_lbo, 1024), smem_desc_sw128(sb + PA_BYTES + k * a_step, a_lbo, 1024),
+                         idesc, (kb | k) != 0, leader);
           umma_commit_pair(cluster_addr_of(&empty[s], 0), leader);
           umma_commit_pair(cluster_addr_of(&empty[s], 1), leader);
           if (++s == TSTAGES) {
@@ -830,7 +858,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
       }
     }
   } else {
-    // ------------------------------ epilogue (warps 2..5 of both CTAs): lane = column of C ------------------------------
+    // ------------------------------ epilogue (warps 2.. of both CTAs): lane = column of C ------------------------------
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
     uint32_t tile_i = 0;
     Tile w{};
@@ -845,25 +873,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1) gem
       const int n_tok = min(w.nt, pr.M - w.m0);
       const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + acc * 256;
 #pragma unroll 1
-      for (int c0 = 0; c0 < n_tok; c0 += 32) {
+      for (int c0 = 32 * ((warp - 2) >> 2); c0 < n_tok; c0 += 8 * TALL_EPI_WARPS) {   // the quarter's warps take turns
         uint32_t r[32];
         tmem_ld_x32(taddr + c0, r);
         tmem_ld_wait();
+        const int left = col < pr.N ? n_tok - c0 : 0;
         if (pr.out_f32) {
           float* dst = reinterpret_cast<float*>(pr.c) + size_t(w.m0 + c0) * pr.ldc + col;
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (c0 + i < n_tok && col < pr.N)
-              dst[size_t(i) * pr.ldc] = __uint_as_float(pr.out_f32 == OUT_F32_OF_BF16 ? bf16_bits_f32(__uint_as_float(r[i])) : r[i]);
+          for (int i = 0; i < 32; ++i, dst += pr.ldc)
+            if (i < left) *dst = __uint_as_float(pr.out_f32 == OUT_F32_OF_BF16 ? bf16_bits_f32(__uint_as_float(r[i])) : r[i]);
         } else {
           // two tokens at a time: even lanes end up with two columns of the first, odd lanes with two of the second
           const int odd = lane & 1;
           __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(pr.c) + size_t(w.m0 + c0 + odd) * pr.ldc + (col - odd);
 #pragma unroll
-          for (int i = 0; i < 32; i += 2) {
+          for (int i = 0; i < 32; i += 2, dst += 2 * pr.ldc) {
             const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? r[i] : r[i + 1], 1);
             const float lo = __uint_as_float(odd ? got : r[i]), hi = __uint_as_float(odd ? r[i + 1] : got);
-            if (c0 + i + odd < n_tok && col < pr.N) *reinterpret_cast<uint32_t*>(dst + size_t(i) * pr.ldc) = pack_bf16(lo, hi);
+            if (i + odd < left) *reinterpret_cast<uint32_t*>(dst) = pack_bf16(lo, hi);
           }
         }
       }
@@ -910,33 +938,13 @@ int check_problem(const GemmProblem& g) {
   return KVP_OK;
 }
 
-// Tensor maps of one operand pair; the box depends on the operand mode and on the rows of B one CTA loads.
-int encode_segment(const GemmProblem& g, const GemmSeg& e, CUtensorMap* map_a, CUtensorMap* map_b, uint32_t b_rows) {
-  int rc;
-  if (g.a_mn == 0) {
-    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.M)};
-    uint64_t strides[1] = {uint64_t(e.lda) * 2};
-    uint32_t box[2] = {BK, BM};
-    rc = make_tensor_map(map_a, e.a, 2, 2, dims, strides, box, true);
-  } else {
-    uint64_t dims[2] = {uint64_t(g.M), uint64_t(e.K)};
-    uint64_t strides[1] = {uint64_t(e.lda) * 2};
-    uint32_t box[2] = {64, BK};
-    rc = make_tensor_map(map_a, e.a, 2, 2, dims, strides, box, true);
-  }
-  if (rc != KVP_OK) return rc;
-  if (g.b_mn == 0) {
-    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.N)};
-    uint64_t strides[1] = {uint64_t(e.ldb) * 2};
-    uint32_t box[2] = {BK, b_rows};
-    rc = make_tensor_map(map_b, e.b, 2, 2, dims, strides, box, true);
-  } else {
-    uint64_t dims[2] = {uint64_t(g.N), uint64_t(e.K)};
-    uint64_t strides[1] = {uint64_t(e.ldb) * 2};
-    uint32_t box[2] = {64, BK};
-    rc = make_tensor_map(map_b, e.b, 2, 2, dims, strides, box, true);
-  }
-  return rc;
+// Tensor map of one operand with `rows` rows (of A) or columns (of B): K-major boxes hold box_rows of them by BK, MN-major
+// ones 64 by BK.
+int encode_operand(CUtensorMap* map, const void* base, int64_t ld, int rows, int K, int mn, uint32_t box_rows) {
+  uint64_t dims[2] = {uint64_t(mn ? rows : K), uint64_t(mn ? K : rows)};
+  uint64_t strides[1] = {uint64_t(ld) * 2};
+  uint32_t box[2] = {mn ? 64u : uint32_t(BK), mn ? uint32_t(BK) : box_rows};
+  return make_tensor_map(map, base, 2, 2, dims, strides, box, true);
 }
 
 int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withhold_at, unsigned long long wait_limit_ns,
@@ -967,7 +975,9 @@ int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withh
       q.total_kb += q.kblocks[s];
       q.map_a[s] = short(n_maps);
       q.map_b[s] = short(n_maps + 1);
-      const int rc = encode_segment(g, g.segs[s], &p.maps[n_maps], &p.maps[n_maps + 1], pair ? PHALF : BN);
+      const GemmSeg& e = g.segs[s];
+      int rc = encode_operand(&p.maps[n_maps], e.a, e.lda, g.M, e.K, g.a_mn, BM);
+      if (rc == KVP_OK) rc = encode_operand(&p.maps[n_maps + 1], e.b, e.ldb, g.N, e.K, g.b_mn, pair ? PHALF : BN);
       if (rc != KVP_OK) return rc;
       n_maps += 2;
     }
@@ -999,9 +1009,9 @@ constexpr int SPLIT_MAX_ROWS = 128;
 constexpr int SPLIT_MAX_PROB = 32;
 
 // Both operands K-major, one segment: the shape of every forward projection.
-bool split_applies(const GemmProblem* probs, int n) {
+bool k_major(const GemmProblem* probs, int n) {
   for (int i = 0; i < n; ++i)
-    if (probs[i].M > SPLIT_MAX_ROWS || probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
+    if (probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
   return n > 0;
 }
 
@@ -1041,14 +1051,8 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
     q.ldc = g.ldc;
     q.c = g.c;
     const GemmSeg& e = g.segs[0];
-    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.M)}, strides[1] = {uint64_t(e.lda) * 2};
-    uint32_t box[2] = {BK, uint32_t(cfg.nt)};
-    int rc = make_tensor_map(&p.map_a[i], e.a, 2, 2, dims, strides, box, true);
-    if (rc != KVP_OK) return rc;
-    dims[1] = uint64_t(g.N);
-    strides[0] = uint64_t(e.ldb) * 2;
-    box[1] = SROWS;
-    rc = make_tensor_map(&p.map_b[i], e.b, 2, 2, dims, strides, box, true);
+    int rc = encode_operand(&p.map_a[i], e.a, e.lda, g.M, e.K, 0, uint32_t(cfg.nt));
+    if (rc == KVP_OK) rc = encode_operand(&p.map_b[i], e.b, e.ldb, g.N, e.K, 0, SROWS);
     if (rc != KVP_OK) return rc;
   }
   p.nt = cfg.nt;
@@ -1068,54 +1072,67 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
-template <int NP>
+template <int NP, int NSEG>
 int launch_tall(const GemmProblem* probs, int n, int nt, cudaStream_t stream) {
-  TallParams<NP> p;
-  int lists = 0, tiles = 0;
+  TallParams<NP, NSEG> p;
+  int lists = 0, tiles = 0, maps_a = 0, maps_b = 0;
   for (int i = 0; i < n; ++i) {
     const GemmProblem& g = probs[i];
-    const GemmSeg& e = g.segs[0];
-    p.prob[i] = TallProblem{g.M, g.N, (e.K + BK - 1) / BK, g.out_f32, g.ldc, g.c};
-    uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.N)}, strides[1] = {uint64_t(e.ldb) * 2};
-    uint32_t box[2] = {BK, 128};
-    const int rc = make_tensor_map(&p.map_b[i], e.b, 2, 2, dims, strides, box, true);
-    if (rc != KVP_OK) return rc;
+    TallProblem& q = p.prob[i];
+    q.M = g.M;
+    q.N = g.N;
+    q.nseg = g.nseg;
+    q.total_kb = 0;
+    q.a_mn = g.a_mn;
+    q.b_mn = g.b_mn;
+    q.out_f32 = g.out_f32;
+    q.ldc = g.ldc;
+    q.c = g.c;
+    for (int e = 0; e < g.nseg; ++e) {
+      const GemmSeg& sg = g.segs[e];
+      q.kblocks[e] = (sg.K + BK - 1) / BK;
+      q.total_kb += q.kblocks[e];
+      q.map_b[e] = short(maps_b);
+      const int rc = encode_operand(&p.map_b[maps_b++], sg.b, sg.ldb, g.N, sg.K, g.b_mn, 128);
+      if (rc != KVP_OK) return rc;
+    }
   }
   // the whole tiles of all problems first, then the remainders
   for (int part = 0; part < 2; ++part)
     for (int i = 0; i < n; ++i) {
       const GemmProblem& g = probs[i];
-      const GemmSeg& e = g.segs[0];
-      const int whole = g.M / nt, rest = g.M - whole * nt;
-      TallList l;
+      const int whole = g.M / nt, rest = g.M - whole * nt, unit = g.a_mn ? 128 : 32;
+      TallList l{};
       l.prob = i;
-      l.nt = part == 0 ? nt : (rest + 31) / 32 * 32;
+      l.nt = part == 0 ? nt : (rest + unit - 1) / unit * unit;
       l.m_first = part == 0 ? 0 : whole * nt;
       l.n_tok = part == 0 ? whole : (rest > 0 ? 1 : 0);
       if (l.n_tok == 0) continue;
       tiles += l.n_tok * ((g.N + TCOLS - 1) / TCOLS);
       l.tile_end = tiles;
-      l.idesc = umma_idesc_bf16(256, l.nt, 0, 0);
-      uint64_t dims[2] = {uint64_t(e.K), uint64_t(g.M)}, strides[1] = {uint64_t(e.lda) * 2};
-      uint32_t box[2] = {BK, uint32_t(l.nt / 2)};
-      const int rc = make_tensor_map(&p.map_a[lists], e.a, 2, 2, dims, strides, box, true);
-      if (rc != KVP_OK) return rc;
+      l.idesc = umma_idesc_bf16(256, l.nt, g.b_mn, g.a_mn);
+      for (int e = 0; e < g.nseg; ++e) {
+        l.map_a[e] = short(maps_a);
+        const int rc = encode_operand(&p.map_a[maps_a++], g.segs[e].a, g.segs[e].lda, g.M, g.segs[e].K, g.a_mn, uint32_t(l.nt / 2));
+        if (rc != KVP_OK) return rc;
+      }
       p.list[lists++] = l;
     }
   p.total_tiles = tiles;
-  if (allow_smem<gemm_tall_kernel<NP>>(int(TALL_SMEM)) != cudaSuccess) return KVP_ERR_CUDA;
+  if (allow_smem<gemm_tall_kernel<NP, NSEG>>(int(TALL_SMEM)) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
-  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP>, 2 * std::min(tiles, sm_count() / 2), GEMM_THREADS, TALL_SMEM, stream, 1, p);
+  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * std::min(tiles, sm_count() / 2), TALL_THREADS, TALL_SMEM, stream, 1, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
-// 0: single-CTA tiles only; 1: CTA pairs where the caller prefers them (forward GEMMs); 2: CTA pairs everywhere.
-// Pairs are never used for a group with a problem of at most 128 rows (half of every pair tile would be padding).
+// 0: single-CTA tiles only; 1: whichever kernel suits the sizes; 2: CTA pairs (gemm_pair_kernel) everywhere.
+// In modes 1 and 2 pairs are never used for a group with a problem of at most 128 rows (half of every pair tile would be
+// padding).
 int g_pair_mode = 1;
 
-bool use_pair(const GemmProblem* probs, int n, bool prefer_pair) {
-  if (g_pair_mode == 0 || (g_pair_mode == 1 && !prefer_pair)) return false;
+bool use_pair(const GemmProblem* probs, int n) {
+  if (g_pair_mode == 0) return false;
   for (int i = 0; i < n; ++i)
     if (probs[i].M <= BM) return false;
   return true;
@@ -1190,18 +1207,39 @@ Choice choose_forward(const GemmProblem* probs, int n) {
   return best;
 }
 
-bool k_major(const GemmProblem* probs, int n) {
-  for (int i = 0; i < n; ++i)
-    if (probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
-  return n > 0;
-}
-
 template <typename F1, typename F4, typename F32>
 int by_count(int n, F1 one, F4 four, F32 many) { return n == 1 ? one() : n <= 4 ? four() : many(); }
 
-// A forward GEMM (pair mode 1, K-major operands, one segment): -1 when the tile kernels take it
+// The gradient GEMMs of a launch (pair mode 1) run on gemm_tall_kernel, in tiles of 256 rows; of 128 where those would
+// leave half of the pairs idle.  Measured (us, all weight and input gradients of a backward pass: gemm_kernel / tiles of
+// 128 / 256): 256 tokens x 256, four layers 15.6 / 6.9 / 9.1; 400 x 4096, two layers 33.6 / 29.2 / 24.0; 1984 x 1024, six
+// layers 72.7 / 74.5 / 60.2; 1664 x 4096, five layers 141 / 150 / 121; 4096 x 4096, one layer 300 / 352 / 286.
+// Launches of more than GRADIENT_MAX_FLOP (about 0.3 ms) stay on gemm_kernel, although by themselves they too are a little
+// faster on pairs (4096 x 4096, four layers, 0.8 TFLOP: 1140 / - / 1030): they belong to steps of many milliseconds, which
+// the board's power limit bounds, and there the rest of the step slows by more than the pairs gain (training step of eight
+// layers, 2 x 8192 tokens: 46.2 -> 47.8 ms; of four layers with output projections, 8 x 4096: 39.9 -> 41.4 ms).
+constexpr double GRADIENT_MAX_FLOP = 5e11;
+int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
+  int tiles = 0, segs = 0;
+  double flop = 0;
+  for (int i = 0; i < n; ++i) {
+    const GemmProblem& g = probs[i];
+    tiles += ((g.M + 255) / 256) * ((g.N + TCOLS - 1) / TCOLS);
+    segs += g.nseg;
+    for (int e = 0; e < g.nseg; ++e) flop += 2.0 * g.M * g.N * g.segs[e].K;
+  }
+  if (flop > GRADIENT_MAX_FLOP) return launch_group(probs, n, stream, 0, 0, false);
+  const int nt = 4 * tiles <= sm_count() ? 128 : 256;
+  if (segs == 1) return launch_tall<1, 1>(probs, n, nt, stream);
+  if (segs <= 4) return launch_tall<4, 4>(probs, n, nt, stream);
+  return launch_tall<MAX_PROB, MAX_MAPS / 2>(probs, n, nt, stream);
+}
+
+// A forward GEMM (K-major operands, one segment): -1 when the tile kernels take it
 int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
-  if (split_applies(probs, n)) {
+  int rows = 0;
+  for (int i = 0; i < n; ++i) rows = std::max(rows, probs[i].M);
+  if (rows <= SPLIT_MAX_ROWS) {
     for (int begin = 0; begin < n; begin += SPLIT_MAX_PROB) {
       const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
       const GemmProblem* g = probs + begin;
@@ -1212,17 +1250,15 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
     }
     return KVP_OK;
   }
-  if (g_pair_mode != 1 || !k_major(probs, n)) return -1;
-  for (int i = 0; i < n; ++i)
-    if (probs[i].M > CHOICE_MAX_ROWS) return -1;
+  if (g_pair_mode != 1 || rows > CHOICE_MAX_ROWS) return -1;
   for (int begin = 0; begin < n; begin += MAX_PROB) {
     const int cnt = std::min(MAX_PROB, n - begin);
     const GemmProblem* g = probs + begin;
     const Choice c = choose_forward(g, cnt);
     int rc;
     if (c.kind == Choice::kTall) {
-      rc = by_count(cnt, [&] { return launch_tall<1>(g, cnt, c.nt, stream); }, [&] { return launch_tall<4>(g, cnt, c.nt, stream); },
-                    [&] { return launch_tall<MAX_PROB>(g, cnt, c.nt, stream); });
+      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, stream); },
+                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
       rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
@@ -1237,13 +1273,14 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
 
 }  // namespace
 
-int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool prefer_pair) {
+int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream) {
   if (n < 0 || (n > 0 && probs == nullptr)) return KVP_ERR_INVALID_ARG;
   for (int i = 0; i < n; ++i) {
     const int rc = check_problem(probs[i]);
     if (rc != KVP_OK) return rc;
   }
-  if (prefer_pair || split_applies(probs, n)) {
+  const bool forward = k_major(probs, n);
+  if (forward) {
     const int rc = gemm_forward(probs, n, stream);
     if (rc >= 0) return rc;
   }
@@ -1252,7 +1289,9 @@ int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool pref
   while (begin < n) {
     int end = begin, maps = 0;
     while (end < n && end - begin < MAX_PROB && maps + 2 * probs[end].nseg <= MAX_MAPS) maps += 2 * probs[end++].nseg;
-    const int rc = launch_group(probs + begin, end - begin, stream, 0, 0, use_pair(probs + begin, end - begin, prefer_pair));
+    const int rc = !forward && g_pair_mode == 1
+                       ? gemm_gradient(probs + begin, end - begin, stream)
+                       : launch_group(probs + begin, end - begin, stream, 0, 0, use_pair(probs + begin, end - begin));
     if (rc != KVP_OK) return rc;
     begin = end;
   }
@@ -1260,7 +1299,7 @@ int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool pref
 }
 
 int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, void* c, int64_t ldc, int out_f32,
-              cudaStream_t stream, int withhold_at, unsigned long long wait_limit_ns, bool prefer_pair) {
+              cudaStream_t stream, int withhold_at, unsigned long long wait_limit_ns) {
   if (nseg < 1 || nseg > MAX_SEG || segs == nullptr) return KVP_ERR_INVALID_ARG;
   GemmProblem g{};
   g.M = M;
@@ -1272,13 +1311,9 @@ int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, v
   g.c = c;
   g.ldc = ldc;
   g.out_f32 = out_f32;
+  if (withhold_at == 0) return gemm_grouped(&g, 1, stream);
   const int rc = check_problem(g);
-  if (rc != KVP_OK) return rc;
-  if (withhold_at == 0 && (prefer_pair || split_applies(&g, 1))) {
-    const int forward = gemm_forward(&g, 1, stream);
-    if (forward >= 0) return forward;
-  }
-  return launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1, prefer_pair));
+  return rc == KVP_OK ? launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1)) : rc;
 }
 
 }  // namespace kvp

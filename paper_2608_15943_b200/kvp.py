@@ -377,8 +377,8 @@ lib.kvp_set_gemm_pair_mode.argtypes = [C.c_int]
 
 
 def set_gemm_pair_mode(mode: int) -> None:
-    """kvp_set_gemm_pair_mode: 1 = CTA-pair tiles for the forward GEMMs (default), 0 = single-CTA tiles everywhere,
-    2 = CTA pairs everywhere."""
+    """kvp_set_gemm_pair_mode: 1 = the kernel that suits the sizes (default), 0 = single-CTA tiles everywhere,
+    2 = 256 x 256 tiles on CTA pairs everywhere."""
     lib.kvp_set_gemm_pair_mode(int(mode))
 
 

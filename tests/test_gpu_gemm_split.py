@@ -1,5 +1,5 @@
 """GEMMs with few rows of A (decode-step projections, prompts): operands swapped, K split over a cluster of CTAs, or tiles
-of tokens on CTA pairs."""
+of tokens on CTA pairs; and the weight and input gradients, which take those pairs too."""
 import pytest
 import torch
 
@@ -58,3 +58,40 @@ def test_few_rows_grouped_projections():
             ref = x[l].double() @ w[n][l].double().T
             got = out[n][l].view(B, -1).double()
             assert ((got - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4).all(), (n, l)   # bf16 storage; 256 terms of size 0.02
+
+
+@pytest.mark.parametrize("L,own,S,D,Hq,Hkv", [
+    (1, 1, 8, 64, 1, 1),          # the fewest tokens: less than one k-block along them, eight rows of dX
+    (4, 1, 136, 320, 2, 1),       # tiles of 128 rows, remainders rounded up to 32 (dX) and to 128 (MN-major A)
+    (5, 2, 392, 1088, 6, 3),      # tiles of 256 rows, one and three K segments
+    (20, 8, 104, 576, 4, 1),       # more problems than one launch holds
+    (1, 1, 7048, 4096, 64, 16),   # above the line to single-CTA tiles
+])
+def test_gradient_gemms(L, own, S, D, Hq, Hkv):
+    from paper_2608_15943_b200 import kvp
+    dh, T = 64, S
+    donor = [min(l, own - 1) for l in range(L)]
+    sh = kvp.Shape(L, 1, S, D, Hq, Hkv, dh)
+    x = [synth.normal((T, D), 33, synth.tid(0, l), 1.0, "cuda") for l in range(L)]
+    w = {n: [synth.normal((h * dh, D), 33, synth.tid(i, l), 0.5, "cuda") for l in range(L)]
+         for i, (n, h) in enumerate((("q", Hq), ("k", Hkv), ("v", Hkv)), 1)}
+    dq = [synth.normal((T, Hq * dh), 33, synth.tid(4, l), 1.0, "cuda") for l in range(L)]
+    dkv = [[synth.normal((T, Hkv * dh), 33, synth.tid(i, l), 1.0, "cuda").float() if l < own else None for l in range(L)] for i in (5, 6)]
+    ws = torch.empty(kvp.workspace_bytes(kvp.OP_PROJ_BWD, sh, donor), dtype=torch.uint8, device="cuda")
+    gd = Guarded()
+    dw = {n: [gd.empty((h * dh, D), torch.float32, float("nan")) if n == "q" or l < own else None for l in range(L)]
+          for n, h in (("q", Hq), ("k", Hkv), ("v", Hkv))}
+    dx = [gd.empty((T, D), torch.bfloat16, float("nan")) for _ in range(L)]
+    kvp.proj_bwd(sh, donor, x, w["q"], w["k"], w["v"], dq, dkv[0], dkv[1], dw["q"], dw["k"], dw["v"], dx, ws)
+    gd.check()
+    assert kvp.device_status() == kvp.OK
+    for l in range(L):
+        parts = [("q", dq[l])] + ([("k", dkv[0][l]), ("v", dkv[1][l])] if l < own else [])
+        # as test_few_rows: K 2^-24 sum|a b| for the fp32 sums, half an ulp of bf16 for dX
+        for n, d in parts:
+            bound = T * 2.0 ** -24 * (d.double().abs().T @ x[l].double().abs()) + 1e-30
+            assert ((dw[n][l].double() - d.double().T @ x[l].double()).abs() <= bound).all(), (n, l)
+        ref = sum(d.double() @ w[n][l].double() for n, d in parts)
+        K = sum(d.shape[1] for _, d in parts)
+        bound = K * 2.0 ** -24 * sum(d.double().abs() @ w[n][l].double().abs() for n, d in parts)
+        assert ((dx[l].double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all(), l
