@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       uint32_t it = 0;    // items so far
       uint32_t jg = 0;    // key tiles of earlier items (ring position of this item's tile 0)
       uint32_t g0 = 0;    // sub-blocks of earlier items of this query tile (always even)
+      uint32_t n_o = 0;   // earlier items in which this query tile existed
       bool ok = true;
       for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
         const int t = fwd_item_index(round);
@@ -270,8 +271,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
           if (c < n_cx) issue_s(c);
         umma_commit(&k_empty[k_stage(0)], leader);
         if (n_cx <= 2) umma_commit(q_empty, leader);  // no further score MMAs of this item from this warp
-        // O_x is overwritten by the first P V product: the softmax warps must have read the previous item's out
-        if (it > 0 && !mbar_wait(&o_free[x], (it - 1) & 1, err)) { ok = false; break; }
+        // O_x is overwritten by the first P V product: the softmax warps must have read the last one out.  Only items
+        // that have this tile count on o_free: softmax warps that also arrived for the others could run several items
+        // ahead of this warp, past the phase that it waits for.
+        if (n_cx > 0 && n_o > 0 && !mbar_wait(&o_free[x], (n_o - 1) & 1, err)) { ok = false; break; }
         // Every round releases its K / V stages from this warp too when this tile has run out of sub-blocks (the
         // other tile may be one key tile longer): an arrival with nothing outstanding completes at once.
         for (int c = 0; c < n_cmax && ok; ++c) {
@@ -299,6 +302,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
         }
         jg += w.n_max;
         g0 += n_cx;
+        n_o += n_cx > 0 ? 1 : 0;
         ++it;
       }
     }
@@ -439,8 +443,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
           }
         }
         if (valid) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
-      } else if (ok) {
-        mbar_arrive(&o_free[x]);  // this query tile does not exist in this item: nothing to read out
       }
       g0 += my_c;
       n_done += my_n > 0 ? 1 : 0;
