@@ -18,6 +18,12 @@
 //               == row, so the row maximum and sum need no cross-thread traffic), packed fp32x2
 //               arithmetic, O rescaled in TMEM only when the running maximum moved by more than 2^8 (and
 //               then only after the P V product still in flight has completed)
+//   warps 12-15 epilogue of both tiles: they wait for the item's last product, normalise and store O while the
+//               softmax warps are at the next item's scores already.  (us, softmax warps storing O themselves -> this:
+//               4 x 512 tokens, 16 heads of 128, three layers 29.0 -> 26.9; 4 x 4096, 32 heads of 128 491 -> 482;
+//               full attention 4 x 1000, 16 heads of 64, two layers 67.9 -> 65.4; causal, heads of 64: no change)
+// What bounds it: the exponentials (special-function pipe 69 % busy at heads of 64, 63 % at 128, where the tensor pipe
+// is 62 % busy) together with their waits, and at 8192 tokens x 32 heads the board's power.
 // While one tile's exponentials run, the tensor pipe works on the other tile and on the next scores of this one.
 #include <math.h>
 
@@ -29,7 +35,7 @@ namespace {
 
 constexpr int BQ = 128, BKV = 128;
 constexpr int BC = 64;            // keys per sub-block (one score buffer)
-constexpr int FWD_THREADS = 384;
+constexpr int FWD_THREADS = 512;
 constexpr int FWD_KSTAGES = 3;
 constexpr int FWD_VSTAGES = 2;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
@@ -45,7 +51,8 @@ struct FwdSmem {
   static constexpr int OFF_K = OFF_Q + 2 * Q_BYTES;
   static constexpr int OFF_V = OFF_K + FWD_KSTAGES * KV_BYTES;
   static constexpr int OFF_BAR = OFF_V + FWD_VSTAGES * KV_BYTES;
-  static constexpr int TOTAL = OFF_BAR + 256 + 1024;  // + alignment slack
+  static constexpr int OFF_INV = OFF_BAR + 256; // [2][128] fp32: 1 / row sum of each query row
+  static constexpr int TOTAL = OFF_INV + 2 * BQ * 4 + 1024;  // + alignment slack
 };
 
 constexpr int FWD_MAX_LAYERS = 8;   // layers per launch
@@ -119,8 +126,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
   uint64_t* p_ready = s_full + 4;               // [2][2] per query tile and score buffer (128 arrivals)
   uint64_t* pv_done = p_ready + 4;              // [2] per query tile: one completion per sub-block's P V product
   uint64_t* o_done = pv_done + 2;               // [2] per query tile: the item's last P V product has completed
-  uint64_t* o_free = o_done + 2;                // [2] per query tile: the softmax warps have read O out (128 arrivals)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 2);
+  uint64_t* o_free = o_done + 2;                // [2] per query tile: the epilogue warps have read O out (128 arrivals)
+  uint64_t* l_ready = o_free + 2;               // [2] per query tile: the softmax warps have left 1 / row sum (128 arrivals)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(l_ready + 2);
+  float* inv_sum = reinterpret_cast<float*>(smem + L::OFF_INV);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -149,6 +158,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       mbar_init(&pv_done[i], 1);
       mbar_init(&o_done[i], 1);
       mbar_init(&o_free[i], 128);
+      mbar_init(&l_ready[i], 128);
     }
     mbar_fence_init();
   }
@@ -306,8 +316,60 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
         ++it;
       }
     }
+  } else if (warp >= 12) {
+    // ------------------------------ epilogue: O / row sum of both tiles ------------------------------
+    const int quarter = warp & 3;
+    const int r = quarter * 32 + lane;
+    uint32_t n_done[2] = {0, 0};
+    bool ok = true;
+    for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
+      const int t = fwd_item_index(round);
+      if (t >= n_items) continue;
+      const FwdItem w = fwd_item(p, t, n_pairs);
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (w.n_kv[x] == 0 || !ok) continue;
+        ok = mbar_wait(&l_ready[x], n_done[x] & 1, err) && mbar_wait(&o_done[x], n_done[x] & 1, err);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        ++n_done[x];
+        tc_fence_after_sync();
+        const float inv_l = inv_sum[x * BQ + r];
+        const int q_row = w.q0 + x * BQ + r;
+        const size_t o_at = ((size_t(w.b) * p.S + q_row) * p.Hq + w.hq) * DH;
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+          uint32_t tmp[64];
+          tmem_ld_x32(tmem_base + 256 + x * 128 + (uint32_t(quarter * 32) << 16) + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&tmp[0]));
+          tmem_ld_x32(tmem_base + 256 + x * 128 + (uint32_t(quarter * 32) << 16) + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&tmp[32]));
+          tmem_ld_wait();
+          if (h == HALVES - 1) {   // the next item's first P V product may overwrite O_x, its softmax warps inv_sum
+            tc_fence_before_sync();
+            mbar_arrive(&o_free[x]);
+          }
+          if (q_row < p.S && p.o_f32) {
+            float* dst = reinterpret_cast<float*>(p.o[w.layer]) + o_at + h * 64;
+#pragma unroll
+            for (int i = 0; i < 64; i += 4)
+              *reinterpret_cast<uint4*>(dst + i) =
+                  make_uint4(bf16_bits_f32(__uint_as_float(tmp[i]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[i + 1]) * inv_l),
+                             bf16_bits_f32(__uint_as_float(tmp[i + 2]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[i + 3]) * inv_l));
+          } else if (q_row < p.S) {
+            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.o[w.layer]) + o_at + h * 64;
+#pragma unroll
+            for (int i = 0; i < 64; i += 8)
+              *reinterpret_cast<uint4*>(dst + i) = make_uint4(
+                  pack_bf16(__uint_as_float(tmp[i]) * inv_l, __uint_as_float(tmp[i + 1]) * inv_l),
+                  pack_bf16(__uint_as_float(tmp[i + 2]) * inv_l, __uint_as_float(tmp[i + 3]) * inv_l),
+                  pack_bf16(__uint_as_float(tmp[i + 4]) * inv_l, __uint_as_float(tmp[i + 5]) * inv_l),
+                  pack_bf16(__uint_as_float(tmp[i + 6]) * inv_l, __uint_as_float(tmp[i + 7]) * inv_l));
+          }
+          __syncwarp();
+        }
+      }
+    }
   } else if (warp >= 4) {
-    // ------------------------------ softmax + epilogue ------------------------------
+    // ------------------------------ softmax of query tile x ------------------------------
     const int x = (warp - 4) >> 2;      // query tile of this warpgroup
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;  // row inside the query tile == TMEM lane
@@ -404,45 +466,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       }
       ok = __all_sync(0xffffffffu, ok);
       if (ok && my_n > 0) {
-        bool wt = mbar_wait(&o_done[x], n_done & 1, err);
-        ok = __all_sync(0xffffffffu, wt);
-      }
-      if (ok && my_n > 0) {
-        tc_fence_after_sync();
         const float l_sum = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
-        const float inv_l = 1.f / l_sum;
-        const bool valid = q_row < p.S;
-        const size_t o_at = ((size_t(w.b) * p.S + (valid ? q_row : 0)) * p.Hq + w.hq) * DH;
-        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.o[w.layer]) + o_at;
-#pragma unroll
-        for (int g = 0; g < DH / 32; ++g) {
-          uint32_t tmp[32];
-          tmem_ld_x32(tm_o + g * 32, tmp);
-          tmem_ld_wait();
-          if (g == DH / 32 - 1) {  // O_x has been read out: the next item's first P V product may overwrite it
-            tc_fence_before_sync();
-            mbar_arrive(&o_free[x]);
-          }
-          if (valid && p.o_f32) {
-            float* dst32 = reinterpret_cast<float*>(p.o[w.layer]) + o_at;
-#pragma unroll
-            for (int v4 = 0; v4 < 8; ++v4)
-              *reinterpret_cast<uint4*>(dst32 + g * 32 + v4 * 4) =
-                  make_uint4(bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 0]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 1]) * inv_l),
-                             bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 2]) * inv_l), bf16_bits_f32(__uint_as_float(tmp[4 * v4 + 3]) * inv_l));
-          } else if (valid) {
-#pragma unroll
-            for (int v4 = 0; v4 < 4; ++v4) {
-              uint4 v;
-              v.x = pack_bf16(__uint_as_float(tmp[8 * v4 + 0]) * inv_l, __uint_as_float(tmp[8 * v4 + 1]) * inv_l);
-              v.y = pack_bf16(__uint_as_float(tmp[8 * v4 + 2]) * inv_l, __uint_as_float(tmp[8 * v4 + 3]) * inv_l);
-              v.z = pack_bf16(__uint_as_float(tmp[8 * v4 + 4]) * inv_l, __uint_as_float(tmp[8 * v4 + 5]) * inv_l);
-              v.w = pack_bf16(__uint_as_float(tmp[8 * v4 + 6]) * inv_l, __uint_as_float(tmp[8 * v4 + 7]) * inv_l);
-              *reinterpret_cast<uint4*>(dst + g * 32 + v4 * 8) = v;
-            }
-          }
-        }
-        if (valid) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
+        if (q_row < p.S) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
+        ok = n_done == 0 || mbar_wait(&o_free[x], (n_done - 1) & 1, err);   // the epilogue warps have read the last item's
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        inv_sum[x * BQ + r] = 1.f / l_sum;
+        mbar_arrive(&l_ready[x]);
       }
       g0 += my_c;
       n_done += my_n > 0 ? 1 : 0;
