@@ -672,25 +672,28 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
 //
 // Each pair of CTAs owns 256 columns of C (rows of B: 128 a CTA, the M = 256 of the pair's MMA) and a tile of tokens (the
 // N, split between the CTAs' loads).  256 x 256 tiles of gemm_pair_kernel pad 347 tokens to 512; here the tokens are cut
-// into tiles of 128 to 256, whatever leaves the fewest pairs idle, and one tile of the remainder, a multiple of 32 (of
-// 128 where A is MN-major: its TMA boxes hold 64 rows and each CTA loads half of the tile).  The tiles are walked longest
-// first, pairs taking turns in alternating direction, so the short tiles of the remainder fill the pairs that have no
-// second long one.  A lane of the epilogue holds a column, so a warp stores rows of 64 consecutive bytes, two at a time
-// (128 in fp32), where a lane of gemm_pair_kernel's holds a row.  Roles, ring, segments and barriers are those of
-// gemm_pair_kernel; results are bit-identical to its (same products, same order along K).
-// Bound: the 120 GB/s that an SM draws from L2 (tiles of up to 192 tokens), then the tensor pipe.  Measured (us;
-// gemm_pair_kernel -> this, tokens x columns x K): 200 x 11008 x 4096 29.1 -> 26.5, 512 x 11008 x 4096 51 -> 43,
-// 776 x 11008 x 4096 76 -> 57, 1500 x 4096 x 11008 123 -> 101, 2328 x 4096 x 4096 69 -> 56.  With a short K the stores
-// bound it, and four epilogue warps leave them waiting for one another: sixteen instead of four took fp32 results of
-// 2328 x 1024 x 1024, four problems, from 48 to 24 us and those of 776 tokens, six problems, from 26 to 16 (bf16: 13.8
-// -> 14.6; the same change slowed gemm_kernel and gemm_pair_kernel by 2 to 10 %).
+// into tiles of up to 256, either all of the same size (a multiple of 16) or whole ones and one tile of the remainder (a
+// multiple of 16; of 128 where A is MN-major: its TMA boxes hold 64 rows and each CTA loads half of the tile).  Tiles of
+// one size are walked column by column, so that the columns' weights come from memory once; whole tiles go before all
+// remainders, pairs taking turns in alternating direction, so the short tiles fill the pairs that have no second long
+// one, but weights beyond L2 are read again.  A lane of the epilogue holds a column, so a warp stores rows of 64
+// consecutive bytes, two at a time (128 in fp32), where a lane of gemm_pair_kernel's holds a row.  Roles, segments and
+// barriers are those of gemm_pair_kernel, the ring has as many stages as tiles of the launch's size leave room for;
+// results are bit-identical to its (same products, same order along K).
+// Bound: the 120 GB/s that an SM draws from L2 (tiles of up to 192 tokens), then the tensor pipe.  Measured (us, weights
+// not in L2; gemm_pair_kernel -> whole tiles and remainder -> tiles of one size, tokens x columns x K): 347 x 32000 x 4096
+// 124 -> 98 -> 70, 512 x 11008 x 4096 52 -> 46 -> 40, 776 x 4096 x 4096 x 3 problems 87 -> 75 -> 71, 1500 x 4096 x 11008
+// 142 -> 113 -> 100, 2328 x 4096 x 4096 78 -> 69 -> 61.  A ring of 7 to 9 stages instead of 6 gave 2 to 8 %.  With a
+// short K the stores bound it, and four epilogue warps leave them waiting for one another: sixteen instead of four took
+// fp32 results of 2328 x 1024 x 1024, four problems, from 48 to 24 us and those of 776 tokens, six problems, from 26 to
+// 16 (bf16: 13.8 -> 14.6; the same change slowed gemm_kernel and gemm_pair_kernel by 2 to 10 %).
 // ------------------------------------------------------------------------------------------------------------
 constexpr int TCOLS = 256;                        // columns of C per pair
-constexpr int TSTAGES = 6;
-constexpr int TSTAGE_BYTES = 32 * 1024;           // per CTA: 128 rows of B, up to 128 rows of A
+constexpr int TMAX_STAGES = 10;                   // a stage holds, per CTA, 128 rows of B and half of a tile's rows of A
 constexpr int TALL_EPI_WARPS = 16;                // four for every quarter of the TMEM lanes, taking 32 tokens each in turn
 constexpr int TALL_THREADS = (2 + TALL_EPI_WARPS) * 32;
-constexpr size_t TALL_SMEM = 1024 + size_t(TSTAGES) * TSTAGE_BYTES + 256;
+constexpr int TALL_RING = 224 * 1024;             // the ring takes as many stages as fit
+constexpr int TALL_SMEM = 1024 + TALL_RING + 256;
 
 struct TallList {                                 // the tiles of one problem that have the same number of tokens
   int prob;
@@ -713,6 +716,7 @@ struct TallParams {
   TallProblem prob[NP];
   TallList list[2 * NP];
   int total_tiles;
+  int stages, stage_bytes;
 };
 
 template <int NP, int NSEG>
@@ -720,23 +724,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
     gemm_tall_kernel(const __grid_constant__ TallParams<NP, NSEG> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(TSTAGES) * TSTAGE_BYTES);
-  uint64_t* full = bars;                    // [TSTAGES]  (used in the even CTA)
-  uint64_t* empty = bars + TSTAGES;         // [TSTAGES]
-  uint64_t* acc_full = bars + 2 * TSTAGES;  // [2]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + TALL_RING);
+  uint64_t* full = bars;                        // [stages]  (used in the even CTA)
+  uint64_t* empty = bars + TMAX_STAGES;         // [stages]
+  uint64_t* acc_full = bars + 2 * TMAX_STAGES;  // [2]
   uint64_t* acc_empty = acc_full + 2;       // [2]        (used in the even CTA)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   int* err = &g_gemm_status;
-  const int total_tiles = p.total_tiles;
+  const int total_tiles = p.total_tiles, stages = p.stages, stage_bytes = p.stage_bytes;
   const uint32_t rank = cluster_ctarank();  // 0: issues the MMAs; 1: partner
   const int pair = blockIdx.x >> 1;
   const int n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < TSTAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -793,7 +797,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
         const int nkb = pr.kblocks[seg];
         for (int kb = 0; kb < nkb; ++kb) {
           if (!mbar_wait(&empty[s], ph, err)) { ok = false; break; }
-          uint8_t* sb = smem + size_t(s) * TSTAGE_BYTES;
+          uint8_t* sb = smem + s * stage_bytes;
           uint8_t* sa = sb + PA_BYTES;
           if (rank == 0) mbar_expect_tx_e(&full[s], bytes, leader);
           const uint32_t bar = cluster_addr_of(&full[s], 0);
@@ -808,7 +812,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
           } else {
             for (int j = 0; j < half / 64; ++j) tma_load_2d_pair_e(sa + j * 8192, map_a, bar, m0 + 64 * j, kb * BK, leader);
           }
-          if (++s == TSTAGES) {
+          if (++s == stages) {
             s = 0;
             ph ^= 1;
           }
@@ -838,14 +842,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
         for (int kb = 0; kb < nkb; ++kb) {
           if (!mbar_wait(&full[s], ph, err)) { ok = false; break; }
           tc_fence_after_sync();
-          const uint32_t sb = smem_u32(smem + size_t(s) * TSTAGE_BYTES);
+          const uint32_t sb = smem_u32(smem + s * stage_bytes);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             umma_ss_pair(d_tmem, smem_desc_sw128(sb + k * b_step, b_lbo, 1024), smem_desc_sw128(sb + PA_BYTES + k * a_step, a_lbo, 1024),
                          idesc, (kb | k) != 0, leader);
           umma_commit_pair(cluster_addr_of(&empty[s], 0), leader);
           umma_commit_pair(cluster_addr_of(&empty[s], 1), leader);
-          if (++s == TSTAGES) {
+          if (++s == stages) {
             s = 0;
             ph ^= 1;
           }
@@ -1073,7 +1077,7 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
 }
 
 template <int NP, int NSEG>
-int launch_tall(const GemmProblem* probs, int n, int nt, cudaStream_t stream) {
+int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t stream) {
   TallParams<NP, NSEG> p;
   int lists = 0, tiles = 0, maps_a = 0, maps_b = 0;
   for (int i = 0; i < n; ++i) {
@@ -1101,7 +1105,7 @@ int launch_tall(const GemmProblem* probs, int n, int nt, cudaStream_t stream) {
   for (int part = 0; part < 2; ++part)
     for (int i = 0; i < n; ++i) {
       const GemmProblem& g = probs[i];
-      const int whole = g.M / nt, rest = g.M - whole * nt, unit = g.a_mn ? 128 : 32;
+      const int whole = even ? (g.M + nt - 1) / nt : g.M / nt, rest = std::max(0, g.M - whole * nt), unit = g.a_mn ? 128 : 16;
       TallList l{};
       l.prob = i;
       l.nt = part == 0 ? nt : (rest + unit - 1) / unit * unit;
@@ -1119,7 +1123,9 @@ int launch_tall(const GemmProblem* probs, int n, int nt, cudaStream_t stream) {
       p.list[lists++] = l;
     }
   p.total_tiles = tiles;
-  if (allow_smem<gemm_tall_kernel<NP, NSEG>>(int(TALL_SMEM)) != cudaSuccess) return KVP_ERR_CUDA;
+  p.stage_bytes = PA_BYTES + nt / 2 * (BK * 2);
+  p.stages = std::min(TMAX_STAGES, TALL_RING / p.stage_bytes);
+  if (allow_smem<gemm_tall_kernel<NP, NSEG>>(TALL_SMEM) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * std::min(tiles, sm_count() / 2), TALL_THREADS, TALL_SMEM, stream, 1, p);
   timing_after(KVP_KERNEL_GEMM, stream);
@@ -1147,15 +1153,16 @@ namespace {
 
 // ------------------------------------------------------------------------------------------------------------
 // Which kernel a forward GEMM of more than 128 rows runs on.  The times (us) of each are estimated from a model with the
-// terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe -- whose
-// constants were fitted to 4000 measurements (13 column counts x 27 row counts, one launch behind the other); the
-// choice it makes costs 1.9 % more than the best of all choices on average, and 31 % less than CTA pairs always.
+// terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe, memory -- whose
+// constants were fitted to 3400 measurements (11 weight shapes x 24 row counts, weights not in L2).  The choice it makes
+// costs 1.1 % more than the best of all choices on average; without tiles of equal size 5.1 %, CTA pairs always 33 %.
 // Above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand.
 // ------------------------------------------------------------------------------------------------------------
 constexpr int CHOICE_MAX_ROWS = 4096;
 struct Choice {
   enum Kind { kSingle, kPair, kTall, kSplit } kind = kPair;
   int nt = 0;         // tokens per tile (tall, split)
+  bool even = false;  // tall: tiles of nt only
   int split = 1;
   float us = 1e30f;
 };
@@ -1172,37 +1179,54 @@ float makespan(int n1, float c1, int n2, float c2, int pairs) {
 
 Choice choose_forward(const GemmProblem* probs, int n) {
   int M = 0, kb = 0, cols128 = 0, cols256 = 0;
+  float weights = 0.f, rows = 0.f;   // bytes of B, of A and C
   for (int i = 0; i < n; ++i) {
-    M = std::max(M, probs[i].M);
-    kb = std::max(kb, (probs[i].segs[0].K + BK - 1) / BK);
-    cols128 += (probs[i].N + 127) / 128;
-    cols256 += (probs[i].N + 255) / 256;
+    const GemmProblem& g = probs[i];
+    M = std::max(M, g.M);
+    kb = std::max(kb, (g.segs[0].K + BK - 1) / BK);
+    cols128 += (g.N + 127) / 128;
+    cols256 += (g.N + 255) / 256;
+    weights += 2.f * g.N * g.segs[0].K;
+    rows += 2.f * g.M * g.N + (i == 0 ? 2.f * g.M * g.segs[0].K : 0.f);
   }
   const int sms = sm_count(), pairs = sms / 2;
   Choice best;
-  auto consider = [&](Choice::Kind kind, int nt, int split, float us) {
+  auto consider = [&](Choice::Kind kind, int nt, bool even, int split, float us) {
     if (us >= best.us) return;
     best.kind = kind;
     best.nt = nt;
+    best.even = even;
     best.split = split;
     best.us = us;
   };
   auto up = [](int x, int y) { return (x + y - 1) / y; };
-  consider(Choice::kSingle, 0, 1, up(up(M, BM) * cols256, sms) * (kb * 0.388f + 3.8f));
-  consider(Choice::kPair, 0, 1, up(up(M, PBM) * cols256, pairs) * (kb * 0.320f + 5.5f));
-  auto tall_tile = [&](int nt) { return nt == 0 ? 0.f : kb * std::max(0.125f * (1.f + nt / 256.f), 0.0013f * nt) + 3.1f; };
+  const float memory = (weights + rows) / 5.5e6f;
+  consider(Choice::kSingle, 0, false, 1, 2.1f + std::max(up(up(M, BM) * cols256, sms) * (kb * 0.403f + 4.2f), memory));
+  consider(Choice::kPair, 0, false, 1, 3.2f + std::max(up(up(M, PBM) * cols256, pairs) * (kb * 0.346f + 4.3f), memory));
+  auto tall_tile = [&](int nt) { return nt == 0 ? 0.f : kb * std::max(0.147f * (1.f + nt / 256.f), 0.00136f * nt) + 2.6f; };
+  // tiles of equal size along the tokens
+  const int fewest = up(M, 256);
+  for (int k = fewest; k < fewest + 4 + fewest / 3; ++k) {
+    const int nt = up(up(M, k), 16) * 16;
+    if (k > fewest && nt < 80) break;
+    consider(Choice::kTall, nt, true, 1, 3.5f + std::max(makespan(up(M, nt) * cols256, tall_tile(nt), 0, 0.f, pairs), memory));
+  }
+  // whole tiles, then those of the remainder: weights of which little stays in L2 in between are read twice
+  const float again = weights > 60e6f ? (weights - 60e6f) / 5.5e6f : 0.f;
   for (int nt = 128; nt <= 256; nt += 32) {
-    const int whole = M / nt, rest = up(M - whole * nt, 32) * 32;
-    consider(Choice::kTall, nt, 1, 2.9f + makespan(whole * cols256, tall_tile(nt), rest > 0 ? cols256 : 0, tall_tile(rest), pairs));
+    const int whole = M / nt, rest = up(M - whole * nt, 16) * 16;
+    if (whole == 0 || rest == 0) continue;
+    consider(Choice::kTall, nt, false, 1,
+             1.04f * (3.5f + std::max(makespan(whole * cols256, tall_tile(nt), cols256, tall_tile(rest), pairs), memory + again)));
   }
   // split kernel: one CTA per SM; clusters of four do not fill every GPC
   for (int split = 1; split <= 4 && 2 * split <= kb; split *= 2) {
     const int most = (split == 4 ? sms - 16 : sms) / (split * cols128);   // token tiles that fit
     if (most < 1) break;
-    const int nt = up(up(M, most), 16) * 16 < 48 ? 48 : up(up(M, most), 16) * 16;
+    const int nt = std::max(48, up(up(M, most), 16) * 16);
     if (nt > 256) continue;
-    consider(Choice::kSplit, nt, split, 4.5f + float(kb) / split * std::max(0.120f * (1.f + nt / 128.f), 0.0012f * nt) + 0.01f * nt +
-                                            (split > 1 ? 0.013f * nt + 0.4f : 0.f));
+    consider(Choice::kSplit, nt, false, split, 4.f + std::max(float(kb) / split * 0.109f * (1.f + nt / 128.f), (weights + rows) / 7.8e6f) +
+                                                   0.031f * nt + (split > 1 ? 0.6f : 0.f));
   }
   return best;
 }
@@ -1212,8 +1236,8 @@ int by_count(int n, F1 one, F4 four, F32 many) { return n == 1 ? one() : n <= 4 
 
 // The gradient GEMMs of a launch (pair mode 1) run on gemm_tall_kernel, in tiles of 256 rows; of 128 where those would
 // leave half of the pairs idle.  Measured (us, all weight and input gradients of a backward pass: gemm_kernel / tiles of
-// 128 / 256): 256 tokens x 256, four layers 15.6 / 6.9 / 9.1; 400 x 4096, two layers 33.6 / 29.2 / 24.0; 1984 x 1024, six
-// layers 72.7 / 74.5 / 60.2; 1664 x 4096, five layers 141 / 150 / 121; 4096 x 4096, one layer 300 / 352 / 286.
+// 128 / 256): 256 tokens x 256, four layers 14.4 / 7.0 / 9.0; 400 x 4096, two layers 32.1 / 28.9 / 23.2; 1984 x 1024, six
+// layers 70.6 / 72.8 / 59.3; 1664 x 4096, five layers 140 / 147 / 120; 4096 x 4096, one layer 303 / 352 / 282.
 // Launches of more than GRADIENT_MAX_FLOP (about 0.3 ms) stay on gemm_kernel, although by themselves they too are a little
 // faster on pairs (4096 x 4096, four layers, 0.8 TFLOP: 1140 / - / 1030): they belong to steps of many milliseconds, which
 // the board's power limit bounds, and there the rest of the step slows by more than the pairs gain (training step of eight
@@ -1230,9 +1254,9 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
   }
   if (flop > GRADIENT_MAX_FLOP) return launch_group(probs, n, stream, 0, 0, false);
   const int nt = 4 * tiles <= sm_count() ? 128 : 256;
-  if (segs == 1) return launch_tall<1, 1>(probs, n, nt, stream);
-  if (segs <= 4) return launch_tall<4, 4>(probs, n, nt, stream);
-  return launch_tall<MAX_PROB, MAX_MAPS / 2>(probs, n, nt, stream);
+  if (segs == 1) return launch_tall<1, 1>(probs, n, nt, false, stream);
+  if (segs <= 4) return launch_tall<4, 4>(probs, n, nt, false, stream);
+  return launch_tall<MAX_PROB, MAX_MAPS / 2>(probs, n, nt, false, stream);
 }
 
 // A forward GEMM (K-major operands, one segment): -1 when the tile kernels take it
@@ -1257,8 +1281,8 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
     const Choice c = choose_forward(g, cnt);
     int rc;
     if (c.kind == Choice::kTall) {
-      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, stream); },
-                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, stream); });
+      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, c.even, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, c.even, stream); },
+                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, c.even, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
       rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
