@@ -1,19 +1,23 @@
-"""In-tree build of the CUDA library: nvcc for sm_100a -> libkvp.so next to this file.
+"""In-tree build of the CUDA library: nvcc for sm_100a -> libkvp.so next to this file; and of the binding's argument
+packing: g++ against torch's headers -> _pack.so.
 
 Run as ``python -m paper_2608_15943_b200.build`` or call ``build()``.  Objects are rebuilt only
 when a source or header is newer than the object.
 """
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libkvp.so")
+PACK = os.path.join(HERE, "_pack.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 SOURCES = ["kvp_common.cu", "kvp_plan.cu", "kvp_gemm.cu", "kvp_attn_fwd.cu", "kvp_attn_bwd.cu", "kvp_decode.cu", "kvp_misc.cu", "kvp_stage.cu",
@@ -42,11 +46,27 @@ def _compile(src: str, force: bool) -> str:
     return obj
 
 
+def _build_pack(force: bool) -> None:
+    src = os.path.join(CSRC, "kvp_pack.cpp")
+    if not force and os.path.exists(PACK) and os.path.getmtime(PACK) > os.path.getmtime(src):
+        return
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-w", "-I" + sysconfig.get_paths()["include"],
+           "-I" + inc, "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), src, "-o", PACK, "-L" + lib,
+           "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath," + lib]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{cmd[0]} failed for {src}:\n{r.stdout}\n{r.stderr}")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     srcs = [s for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
-    with ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with ThreadPoolExecutor(max_workers=min(8, len(srcs) + 1)) as ex:
+        pack = ex.submit(_build_pack, force)
         objs = list(ex.map(lambda s: _compile(s, force), srcs))
+        pack.result()
     if force or not os.path.exists(LIB) or any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
         cmd = [NVCC, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a", "-lcudart_static",
                "-ldl", "-lpthread", "-lrt"]
