@@ -1,8 +1,8 @@
 // Causal GQA flash-attention forward over a donor map (Eq. 2-3 of the paper): layer l attends
 // with its own queries to the keys/values of layer donor[l].
 //
-// A work item is TWO adjacent 128-row query tiles (A, B) of one (batch, query head); the CTA walks the
-// donor's K/V tiles once for both, so every K/V tile fetched by TMA feeds twice the tensor work.  CTAs are
+// A work item is TWO adjacent 128-row query tiles (A, B) of one (batch, query head), or the last tiles of two heads; the
+// CTA walks the donor's K/V tiles once for both, so every K/V tile fetched by TMA feeds twice the tensor work.  CTAs are
 // persistent (one per SM) and take a balanced list of items each.
 //   warp 0      TMA producer: Q_A, Q_B once, then K_j / V_j rings
 //   warps 1, 2  tcgen05.mma issuers, one per query tile (on two different warp schedulers: issuing an MMA costs
@@ -65,6 +65,7 @@ struct FwdParams {
   int n_layers;
   int o_f32;
   int B, S, Hq, Hkv;
+  int odd_by_heads;                 // the last of an odd number of query tiles: two heads' make an item
   int causal;
   float scale_log2;                 // scale * log2(e)
 };
@@ -82,29 +83,50 @@ __device__ __forceinline__ int fwd_item_index(int round) {
   const int g = int(gridDim.x), i = int(blockIdx.x);
   return round * g + ((round & 1) ? g - 1 - i : i);
 }
+// The last of an odd number of query tiles comes first, by itself or (odd_by_heads) with that of the next query head, which
+// reads the same keys: half as many of the items that keep only one of the two softmax warpgroups busy.  (us, before ->
+// after, 16 heads on 4: 12 x 128 tokens, dh 64, 3 layers 16.6 -> 12.7; 12 x 100, dh 128, 4 layers 24.8 -> 18.8; 8 x 640,
+// dh 128, 2 layers 52.2 -> 47.4; 4 x 1664, dh 64, 2 layers 91.1 -> 84.5.  All tiles paired by heads instead: an even
+// number of them takes 2 to 3 % longer, the two tiles of an item then end at the same time.)
 struct FwdItem {
-  int layer, b, hq, hk, q0;
-  int n_kv[2];  // key tiles each query tile walks (tile B may not exist at a ragged end)
-  int n_max;
+  int layer, b, hq, hk, q0;     // of tile A
+  int dhq, dq0;                 // tile B: dhq heads and dq0 rows further on
+  int n_a, n_b;                 // key tiles each query tile walks (0: there is no tile B)
+  __device__ __forceinline__ int n_kv(int x) const { return x == 0 ? n_a : n_b; }
+  __device__ __forceinline__ int n_max() const { return max(n_a, n_b); }
 };
-__device__ __forceinline__ FwdItem fwd_item(const FwdParams& p, int t, int n_pairs) {
+__device__ __forceinline__ FwdItem fwd_item(const FwdParams& p, int t, int n_qtiles) {
   FwdItem w;
-  const int bh = p.B * p.Hq, lbh = p.n_layers * bh;
-  const int pair = n_pairs - 1 - t / lbh;
-  const int r = t % lbh;
-  w.layer = r / bh;
-  w.hq = r % p.Hq;
-  w.b = (r % bh) / p.Hq;
-  w.hk = w.hq / (p.Hq / p.Hkv);
-  w.q0 = pair * 2 * BQ;  // first row of tile A; tile B starts at q0 + 128
-#pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const int qs = w.q0 + x * BQ;
-    const int kv_end = p.causal ? min(p.S, qs + BQ) : p.S;
-    w.n_kv[x] = qs < p.S ? (kv_end + BKV - 1) / BKV : 0;
+  int heads = p.Hq, row = 0;
+  const int lb = p.n_layers * p.B, n_odd = (n_qtiles & 1) ? lb * p.Hq >> p.odd_by_heads : 0;
+  w.dhq = 0;
+  w.dq0 = BQ;
+  if (t < n_odd) {
+    row = n_qtiles - 1;
+    heads >>= p.odd_by_heads;
+    w.dhq = p.odd_by_heads;
+    w.dq0 = p.odd_by_heads ? 0 : BQ;
+  } else {
+    t -= n_odd;
+    row = (n_qtiles & ~1) - 2 - t / (lb * heads) * 2;
   }
-  w.n_max = max(w.n_kv[0], w.n_kv[1]);
+  const int r = t % (lb * heads);
+  w.layer = r / (p.B * heads);
+  w.b = r / heads % p.B;
+  w.hq = r % heads << w.dhq;
+  w.hk = w.hq / (p.Hq / p.Hkv);
+  w.q0 = row * BQ;
+  auto key_tiles = [&](int qs) {
+    const int kv_end = p.causal ? min(p.S, qs + BQ) : p.S;
+    return qs < p.S ? (kv_end + BKV - 1) / BKV : 0;
+  };
+  w.n_a = key_tiles(w.q0);
+  w.n_b = key_tiles(w.q0 + w.dq0);
   return w;
+}
+// number of work items
+__host__ __device__ __forceinline__ long long fwd_items(long long lbh, int n_qtiles, int odd_by_heads) {
+  return lbh * (n_qtiles / 2) + ((n_qtiles & 1) ? lbh >> odd_by_heads : 0);
 }
 
 template <int DH>
@@ -136,8 +158,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
   int* err = &g_fwd_status;
 
   const int n_qtiles = (p.S + BQ - 1) / BQ;
-  const int n_pairs = (n_qtiles + 1) / 2;
-  const int n_items = n_pairs * p.n_layers * p.B * p.Hq;
+  const int n_items = int(fwd_items(p.n_layers * p.B * p.Hq, n_qtiles, p.odd_by_heads));
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -189,14 +210,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
         const int t = fwd_item_index(round);
         if (t >= n_items) continue;   // only the last round can be short
-        const FwdItem w = fwd_item(p, t, n_pairs);
+        const FwdItem w = fwd_item(p, t, n_qtiles);
         if (!mbar_wait(q_empty, (it & 1) ^ 1, err)) { ok = false; break; }
         mbar_expect_tx_e(q_full, 2 * L::Q_BYTES, leader);  // rows beyond the sequence are zero-filled
 #pragma unroll
         for (int x = 0; x < 2; ++x)
 #pragma unroll
           for (int h = 0; h < HALVES; ++h)
-            tma_load_4d_e(smem + L::OFF_Q + x * L::Q_BYTES + h * HALF_BYTES, &p.map_q[w.layer], q_full, h * 64, w.hq, w.q0 + x * BQ, w.b, leader);
+            tma_load_4d_e(smem + L::OFF_Q + x * L::Q_BYTES + h * HALF_BYTES, &p.map_q[w.layer], q_full, h * 64, w.hq + x * w.dhq, w.q0 + x * w.dq0, w.b, leader);
         auto load_k = [&](int j) -> bool {
           const int s = kg % FWD_KSTAGES;
           if (!mbar_wait(&k_empty[s], ((kg / FWD_KSTAGES) & 1) ^ 1, err)) return false;
@@ -218,8 +239,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
           return true;
         };
         ok = load_k(0);
-        for (int j = 0; j < w.n_max && ok; ++j) {
-          if (j + 1 < w.n_max) ok = load_k(j + 1);  // scores run one tile ahead of the P V products
+        for (int j = 0; j < w.n_max() && ok; ++j) {
+          if (j + 1 < w.n_max()) ok = load_k(j + 1);  // scores run one tile ahead of the P V products
           if (ok) ok = load_v(j);
         }
         ++it;
@@ -246,9 +267,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
         const int t = fwd_item_index(round);
         if (t >= n_items) continue;
-        const FwdItem w = fwd_item(p, t, n_pairs);
-        const int n_cx = 2 * w.n_kv[x];
-        const int n_cmax = 2 * w.n_max;
+        const FwdItem w = fwd_item(p, t, n_qtiles);
+        const int n_cx = 2 * w.n_kv(x);
+        const int n_cmax = 2 * w.n_max();
         auto k_stage = [&](int j) { return (jg + j) % FWD_KSTAGES; };
         auto k_parity = [&](int j) { return ((jg + j) / FWD_KSTAGES) & 1; };
         auto v_stage = [&](int j) { return (jg + j) % FWD_VSTAGES; };
@@ -310,7 +331,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
           if (u == 1) umma_commit(&v_empty[v_stage(j)], leader);
           if (cn < n_cmax && (cn & 1) == 1) umma_commit(&k_empty[k_stage(jn)], leader);
         }
-        jg += w.n_max;
+        jg += w.n_max();
         g0 += n_cx;
         n_o += n_cx > 0 ? 1 : 0;
         ++it;
@@ -325,18 +346,18 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
     for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
       const int t = fwd_item_index(round);
       if (t >= n_items) continue;
-      const FwdItem w = fwd_item(p, t, n_pairs);
+      const FwdItem w = fwd_item(p, t, n_qtiles);
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
-        if (w.n_kv[x] == 0 || !ok) continue;
+        if (w.n_kv(x) == 0 || !ok) continue;
         ok = mbar_wait(&l_ready[x], n_done[x] & 1, err) && mbar_wait(&o_done[x], n_done[x] & 1, err);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         ++n_done[x];
         tc_fence_after_sync();
         const float inv_l = inv_sum[x * BQ + r];
-        const int q_row = w.q0 + x * BQ + r;
-        const size_t o_at = ((size_t(w.b) * p.S + q_row) * p.Hq + w.hq) * DH;
+        const int q_row = w.q0 + x * w.dq0 + r;
+        const size_t o_at = ((size_t(w.b) * p.S + q_row) * p.Hq + w.hq + x * w.dhq) * DH;
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) {
           uint32_t tmp[64];
@@ -383,9 +404,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
     for (int round = 0; round * int(gridDim.x) < n_items && ok; ++round) {
       const int t = fwd_item_index(round);
       if (t >= n_items) continue;
-      const FwdItem w = fwd_item(p, t, n_pairs);
-      const int q_row = w.q0 + x * BQ + r;
-      const int my_n = w.n_kv[x];
+      const FwdItem w = fwd_item(p, t, n_qtiles);
+      const int q0 = w.q0 + x * w.dq0, q_row = q0 + r;
+      const int my_n = w.n_kv(x);
       const int my_c = 2 * my_n;
       float m_used = -INFINITY;  // running maximum (log2 domain) the exponentials are taken against
       uint64_t l2 = 0ull, l2b = 0ull;  // four partial row sums (two packed pairs, for independent add chains)
@@ -404,7 +425,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
         int lim = p.S - kv0;
         if (p.causal) lim = min(lim, q_row - kv0 + 1);
         // (no vote for the sub-blocks that every row of the tile sees in full: the common case)
-        const bool all_visible = kv0 + BC <= p.S && (!p.causal || kv0 + BC - 1 <= w.q0 + x * BQ);
+        const bool all_visible = kv0 + BC <= p.S && (!p.causal || kv0 + BC - 1 <= q0);
         if (!all_visible && __any_sync(0xffffffffu, lim < BC)) {
 #pragma unroll
           for (int i = 0; i < BC; ++i)
@@ -467,7 +488,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       ok = __all_sync(0xffffffffu, ok);
       if (ok && my_n > 0) {
         const float l_sum = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
-        if (q_row < p.S) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
+        if (q_row < p.S) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq + x * w.dhq) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
         ok = n_done == 0 || mbar_wait(&o_free[x], (n_done - 1) & 1, err);   // the epilogue warps have read the last item's
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         inv_sum[x * BQ + r] = 1.f / l_sum;
@@ -535,7 +556,9 @@ int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* con
   const float sc = scale == 0.f ? 1.f / sqrtf(float(s->dh)) : scale;
   p.scale_log2 = sc * 1.4426950408889634f;
   const int n_qtiles = (s->S + BQ - 1) / BQ;
-  const long long n_items = (long long)n * s->B * s->Hq * ((n_qtiles + 1) / 2);
+  // (with no more items than SMs every tile has an SM to itself)
+  p.odd_by_heads = (s->Hq / s->Hkv) % 2 == 0 && fwd_items((long long)n * s->B * s->Hq, n_qtiles, 0) > sm_count();
+  const long long n_items = fwd_items((long long)n * s->B * s->Hq, n_qtiles, p.odd_by_heads);
   if (n_items > 0x7fffffffLL) return KVP_ERR_UNSUPPORTED;
   // persistent: one CTA per SM walks a list of (layer, b, hq, tile pair) items
   const int grid = int(n_items < (long long)sm_count() ? n_items : (long long)sm_count());

@@ -12,8 +12,12 @@ pytestmark = pytest.mark.gpu
     (13, 104, 12, 12, 64, [0, 0], True),    # one query tile: no item has a second one
     (10, 384, 16, 16, 128, [0], True),      # three: every CTA starts with an item without, some have two in a row
     (6, 264, 15, 3, 64, [0, 0], False),     # the same in full attention, five heads to a KV head
+    (13, 104, 12, 6, 64, [0, 0], True),     # an even number of heads to a KV head: two heads' last tiles make an item
+    (5, 392, 16, 4, 128, [0, 1], True),
+    (4, 257, 20, 10, 64, [0, 0], False),    # one query in the last tile
+    (2, 264, 8, 2, 128, [0], True),         # fewer items than SMs: the last tiles stay by themselves
 ])
-def test_items_without_a_second_tile(B, S, Hq, Hkv, dh, donor, causal):
+def test_items_of_an_odd_number_of_query_tiles(B, S, Hq, Hkv, dh, donor, causal):
     from paper_2608_15943_b200 import kvp
     L = len(donor)
     q, k, v, _ = attn_inputs(B, S, Hq, Hkv, dh, donor)
