@@ -1,5 +1,5 @@
-"""RMSNorm and rotary embedding at the edges of how they share the work out: one row or two per block, all heads or a
-few per thread."""
+"""RMSNorm, rotary embedding, add and SwiGLU at the edges of how they share the work out: rows per block, heads and pieces
+per thread."""
 import numpy as np
 import pytest
 import torch
@@ -32,3 +32,17 @@ def test_rope_heads_per_thread(B, S, H, dh, pos0):
     x = synth.normal((B, S, H, dh), 62, 1, 1.0, "cuda")
     ref = ST.rope(x.double().cpu().numpy(), 10000.0, pos0)
     bf16_close(kvp.rope(x, 10000.0, pos0), ref)
+
+
+@pytest.mark.parametrize("n8", [1, 255, 148 * 2048, 148 * 2048 + 1, 2 * 148 * 2048, 2 * 148 * 2048 + 1])
+def test_add_and_swiglu_pieces_per_thread(n8):
+    """One, two and three 16-byte pieces per thread on a device of 148 SMs, and one more than fits each."""
+    from paper_2608_15943_b200 import kvp
+    a, b = synth.normal((n8 * 8,), 63, 1, 1.0, "cuda"), synth.normal((n8 * 8,), 63, 2, 1.0, "cuda")
+    an, bn = a.double().cpu().numpy(), b.double().cpu().numpy()
+    y = torch.full((n8 * 8 + 64,), 7.0, dtype=torch.bfloat16, device="cuda")
+    for op, ref in ((kvp.add, an + bn), (kvp.swiglu, ST.swiglu(an, bn))):
+        y.fill_(7.0)
+        op(a, b, y[:n8 * 8])
+        bf16_close(y[:n8 * 8], ref)
+        assert (y[n8 * 8:] == 7.0).all()
