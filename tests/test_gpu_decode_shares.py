@@ -67,3 +67,64 @@ def test_decode_shares(L, donor, B, Hq, Hkv, dh, page, lens, static):
         assert np.linalg.norm(got - ro[l]) <= REL * np.linalg.norm(ro[l])
         assert np.abs(got - ro[l]).max() <= ABS
         assert np.abs(f64(lse[l]) - rl[l]).max() <= LSE_TOL
+
+
+def paged(lens, Hkv, dh, page, seed):
+    """Pools of one layer with the pages of each sequence in a row, their block table and max_pages."""
+    need = [(n + page - 1) // page for n in lens]
+    bt, at = torch.zeros(len(lens), max(need), dtype=torch.int32), 0
+    for b, k in enumerate(need):
+        bt[b, :k] = torch.arange(at, at + k)
+        at += k
+    return [synth.normal((at, Hkv, page, dh), seed, i, 1.0, "cuda") for i in (1, 2)] + [bt]
+
+
+def exact_on_gpu(q, kc, vc, bt, lens, page):
+    """The oracle's decode in 64 bits for sizes that take numpy too long: outputs [B, Hq, dh] and LSE [B, Hq]."""
+    B, Hq, dh = q.shape
+    Hkv = kc.shape[1]
+    o, lse = torch.empty(B, Hq, dh, dtype=torch.float64, device="cuda"), torch.empty(B, Hq, dtype=torch.float64, device="cuda")
+    for b, n in enumerate(lens):
+        k, v = (p[bt[b, :(n + page - 1) // page].long().cuda()].permute(1, 0, 2, 3).reshape(Hkv, -1, dh)[:, :n].double() for p in (kc, vc))
+        s = torch.einsum("hgd,hnd->hgn", q[b].double().view(Hkv, Hq // Hkv, dh), k) * dh ** -0.5
+        o[b] = torch.einsum("hgn,hnd->hgd", torch.softmax(s, -1), v).reshape(Hq, dh)
+        lse[b] = torch.logsumexp(s, -1).reshape(Hq)
+    return o, lse
+
+
+def decode_one_layer(q, kc, vc, bt, lens, page, num_splits=0):
+    from paper_2608_15943_b200 import kvp
+    B, Hq, dh = q.shape
+    desc = kvp.DecodeDesc(1, B, Hq, kc.shape[1], dh, page, bt.shape[1], kc.shape[0], num_splits)
+    o, lse = torch.full_like(q, float("nan")), torch.full((B, Hq), float("nan"), device="cuda")
+    ws = torch.empty(kvp.decode_workspace_bytes(desc, [0]), dtype=torch.uint8, device="cuda")
+    kvp.decode(desc, [0], [q], [kc], [vc], bt.cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda"), [o], [lse], ws)
+    assert kvp.device_status() == kvp.OK
+    return o.double(), lse.double()
+
+
+def test_error_does_not_grow_with_the_share():
+    """Shares of 166 granules are no further from 64 bits than splits of 128 (2048 tokens): a warp's 41 granules against 32.
+    With 32768 outputs two draws of the same error differ by 0.4 % (one sigma); 1 % is allowed."""
+    lens, page = [16384] * 8, 128
+    kc, vc, bt = paged(lens, 8, 128, page, 71)
+    q = synth.normal((8, 32, 128), 71, 3, 1.0, "cuda")
+    ro, rl = exact_on_gpu(q, kc, vc, bt, lens, page)
+    got, lse = decode_one_layer(q, kc, vc, bt, lens, page)
+    split, _ = decode_one_layer(q, kc, vc, bt, lens, page, num_splits=8)
+    assert (got - ro).norm() <= 1.01 * (split - ro).norm()
+    assert (lse - rl).abs().max() <= 2e-6     # values of about 10: two ulps
+
+
+@pytest.mark.parametrize("at", [0, 700, 4999])
+def test_one_score_far_above_the_others(at):
+    """One token 290 (log2) above the rest, first, in the middle or last: what comes before it vanishes and what comes after
+    it adds nothing, however often the reference of the probabilities falls."""
+    lens, page = [5000], 16
+    kc, vc, bt = paged(lens, 1, 64, page, 72)
+    q = synth.normal((1, 4, 64), 72, 3, 1.0, "cuda")
+    q[:, 1:] = q[:, :1]
+    kc[at // page, 0, at % page] = q[0, 0] * 25.0
+    ro, rl = exact_on_gpu(q, kc, vc, bt, lens, page)
+    got, lse = decode_one_layer(q, kc, vc, bt, lens, page)
+    assert (got - ro).norm() <= REL * ro.norm() and (lse - rl).abs().max() <= 2e-7 * rl.abs().max()
