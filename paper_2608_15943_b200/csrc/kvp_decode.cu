@@ -8,11 +8,12 @@
 //  - The rows of all units form one list of 16-token granules (8 KB at dh 128: 4 KB of K, 4 KB of V; both contiguous,
 //    a page block of one KV head is), in order of (group, sequence, KV head, position).  The lengths are in device
 //    memory, so every block sums them up itself and takes an equal share of the list, wherever its ends fall: no
-//    part-filled last wave, whatever the batch and the lengths.  Long lists are cut into more shares than blocks that
+//    part-filled last wave, whatever the batch and the lengths.  (kvp_deal.h has the rules; the list has empty places that
+//    stand for the merge of each unit.)  Long lists are cut into more shares than blocks that
 //    fit, so that the block scheduler evens out SMs that draw memory at different rates.
-//  - Short units are not cut: units of 32 granules or fewer on average (64, where there are enough of them) are dealt
-//    out whole, since every piece costs a block a merge of its warps (30 sequences of 500 tokens, 8 groups at dh 64:
-//    46 us by units, 96 us when each was cut in two).
+//  - Short units, none of them much longer than an equal share, are not cut but dealt out whole, since every piece costs a
+//    block a merge of its warps (30 sequences of 500 tokens, 8 groups at dh 64: 46 us by units, 96 us when each was cut in
+//    two).
 //  - The four warps of a block take the granules of a share in turn, each with a ring of its own filled by 16-byte
 //    cp.async copies that are fully coalesced and continue across the ends of units; two blocks per SM.  (A contiguous
 //    share for every warp instead read memory 3 % slower.)  No transposes in HBM -- V fragments come from ldmatrix.trans
@@ -28,6 +29,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "kvp_deal.h"
 #include "kvp_host.h"
 #include "kvp_sm100.cuh"
 
@@ -47,9 +49,6 @@ constexpr int DEC_CTAS_PER_SM = DH == 128 ? 2 : 4;   // as many as shared memory
 // granules a warp, 2.12e-3 so, 0.6 % slower.  Against the largest of each granule by itself: 1.94e-3, 1.2 % slower.)
 constexpr int REFERENCE_GRANULES = 16;
 constexpr float REFERENCE_DROP = 8.f;
-constexpr int MIN_SHARE = 8;       // granules of a share at least: a piece costs a block about as much again
-constexpr int LONG_SHARE = 160;    // granules of a share at least where there are more shares than blocks that fit
-constexpr int MAX_ROUNDS = 16;     // shares per block that fits, at most
 constexpr int MAX_DEC_GROUPS = 64;
 constexpr int MAX_MEMBERS = 4;     // layers of a donor group served by one pass (rows = members * G <= 16)
 
@@ -86,31 +85,21 @@ __device__ __forceinline__ int clamped_length(const DecParams& p, int b) {
 }
 __device__ __forceinline__ int granules_of(int len) { return (len + GRAN - 1) / GRAN; }
 
-// Sums over the batch, formed by one warp: granules (of one KV head) of the sequences before b_before, and of all.
-__device__ __forceinline__ void sum_granules(const DecParams& p, int b_before, int& before, int& all) {
-  before = all = 0;
+// Over the batch, formed by one warp: granules (of one KV head) of the sequences before b_before, of all, and of the longest.
+__device__ __forceinline__ void sum_granules(const DecParams& p, int b_before, int& before, int& all, int& longest) {
+  before = all = longest = 0;
   for (int b = threadIdx.x & 31; b < p.B; b += 32) {
     const int n = granules_of(clamped_length(p, b));
     all += n;
+    longest = max(longest, n);
     before += b < b_before ? n : 0;
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     before += __shfl_xor_sync(0xffffffffu, before, s);
     all += __shfl_xor_sync(0xffffffffu, all, s);
+    longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, s));
   }
-}
-__host__ __device__ inline bool dealt_by_units(long long total, long long units, int fit) {
-  return total < 32 * units || (total < 64 * units && units >= fit);
-}
-// Shares a list of `total` granules is dealt out in.
-__host__ __device__ inline int shares_for(int fit, int max_shares, long long total) {
-  long long n = total / MIN_SHARE;
-  if (n > fit) {
-    const long long rounds = total / ((long long)fit * LONG_SHARE);
-    n = (long long)fit * (rounds < 1 ? 1 : rounds > MAX_ROUNDS ? MAX_ROUNDS : rounds);
-  }
-  return int(n < 1 ? 1 : n > max_shares ? max_shares : n);
 }
 // The first T mod n of n shares of a list of T granules hold one more than the others.
 __device__ __forceinline__ uint32_t div_long(long long a, uint32_t b) {   // quotients here fit 32 bits; so do nearly all dividends
@@ -205,7 +194,7 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     int id;                                        // the unit's number, where units are dealt out
   };
   Cursor c;                                        // start of the block's next piece
-  int todo;                                        // granules of the block's share of a group's list still to do
+  int todo;                                        // places of the block's share of the list still to do
   const bool caller_splits = p.num_splits > 0;
   auto go_to_unit = [&](Cursor& x, int id) {       // (past the last unit: grp >= n_groups)
     x.id = id;
@@ -218,11 +207,14 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
   };
   long long per_group = 0;
   bool by_units = p.by_units != 0;
+  int rest = 0;                                    // places behind the granules of a unit
   if (!caller_splits && !by_units) {
-    int before, all;
-    sum_granules(p, 0, before, all);
-    per_group = (long long)all * p.Hkv;
-    by_units = dealt_by_units(per_group * p.n_groups, (long long)p.n_groups * p.B * p.Hkv, p.fit);
+    int before, all, longest;
+    sum_granules(p, 0, before, all, longest);
+    const long long granules = (long long)all * p.Hkv * p.n_groups;
+    by_units = dealt_by_units(DH, granules, (long long)p.n_groups * p.B * p.Hkv, longest, p.fit);
+    rest = by_units ? 0 : unit_rest(DH, granules, p.fit);
+    per_group = ((long long)all + (long long)p.B * rest) * p.Hkv;
   }
   if (caller_splits) {
     const int split = blockIdx.x % p.num_splits;
@@ -236,7 +228,7 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     todo = c.ng;
   } else {
     const long long total = per_group * p.n_groups;
-    const int n_shares = shares_for(p.fit, p.max_shares, total);
+    const int n_shares = shares_for(DH, p.fit, p.max_shares, total);
     if (blockIdx.x >= n_shares) return;
     const Dealt dealt(total, n_shares);
     long long at = dealt.begin(blockIdx.x);
@@ -245,7 +237,7 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     c.grp = int(div_long(at, uint32_t(per_group)));
     at -= c.grp * per_group;                       // inside the group: find the sequence, 32 lengths at a time
     for (int b0 = 0;; b0 += 32) {
-      const int mine = b0 + lane < p.B ? granules_of(clamped_length(p, b0 + lane)) : 0;
+      const int mine = b0 + lane < p.B ? granules_of(clamped_length(p, b0 + lane)) + rest : 0;
       int upto = mine;
 #pragma unroll
       for (int s = 1; s < 32; s <<= 1) {
@@ -263,8 +255,8 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     }
     c.len = clamped_length(p, c.b);
     c.ng = granules_of(c.len);
-    c.hk = int(at) / c.ng;                         // (a sequence's granules of all KV heads fit 32 bits)
-    c.gran = int(at) % c.ng;
+    c.hk = int(at) / (c.ng + rest);                // (a sequence's places of all KV heads fit 32 bits)
+    c.gran = int(at) % (c.ng + rest);
   }
 
   uint8_t* ring = dsmem + size_t(warp) * STAGES * STAGE_BYTES;
@@ -282,9 +274,9 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
       x.ng = granules_of(x.len);
     }
   };
-  // The piece behind the one at x, of the `left` granules of the block's share from x on; past the end: grp >= n_groups.
+  // The piece behind the one at x, of the `left` places of the block's share from x on; past the end: grp >= n_groups.
   auto next_piece = [&](Cursor& x, int& left) {
-    left -= min(left, x.ng - x.gran);
+    left -= min(left, x.ng + rest - x.gran);
     if (left > 0) {
       next_unit(x);
     } else if (by_units && !caller_splits) {
@@ -295,9 +287,14 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     }
   };
 
+  if (c.gran >= c.ng && !caller_splits) {          // the share begins behind the granules of a unit
+    next_piece(c, todo);
+    if (c.grp >= p.n_groups) return;
+  }
+
   // ---- copies: a cursor of their own, STAGES - 1 of this warp's granules ahead of the arithmetic ----
   Cursor f = c;                                    // start of the piece the copies are in
-  int f_todo = todo;                               // granules of the share from there on
+  int f_todo = todo;                               // places of the share from there on
   int f_left;                                      // granules of the piece from this warp's next one on (<= 0: none)
   const int gran_per_page = p.page_size / GRAN;
   const uint8_t *kbase = nullptr, *vbase = nullptr;   // the group's pools
@@ -622,12 +619,14 @@ __global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const _
     w0 = unit * p.num_splits;
     w1 = w0 + p.num_splits - 1;
   } else {
-    int before, all;
-    sum_granules(p, b, before, all);
-    const long long per_group = (long long)all * p.Hkv, total = per_group * p.n_groups;
-    if (dealt_by_units(total, (long long)p.n_groups * p.B * p.Hkv, p.fit)) return;   // finished by the blocks that held them
-    const int n = shares_for(p.fit, p.max_shares, total), ng = granules_of(clamped_length(p, b));
-    const long long first = gi * per_group + (long long)before * p.Hkv + (long long)hk * ng;
+    int before, all, longest;
+    sum_granules(p, b, before, all, longest);
+    const long long granules = (long long)all * p.Hkv * p.n_groups;
+    if (dealt_by_units(DH, granules, (long long)p.n_groups * p.B * p.Hkv, longest, p.fit)) return;   // finished by the blocks that held them
+    const int rest = unit_rest(DH, granules, p.fit), ng = granules_of(clamped_length(p, b));
+    const long long per_group = ((long long)all + (long long)p.B * rest) * p.Hkv, total = per_group * p.n_groups;
+    const int n = shares_for(DH, p.fit, p.max_shares, total);
+    const long long first = gi * per_group + ((long long)before + (long long)b * rest) * p.Hkv + (long long)hk * (ng + rest);
     const Dealt dealt(total, n);
     w0 = dealt.share_of(first);
     w1 = dealt.share_of(first + ng - 1);
@@ -802,9 +801,8 @@ int blocks_that_fit(int dh) { return sm_count() * (dh == 128 ? DEC_CTAS_PER_SM<1
 size_t piece_bytes(const kvp_decode_desc* d, size_t pieces, int rows) {
   return align256(pieces * rows * d->dh * 4) + align256(pieces * rows * 2 * 4);
 }
-long long longest_list(const kvp_decode_desc* d, int n_groups) {
-  return (long long)n_groups * d->B * d->Hkv * ((long long)d->max_pages * d->page_size / GRAN);
-}
+long long longest_unit(const kvp_decode_desc* d) { return (long long)d->max_pages * d->page_size / GRAN; }
+long long longest_list(const kvp_decode_desc* d, int n_groups) { return (long long)n_groups * d->B * d->Hkv * longest_unit(d); }
 struct Scratch {
   int max_shares = 0, rows = 0;
   size_t pieces = 0, bytes = 0;
@@ -815,7 +813,8 @@ Scratch plan_scratch(const kvp_decode_desc* d, const SubGroup* subs, int n_sub, 
   const int per_launch = n_sub < MAX_DEC_GROUPS ? n_sub : MAX_DEC_GROUPS;
   for (int i = 0; i < n_sub; ++i) s.rows = std::max(s.rows, subs[i].n * (d->Hq / d->Hkv));
   const int fit = blocks_that_fit(d->dh);
-  s.max_shares = shares_for(fit, fit * MAX_ROUNDS, longest_list(d, per_launch));
+  const long long longest = longest_list(d, per_launch);
+  s.max_shares = shares_for(d->dh, fit, fit * max_rounds(d->dh), longest + (long long)per_launch * d->B * d->Hkv * unit_rest(d->dh, longest, fit));
   for (;;) {
     s.pieces = d->num_splits > 0 ? size_t(per_launch) * d->B * d->Hkv * d->num_splits : size_t(s.max_shares) * 2;
     s.bytes = piece_bytes(d, s.pieces, s.rows);
@@ -965,10 +964,11 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
     // a block for every share of the longest list; shares go by the lengths on the device, and so does whether whole units
     // are dealt out instead
     const long long blocks = d->num_splits > 0 ? units * d->num_splits
-                                               : std::max((long long)sc_plan.max_shares, std::min(units, (long long)p.fit * MAX_ROUNDS));
+                                               : std::max((long long)sc_plan.max_shares, std::min(units, (long long)p.fit * max_rounds(d->dh)));
     if (units > 0x7fffffffLL || blocks > 0x7fffffffLL) return KVP_ERR_UNSUPPORTED;
     p.n_groups = n;
-    p.by_units = dealt_by_units(longest_list(d, n), units, p.fit);
+    // (units that are short on average in a full table are so at any lengths)
+    p.by_units = dealt_by_units(d->dh, longest_list(d, n), units, longest_unit(d), p.fit);
     const long long unit_pieces = d->num_splits > 0 ? d->num_splits : sc_plan.max_shares / units;
     const int wpr = unit_pieces > 8 ? 8 : 1;   // many pieces a unit: eight warps share those of a row
     const int rows_per_block = COMBINE_THREADS / 32 / wpr;

@@ -128,3 +128,16 @@ def test_one_score_far_above_the_others(at):
     ro, rl = exact_on_gpu(q, kc, vc, bt, lens, page)
     got, lse = decode_one_layer(q, kc, vc, bt, lens, page)
     assert (got - ro).norm() <= REL * ro.norm() and (lse - rl).abs().max() <= 2e-7 * rl.abs().max()
+
+
+@pytest.mark.parametrize("lens,Hkv,dh,page", [
+    ([32768] + [300] * 63, 8, 128, 128),                  # short units on average, one of 2048 granules
+    ([200] * 20 + [30000] + [200] * 19, 4, 64, 16),
+    ([5, 1100, 1, 1009, 1], 1, 128, 16),                  # units just above and below those a block takes whole
+])
+def test_a_long_sequence_among_short_ones(lens, Hkv, dh, page):
+    kc, vc, bt = paged(lens, Hkv, dh, page, 73)
+    q = synth.normal((len(lens), 4 * Hkv, dh), 73, 3, 1.0, "cuda")
+    ro, rl = exact_on_gpu(q, kc, vc, bt, lens, page)
+    got, lse = decode_one_layer(q, kc, vc, bt, lens, page)
+    assert ((got - ro).norm(dim=(1, 2)) <= REL * ro.norm(dim=(1, 2))).all() and (lse - rl).abs().max() <= 2e-6
