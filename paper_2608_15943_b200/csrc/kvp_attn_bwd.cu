@@ -29,14 +29,15 @@
 #include <algorithm>
 #include <vector>
 
+#include "kvp_bwd_shape.h"
 #include "kvp_host.h"
 #include "kvp_sm100.cuh"
 
 namespace kvp {
 namespace {
 
-constexpr int BT = 128;    // key rows per tile
-constexpr int BQ2 = 64;    // query rows per step
+constexpr int BT = BWD_KEYS;        // key rows per tile
+constexpr int BQ2 = BWD_QUERIES;    // query rows per step
 constexpr int MAX_CLASSES = 128;
 constexpr int MAX_GROUP = 8;  // layers of one donor group per launch
 constexpr uint32_t HALF_BYTES = 128 * 128;  // [128 rows x 128 B] block
@@ -54,21 +55,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
 constexpr int BWD_THREADS = 448;
 constexpr int BWD_STAGES = 3;        // ring of (Q, dO) 64-row tiles
 constexpr int DQ_STAGE_BYTES = BQ2 * 32 * 4;  // one drain warp's share of a step: [64 queries x 32 columns] fp32
-// A CTA's window of query tiles is sized so that it runs about this many steps (window x streams): long enough
-// to amortise its prologue and its dK / dV reduction, short enough that a wave's footprint stays in L2.
-constexpr int kStepsPerCta = 256;
-constexpr int kMinWindow = 16;
-// A CTA costs about seven steps besides its steps (prologue, dK / dV reduction, gap between two CTAs), and the last CTAs of
-// a launch leave the device idle for some part of their length: with n steps per SM in all, n * 7 / t + 0.3 t is least at
-// t = sqrt(24 n), and there is nothing to gain from fewer CTAs than one for every SM (1.5 n).  Up to kLongestFirst steps per SM the CTAs are dispatched longest first; beyond, in an order that keeps
-// what a wave touches in L2 (2 layers of 4 x 4096 tokens, dh 64: 1970 us in that order, 2010 longest first).
-// Measured (us; always 256 steps, index order -> this): B3 S776 H16/4 dh64, 3 layers 119 -> 80; B4 S632 H8/2 dh128, 8
-// layers 201 -> 107; B1 S2048 H8/8 dh128, 1 layer 50 -> 44; B1 S4096 H32/8 dh128, 1 layer 445 -> 345.  From about 2700
-// steps per SM on the 256 stand.
-constexpr float kTailFactor = 24.f;
-constexpr int kMinSteps = 2;
-constexpr float kLongestFirst = 512.f;
-
 template <int DH>
 struct BwdSmem {
   static constexpr int KV_TILE = BT * DH * 2;
@@ -787,10 +773,8 @@ int make_map_sum(CUtensorMap* m, const void* base, int B, int S, int H, int dh) 
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Orders the CTAs of a launch by their number of steps, longest first, so that the short ones (diagonal key tiles, last
-// windows) fill in at the end; 0 when there are more classes than the parameter block holds.  Only for launches that do
-// not run long enough for the order to cost L2 locality.  Three layers of 3 x 776 tokens, dh 64: 95 us in index
-// order, 79 longest first.
+// Orders the CTAs of a launch by their number of steps, longest first; 0 when there are more classes than the parameter
+// block holds.  Three layers of 3 x 776 tokens, dh 64: 95 us in index order, 79 longest first.
 int longest_first(BwdParams& p, int n_groups, int n_pairs, int n_jt, int n_qt, int G, int causal) {
   struct Class {
     int steps, ctas;
@@ -880,11 +864,9 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b) { return a.n > b.n; });
   const int n_jt = (s->S + BT - 1) / BT, n_qt = (s->S + BQ2 - 1) / BQ2, n_pairs = s->Hkv * s->B;
   const int G = s->Hq / s->Hkv;
-  // steps of one query stream of one (batch, KV head), and the steps one CTA should run
-  long long stream_steps = 0;
-  for (int j = 0; j < n_jt; ++j) stream_steps += causal ? n_qt - j * (BT / BQ2) : n_qt;
-  const float steps_per_sm = float(stream_steps) * n_pairs * s->L * G / sm_count();
-  const int target = std::max(kMinSteps, int(std::min(std::min(float(kStepsPerCta), 1.5f * steps_per_sm), sqrtf(kTailFactor * steps_per_sm))));
+  const BwdSizes sizes{n_jt, n_qt, n_pairs, G, causal != 0, sm_count()};
+  const double steps_per_sm = bwd_steps_per_sm(sizes, s->L);
+  const int target = bwd_target_steps(steps_per_sm);
   size_t gi = 0;
   while (gi < groups.size()) {
     BwdParams p;
@@ -917,16 +899,9 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       rc = make_map_sum(&p.map_dk[ng], dk_sum[g.owner], s->B, s->S, s->Hkv, dh);
       if (rc == KVP_OK) rc = make_map_sum(&p.map_dv[ng], dv_sum[g.owner], s->B, s->S, s->Hkv, dh);
       if (rc != KVP_OK) return rc;
-      // Windows first (a CTA that serves all streams of its window loads K and V once for them), then parts of the streams
-      // where even the smallest window holds more steps than a CTA should run.
-      const int streams = g.n * G;
-      int window = std::max(std::max(1, target / (kStepsPerCta / kMinWindow)), (target + streams - 1) / streams);
-      if (window > 1) window += window & 1;   // whole key tiles of two query tiles: no CTA for half of a diagonal tile
-      p.window[ng] = std::min(n_qt, window);
-      p.parts[ng] = target < kStepsPerCta ? std::max(1, std::min(streams, (streams * p.window[ng] + (p.window[ng] == 1 ? target - 1 : target / 2)) / target)) : 1;
-      // Up to 128 tokens dQ has one term, and two CTAs' terms of dK / dV add up to the same value in either order: such
-      // short sequences keep results that do not differ from run to run.
-      if (n_jt == 1) p.parts[ng] = std::min(p.parts[ng], p.window[ng] < n_qt ? 1 : 2);
+      const BwdCut cut = bwd_cut(sizes, g.n * G, target);
+      p.window[ng] = cut.window;
+      p.parts[ng] = cut.parts;
       p.ctas_per_pair[ng] = 0;
       for (int w = 0; w * p.window[ng] < n_qt; ++w)
         p.ctas_per_pair[ng] += causal ? std::min(n_jt, ((w + 1) * p.window[ng] * BQ2 + BT - 1) / BT) : n_jt;
@@ -954,7 +929,9 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       p.first_slot[i + 1] = slots;
       p.cta_begin[i + 1] = p.cta_begin[ng];
     }
-    p.n_classes = steps_per_sm <= kLongestFirst ? longest_first(p, ng, n_pairs, n_jt, n_qt, G, causal) : 0;
+    p.n_classes = bwd_longest_first(sizes, slots, steps_per_sm, (long long)s->B * s->S * s->Hq, dh)
+                      ? longest_first(p, ng, n_pairs, n_jt, n_qt, G, causal)
+                      : 0;
     p.n_groups = ng;
     p.B = s->B;
     p.S = s->S;
