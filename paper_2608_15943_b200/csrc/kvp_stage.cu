@@ -28,7 +28,10 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 // y = x / sqrt(mean(x^2) + eps) * w.  One CTA of 256 threads takes ROWS rows at a time, held in registers between the
 // reduction and the scaling; the next rows are requested before these are reduced.  Two rows share a block barrier (one,
 // since the partial sums alternate between two buffers) and the weights stay in registers: 8192 x 4096 25.3 -> 22.0 us,
-// 2400 x 4096 10.2 -> 7.8.  Up to eight rows per SM go one to a CTA (347 rows 2.9 -> 2.2).  Bound: HBM.
+// 2400 x 4096 10.2 -> 7.8.  Up to eight rows per SM go one to a CTA (347 rows 2.9 -> 2.2).  Rows of more than 4096 elements
+// leave no registers for that: their weights come from L1 for every row, with four CTAs an SM up to 6144 elements and three
+// up to 8192 (us, weights in registers and two CTAs -> so: 16384 x 5120 64.2 -> 52.4, 8192 x 5120 33.6 -> 27.6, 16384 x 8192
+// 86.7 -> 82.5).  Bound: HBM.
 constexpr int kNormThreads = 256;
 constexpr int kMaxChunks = 4;  // D <= 8192
 template <int CHUNKS, int ROWS>
@@ -47,13 +50,17 @@ __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __re
         if (i < D8 && row + r < T) v[r][c] = x[size_t(row + r) * D8 + i];
       }
   };
+  constexpr bool KEEP = CHUNKS <= 2;          // the weights in registers
   uint4 v[ROWS][CHUNKS], vn[ROWS][CHUNKS], g[CHUNKS];
   load_rows(first, v);
+  auto load_weights = [&]() {
 #pragma unroll
-  for (int c = 0; c < CHUNKS; ++c) {
-    const int i = c * kNormThreads + threadIdx.x;
-    if (i < D8) g[c] = w[i];
-  }
+    for (int c = 0; c < CHUNKS; ++c) {
+      const int i = c * kNormThreads + threadIdx.x;
+      if (i < D8) g[c] = w[i];
+    }
+  };
+  if (KEEP) load_weights();
   int buf = 0;
   for (int row = first; row < T; row += stride, buf ^= 1) {
     if (row + stride < T) load_rows(row + stride, vn);
@@ -72,6 +79,7 @@ __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __re
       for (int s = 16; s > 0; s >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, s);
       if ((threadIdx.x & 31) == 0) part[buf][r][threadIdx.x >> 5] = ss;
     }
+    if (!KEEP) load_weights();
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
@@ -240,12 +248,13 @@ extern "C" int kvp_rmsnorm(int32_t T, int32_t D, const void* x, const void* w, f
   if (D % 8 != 0 || D > 8 * kNormThreads * kMaxChunks || !is_aligned16(x) || !is_aligned16(w) || !is_aligned16(y)) return KVP_ERR_UNSUPPORTED;
   if (T == 0) return KVP_OK;
   const int d8 = D / 8, sms = sm_count();
-  const int chunks = d8 <= kNormThreads ? 1 : d8 <= 2 * kNormThreads ? 2 : kMaxChunks;
+  const int chunks = (d8 + kNormThreads - 1) / kNormThreads;
   const bool two = T > 8 * sms && chunks <= 2;   // wider rows: the registers of two would leave one CTA per SM
   auto* const kernel = chunks == 1 ? (two ? rmsnorm_kernel<1, 2> : rmsnorm_kernel<1, 1>)
                        : chunks == 2 ? (two ? rmsnorm_kernel<2, 2> : rmsnorm_kernel<2, 1>)
+                       : chunks == 3 ? rmsnorm_kernel<3, 1>
                                      : rmsnorm_kernel<kMaxChunks, 1>;
-  const int resident = chunks == 1 ? 5 : chunks == 2 ? 3 : 2;   // CTAs per SM by registers
+  const int resident = chunks == 1 ? 5 : chunks == 2 ? 3 : chunks == 3 ? 4 : 3;   // CTAs per SM by registers
   const int blocks = T <= 8 * sms && chunks <= 2 ? T : std::min(two ? (T + 1) / 2 : T, sms * resident);
   const cudaError_t e = launch_kernel(kernel, blocks, kNormThreads, 0, reinterpret_cast<cudaStream_t>(stream), 1,
       reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), reinterpret_cast<uint4*>(y), T, d8, 1.f / float(D), eps);

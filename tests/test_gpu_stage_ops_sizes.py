@@ -46,3 +46,14 @@ def test_add_and_swiglu_pieces_per_thread(n8):
         op(a, b, y[:n8 * 8])
         bf16_close(y[:n8 * 8], ref)
         assert (y[n8 * 8:] == 7.0).all()
+
+
+@pytest.mark.parametrize("T,D", [(1, 4104), (593, 5120), (1777, 6144), (445, 6152), (1333, 8184)])
+def test_rmsnorm_wide_rows(T, D):
+    """Three and four pieces of a row per thread, one row more than a round of CTAs (four and three per SM)."""
+    from paper_2608_15943_b200 import kvp
+    x, w = synth.normal((T, D), 64, 1, 1.0, "cuda"), synth.normal((D,), 64, 2, 1.0, "cuda")
+    y = torch.full((T + 1, D), 7.0, dtype=torch.bfloat16, device="cuda")
+    kvp.rmsnorm(x, w, 1e-5, y[:T])
+    bf16_close(y[:T], ST.rmsnorm(x.double().cpu().numpy(), w.double().cpu().numpy(), 1e-5))
+    assert (y[T:] == 7.0).all()
