@@ -13,13 +13,14 @@
 // backward pass, and the SMs idle only behind the last tile of the list instead of behind each GEMM's last wave.
 #include <algorithm>
 
+#include "kvp_gemm_choice.h"
 #include "kvp_host.h"
 #include "kvp_sm100.cuh"
 
 namespace kvp {
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int BM = GEMM_BM, BN = 256, BK = GEMM_BK, STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;            // 16 KB
 constexpr int B_BYTES = BN * BK * 2;            // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_cons
 // loads; empty[s] and acc_full[a] exist in both CTAs and receive one MMA-completion arrival each; acc_empty[a]
 // lives in the even CTA and collects the eight epilogue warps of the pair.
 // ------------------------------------------------------------------------------------------------------------
-constexpr int PBM = 256;                          // tile rows per pair
+constexpr int PBM = GEMM_PAIR_BM;                 // tile rows per pair
 constexpr int PHALF = 128;                        // rows of A, and rows of B, per CTA
 constexpr int PSTAGES = 6;
 constexpr int PA_BYTES = PHALF * BK * 2;          // 16 KB
@@ -498,10 +499,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 // tokens 28.7 -> 11.6 (5.2), 4096 x 11008 at 16 30.8 -> 20.6 (13.9), 11008 x 4096 at 16 65.5 -> 20.6 (13.9), 4096 x
 // 4096 at 128 28.9 -> 14.5 (5.5); a launch that does almost nothing takes 6.
 // ------------------------------------------------------------------------------------------------------------
-constexpr int SROWS = 128;                       // rows of B (output columns) per tile: the M of the MMA
-constexpr int SB_BYTES = SROWS * BK * 2;         // 16 KB
+constexpr int SROWS = SPLIT_COLS;                // rows of B (output columns) per tile: the M of the MMA
+constexpr int SB_BYTES = SPLIT_B_BYTES;          // 16 KB
 constexpr int SPLIT_THREADS = 192;
-constexpr int SPLIT_MAX_STAGES = 8;
 // k-blocks of B a CTA asks into L2 before the kernels ahead of it have finished (a token step's 56 kernels: 601 us
 // without, 595 with 8, 613 with 32)
 constexpr int SPLIT_PREFETCH = 8;
@@ -1003,39 +1003,13 @@ int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withh
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
-struct SplitConfig {
-  int nt;       // tokens per tile
-  int split;    // CTAs of a cluster along K
-  int stages;
-};
-
-constexpr int SPLIT_MAX_ROWS = 128;
-constexpr int SPLIT_MAX_PROB = 32;
+constexpr int SPLIT_MAX_PROB = MAX_PROB;
 
 // Both operands K-major, one segment: the shape of every forward projection.
 bool k_major(const GemmProblem* probs, int n) {
   for (int i = 0; i < n; ++i)
     if (probs[i].nseg != 1 || probs[i].a_mn != 0 || probs[i].b_mn != 0) return false;
   return n > 0;
-}
-
-// The smallest split that gives 128 CTAs: enough of them to draw the full memory bandwidth, and no partial more than
-// that needs (at N = K = 4096 and 16 tokens a split of 2 / 4 / 8 measured 12.3 / 11.6 / 10.8 us, at 64 tokens and 4 / 8
-// it measured 12.5 / 14.3).  One CTA per SM takes a ring as deep as fits; more CTAs than SMs share them in twos.
-SplitConfig split_config(const GemmProblem* probs, int n) {
-  int rows = 0, tiles = 0, kblocks = 1 << 30;
-  for (int i = 0; i < n; ++i) {
-    rows = std::max(rows, probs[i].M);
-    tiles += (probs[i].N + SROWS - 1) / SROWS;
-    kblocks = std::min(kblocks, (probs[i].segs[0].K + BK - 1) / BK);
-  }
-  SplitConfig c;
-  c.nt = (rows + 15) / 16 * 16;
-  c.split = 1;
-  while (c.split < 8 && 2 * c.split <= kblocks && tiles * c.split < 128) c.split *= 2;
-  const int ring_bytes = (tiles * c.split <= sm_count() ? 220 : 110) * 1024;
-  c.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SB_BYTES + c.nt * BK * 2));
-  return c;
 }
 
 template <int NP>
@@ -1151,86 +1125,6 @@ int gemm_pair_mode() { return g_pair_mode; }
 
 namespace {
 
-// ------------------------------------------------------------------------------------------------------------
-// Which kernel a forward GEMM of more than 128 rows runs on.  The times (us) of each are estimated from a model with the
-// terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe, memory -- whose
-// constants were fitted to 3400 measurements (11 weight shapes x 24 row counts, weights not in L2).  The choice it makes
-// costs 1.1 % more than the best of all choices on average; without tiles of equal size 5.1 %, CTA pairs always 33 %.
-// Above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand.
-// ------------------------------------------------------------------------------------------------------------
-constexpr int CHOICE_MAX_ROWS = 4096;
-struct Choice {
-  enum Kind { kSingle, kPair, kTall, kSplit } kind = kPair;
-  int nt = 0;         // tokens per tile (tall, split)
-  bool even = false;  // tall: tiles of nt only
-  int split = 1;
-  float us = 1e30f;
-};
-
-// Longest pair of `pairs`, n1 tiles of cost c1 dealt out before n2 of cost c2 <= c1, rounds in alternating direction.
-float makespan(int n1, float c1, int n2, float c2, int pairs) {
-  const int rem = n1 % pairs, a = n1 / pairs;
-  if (rem == 0) return a * c1 + ((n2 + pairs - 1) / pairs) * c2;
-  const int left = n2 - (pairs - rem);            // short tiles that do not fit beside the last round of long ones
-  if (left <= 0) return std::max((a + 1) * c1, a * c1 + (n2 > 0 ? c2 : 0.f));
-  const int rounds = left / pairs, over = left % pairs;
-  return std::max((a + 1) * c1 + (rounds + (over > pairs - rem ? 1 : 0)) * c2, a * c1 + (1 + rounds + (over > 0 ? 1 : 0)) * c2);
-}
-
-Choice choose_forward(const GemmProblem* probs, int n) {
-  int M = 0, kb = 0, cols128 = 0, cols256 = 0;
-  float weights = 0.f, rows = 0.f;   // bytes of B, of A and C
-  for (int i = 0; i < n; ++i) {
-    const GemmProblem& g = probs[i];
-    M = std::max(M, g.M);
-    kb = std::max(kb, (g.segs[0].K + BK - 1) / BK);
-    cols128 += (g.N + 127) / 128;
-    cols256 += (g.N + 255) / 256;
-    weights += 2.f * g.N * g.segs[0].K;
-    rows += 2.f * g.M * g.N + (i == 0 ? 2.f * g.M * g.segs[0].K : 0.f);
-  }
-  const int sms = sm_count(), pairs = sms / 2;
-  Choice best;
-  auto consider = [&](Choice::Kind kind, int nt, bool even, int split, float us) {
-    if (us >= best.us) return;
-    best.kind = kind;
-    best.nt = nt;
-    best.even = even;
-    best.split = split;
-    best.us = us;
-  };
-  auto up = [](int x, int y) { return (x + y - 1) / y; };
-  const float memory = (weights + rows) / 5.5e6f;
-  consider(Choice::kSingle, 0, false, 1, 2.1f + std::max(up(up(M, BM) * cols256, sms) * (kb * 0.403f + 4.2f), memory));
-  consider(Choice::kPair, 0, false, 1, 3.2f + std::max(up(up(M, PBM) * cols256, pairs) * (kb * 0.346f + 4.3f), memory));
-  auto tall_tile = [&](int nt) { return nt == 0 ? 0.f : kb * std::max(0.147f * (1.f + nt / 256.f), 0.00136f * nt) + 2.6f; };
-  // tiles of equal size along the tokens
-  const int fewest = up(M, 256);
-  for (int k = fewest; k < fewest + 4 + fewest / 3; ++k) {
-    const int nt = up(up(M, k), 16) * 16;
-    if (k > fewest && nt < 80) break;
-    consider(Choice::kTall, nt, true, 1, 3.5f + std::max(makespan(up(M, nt) * cols256, tall_tile(nt), 0, 0.f, pairs), memory));
-  }
-  // whole tiles, then those of the remainder: weights of which little stays in L2 in between are read twice
-  const float again = weights > 60e6f ? (weights - 60e6f) / 5.5e6f : 0.f;
-  for (int nt = 128; nt <= 256; nt += 32) {
-    const int whole = M / nt, rest = up(M - whole * nt, 16) * 16;
-    if (whole == 0 || rest == 0) continue;
-    consider(Choice::kTall, nt, false, 1,
-             1.04f * (3.5f + std::max(makespan(whole * cols256, tall_tile(nt), cols256, tall_tile(rest), pairs), memory + again)));
-  }
-  // split kernel: one CTA per SM; clusters of four do not fill every GPC
-  for (int split = 1; split <= 4 && 2 * split <= kb; split *= 2) {
-    const int most = (split == 4 ? sms - 16 : sms) / (split * cols128);   // token tiles that fit
-    if (most < 1) break;
-    const int nt = std::max(48, up(up(M, most), 16) * 16);
-    if (nt > 256) continue;
-    consider(Choice::kSplit, nt, false, split, 4.f + std::max(float(kb) / split * 0.109f * (1.f + nt / 128.f), (weights + rows) / 7.8e6f) +
-                                                   0.031f * nt + (split > 1 ? 0.6f : 0.f));
-  }
-  return best;
-}
-
 template <typename F1, typename F4, typename F32>
 int by_count(int n, F1 one, F4 four, F32 many) { return n == 1 ? one() : n <= 4 ? four() : many(); }
 
@@ -1263,11 +1157,16 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
 int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
   int rows = 0;
   for (int i = 0; i < n; ++i) rows = std::max(rows, probs[i].M);
+  GemmSize sizes[MAX_PROB];
+  auto sizes_of = [&](const GemmProblem* g, int cnt) {
+    for (int i = 0; i < cnt; ++i) sizes[i] = GemmSize{g[i].M, g[i].N, g[i].segs[0].K};
+    return sizes;
+  };
   if (rows <= SPLIT_MAX_ROWS) {
     for (int begin = 0; begin < n; begin += SPLIT_MAX_PROB) {
       const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
       const GemmProblem* g = probs + begin;
-      const SplitConfig cfg = split_config(g, cnt);
+      const SplitConfig cfg = split_config(sizes_of(g, cnt), cnt, sm_count());
       const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
                               [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream); });
       if (rc != KVP_OK) return rc;
@@ -1278,7 +1177,7 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
   for (int begin = 0; begin < n; begin += MAX_PROB) {
     const int cnt = std::min(MAX_PROB, n - begin);
     const GemmProblem* g = probs + begin;
-    const Choice c = choose_forward(g, cnt);
+    const Choice c = choose_forward(sizes_of(g, cnt), cnt, sm_count());
     int rc;
     if (c.kind == Choice::kTall) {
       rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, c.even, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, c.even, stream); },
