@@ -672,18 +672,17 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
 //
 // Each pair of CTAs owns 256 columns of C (rows of B: 128 a CTA, the M = 256 of the pair's MMA) and a tile of tokens (the
 // N, split between the CTAs' loads).  256 x 256 tiles of gemm_pair_kernel pad 347 tokens to 512; here the tokens are cut
-// into tiles of up to 256, either all of the same size (a multiple of 16) or whole ones and one tile of the remainder (a
-// multiple of 16; of 128 where A is MN-major: its TMA boxes hold 64 rows and each CTA loads half of the tile).  Tiles of
-// one size are walked column by column, so that the columns' weights come from memory once; whole tiles go before all
-// remainders, pairs taking turns in alternating direction, so the short tiles fill the pairs that have no second long
-// one, but weights beyond L2 are read again.  A lane of the epilogue holds a column, so a warp stores rows of 64
+// into tiles of up to 256, in steps of 32.  Forward they are all of one size, walked column by column, so that the columns'
+// weights come from memory once.  Gradients have whole tiles and one of the remainder (in steps of 128 where A is MN-major:
+// its TMA boxes hold 64 rows and each CTA loads half of the tile); the whole tiles go before all remainders, pairs taking
+// turns in alternating direction, so that the short ones fill the pairs that have no second long one.  A lane of the
+// epilogue holds a column, so a warp stores rows of 64
 // consecutive bytes, two at a time (128 in fp32), where a lane of gemm_pair_kernel's holds a row.  Roles, segments and
 // barriers are those of gemm_pair_kernel, the ring has as many stages as tiles of the launch's size leave room for;
 // results are bit-identical to its (same products, same order along K).
 // Bound: the 120 GB/s that an SM draws from L2 (tiles of up to 192 tokens), then the tensor pipe.  Measured (us, weights
-// not in L2; gemm_pair_kernel -> whole tiles and remainder -> tiles of one size, tokens x columns x K): 347 x 32000 x 4096
-// 124 -> 98 -> 70, 512 x 11008 x 4096 52 -> 46 -> 40, 776 x 4096 x 4096 x 3 problems 87 -> 75 -> 71, 1500 x 4096 x 11008
-// 142 -> 113 -> 100, 2328 x 4096 x 4096 78 -> 69 -> 61.  A ring of 7 to 9 stages instead of 6 gave 2 to 8 %.  With a
+// not in L2; gemm_pair_kernel -> this, tokens x columns x K): 347 x 32000 x 4096 102 -> 82, 512 x 11008 x 4096 51 -> 40, 1500 x
+// 4096 x 11008 155 -> 121, 2328 x 4096 x 4096 90 -> 70.  A ring of 7 to 9 stages instead of 6 gave 2 to 8 %.  With a
 // short K the stores bound it, and four epilogue warps leave them waiting for one another: sixteen instead of four took
 // fp32 results of 2328 x 1024 x 1024, four problems, from 48 to 24 us and those of 776 tokens, six problems, from 26 to
 // 16 (bf16: 13.8 -> 14.6; the same change slowed gemm_kernel and gemm_pair_kernel by 2 to 10 %).
@@ -1079,7 +1078,7 @@ int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t
   for (int part = 0; part < 2; ++part)
     for (int i = 0; i < n; ++i) {
       const GemmProblem& g = probs[i];
-      const int whole = even ? (g.M + nt - 1) / nt : g.M / nt, rest = std::max(0, g.M - whole * nt), unit = g.a_mn ? 128 : 16;
+      const int whole = even ? (g.M + nt - 1) / nt : g.M / nt, rest = std::max(0, g.M - whole * nt), unit = g.a_mn ? 128 : TALL_UNIT;
       TallList l{};
       l.prob = i;
       l.nt = part == 0 ? nt : (rest + unit - 1) / unit * unit;
@@ -1180,8 +1179,8 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
     const Choice c = choose_forward(sizes_of(g, cnt), cnt, sm_count());
     int rc;
     if (c.kind == Choice::kTall) {
-      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, c.even, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, c.even, stream); },
-                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, c.even, stream); });
+      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, true, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, true, stream); },
+                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, true, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
       rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },

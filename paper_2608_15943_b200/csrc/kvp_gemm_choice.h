@@ -14,6 +14,8 @@ constexpr int GEMM_BK = 64;                      // depth of a k-block
 constexpr int GEMM_BM = 128, GEMM_PAIR_BM = 256; // rows of a tile of the single-CTA and the CTA-pair kernel
 constexpr int SPLIT_COLS = 128;                  // columns of a tile of the split kernel: the M of its MMA
 constexpr int SPLIT_MAX_STAGES = 8;
+// Tokens of a tile of the column-owning pairs: the N of an MMA with M = 256 on a CTA pair goes in steps of 32.
+constexpr int TALL_UNIT = 32;
 constexpr int SPLIT_B_BYTES = SPLIT_COLS * GEMM_BK * 2;
 constexpr int SPLIT_MAX_ROWS = 128;       // up to here always the split kernel
 
@@ -45,28 +47,19 @@ inline SplitConfig split_config(const GemmSize* probs, int n, int sms) {
 // ------------------------------------------------------------------------------------------------------------
 // Which kernel a forward GEMM of more than 128 rows runs on.  The times (us) of each are estimated from a model with the
 // terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe, memory -- whose
-// constants were fitted to 3400 measurements (11 weight shapes x 24 row counts, weights not in L2).  The choice it makes
-// costs 1.1 % more than the best of all choices on average; without tiles of equal size 5.1 %, CTA pairs always 33 %.
-// Above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand.
+// constants were fitted to 3400 measurements (11 weight shapes x 28 row counts, weights not in L2).  The choice it makes
+// costs 0.7 % more than the best of all choices on average, CTA pairs always 50 %.  From PAIR_ROUNDS rounds of pair tiles on
+// and above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand: 3000 rows x 32000 x 4096 508
+// us on them, 597 in tiles of one size.
 // ------------------------------------------------------------------------------------------------------------
+constexpr int PAIR_ROUNDS = 16;
 constexpr int CHOICE_MAX_ROWS = 4096;
 struct Choice {
   enum Kind { kSingle, kPair, kTall, kSplit } kind = kPair;
   int nt = 0;         // tokens per tile (tall, split)
-  bool even = false;  // tall: tiles of nt only
   int split = 1;
   float us = 1e30f;
 };
-
-// Longest pair of `pairs`, n1 tiles of cost c1 dealt out before n2 of cost c2 <= c1, rounds in alternating direction.
-inline float makespan(int n1, float c1, int n2, float c2, int pairs) {
-  const int rem = n1 % pairs, a = n1 / pairs;
-  if (rem == 0) return a * c1 + ((n2 + pairs - 1) / pairs) * c2;
-  const int left = n2 - (pairs - rem);            // short tiles that do not fit beside the last round of long ones
-  if (left <= 0) return std::max((a + 1) * c1, a * c1 + (n2 > 0 ? c2 : 0.f));
-  const int rounds = left / pairs, over = left % pairs;
-  return std::max((a + 1) * c1 + (rounds + (over > pairs - rem ? 1 : 0)) * c2, a * c1 + (1 + rounds + (over > 0 ? 1 : 0)) * c2);
-}
 
 inline Choice choose_forward(const GemmSize* probs, int n, int sms) {
   int M = 0, kb = 0, shallowest = 1 << 30, cols128 = 0, cols256 = 0;
@@ -83,42 +76,34 @@ inline Choice choose_forward(const GemmSize* probs, int n, int sms) {
   }
   const int pairs = sms / 2;
   Choice best;
-  auto consider = [&](Choice::Kind kind, int nt, bool even, int split, float us) {
+  if ((M + GEMM_PAIR_BM - 1) / GEMM_PAIR_BM * cols256 > PAIR_ROUNDS * pairs) return best;
+  auto consider = [&](Choice::Kind kind, int nt, int split, float us) {
     if (us >= best.us) return;
     best.kind = kind;
     best.nt = nt;
-    best.even = even;
     best.split = split;
     best.us = us;
   };
   auto up = [](int x, int y) { return (x + y - 1) / y; };
-  const float memory = (weights + rows) / 5.5e6f;
-  consider(Choice::kSingle, 0, false, 1, 2.1f + std::max(up(up(M, GEMM_BM) * cols256, sms) * (kb * 0.403f + 4.2f), memory));
-  consider(Choice::kPair, 0, false, 1, 3.2f + std::max(up(up(M, GEMM_PAIR_BM) * cols256, pairs) * (kb * 0.346f + 4.3f), memory));
-  auto tall_tile = [&](int nt) { return nt == 0 ? 0.f : kb * std::max(0.147f * (1.f + nt / 256.f), 0.00136f * nt) + 2.6f; };
-  // tiles of equal size along the tokens
+  const float memory = (weights + rows) / 5.95e6f;
+  consider(Choice::kSingle, 0, 1, 2.3f + std::max(up(up(M, GEMM_BM) * cols256, sms) * (kb * 0.361f + 4.3f), memory));
+  consider(Choice::kPair, 0, 1, 3.2f + std::max(up(up(M, GEMM_PAIR_BM) * cols256, pairs) * (kb * 0.338f + 4.3f), memory));
+  // column-owning pairs, tiles of equal size along the tokens
   const int fewest = up(M, 256);
   for (int k = fewest; k < fewest + 4 + fewest / 3; ++k) {
-    const int nt = up(up(M, k), 16) * 16;
+    const int nt = up(up(M, k), TALL_UNIT) * TALL_UNIT;
     if (k > fewest && nt < 80) break;
-    consider(Choice::kTall, nt, true, 1, 3.5f + std::max(makespan(up(M, nt) * cols256, tall_tile(nt), 0, 0.f, pairs), memory));
-  }
-  // whole tiles, then those of the remainder: weights of which little stays in L2 in between are read twice
-  const float again = weights > 60e6f ? (weights - 60e6f) / 5.5e6f : 0.f;
-  for (int nt = 128; nt <= 256; nt += 32) {
-    const int whole = M / nt, rest = up(M - whole * nt, 16) * 16;
-    if (whole == 0 || rest == 0) continue;
-    consider(Choice::kTall, nt, false, 1,
-             1.04f * (3.5f + std::max(makespan(whole * cols256, tall_tile(nt), cols256, tall_tile(rest), pairs), memory + again)));
+    const float tile = kb * std::max(0.157f * (1.f + nt / 256.f), 0.00139f * nt) + 2.5f;
+    consider(Choice::kTall, nt, 1, 3.7f + std::max(up(up(M, nt) * cols256, pairs) * tile, memory));
   }
   // split kernel: one CTA per SM; clusters of four do not fill every GPC; every CTA has k-blocks of every problem
   for (int split = 1; split <= 4 && 2 * split <= shallowest; split *= 2) {
     const int most = (split == 4 ? sms - 16 : sms) / (split * cols128);   // token tiles that fit
     if (most < 1) break;
     const int nt = std::max(48, up(up(M, most), 16) * 16);
-    if (nt > 256) continue;
-    consider(Choice::kSplit, nt, false, split, 4.f + std::max(float(kb) / split * 0.109f * (1.f + nt / 128.f), (weights + rows) / 7.8e6f) +
-                                                   0.031f * nt + (split > 1 ? 0.6f : 0.f));
+    if (nt > 224) continue;   // (longer tiles draw more from L2 than the model says: 900 x 4096 x 11008 76 us for 65)
+    consider(Choice::kSplit, nt, split, 4.7f + std::max(float(kb) / split * 0.11f * (1.f + nt / 128.f), (weights + rows) / 9.6e6f) +
+                                                   0.027f * nt + (split > 1 ? 0.75f : 0.f));
   }
   return best;
 }

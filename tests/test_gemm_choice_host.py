@@ -12,7 +12,7 @@ SINGLE, PAIR, TALL, SPLIT = range(4)
 
 
 def compiled(folder):
-    """choose(list of (M, N, K)) -> (kernel, tokens per tile, tiles of that size only, K split)."""
+    """choose(list of (M, N, K)) -> (kernel, tokens per tile, K split)."""
     (folder / "c.cpp").write_text("""#include "kvp_gemm_choice.h"
 using namespace kvp;
 extern "C" void choose(const int* mnk, int n, int* out) {
@@ -24,12 +24,12 @@ extern "C" void choose(const int* mnk, int n, int* out) {
   }
   if (rows <= SPLIT_MAX_ROWS) {
     const SplitConfig c = split_config(g, n, 148);
-    out[0] = Choice::kSplit, out[1] = c.nt, out[2] = 1, out[3] = c.split;
+    out[0] = Choice::kSplit, out[1] = c.nt, out[2] = c.split;
   } else if (rows > CHOICE_MAX_ROWS) {
-    out[0] = Choice::kPair, out[1] = 0, out[2] = 0, out[3] = 1;
+    out[0] = Choice::kPair, out[1] = 0, out[2] = 1;
   } else {
     const Choice c = choose_forward(g, n, 148);
-    out[0] = c.kind, out[1] = c.nt, out[2] = c.even, out[3] = c.split;
+    out[0] = c.kind, out[1] = c.nt, out[2] = c.split;
   }
 }
 """)
@@ -37,9 +37,9 @@ extern "C" void choose(const int* mnk, int n, int* out) {
     lib = C.CDLL(str(folder / "c.so"))
 
     def choose(problems):
-        out, flat = (C.c_int * 4)(), [x for p in problems for x in p]
+        out, flat = (C.c_int * 3)(), [x for p in problems for x in p]
         lib.choose((C.c_int * len(flat))(*flat), len(problems), out)
-        return out[0], out[1], bool(out[2]), out[3]
+        return tuple(out)
     return choose
 
 
@@ -59,7 +59,20 @@ def test_every_cta_of_a_split_has_k_blocks(choose):
     """Problems of different depth in one launch: the shallowest bounds the split, an empty range would add whatever the
     accumulator held."""
     for problems in some_lists(1):
-        kind, nt, _, split = choose(problems)
+        kind, nt, split = choose(problems)
         if kind == SPLIT:
             assert split <= min((k + 63) // 64 for _, _, k in problems), problems
             assert 16 <= nt <= 256 and nt % 16 == 0
+
+
+def test_pair_tiles_go_in_steps_of_32_tokens(choose):
+    """The N of an MMA of M = 256 on a CTA pair; the kernel's remainders use the same unit."""
+    seen = 0
+    for problems in some_lists(2):
+        kind, nt, _ = choose(problems)
+        if kind == TALL:
+            seen += 1
+            assert 32 <= nt <= 256 and nt % 32 == 0, problems
+    assert seen > 300
+    source = open(os.path.join(CSRC, "kvp_gemm.cu")).read()
+    assert "unit = g.a_mn ? 128 : TALL_UNIT" in source
