@@ -97,3 +97,27 @@ def test_gradient_gemms(L, own, S, D, Hq, Hkv):
         K = sum(d.shape[1] for _, d in parts)
         bound = K * 2.0 ** -24 * sum(d.double().abs() @ w[n][l].double().abs() for n, d in parts)
         assert ((dx[l].double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all(), l
+
+
+@pytest.fixture(scope="module")
+def choose(tmp_path_factory):
+    from test_gemm_choice_host import compiled
+    return compiled(tmp_path_factory.mktemp("choice"))
+
+
+# (kernel, tokens per tile, K split) that a launch is to take: a change of the rules that moves a case off the edge it is
+# here for fails instead of passing somewhere else
+@pytest.mark.parametrize("M,N,K,kernel", [
+    (193, 264, 8, ("tall", 96, 1)), (207, 264, 8, ("tall", 96, 1)), (209, 1032, 8, ("tall", 96, 1)),    # last tiles of 1, 15, 17 tokens
+    (1345, 9688, 136, ("tall", 224, 1)), (1360, 9688, 136, ("tall", 224, 1)), (1375, 9688, 136, ("tall", 224, 1)),   # 1, 16, 31; 38 columns of 7 tiles
+    (961, 5512, 200, ("tall", 192, 1)), (1280, 9688, 136, ("tall", 256, 1)),                             # the largest tile, no remainder
+    (145, 264, 2056, ("split", 48, 4)), (159, 520, 1032, ("split", 48, 4)), (401, 520, 1032, ("split", 48, 2)), (192, 1032, 520, ("split", 48, 1)),
+    (279, 9688, 8, ("single", 0, 1)), (290, 9608, 16, ("single", 0, 1)),                                # single-CTA tiles, last of 23 and 34 rows
+    (3897, 19016, 8, ("pair", 0, 1)),                                                                   # CTA pairs, last rows 57, last columns 72
+    (4097, 520, 72, ("pair", 0, 1)), (4224, 264, 136, ("pair", 0, 1)),                                  # the first row counts without a choice
+])
+def test_each_forward_kernel_at_its_edges(choose, M, N, K, kernel):
+    from paper_2608_15943_b200 import kvp
+    kind, nt, split = choose([(M, N, K)])
+    assert (("single", "pair", "tall", "split")[kind], nt, split) == kernel
+    test_few_rows(M, N, K)
