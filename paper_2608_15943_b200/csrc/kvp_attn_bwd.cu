@@ -649,7 +649,7 @@ template <int DH>
 __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   constexpr int TPR = DH / 8;  // threads per query row
   grid_dep_wait();
-  const float* __restrict__ acc = p.dq_acc[blockIdx.y];
+  const float* acc = p.dq_acc[blockIdx.y];
   const int S = p.S, Hq = p.Hq;
   const float scale = p.scale;
   const int n_qt = (S + BQ2 - 1) / BQ2;
@@ -706,9 +706,9 @@ __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
     clear(p.dk_sum[slot], p.kv_v4);
     clear(p.dv_sum[slot], p.kv_v4);
   }
-  const __nv_bfloat16* __restrict__ o = p.o[slot];
-  const __nv_bfloat16* __restrict__ d_o = p.d_o[slot];
-  float* __restrict__ delta = p.delta[slot];
+  const __nv_bfloat16* o = p.o[slot];
+  const __nv_bfloat16* d_o = p.d_o[slot];
+  float* delta = p.delta[slot];
   const int S = p.S, Hq = p.Hq;
   const size_t rows = size_t(p.B) * S * Hq;
   const int lane = threadIdx.x & 31;

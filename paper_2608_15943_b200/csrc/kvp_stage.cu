@@ -35,8 +35,8 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 constexpr int kNormThreads = 256;
 constexpr int kMaxChunks = 4;  // D <= 8192
 template <int CHUNKS, int ROWS>
-__global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
-                                                               uint4* __restrict__ y, int T, int D8, float inv_d, float eps) {
+__global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* x, const uint4* w,
+                                                               uint4* y, int T, int D8, float inv_d, float eps) {
   __shared__ float part[2][ROWS][kNormThreads / 32];
   grid_dep_wait();
   const int first = blockIdx.x * ROWS, stride = gridDim.x * ROWS;
@@ -122,7 +122,7 @@ constexpr uint32_t kRopeUnroll = 4;
 struct RopeFreq {
   float2 f[kMaxRopePairs];
 };
-__global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, uint32_t H, uint32_t dh8, uint32_t group,
+__global__ void rope_kernel(uint4* x, uint32_t n_work, uint32_t S, uint32_t H, uint32_t dh8, uint32_t group,
                             int pos0, const __grid_constant__ RopeFreq fr) {
   // lanes of a warp need different table entries: shared memory serves them in one pass, the constant bank
   // that holds kernel parameters would replay once per distinct address
@@ -187,7 +187,7 @@ __global__ void rope_kernel(uint4* __restrict__ x, uint32_t n_work, uint32_t S, 
 // set-up), so that it takes the loop where a thread has a single piece.  Both stay within 32 registers: with 48, five
 // blocks an SM instead of eight, swiglu of 8192 x 4096 took 37.2 instead of 33.4.
 template <bool TWO, typename F>
-__device__ __forceinline__ void zip8(const uint4* __restrict__ a, const uint4* __restrict__ b, uint4* __restrict__ out, size_t n8, F f) {
+__device__ __forceinline__ void zip8(const uint4* a, const uint4* b, uint4* out, size_t n8, F f) {
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
   auto piece = [&](const uint4& p, const uint4& q) {
@@ -222,14 +222,14 @@ __device__ __forceinline__ void zip8(const uint4* __restrict__ a, const uint4* _
 constexpr int kStreamThreads = 256, kStreamResident = 8;   // CTAs per SM
 template <bool TWO>
 __global__ void __launch_bounds__(kStreamThreads, kStreamResident)
-    swiglu_kernel(const uint4* __restrict__ gate, const uint4* __restrict__ up, uint4* __restrict__ out, size_t n8) {
+    swiglu_kernel(const uint4* gate, const uint4* up, uint4* out, size_t n8) {
   grid_dep_wait();
   zip8<TWO>(gate, up, out, n8, [](float g, float u) { return g * __frcp_rn(1.f + __expf(-g)) * u; });
 }
 
 template <bool TWO>
 __global__ void __launch_bounds__(kStreamThreads, kStreamResident)
-    add_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b, uint4* __restrict__ out, size_t n8) {
+    add_kernel(const uint4* a, const uint4* b, uint4* out, size_t n8) {
   grid_dep_wait();
   zip8<TWO>(a, b, out, n8, [](float x, float y) { return x + y; });
 }

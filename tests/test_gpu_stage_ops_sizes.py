@@ -57,3 +57,29 @@ def test_rmsnorm_wide_rows(T, D):
     kvp.rmsnorm(x, w, 1e-5, y[:T])
     bf16_close(y[:T], ST.rmsnorm(x.double().cpu().numpy(), w.double().cpu().numpy(), 1e-5))
     assert (y[T:] == 7.0).all()
+
+
+@pytest.mark.parametrize("T,D", [(5, 256), (347, 4096), (2400, 1024)])
+def test_back_to_back_calls_see_what_the_one_before_wrote(T, D):
+    """GEMM, SwiGLU in place, add in place, RMSNorm in place, again and again: the same bits as with a synchronisation after
+    every call, although each kernel comes up while the one ahead of it still runs."""
+    from paper_2608_15943_b200 import kvp
+    w = [synth.normal((D, D), 65, i, 2.0 * D ** -0.5, "cuda") for i in range(2)]
+    n = 1.0 + synth.normal((D,), 65, 2, 0.1, "cuda")
+    x0 = synth.normal((T, D), 65, 3, 1.0, "cuda")
+
+    def chain(wait):
+        x, gate, up = x0.clone(), torch.empty_like(x0), torch.empty_like(x0)
+        for _ in range(6):
+            for call in (lambda: kvp.gemm(x, w[0], gate), lambda: kvp.gemm(x, w[1], up), lambda: kvp.swiglu(gate, up, gate),
+                         lambda: kvp.add(gate, x, x), lambda: kvp.rmsnorm(x, n, 1e-5, x)):
+                call()
+                if wait:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return x, gate
+    want = chain(True)
+    assert torch.isfinite(want[0]).all()
+    for _ in range(5):
+        for got, ref in zip(chain(False), want):
+            assert torch.equal(got, ref)

@@ -1,4 +1,5 @@
-"""What the build says of the stage operators' kernels."""
+"""What the sources and the build say of the kernels."""
+import glob
 import os
 import re
 
@@ -22,3 +23,12 @@ def registers():
 def test_rmsnorm_ctas_fit_an_sm(registers, pieces, rows, ctas):
     """As many CTAs of 256 threads as the launch counts on; rows of more than 4096 elements need four and three of them."""
     assert ctas * 256 * registers[(pieces, rows)] <= 65536
+
+
+def test_no_input_is_taken_for_constant():
+    """Kernels come up while the ones ahead still write their inputs (programmatic dependent launch), and the element-wise
+    operators may work in place: neither allows a pointer that promises nobody else writes, nor a read-only load."""
+    from paper_2608_15943_b200 import build
+    for path in glob.glob(os.path.join(build.CSRC, "*.cu*")):
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        assert not re.search(r"__restrict__|__ldg\b|ld\.global\.nc", code), path
