@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "kvp_host.h"
+#include "kvp_rope_freq.h"
 #include "kvp_sm100.cuh"
 
 namespace kvp {
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint4* x, c
 // not: 347 tokens x 32 heads went to 22 blocks, each thread eight rounds of loads and stores one after the other (5.2 ->
 // 2.3 us; 16 tokens 4.9 -> 1.7, 8192 tokens 25.3 -> 22.6).  The rotations need no memory and are formed before the kernel
 // waits for the one ahead of it.
-// The frequencies arrive as float pairs hi + lo rounded from the host's double values; the angle pos * f is formed as an
+// The frequencies arrive as float pairs hi + lo (kvp_rope_freq.h); the angle pos * f is formed as an
 // exact product p = pos * hi plus its rounding error and the lo term, sine and cosine of the float p are taken after an
 // exact range reduction, and the small remainder is applied as a second-order correction.
 constexpr int kMaxRopePairs = 128;
@@ -267,14 +268,8 @@ extern "C" int kvp_rope(int32_t B, int32_t S, int32_t H, int32_t dh, float theta
   const size_t n8 = size_t(B) * S * H * (dh / 8);
   if (n8 == 0) return KVP_OK;
   RopeFreq fr;
-  // theta^(-2i/dh) by repeated multiplication in double: at most 128 roundings of 2^-53, below the 2^-48 that the hi + lo
-  // float pairs keep; one pow instead of one per pair (3 us of a 13 us call)
-  const double ratio = pow(double(theta), -2.0 / dh);
-  double f = 1.0;
-  for (int i = 0; i < dh / 2; ++i, f *= ratio) {
-    fr.f[i].x = float(f);
-    fr.f[i].y = float(f - double(fr.f[i].x));
-  }
+  static_assert(sizeof(float2) == 2 * sizeof(float), "hi and lo of a pair lie side by side");
+  rope_frequencies(double(theta), dh, &fr.f[0].x, &fr.f[0].y, 2);
   // 16-byte groups are indexed with 32 bits: larger tensors go in slices of whole sequences
   const size_t per_seq = size_t(S) * H * (dh / 8);
   if (per_seq >= (size_t(1) << 31)) return KVP_ERR_UNSUPPORTED;

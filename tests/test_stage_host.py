@@ -2,6 +2,9 @@
 import glob
 import os
 import re
+import subprocess
+from decimal import Decimal, getcontext
+import ctypes as C
 
 import pytest
 
@@ -32,3 +35,21 @@ def test_no_input_is_taken_for_constant():
     for path in glob.glob(os.path.join(build.CSRC, "*.cu*")):
         code = re.sub(r"//[^\n]*", "", open(path).read())
         assert not re.search(r"__restrict__|__ldg\b|ld\.global\.nc", code), path
+
+
+@pytest.mark.parametrize("dh", [8, 64, 128, 192, 256])
+@pytest.mark.parametrize("theta", [1.5, 10000.0, 500000.0, 1e6])
+def test_rope_frequencies_fill_their_float_pairs(tmp_path, dh, theta):
+    """hi + lo against theta^(-2i/dh) in 60 digits: what two floats of 24 bits hold, and no more error than that."""
+    from paper_2608_15943_b200 import build
+    src = tmp_path / "f.cpp"
+    src.write_text('#include "kvp_rope_freq.h"\n'
+                   'extern "C" void freqs(double t, int dh, float* out) { kvp::rope_frequencies(t, dh, out, out + 1, 2); }\n')
+    subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I" + build.CSRC, str(src), "-o", str(tmp_path / "f.so")], check=True)
+    out = (C.c_float * dh)()
+    C.CDLL(str(tmp_path / "f.so")).freqs(C.c_double(theta), dh, out)
+    getcontext().prec = 60
+    for i in range(dh // 2):
+        want = (Decimal(theta).ln() * Decimal(-2 * i) / Decimal(dh)).exp()
+        got = Decimal(out[2 * i]) + Decimal(out[2 * i + 1])
+        assert abs(got / want - 1) <= Decimal(2) ** -48, i
