@@ -2,7 +2,7 @@
 packing: g++ against torch's headers -> _pack.so.
 
 Run as ``python -m paper_2608_15943_b200.build`` or call ``build()``.  Objects are rebuilt only
-when a source or header is newer than the object.
+when a source or header is newer than the object; _pack.so also when it was built for another Python or torch.
 """
 from __future__ import annotations
 
@@ -46,11 +46,20 @@ def _compile(src: str, force: bool) -> str:
     return obj
 
 
+def _pack_key(torch_dir: str) -> str:
+    """What _pack.so is built against: its layout of torch's and Python's objects holds for these alone."""
+    with open(os.path.join(torch_dir, "version.py")) as fh:
+        return f"{sys.version}\n{torch_dir}\n{fh.read()}"
+
+
 def _build_pack(force: bool) -> None:
     src = os.path.join(CSRC, "kvp_pack.cpp")
-    if not force and os.path.exists(PACK) and os.path.getmtime(PACK) > os.path.getmtime(src):
-        return
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    key, key_file = _pack_key(torch_dir), os.path.join(OBJ, "_pack.key")
+    if not force and os.path.exists(PACK) and os.path.getmtime(PACK) > os.path.getmtime(src) and os.path.exists(key_file):
+        with open(key_file) as fh:
+            if fh.read() == key:
+                return
     inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-w", "-I" + sysconfig.get_paths()["include"],
            "-I" + inc, "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), src, "-o", PACK, "-L" + lib,
@@ -58,6 +67,8 @@ def _build_pack(force: bool) -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"{cmd[0]} failed for {src}:\n{r.stdout}\n{r.stderr}")
+    with open(key_file, "w") as fh:
+        fh.write(key)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

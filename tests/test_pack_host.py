@@ -32,3 +32,30 @@ def test_refused():
     for bad, err in (([1.5], AttributeError), (None, TypeError)):
         with pytest.raises(err):
             kvp._ptr_array(bad)
+
+
+def test_packing_is_built_anew_for_another_torch(monkeypatch, tmp_path):
+    """_pack.so is laid out for one Python and one torch: a build for another is not kept, whatever its time."""
+    import os
+    from paper_2608_15943_b200 import build
+    os.makedirs(tmp_path / "obj")
+    monkeypatch.setattr(build, "OBJ", str(tmp_path / "obj"))
+    monkeypatch.setattr(build, "PACK", str(tmp_path / "_pack.so"))
+    runs = []
+
+    class Done:
+        returncode, stdout, stderr = 0, "", ""
+
+    def run(cmd, **kw):
+        runs.append(cmd)
+        open(build.PACK, "w").close()
+        return Done()
+    monkeypatch.setattr(build.subprocess, "run", run)
+    build._build_pack(False)
+    build._build_pack(False)
+    assert len(runs) == 1
+    key = build._pack_key
+    monkeypatch.setattr(build, "_pack_key", lambda d: key(d) + "another")
+    build._build_pack(False)
+    build._build_pack(False)
+    assert len(runs) == 2
