@@ -86,8 +86,8 @@ unsigned long long kvp_launch_count(void);
 int kvp_set_timing_events(int kernel, void** starts, void** stops, int n);
 int kvp_timing_events_used(int kernel);
 /* Measurement switch of the GEMM's tile shape.  1 (the default): forward GEMMs (K-major operands) run on CTA pairs
- * (256 x 256 tiles, one per pair of SMs), or up to 4096 rows on whichever of the library's kernels an estimate of their
- * times prefers; the gradient GEMMs on pairs that own 256 columns, large launches (more than 0.5 TFLOP) on single-CTA
+ * (256 x 256 tiles, one per pair of SMs), or up to 4096 rows and sixteen rounds of such tiles on whichever of the
+ * library's kernels an estimate of their times prefers; the gradient GEMMs on pairs that own 256 columns, large launches (more than 0.5 TFLOP) on single-CTA
  * 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: 256 x 256 tiles on CTA pairs for every launch whose problems all
  * have more than 128 rows.  (K-major problems of at most 128 rows have a kernel of their own in every mode.)  The tile
  * kernels sum the same products in the same order along K in every mode; up to 4096 rows K may be split over a cluster of
@@ -243,7 +243,10 @@ int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal, float sca
 /* Building block of the projections: C[M,N] = A B, bf16 inputs, fp32 accumulate.
  * a_mn == 0: A stored [M,K] row-major, else stored [K,M].  b_mn == 0: B stored [N,K] row-major
  * (C = A B^T in storage terms), else stored [K,N].  out_f32: C fp32, else bf16.  Leading dimensions
- * in elements, multiples of 8; K a multiple of 8.  The paper's 2mkn matrix-multiplication rule. */
+ * in elements, multiples of 8; K a multiple of 8.  The paper's 2mkn matrix-multiplication rule.
+ * The kernel, and whether K is summed in parts, follow from the sizes of the whole launch (K-major operands, up to 4096
+ * rows): a row's last bits can differ between calls with different numbers of rows, never between equal calls.  The
+ * projections (kvp_proj_fwd, kvp_out_proj_fwd) run on the same kernels. */
 int kvp_gemm(int M, int N, int K, const void* a, int64_t lda, int a_mn, const void* b, int64_t ldb, int b_mn,
              void* c, int64_t ldc, int out_f32, kvp_stream_t stream);
 
@@ -295,7 +298,10 @@ int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, const void*
  * the group's query rows fit one pass: min(4, 16 / (Hq/Hkv)) layers; a larger group takes one pass
  * per that many layers.
  * q[l], o[l]: [B,Hq,dh] bf16; lse[l]: [B,Hq] fp32.  lengths outside [1, max_pages*page_size] are
- * clamped.  Workspace: kvp_decode_workspace_bytes. */
+ * clamped.  Workspace: kvp_decode_workspace_bytes.
+ * Results are the same from run to run.  With num_splits == 0 the rows are cut by the lengths of the whole batch and by the
+ * donor groups of the call, so a sequence's last bits (fp32 summation order, rounding of the probabilities to bf16) depend
+ * on the other sequences and on the layer range; with num_splits > 0 they follow from the sequence's own length. */
 int kvp_decode(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q,
                const void* const* k_cache, const void* const* v_cache, const int32_t* block_table,
                const int32_t* lengths, void* const* o, float* const* lse, int layer_begin, int layer_end, void* ws,

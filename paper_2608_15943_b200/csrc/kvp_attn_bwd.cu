@@ -2,10 +2,11 @@
 //
 //  bwd_kernel   KV-stationary.  One CTA owns a 128-row K/V tile of one (batch, KV head) of a DONOR
 //               layer, keeps K and V in shared memory and the dK / dV accumulators in TMEM (fp32)
-//               while it walks every query stream that reads the tile: the donor itself and all its
-//               consumer layers, the Hq/Hkv query heads of the KV head's group, and every 64-row query
-//               tile the causal mask lets see the keys.  dK and dV of the donor are therefore summed on
-//               chip across layers and heads and written to HBM once.  Per step, transposed so that TMEM
+//               while it walks the query streams that read the tile: the donor itself and all its
+//               consumer layers, the Hq/Hkv query heads of the KV head's group, and a window of the 64-row
+//               query tiles the causal mask lets see the keys.  dK and dV of the donor are therefore summed
+//               on chip across layers and heads and added to the fp32 sums in HBM once per CTA; where a key
+//               tile has several (windows, and parts of the streams in small calls), in no fixed order.  Per step, transposed so that TMEM
 //               lane == key row:  S^T = K Q^T, dP^T = V dO^T (tcgen05, operands in shared memory), each
 //               followed by one rank-3 MMA that subtracts the query's LSE/scale resp. Delta (a bf16
 //               three-term split against a tile of ones), so the accumulators already hold the
@@ -14,16 +15,16 @@
 //               TMEM.  dS^T also goes to shared memory, where it is the B operand of the fifth product
 //               dQ^T = K^T dS^T (K read as an MN-major A operand): the step's [dh x 64] partial of dQ
 //               lands in TMEM, a third warpgroup moves it to shared memory and adds it to an fp32
-//               accumulator in global memory with bulk reductions (cp.reduce.async.bulk .add.f32, 2 KB
+//               accumulator in global memory with bulk reductions (cp.reduce.async.bulk .add.f32, 8 KB
 //               each), so S and dP are computed once for all three gradients.
 //
 //  dq_convert_kernel  scales the fp32 dQ accumulators and writes dQ as bf16 [B,S,Hq,dh].
 //
 // Delta = rowsum(dO * O) comes from a small pre-pass.  The dQ accumulators live in the caller's
 // workspace in a blocked layout ([b][hq][64-query tile][32-column quarter][64][32] fp32) so that every
-// reduction is one contiguous 2 KB run; they are cleared before each donor group's launch.  The order in
-// which the key tiles' partials reach an accumulator is not fixed, so dQ (unlike dK, dV) is reproducible
-// only up to fp32 rounding order.
+// reduction is one contiguous 8 KB run; they, and the dK / dV sums, are cleared by the pre-pass of each launch.  The
+// order in which partials reach an accumulator is not fixed, so dQ, dK and dV are reproducible only up to fp32 rounding
+// order (bit for bit up to 128 tokens, where no element has more than two terms).
 #include <math.h>
 
 #include <algorithm>

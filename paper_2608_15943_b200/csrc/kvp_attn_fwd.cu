@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
   // The CTA is persistent: every role walks the same list of items and keeps running counts (items, key tiles,
   // sub-blocks per query tile), from which ring stages, score buffers and barrier parities follow.  The K / V rings
   // simply keep streaming across item boundaries; the next item's query tiles are loaded as soon as the last score
-  // MMAs of the current one have completed, and its first scores are computed while the softmax warps still
+  // MMAs of the current one have completed, and its first scores are computed while the epilogue warps still
   // normalise and store the current output.
 
   if (warp == 0) {
@@ -302,9 +302,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
           if (c < n_cx) issue_s(c);
         umma_commit(&k_empty[k_stage(0)], leader);
         if (n_cx <= 2) umma_commit(q_empty, leader);  // no further score MMAs of this item from this warp
-        // O_x is overwritten by the first P V product: the softmax warps must have read the last one out.  Only items
-        // that have this tile count on o_free: softmax warps that also arrived for the others could run several items
-        // ahead of this warp, past the phase that it waits for.
+        // O_x is overwritten by the first P V product: the epilogue warps must have read the last one out.  Only items
+        // that have this tile count on o_free: arrivals for the others too could run several items ahead of this warp,
+        // past the phase that it waits for.
         if (n_cx > 0 && n_o > 0 && !mbar_wait(&o_free[x], (n_o - 1) & 1, err)) { ok = false; break; }
         // Every round releases its K / V stages from this warp too when this tile has run out of sub-blocks (the
         // other tile may be one key tile longer): an arrival with nothing outstanding completes at once.

@@ -1037,9 +1037,11 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   p.tmem_cols = 32;
   while (p.tmem_cols < cfg.nt) p.tmem_cols *= 2;
   p.idesc = umma_idesc_bf16(SROWS, cfg.nt, 0, 0);
-  // Tensor memory is shared out in proportion to shared memory, so that the CTAs that fit on an SM by the latter never
-  // wait for the former (a CTA of a cluster that waited could hold up a peer that another kernel's CTA waits for); 40 KB
-  // keep it off the SMs of the kernels that take all 512 columns.
+  // Tensor memory is shared out in proportion to shared memory, so that CTAs of this kernel that fit on an SM by the latter
+  // never wait for the former: a CTA that waits holds up the peers of its cluster.  40 KB keep it off the SMs of the GEMM
+  // kernels that take all 512 columns, which have peers too, and of the attention kernels at head size 128.  Those at head
+  // size 64 (114 and 149 KB) can share an SM with it, and one of the two then waits in its allocation until the other
+  // ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
   if (allow_smem<gemm_split_kernel<NP>>(226 * 1024) != cudaSuccess) return KVP_ERR_CUDA;
