@@ -17,9 +17,9 @@ constexpr int kMinWindow = 16;
 // A CTA costs about seven steps besides its steps (prologue, dK / dV reduction, gap between two CTAs), and the last CTAs of
 // a launch leave the device idle for some part of their length: with n steps per SM in all, n * 7 / t + 0.3 t is least at
 // t = sqrt(24 n), and there is nothing to gain from fewer CTAs than one for every SM (1.5 n).
-// Measured (us; always 256 steps -> this): B3 S776 H16/4 dh64, 3 layers 119 -> 80; B4 S632 H8/2 dh128, 8 layers 201 -> 107;
-// B1 S2048 H8/8 dh128, 1 layer 50 -> 44; B1 S4096 H32/8 dh128, 1 layer 445 -> 345.  From about 2700 steps per SM on the
-// 256 stand.
+// Measured (bwd_kernel, us; always 256 steps -> this, in the order below): B3 S776 H16/4 dh64, 3 layers 120 -> 79; B4 S632
+// H8/2 dh128, 8 layers 128 -> 107; B1 S2048 H8/8 dh128, 1 layer 51 -> 42; B1 S4096 H32/8 dh128, 1 layer 458 -> 351.  From
+// about 2700 steps per SM on the 256 stand.
 constexpr float kTailFactor = 24.f;
 constexpr int kMinSteps = 2;
 
