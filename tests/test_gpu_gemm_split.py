@@ -18,9 +18,9 @@ pytestmark = pytest.mark.gpu
     (129, 4104, 2056),    # first row count of the chosen kernels: K split, one ragged column tile
     (347, 520, 2048),     # K split in four, several token tiles, the last one short
     (200, 11016, 136),    # CTA pairs with one short token tile
-    (513, 5512, 1032),    # three token tiles of 176, the last of 161, 22 column tiles
-    (289, 16392, 136),    # more column tiles than pairs, the last of eight columns
-    (2049, 2056, 200),    # a remainder of one token
+    (513, 5512, 1032),    # three token tiles of 192, the last of 129, 22 column tiles
+    (289, 16392, 136),    # more tiles than pairs, the last column tile of eight columns
+    (2049, 2056, 200),    # thirteen token tiles of 160, nine column tiles
     (1300, 8200, 72),     # several rounds of tiles, pairs in alternating direction
 ])
 def test_few_rows(M, N, K):
