@@ -498,6 +498,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 // Measured (us, K x N at M tokens; 128 x 256 tiles -> this kernel; reading B at the copy rate): 4096 x 4096 at 16
 // tokens 28.7 -> 11.6 (5.2), 4096 x 11008 at 16 30.8 -> 20.6 (13.9), 11008 x 4096 at 16 65.5 -> 20.6 (13.9), 4096 x
 // 4096 at 128 28.9 -> 14.5 (5.5); a launch that does almost nothing takes 6.
+// Where a warp has more than two tokens to sum it takes four at a time with the parts of two CTAs: one token and part after
+// the other, each waiting for the other CTA's shared memory, took 4.5 of the 16 us of 347 x 4096 x 4096 (back to back 21.2 ->
+// 16.8; 347 x 4096 x 11008 40.8 -> 32.8).
 // ------------------------------------------------------------------------------------------------------------
 constexpr int SROWS = SPLIT_COLS;                // rows of B (output columns) per tile: the M of the MMA
 constexpr int SB_BYTES = SPLIT_B_BYTES;          // 16 KB
@@ -525,8 +528,9 @@ struct SplitParams {
   uint32_t idesc;
 };
 
-template <int NP>
-__global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
+// WIDE: a warp has more than two tokens to sum.
+template <int NP, bool WIDE>
+__global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t full[SPLIT_MAX_STAGES], empty[SPLIT_MAX_STAGES], acc_full;
@@ -620,12 +624,23 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
     tc_fence_after_sync();
     const int quarter = warp & 3;
     const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16);
-    for (int c0 = 0; c0 < nt; c0 += 16) {
+    float* const dst = part + quarter * 32 + lane;
+    int c0 = 0;
+    if constexpr (WIDE) {
+      for (; c0 + 32 <= nt; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld_x32(taddr + c0, r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) dst[(c0 + i) * SROWS] = __uint_as_float(r[i]);
+      }
+    }
+    for (; c0 < nt; c0 += 16) {
       uint32_t r[16];
       tmem_ld_x16(taddr + c0, r);
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) part[(c0 + i) * SROWS + quarter * 32 + lane] = __uint_as_float(r[i]);
+      for (int i = 0; i < 16; ++i) dst[(c0 + i) * SROWS] = __uint_as_float(r[i]);
     }
     tc_fence_before_sync();
   }
@@ -636,26 +651,49 @@ __global__ void __launch_bounds__(SPLIT_THREADS) gemm_split_kernel(const __grid_
     const int col = n0 + lane * 4;
     const uint32_t mine = smem_u32(part) + lane * 16;
     const int n_tok = min(nt, pr.M - m0);
-    for (int tk = rank + warp * split; tk < n_tok; tk += split * (SPLIT_THREADS / 32)) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (uint32_t j = 0; j < split; ++j) {
-        const float4 v = ld_cluster_f4(cluster_map_addr(mine + tk * (SROWS * 4), j));
-        acc.x += v.x;
-        acc.y += v.y;
-        acc.z += v.z;
-        acc.w += v.w;
+    const int step = int(split) * (SPLIT_THREADS / 32);
+    auto store = [&](int tk, float4 acc) {
+      if (col >= pr.N) return;
+      const size_t at = size_t(m0 + tk) * pr.ldc + col;
+      if (pr.out_f32) {
+        if (pr.out_f32 == OUT_F32_OF_BF16)
+          acc = make_float4(__uint_as_float(bf16_bits_f32(acc.x)), __uint_as_float(bf16_bits_f32(acc.y)),
+                            __uint_as_float(bf16_bits_f32(acc.z)), __uint_as_float(bf16_bits_f32(acc.w)));
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(pr.c) + at) = acc;
+      } else
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(pr.c) + at) =
+            make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+    };
+    // a warp's tokens U at a time, and the parts of J CTAs: the loads of other CTAs' shared memory overlap
+    constexpr int U = WIDE ? 4 : 1, J = WIDE ? 2 : 4;
+    for (int tk = int(rank) + warp * int(split); tk < n_tok; tk += step * U) {
+      float4 acc[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (uint32_t j0 = 0; j0 < split; j0 += J) {
+        float4 v[J][U];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          const uint32_t peer = cluster_map_addr(mine, min(j0 + j, split - 1));
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (tk + u * step < n_tok && j0 + j < split) v[j][u] = ld_cluster_f4(peer + (tk + u * step) * (SROWS * 4));
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (tk + u * step < n_tok && j0 + j < split) {
+              acc[u].x += v[j][u].x;
+              acc[u].y += v[j][u].y;
+              acc[u].z += v[j][u].z;
+              acc[u].w += v[j][u].w;
+            }
       }
-      if (col < pr.N) {
-        const size_t at = size_t(m0 + tk) * pr.ldc + col;
-        if (pr.out_f32) {
-          if (pr.out_f32 == OUT_F32_OF_BF16)
-            acc = make_float4(__uint_as_float(bf16_bits_f32(acc.x)), __uint_as_float(bf16_bits_f32(acc.y)),
-                              __uint_as_float(bf16_bits_f32(acc.z)), __uint_as_float(bf16_bits_f32(acc.w)));
-          *reinterpret_cast<float4*>(reinterpret_cast<float*>(pr.c) + at) = acc;
-        } else
-          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(pr.c) + at) =
-              make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
-      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (tk + u * step < n_tok) store(tk + u * step, acc[u]);
     }
   }
   __syncthreads();
@@ -1044,9 +1082,12 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
-  if (allow_smem<gemm_split_kernel<NP>>(226 * 1024) != cudaSuccess) return KVP_ERR_CUDA;
+  const bool wide = cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
+  if ((wide ? allow_smem<gemm_split_kernel<NP, true>>(226 * 1024) : allow_smem<gemm_split_kernel<NP, false>>(226 * 1024)) != cudaSuccess)
+    return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
-  const cudaError_t e = launch_kernel(gemm_split_kernel<NP>, tiles * cfg.split, SPLIT_THREADS, smem, stream, cfg.split, p);
+  const cudaError_t e = launch_kernel(wide ? gemm_split_kernel<NP, true> : gemm_split_kernel<NP, false>, tiles * cfg.split, SPLIT_THREADS,
+                                      smem, stream, cfg.split, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
