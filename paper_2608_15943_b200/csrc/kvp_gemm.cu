@@ -27,7 +27,8 @@ constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
 constexpr int GEMM_THREADS = 192;
 constexpr int MAX_SEG = 3;
 constexpr int GROUP_M = 16;  // m-tiles per rasterisation group (keeps an A slab resident in L2)
-constexpr size_t GEMM_SMEM = 1024 + size_t(STAGES) * STAGE_BYTES + 256;
+constexpr int EPI_BYTES = 4 * 2 * 4096;         // per epilogue warp two pieces of 32 rows x 128 bytes of C
+constexpr size_t GEMM_SMEM = 1024 + size_t(STAGES) * STAGE_BYTES + EPI_BYTES + 256;
 constexpr int MAX_PROB = 32;   // problems per launch
 constexpr int MAX_MAPS = 96;   // tensor maps per launch (two per segment)
 
@@ -45,12 +46,11 @@ struct Problem {
   int a_mn, b_mn;
   int out_f32;
   uint32_t idesc;
-  long long ldc;
-  void* c;
 };
 
 struct GemmParams {
   CUtensorMap maps[MAX_MAPS];
+  CUtensorMap map_c[MAX_PROB];   // C, box of 32 rows x 128 bytes
   Problem prob[MAX_PROB];
   int nprob;
   int total_tiles;
@@ -71,10 +71,56 @@ __device__ __forceinline__ void tile_coords(int within_problem, int m_tiles, int
   tn = within / gm;
 }
 
+// One warp's 32 rows of a tile of C, from row0 and column n0 on: accumulator -> registers -> shared memory (128-byte
+// swizzle) -> TMA stores of 32 rows x 128 bytes, two of them in flight; `release` when the accumulator has been read.  Stored
+// from registers instead, a lane a row and 16 bytes at a time (half-sectors of 32 lines an instruction), a launch's last tile
+// took 4 us after its last MMA (128 x 256, bf16), and a prompt of 347 tokens through a stage, nine launches of 129 to 144
+// tiles among its 51, 811 us; 796 so.
+template <typename F>
+__device__ __forceinline__ void store_rows(const CUtensorMap* map, uint32_t taddr, int row0, int M, int n0, int N, int out_f32,
+                                           uint8_t* stage, uint32_t& pieces, F release) {
+  const int lane = lane_id();
+  const int step = out_f32 ? 32 : 64;   // columns of 128 bytes
+  const int end = row0 < M ? min(BN, N - n0) : 0;
+  if (end <= 0) release();
+#pragma unroll 1
+  for (int c0 = 0; c0 < end; c0 += step, ++pieces) {
+    uint8_t* const piece = stage + (pieces & 1) * 4096;
+    uint32_t v[32];
+    if (out_f32) {
+      tmem_ld_x32(taddr + c0, v);
+      tmem_ld_wait();
+      if (out_f32 == OUT_F32_OF_BF16)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = bf16_bits_f32(__uint_as_float(v[i]));
+    } else {
+      uint32_t r[64];
+      tmem_ld_x32(taddr + c0, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+      tmem_ld_x32(taddr + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(&r[32]));
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = pack_bf16(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+    }
+    if (c0 + step >= end) release();
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the piece before the last has been read
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      *reinterpret_cast<uint4*>(piece + sw128_offset(lane, j)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_2d(map, piece, n0 + c0, row0);
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+  }
+}
+
 __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(STAGES) * STAGE_BYTES);
+  uint8_t* epi = smem + size_t(STAGES) * STAGE_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(epi + EPI_BYTES);
   uint64_t* full = bars;                  // [STAGES]
   uint64_t* empty = bars + STAGES;        // [STAGES]
   uint64_t* acc_full = bars + 2 * STAGES; // [2]
@@ -194,63 +240,27 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(const __grid_cons
   } else {
     // ------------------------------ epilogue (warps 2..5) ------------------------------
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
-    uint32_t tile_i = 0;
+    uint32_t tile_i = 0, pieces = 0;
     int pi = 0;
     for (int t = blockIdx.x; t < total_tiles; t += gridDim.x, ++tile_i) {
       while (t >= p.prob[pi].tile_end) ++pi;
       const Problem& pr = p.prob[pi];
       int tm, tn;
       tile_coords(t - (pi ? p.prob[pi - 1].tile_end : 0), pr.m_tiles, pr.n_tiles, tm, tn);
-      const int M = pr.M, N = pr.N, out_f32 = pr.out_f32;
-      const long long ldc = pr.ldc;
-      void* const c = pr.c;
       const int acc = tile_i & 1;
       const uint32_t acc_ph = (tile_i >> 1) & 1;
       bool ok = mbar_wait(&acc_full[acc], acc_ph, err, p.wait_limit_ns);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      const int row = tm * BM + quarter * 32 + lane;
-      const int n0 = tn * BN;
-      const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN;
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        if (n0 + c0 >= N) break;  // uniform across the warp
-        uint32_t r[32];
-        tmem_ld_x32(taddr + c0, r);
-        tmem_ld_wait();
-        if (row < M) {
-          if (out_f32) {
-            float* dst = reinterpret_cast<float*>(c) + size_t(row) * ldc + n0 + c0;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              if (n0 + c0 + v * 4 < N) {
-                uint4 val = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-                if (out_f32 == OUT_F32_OF_BF16)
-                  val = make_uint4(bf16_bits_f32(__uint_as_float(val.x)), bf16_bits_f32(__uint_as_float(val.y)),
-                                   bf16_bits_f32(__uint_as_float(val.z)), bf16_bits_f32(__uint_as_float(val.w)));
-                *reinterpret_cast<uint4*>(dst + v * 4) = val;
-              }
-            }
-          } else {
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(c) + size_t(row) * ldc + n0 + c0;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              if (n0 + c0 + v * 8 < N) {
-                uint4 val;
-                val.x = pack_bf16(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1]));
-                val.y = pack_bf16(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3]));
-                val.z = pack_bf16(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5]));
-                val.w = pack_bf16(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7]));
-                *reinterpret_cast<uint4*>(dst + v * 8) = val;
-              }
-            }
-          }
-        }
-      }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      store_rows(&p.map_c[pi], tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN, tm * BM + quarter * 32, pr.M, tn * BN, pr.N,
+                 pr.out_f32, epi + quarter * 8192, pieces, [&]() {
+                   tc_fence_before_sync();
+                   __syncwarp();
+                   if (lane == 0) mbar_arrive(&acc_empty[acc]);
+                 });
     }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // before the shared memory goes away
+    __syncwarp();
   }
 
   // ------------------------------ teardown ------------------------------
@@ -278,13 +288,14 @@ constexpr int PSTAGES = 6;
 constexpr int PA_BYTES = PHALF * BK * 2;          // 16 KB
 constexpr int PB_BYTES = PHALF * BK * 2;          // 16 KB
 constexpr int PSTAGE_BYTES = PA_BYTES + PB_BYTES; // 32 KB per CTA
-constexpr size_t PAIR_SMEM = 1024 + size_t(PSTAGES) * PSTAGE_BYTES + 256;
+constexpr size_t PAIR_SMEM = 1024 + size_t(PSTAGES) * PSTAGE_BYTES + EPI_BYTES + 256;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(PSTAGES) * PSTAGE_BYTES);
+  uint8_t* epi = smem + size_t(PSTAGES) * PSTAGE_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(epi + EPI_BYTES);
   uint64_t* full = bars;                    // [PSTAGES]  (used in the even CTA)
   uint64_t* empty = bars + PSTAGES;         // [PSTAGES]
   uint64_t* acc_full = bars + 2 * PSTAGES;  // [2]
@@ -415,63 +426,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
   } else {
     // ------------------------------ epilogue (warps 2..5 of both CTAs) ------------------------------
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
-    uint32_t tile_i = 0;
+    uint32_t tile_i = 0, pieces = 0;
     int pi = 0;
     for (int t = pair; t < total_tiles; t += n_pairs, ++tile_i) {
       while (t >= p.prob[pi].tile_end) ++pi;
       const Problem& pr = p.prob[pi];
       int tm, tn;
       tile_coords(t - (pi ? p.prob[pi - 1].tile_end : 0), pr.m_tiles, pr.n_tiles, tm, tn);
-      const int M = pr.M, N = pr.N, out_f32 = pr.out_f32;
-      const long long ldc = pr.ldc;
-      void* const c = pr.c;
       const int acc = tile_i & 1;
       const uint32_t acc_ph = (tile_i >> 1) & 1;
       bool ok = mbar_wait(&acc_full[acc], acc_ph, err, p.wait_limit_ns);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      const int row = tm * PBM + int(rank) * PHALF + quarter * 32 + lane;
-      const int n0 = tn * BN;
-      const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN;
-#pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        if (n0 + c0 >= N) break;  // uniform across the warp
-        uint32_t r[32];
-        tmem_ld_x32(taddr + c0, r);
-        tmem_ld_wait();
-        if (row < M) {
-          if (out_f32) {
-            float* dst = reinterpret_cast<float*>(c) + size_t(row) * ldc + n0 + c0;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-              if (n0 + c0 + v * 4 < N) {
-                uint4 val = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-                if (out_f32 == OUT_F32_OF_BF16)
-                  val = make_uint4(bf16_bits_f32(__uint_as_float(val.x)), bf16_bits_f32(__uint_as_float(val.y)),
-                                   bf16_bits_f32(__uint_as_float(val.z)), bf16_bits_f32(__uint_as_float(val.w)));
-                *reinterpret_cast<uint4*>(dst + v * 4) = val;
-              }
-            }
-          } else {
-            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(c) + size_t(row) * ldc + n0 + c0;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              if (n0 + c0 + v * 8 < N) {
-                uint4 val;
-                val.x = pack_bf16(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1]));
-                val.y = pack_bf16(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3]));
-                val.z = pack_bf16(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5]));
-                val.w = pack_bf16(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7]));
-                *reinterpret_cast<uint4*>(dst + v * 8) = val;
-              }
-            }
-          }
-        }
-      }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(cluster_addr_of(&acc_empty[acc], 0));
+      store_rows(&p.map_c[pi], tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN, tm * PBM + int(rank) * PHALF + quarter * 32, pr.M, tn * BN, pr.N,
+                 pr.out_f32, epi + quarter * 8192, pieces, [&]() {
+                   tc_fence_before_sync();
+                   __syncwarp();
+                   if (lane == 0) mbar_arrive_cluster(cluster_addr_of(&acc_empty[acc], 0));
+                 });
     }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // before the shared memory goes away
+    __syncwarp();
   }
 
   // ------------------------------ teardown ------------------------------
@@ -1026,8 +1001,12 @@ int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withh
     q.b_mn = g.b_mn;
     q.out_f32 = g.out_f32;
     q.idesc = umma_idesc_bf16(bm, BN, g.a_mn, g.b_mn);
-    q.ldc = g.ldc;
-    q.c = g.c;
+    const int elem = g.out_f32 ? 4 : 2;
+    const uint64_t dims[2] = {uint64_t(g.N), uint64_t(g.M)};
+    const uint64_t strides[1] = {uint64_t(g.M > 1 ? g.ldc : (g.N + 7) / 8 * 8) * elem};
+    const uint32_t box[2] = {uint32_t(128 / elem), 32};
+    const int rc = make_tensor_map(&p.map_c[i], g.c, elem, 2, dims, strides, box, true);
+    if (rc != KVP_OK) return rc;
   }
   for (int i = n; i < MAX_PROB; ++i) p.prob[i] = p.prob[n - 1];
   p.total_tiles = tiles;

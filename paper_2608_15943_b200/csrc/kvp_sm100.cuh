@@ -155,6 +155,11 @@ __device__ __forceinline__ void tma_load_4d_e(void* dst, const CUtensorMap* map,
       "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(leader)
       : "memory");
 }
+// writes a shared-memory tile to global memory (bulk group completion); what lies outside the tensor is left out
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(smem_u32(src)), "r"(x), "r"(y)
+               : "memory");
+}
 // adds a shared-memory tile to global memory (fp32, bulk group completion); rows outside the tensor are left out
 __device__ __forceinline__ void tma_reduce_add_4d(const CUtensorMap* map, const void* src, int x, int y, int z, int w) {
   asm volatile("cp.reduce.async.bulk.tensor.4d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(map),

@@ -121,3 +121,26 @@ def test_each_forward_kernel_at_its_edges(choose, M, N, K, kernel):
     kind, nt, split = choose([(M, N, K)])
     assert (("single", "pair", "tall", "split")[kind], nt, split) == kernel
     test_few_rows(M, N, K)
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("M,N,K,cols", [(129, 8, 72, 24), (160, 264, 136, 520), (300, 520, 64, 528), (513, 296, 200, 304)])
+def test_results_inside_a_wider_matrix(mode, M, N, K, cols):
+    """C is a block of columns of a wider matrix: the tile kernels store whole boxes of it, and nothing beside it."""
+    from paper_2608_15943_b200 import kvp
+    a, b = synth.normal((M, K), 34, 1, 1.0, "cuda"), synth.normal((N, K), 34, 2, 1.0, "cuda")
+    ref = a.double() @ b.double().T
+    bound = K * 2.0 ** -24 * (a.double().abs() @ b.double().abs().T) + 1e-30   # as test_few_rows
+    kvp.set_gemm_pair_mode(mode)
+    try:
+        for dtype in (torch.bfloat16, torch.float32):
+            whole = torch.full((M + 3, cols), 7.0, dtype=dtype, device="cuda")
+            c = whole[1:M + 1, 8:8 + N]
+            kvp.gemm(a, b, c)
+            assert kvp.device_status() == kvp.OK
+            half_ulp = 2.0 ** -8 * ref.abs() if dtype == torch.bfloat16 else 0.0
+            assert ((c.double() - ref).abs() <= bound + half_ulp).all()
+            c.fill_(7.0)
+            assert (whole == 7.0).all()
+    finally:
+        kvp.set_gemm_pair_mode(1)
