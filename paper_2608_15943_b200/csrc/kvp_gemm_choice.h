@@ -2,6 +2,8 @@
 // dependency: a host-only test uses the same rules).
 #pragma once
 
+#include <math.h>
+
 #include <algorithm>
 
 namespace kvp {
@@ -25,23 +27,48 @@ struct SplitConfig {
   int stages;
 };
 
-// The smallest split that gives 128 CTAs: enough of them to draw the full memory bandwidth, and no partial more than
-// that needs (at N = K = 4096 and 16 tokens a split of 2 / 4 / 8 measured 12.3 / 11.6 / 10.8 us, at 64 tokens and 4 / 8
-// it measured 12.5 / 14.3).  One CTA per SM takes a ring as deep as fits; more CTAs than SMs share them in twos.
+// Up to SPLIT_MAX_ROWS rows: tokens per tile and K split by an estimate of the time (us), whose constants were fitted to 1100
+// launches (15 weight shapes x 9 row counts, weights not in L2, each behind an element-wise kernel, replayed from a graph;
+// the choice it makes costs 0.5 % more than the best of all on average).  A CTA's k-blocks and the memory both count, as the
+// root of the sum of their squares; a cluster costs up to a microsecond, and clusters of eight do not all fit at once from
+// about seven tenths of the SMs on; more CTAs than SMs share them in twos, with half the ring.  The smallest split that gave
+// 128 CTAs, with all tokens in one tile, was 15 % slower on average (16 x 2048 x 2048 13.4 us -> 8.2, 16 x 2048 x 5504 15.4 ->
+// 9.7, 128 x 1024 x 1024 9.4 -> 6.7, 128 x 5504 x 2048 15.0 -> 11.4).
 inline SplitConfig split_config(const GemmSize* probs, int n, int sms) {
-  int rows = 0, tiles = 0, kblocks = 1 << 30;
+  int rows = 0, columns = 0, deepest = 0, shallowest = 1 << 30;
+  float weights = 0.f;
   for (int i = 0; i < n; ++i) {
+    const int kb = (probs[i].K + GEMM_BK - 1) / GEMM_BK;
     rows = std::max(rows, probs[i].M);
-    tiles += (probs[i].N + SPLIT_COLS - 1) / SPLIT_COLS;
-    kblocks = std::min(kblocks, (probs[i].K + GEMM_BK - 1) / GEMM_BK);
+    columns += (probs[i].N + SPLIT_COLS - 1) / SPLIT_COLS;
+    deepest = std::max(deepest, kb);
+    shallowest = std::min(shallowest, kb);
+    weights += 2.f * probs[i].N * probs[i].K;
   }
-  SplitConfig c;
-  c.nt = (rows + 15) / 16 * 16;
-  c.split = 1;
-  while (c.split < 8 && 2 * c.split <= kblocks && tiles * c.split < 128) c.split *= 2;
-  const int ring_bytes = (tiles * c.split <= sms ? 220 : 110) * 1024;
-  c.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SPLIT_B_BYTES + c.nt * GEMM_BK * 2));
-  return c;
+  auto up = [](int x, int y) { return (x + y - 1) / y; };
+  SplitConfig best{0, 1, 0};
+  float best_us = 1e30f;
+  int ctas = 0;
+  for (int tok_tiles = 1; tok_tiles <= 4; tok_tiles *= 2) {
+    const int nt = up(up(rows, tok_tiles), 16) * 16, tiles = columns * tok_tiles;
+    if (up(rows, nt) != tok_tiles) continue;
+    for (int split = 1; split <= 8; split *= 2) {
+      if (split > 1 && 2 * split > shallowest) break;
+      if (tiles * split > (tok_tiles == 1 && split < 8 ? 2 * sms : sms) && (tok_tiles > 1 || split > 1)) break;
+      const float over = std::max(0.f, float(tiles * split) / sms - 1.f);   // CTAs that share an SM
+      const float main = up(deepest, split) * (0.144f + 0.017f * nt / 128.f) * (1.f + 3.7f * over), memory = weights / 7.2e6f;
+      const float cluster = split == 1 ? 0.f : split == 2 ? 0.6f : split == 4 ? 0.83f : 10 * tiles * split > 7 * sms ? 6.6f : 0.88f;
+      const float us = sqrtf(main * main + memory * memory) + 0.0277f * nt + cluster + 0.098f * nt * over;
+      if (us >= best_us) continue;
+      best_us = us;
+      best.nt = nt;
+      best.split = split;
+      ctas = tiles * split;
+    }
+  }
+  const int ring_bytes = (ctas <= sms ? 220 : 110) * 1024;
+  best.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SPLIT_B_BYTES + best.nt * GEMM_BK * 2));
+  return best;
 }
 
 // ------------------------------------------------------------------------------------------------------------

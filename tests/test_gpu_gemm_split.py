@@ -123,6 +123,17 @@ def test_each_forward_kernel_at_its_edges(choose, M, N, K, kernel):
     test_few_rows(M, N, K)
 
 
+# tokens per tile and K split of the kernel of few rows, at both sides of the line from which a warp sums several tokens
+# (more than twelve per CTA of the cluster), with short last tiles of tokens, columns and k-blocks
+@pytest.mark.parametrize("M,N,K,nt,split", [
+    (16, 136, 1032, 16, 8), (16, 8200, 520, 16, 1), (30, 2056, 2056, 16, 4), (33, 136, 1032, 32, 8), (33, 1032, 1032, 32, 4),
+    (70, 5512, 2056, 80, 2), (97, 4104, 4104, 64, 2), (128, 2056, 2056, 32, 2),
+])
+def test_few_rows_sums(choose, M, N, K, nt, split):
+    assert choose([(M, N, K)]) == (3, nt, split)
+    test_few_rows(M, N, K)
+
+
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("M,N,K,cols", [(129, 8, 72, 24), (160, 264, 136, 520), (300, 520, 64, 528), (513, 296, 200, 304)])
 def test_results_inside_a_wider_matrix(mode, M, N, K, cols):
