@@ -141,3 +141,33 @@ def test_a_long_sequence_among_short_ones(lens, Hkv, dh, page):
     ro, rl = exact_on_gpu(q, kc, vc, bt, lens, page)
     got, lse = decode_one_layer(q, kc, vc, bt, lens, page)
     assert ((got - ro).norm(dim=(1, 2)) <= REL * ro.norm(dim=(1, 2))).all() and (lse - rl).abs().max() <= 2e-6
+
+
+@pytest.mark.parametrize("first,second,Hkv,dh,page", [
+    ([20000], [777], 1, 128, 128),                        # many shares, few
+    ([300, 5000, 1100], [4000, 200, 129], 2, 128, 16),
+    ([130] * 32, [130] * 31 + [9000], 2, 64, 16),         # whole units, shares
+    ([700] * 33, [700] * 32 + [8000], 2, 64, 16),         # more lengths than a warp's lanes
+])
+def test_lengths_written_by_the_kernel_ahead(first, second, Hkv, dh, page):
+    """The lengths are looked at before the kernel ahead has finished; what it writes counts.  It is the library's own add
+    (whose CTAs let the next kernel come up early) over the lengths' bits as bf16 numbers, plus zero."""
+    from paper_2608_15943_b200 import kvp
+    longest = [max(a, b) for a, b in zip(first, second)]
+    kc, vc, bt = paged(longest, Hkv, dh, page, 74)
+    q = synth.normal((len(first), 4 * Hkv, dh), 74, 3, 1.0, "cuda")
+    want = [exact_on_gpu(q, kc, vc, bt, lens, page) for lens in (first, second)]
+    pad = -len(first) % 4                                 # 16-byte pieces
+    bits = [torch.tensor(lens + [0] * pad, dtype=torch.int32, device="cuda").view(torch.bfloat16) for lens in (first, second)]
+    lengths, zero = bits[1].clone(), torch.zeros_like(bits[0])
+    desc = kvp.DecodeDesc(1, len(first), 4 * Hkv, Hkv, dh, page, bt.shape[1], kc.shape[0])
+    ws = torch.empty(kvp.decode_workspace_bytes(desc, [0]), dtype=torch.uint8, device="cuda")
+    table = bt.cuda()
+    out = [(torch.full_like(q, float("nan")), torch.full(q.shape[:2], float("nan"), device="cuda")) for _ in range(20)]
+    for i, (o, lse) in enumerate(out):
+        kvp.add(bits[i % 2], zero, lengths)
+        kvp.decode(desc, [0], [q], [kc], [vc], table, lengths.view(torch.int32)[:len(first)], [o], [lse], ws)
+    assert kvp.device_status() == kvp.OK
+    for i, (o, lse) in enumerate(out):
+        ro, rl = want[i % 2]
+        assert (o.double() - ro).norm() <= REL * ro.norm() and (lse.double() - rl).abs().max() <= 2e-6, i
