@@ -1,8 +1,12 @@
 """Attention forward with more work items than CTAs: the roles of a CTA walk several items in a row."""
+import ctypes as C
+import subprocess
+
 import pytest
 import torch
 
 from oracle import attention as A
+from test_bwd_shape_host import CSRC
 from test_gpu_parity import attn_inputs, close, f64l, lse_close
 
 pytestmark = pytest.mark.gpu
@@ -30,3 +34,36 @@ def test_items_of_an_odd_number_of_query_tiles(B, S, Hq, Hkv, dh, donor, causal)
     for l in range(L):
         close(f"o[{l}]", o[l], ro[l])
         lse_close(f"lse[{l}]", lse[l], rl[l])
+
+
+@pytest.fixture(scope="module")
+def pack_of(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fwd")
+    (d / "r.cpp").write_text("""#include "kvp_fwd_shape.h"
+extern "C" int pack_of(int B, int S, int Hq, int Hkv, int L, int causal) {
+  return kvp::fwd_pack(kvp::FwdSizes{S, Hq / Hkv, causal != 0, (long long)L * B * Hkv, 148});
+}
+""")
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, str(d / "r.cpp"), "-o", str(d / "r.so")], check=True)
+    return C.CDLL(str(d / "r.so")).pack_of
+
+
+# tiles of 1 << pack heads; the sequence ends in a tile's first token, its last, or between
+@pytest.mark.parametrize("B,S,Hq,Hkv,dh,donor,causal,pack", [
+    (20, 257, 4, 2, 64, [0], True, 1),       # 64 tokens of two heads: five tiles, the last of one token
+    (9, 161, 24, 4, 128, [0], True, 1),      # six heads to a KV head: three groups of two
+    (6, 140, 16, 8, 64, [0, 0], False, 1),   # full attention
+    (9, 129, 8, 2, 128, [0, 1], True, 2),    # 32 tokens of four heads, the last tile of one token
+    (10, 264, 8, 2, 64, [0], True, 2),
+    (12, 33, 32, 2, 128, [0, 0], True, 4),   # eight tokens of sixteen heads, five tiles for one key tile
+    (5, 264, 32, 2, 64, [0], False, 4),      # every tile full
+])
+def test_tiles_of_several_heads(pack_of, B, S, Hq, Hkv, dh, donor, causal, pack):
+    assert pack_of(B, S, Hq, Hkv, len(donor), int(causal)) == pack
+    test_items_of_an_odd_number_of_query_tiles(B, S, Hq, Hkv, dh, donor, causal)
+
+
+def test_heads_stay_by_themselves_where_nothing_is_gained(pack_of):
+    assert pack_of(1, 300, 16, 4, 1, 1) == 0      # 20 items instead of 32, and longer ones
+    assert pack_of(2, 512, 32, 8, 2, 1) == 0
+    assert pack_of(2, 8192, 32, 8, 8, 1) == 0 and pack_of(4, 347, 32, 32, 1, 1) == 0
