@@ -83,3 +83,21 @@ def test_back_to_back_calls_see_what_the_one_before_wrote(T, D):
     for _ in range(5):
         for got, ref in zip(chain(False), want):
             assert torch.equal(got, ref)
+
+
+@pytest.mark.parametrize("n8", [16 * 148 * 2048, 16 * 148 * 2048 + 1])
+def test_swiglu_reciprocal(n8):
+    """The last size with the reciprocal of one instruction on 148 SMs and the first without, gates over the whole range of
+    exp(-g): overflow, subnormal reciprocals, both infinities."""
+    from paper_2608_15943_b200 import kvp
+    g, u = synth.normal((n8 * 8,), 66, 1, 8.0, "cuda"), synth.normal((n8 * 8,), 66, 2, 1.0, "cuda")
+    special = torch.tensor([0.0, -0.0, 88.0, -86.5, -87.5, -88.0, -88.5, -89.0, -104.0, -3e38, float("inf"), 1e-30], device="cuda").bfloat16()
+    g[:12] = special
+    g[-12:] = special
+    u[:12] = u[-12:] = 1.0
+    y = kvp.swiglu(g, u, torch.full_like(g, float("nan")))
+    e = torch.exp(-g.double())
+    ref = torch.where(e > 3.4028235677973366e38, -0.0, g.double() / (1.0 + e) * u.double())    # exp(-g) overflows in fp32
+    # bf16 storage, and exp(-g) to a few ulps of its argument (|g| 2^-23, at most 2^-16)
+    near = (y.double() - ref).abs() <= (2.0 ** -8 + 2.0 ** -15) * ref.abs() + 1e-37
+    assert (near | (y.double() == ref)).all()    # (infinity: equal, but no distance)
