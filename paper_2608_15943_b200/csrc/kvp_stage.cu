@@ -221,24 +221,14 @@ __device__ __forceinline__ void zip8(const uint4* a, const uint4* b, uint4* out,
 }
 
 constexpr int kStreamThreads = 256, kStreamResident = 8;   // CTAs per SM
-// APPROX: the reciprocal by one instruction (at most one ulp off; 2^-23 beside the 2^-9 of the result's type) instead of the
-// correctly rounded one, whose dozen bound launches of up to a few rounds: 16 x 11008 1.73 -> 1.27 us, 347 x 11008 5.9 -> 5.05,
-// 2048 x 11008 22.6 -> 21.7, 8192 x 4096 32.6 -> 31.6.  From 27 rounds on the memory is faster with fewer loads asked for at a
-// time: 6000 x 11008 62.6 / 63.4, 8192 x 11008 84.8 / 89.4.
-__device__ __forceinline__ float approx_rcp(float x) {
-  float y;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-constexpr int kApproxRounds = 16;
-template <bool TWO, bool APPROX>
+// The correctly rounded reciprocal at every size: an element's result depends on its two inputs alone.  (rcp.approx, up to an ulp
+// off, is a dozen instructions less, but moves results that lie near a tie of the bf16 rounding, five in a million.  It gained
+// 0.5 to 1.0 us a launch up to sixteen pieces a thread, 16 x 11008 1.73 -> 1.27, 2048 x 11008 22.6 -> 21.7, and lost beyond.)
+template <bool TWO>
 __global__ void __launch_bounds__(kStreamThreads, kStreamResident)
     swiglu_kernel(const uint4* gate, const uint4* up, uint4* out, size_t n8) {
   grid_dep_wait();
-  zip8<TWO>(gate, up, out, n8, [](float g, float u) {
-    const float d = 1.f + __expf(-g);
-    return g * (APPROX ? approx_rcp(d) : __frcp_rn(d)) * u;
-  });
+  zip8<TWO>(gate, up, out, n8, [](float g, float u) { return g * __frcp_rn(1.f + __expf(-g)) * u; });
 }
 
 template <bool TWO>
@@ -303,11 +293,9 @@ extern "C" int kvp_swiglu(int64_t n, const void* gate, const void* up, void* out
   if (n < 0 || gate == nullptr || up == nullptr || out == nullptr) return KVP_ERR_INVALID_ARG;
   if (n % 8 != 0 || !is_aligned16(gate) || !is_aligned16(up) || !is_aligned16(out)) return KVP_ERR_UNSUPPORTED;
   if (n == 0) return KVP_OK;
-  const size_t n8 = size_t(n / 8), round = one_round();
-  auto* const kernel = n8 > round && n8 <= 2 * round ? swiglu_kernel<true, true>
-                       : n8 <= kApproxRounds * round ? swiglu_kernel<false, true>
-                                                     : swiglu_kernel<false, false>;
-  const cudaError_t e = launch_kernel(kernel, streaming_blocks(n8), kStreamThreads, 0, reinterpret_cast<cudaStream_t>(stream), 1,
+  const size_t n8 = size_t(n / 8);
+  const cudaError_t e = launch_kernel(n8 > one_round() && n8 <= 2 * one_round() ? swiglu_kernel<true> : swiglu_kernel<false>, streaming_blocks(n8),
+      kStreamThreads, 0, reinterpret_cast<cudaStream_t>(stream), 1,
       reinterpret_cast<const uint4*>(gate), reinterpret_cast<const uint4*>(up), reinterpret_cast<uint4*>(out), n8);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }

@@ -85,19 +85,38 @@ def test_back_to_back_calls_see_what_the_one_before_wrote(T, D):
             assert torch.equal(got, ref)
 
 
-@pytest.mark.parametrize("n8", [16 * 148 * 2048, 16 * 148 * 2048 + 1])
-def test_swiglu_reciprocal(n8):
-    """The last size with the reciprocal of one instruction on 148 SMs and the first without, gates over the whole range of
-    exp(-g): overflow, subnormal reciprocals, both infinities."""
+def one_round():
+    """16-byte pieces with one for every thread of a full grid of the streaming kernels."""
+    return torch.cuda.get_device_properties(0).multi_processor_count * 8 * 256
+
+
+@pytest.mark.parametrize("rounds,more", [(0, 24), (1, 0), (1, 1), (2, 0), (2, 1), (16, 0), (16, 1)])
+def test_swiglu_range_of_gates(rounds, more):
+    """Gates over the whole range of exp(-g): overflow, subnormal reciprocals, both infinities (of which the lower has no
+    value: -inf / (1 + inf))."""
     from paper_2608_15943_b200 import kvp
+    n8 = rounds * one_round() + more
     g, u = synth.normal((n8 * 8,), 66, 1, 8.0, "cuda"), synth.normal((n8 * 8,), 66, 2, 1.0, "cuda")
-    special = torch.tensor([0.0, -0.0, 88.0, -86.5, -87.5, -88.0, -88.5, -89.0, -104.0, -3e38, float("inf"), 1e-30], device="cuda").bfloat16()
-    g[:12] = special
-    g[-12:] = special
-    u[:12] = u[-12:] = 1.0
-    y = kvp.swiglu(g, u, torch.full_like(g, float("nan")))
+    special = torch.tensor([0.0, -0.0, 88.0, -86.5, -87.5, -88.0, -88.5, -89.0, -104.0, -3e38, float("inf"), 1e-30, float("-inf")],
+                           device="cuda").bfloat16()
+    g[:13] = special
+    g[-13:] = special
+    u[:13] = u[-13:] = 1.0
+    y = kvp.swiglu(g, u, torch.full_like(g, 7.0))
     e = torch.exp(-g.double())
-    ref = torch.where(e > 3.4028235677973366e38, -0.0, g.double() / (1.0 + e) * u.double())    # exp(-g) overflows in fp32
+    ref = torch.where((e > 3.4028235677973366e38) & (e < float("inf")), -0.0, g.double() / (1.0 + e) * u.double())   # exp(-g) overflows in fp32
     # bf16 storage, and exp(-g) to a few ulps of its argument (|g| 2^-23, at most 2^-16)
     near = (y.double() - ref).abs() <= (2.0 ** -8 + 2.0 ** -15) * ref.abs() + 1e-37
-    assert (near | (y.double() == ref)).all()    # (infinity: equal, but no distance)
+    assert (near | (y.double() == ref) | (y.isnan() & g.isneginf())).all()    # (infinity: equal, but no distance)
+    assert y.isnan().sum() == 2
+
+
+def test_swiglu_does_not_depend_on_the_size():
+    """An element's bits are the same in calls of every size: one piece, and either side of one, two and sixteen rounds."""
+    from paper_2608_15943_b200 import kvp
+    n = (16 * one_round() + 1) * 8
+    g, u = synth.normal((n,), 67, 1, 2.0, "cuda"), synth.normal((n,), 67, 2, 1.0, "cuda")
+    whole = kvp.swiglu(g, u, torch.full_like(g, float("nan")))
+    for n8 in (1, 255, one_round(), one_round() + 1, 2 * one_round(), 2 * one_round() + 1, 16 * one_round()):
+        part = kvp.swiglu(g[:n8 * 8], u[:n8 * 8], torch.full((n8 * 8,), float("nan"), dtype=torch.bfloat16, device="cuda"))
+        assert torch.equal(part, whole[:n8 * 8]), n8
