@@ -467,9 +467,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 // With at most 128 rows of A the product is bound by reading B once, and the 128 x 256 tiles above put it on N / 256
 // CTAs: 16 of 148 SMs at N = 4096, 29 us for 33.5 MB.  Here B supplies the M = 128 side of the MMA and the tokens its
 // N side (a multiple of 16, so 16 tokens cost 16 columns and not 128 rows), and the k-blocks of a tile are dealt to
-// the CTAs of a cluster, each with its own ring.  The partials meet in shared memory: every CTA moves its accumulator
-// from TMEM to shared memory as [token][128 columns] fp32 and sums its share of the tokens over the cluster's CTAs
-// through distributed shared memory, in rank order, so results do not depend on timing.
+// the CTAs of a cluster, each with its own ring and one or two accumulators.  The partials meet in shared memory: every CTA
+// moves its accumulators from TMEM to shared memory as [token][128 columns] fp32 and sums its share of the tokens over the
+// cluster's accumulators through distributed shared memory, in their order along K, so results depend neither on timing nor on
+// how many accumulators a CTA has.
 // Measured (us, K x N at M tokens; 128 x 256 tiles -> this kernel; reading B at the copy rate): 4096 x 4096 at 16
 // tokens 28.7 -> 11.6 (5.2), 4096 x 11008 at 16 30.8 -> 20.6 (13.9), 11008 x 4096 at 16 65.5 -> 20.6 (13.9), 4096 x
 // 4096 at 128 28.9 -> 14.5 (5.5); a launch that does almost nothing takes 6.
@@ -503,8 +504,8 @@ struct SplitParams {
   uint32_t idesc;
 };
 
-// WIDE: a warp has more than two tokens to sum.
-template <int NP, bool WIDE>
+// WIDE: a warp has more than two tokens to sum.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.
+template <int NP, bool WIDE, int PARTS>
 __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -526,7 +527,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
   const int within = t - (pi ? p.prob[pi - 1].tile_end : 0);
   const int n0 = (within / pr.tok_tiles) * SROWS;   // first output column (row of B)
   const int m0 = (within % pr.tok_tiles) * nt;      // first token
-  const int kb0 = int(rank) * pr.kblocks / int(split), kb1 = (int(rank) + 1) * pr.kblocks / int(split);
+  const int pieces = int(split) * PARTS, piece = int(rank) * PARTS;   // of K, and this CTA's first
+  const int kb0 = piece * pr.kblocks / pieces, kb1 = (piece + PARTS) * pr.kblocks / pieces;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -572,15 +574,17 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
     int s = 0;
     uint32_t ph = 0;
     bool ok = true;
+    const int kb_second = PARTS == 2 ? (piece + 1) * pr.kblocks / pieces : kb1;
     for (int kb = kb0; kb < kb1; ++kb) {
       if (!mbar_wait(&full[s], ph, err)) { ok = false; break; }
       tc_fence_after_sync();
+      const uint32_t acc = kb < kb_second ? tmem_base : tmem_base + p.tmem_cols / 2;
       const uint32_t b_lo = desc_lo_sw128(smem_u32(smem + s * stage_bytes), 0);
       const uint32_t a_lo = desc_lo_sw128(smem_u32(smem + s * stage_bytes + SB_BYTES), 0);
 #pragma unroll
       for (int k = 0; k < BK / 16; ++k)
-        umma_ss_w(tmem_base, desc_lo_add(b_lo, k * 32), desc_lo_add(a_lo, k * 32), desc_hi_sw128(1024), p.idesc,
-                  kb != kb0 || k != 0, leader);
+        umma_ss_w(acc, desc_lo_add(b_lo, k * 32), desc_lo_add(a_lo, k * 32), desc_hi_sw128(1024), p.idesc,
+                  (kb != kb0 && (PARTS == 1 || kb != kb_second)) || k != 0, leader);
       umma_commit(&empty[s], leader);
       if (++s == stages) {
         s = 0;
@@ -589,8 +593,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
     }
     if (ok) umma_commit(&acc_full, leader);
   }
-  // every warp waits for the accumulator; the four warps that own its lanes move it to shared memory as [token][128]
-  // fp32 (the ring is idle now)
+  // every warp waits for the accumulators; the four warps that own their lanes move them to shared memory as [token][128]
+  // fp32 (the ring is idle now), one behind the other
   __syncwarp();
   float* part = reinterpret_cast<float*>(smem);
   bool ok = mbar_wait(&acc_full, 0, err);
@@ -598,30 +602,33 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
   if (ok && warp >= 2) {
     tc_fence_after_sync();
     const int quarter = warp & 3;
-    const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16);
-    float* const dst = part + quarter * 32 + lane;
-    int c0 = 0;
-    if constexpr (WIDE) {
-      for (; c0 + 32 <= nt; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_x32(taddr + c0, r);
+    uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16);
+    float* dst = part + quarter * 32 + lane;
+#pragma unroll 1
+    for (int i = 0; i < PARTS; ++i, taddr += p.tmem_cols / 2, dst += nt * SROWS) {
+      int c0 = 0;
+      if constexpr (WIDE) {
+        for (; c0 + 32 <= nt; c0 += 32) {
+          uint32_t r[32];
+          tmem_ld_x32(taddr + c0, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 32; ++k) dst[(c0 + k) * SROWS] = __uint_as_float(r[k]);
+        }
+      }
+      for (; c0 < nt; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld_x16(taddr + c0, r);
         tmem_ld_wait();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) dst[(c0 + i) * SROWS] = __uint_as_float(r[i]);
+        for (int k = 0; k < 16; ++k) dst[(c0 + k) * SROWS] = __uint_as_float(r[k]);
       }
-    }
-    for (; c0 < nt; c0 += 16) {
-      uint32_t r[16];
-      tmem_ld_x16(taddr + c0, r);
-      tmem_ld_wait();
-#pragma unroll
-      for (int i = 0; i < 16; ++i) dst[(c0 + i) * SROWS] = __uint_as_float(r[i]);
     }
     tc_fence_before_sync();
   }
   __syncthreads();
   if (split > 1) cluster_sync_all();
-  // each CTA of the cluster sums its share of the tokens over all partials, always in rank order
+  // each CTA of the cluster sums its share of the tokens over all partials, always in their order along K
   if (ok) {
     const int col = n0 + lane * 4;
     const uint32_t mine = smem_u32(part) + lane * 16;
@@ -639,27 +646,28 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
         *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(pr.c) + at) =
             make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
     };
-    // a warp's tokens U at a time, and the parts of J CTAs: the loads of other CTAs' shared memory overlap
+    // a warp's tokens U at a time, and J partials: the loads of other CTAs' shared memory overlap
     constexpr int U = WIDE ? 4 : 1, J = WIDE ? 2 : 4;
     for (int tk = int(rank) + warp * int(split); tk < n_tok; tk += step * U) {
       float4 acc[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-      for (uint32_t j0 = 0; j0 < split; j0 += J) {
+      for (int j0 = 0; j0 < pieces; j0 += J) {
         float4 v[J][U];
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-          const uint32_t peer = cluster_map_addr(mine, min(j0 + j, split - 1));
+          const int from = min(j0 + j, pieces - 1);
+          const uint32_t peer = cluster_map_addr(mine + from % PARTS * (nt * SROWS * 4), from / PARTS);
 #pragma unroll
           for (int u = 0; u < U; ++u)
-            if (tk + u * step < n_tok && j0 + j < split) v[j][u] = ld_cluster_f4(peer + (tk + u * step) * (SROWS * 4));
+            if (tk + u * step < n_tok && j0 + j < pieces) v[j][u] = ld_cluster_f4(peer + (tk + u * step) * (SROWS * 4));
         }
 #pragma unroll
         for (int j = 0; j < J; ++j)
 #pragma unroll
           for (int u = 0; u < U; ++u)
-            if (tk + u * step < n_tok && j0 + j < split) {
+            if (tk + u * step < n_tok && j0 + j < pieces) {
               acc[u].x += v[j][u].x;
               acc[u].y += v[j][u].y;
               acc[u].z += v[j][u].z;
@@ -1028,6 +1036,11 @@ bool k_major(const GemmProblem* probs, int n) {
   return n > 0;
 }
 
+template <int NP, bool WIDE, int PARTS>
+auto split_kernel() -> decltype(&gemm_split_kernel<NP, WIDE, PARTS>) {
+  return allow_smem<gemm_split_kernel<NP, WIDE, PARTS>>(226 * 1024) == cudaSuccess ? &gemm_split_kernel<NP, WIDE, PARTS> : nullptr;
+}
+
 template <int NP>
 int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaStream_t stream) {
   SplitParams<NP> p;
@@ -1051,22 +1064,22 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   }
   p.nt = cfg.nt;
   p.stages = cfg.stages;
-  p.tmem_cols = 32;
-  while (p.tmem_cols < cfg.nt) p.tmem_cols *= 2;
+  p.tmem_cols = 32 * cfg.parts;
+  while (p.tmem_cols < cfg.nt * cfg.parts) p.tmem_cols *= 2;
   p.idesc = umma_idesc_bf16(SROWS, cfg.nt, 0, 0);
   // Tensor memory is shared out in proportion to shared memory, so that CTAs of this kernel that fit on an SM by the latter
   // never wait for the former: a CTA that waits holds up the peers of its cluster.  40 KB keep it off the SMs of the GEMM
   // kernels that take all 512 columns, which have peers too, and of the attention kernels at head size 128.  Those at head
   // size 64 (114 and 149 KB) can share an SM with it, and one of the two then waits in its allocation until the other
   // ends; it does end, for a CTA of the attention waits for no other CTA.
-  const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.nt * SROWS * 4;
+  const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.parts * cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
   const bool wide = cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
-  if ((wide ? allow_smem<gemm_split_kernel<NP, true>>(226 * 1024) : allow_smem<gemm_split_kernel<NP, false>>(226 * 1024)) != cudaSuccess)
-    return KVP_ERR_CUDA;
+  auto* const kernel = cfg.parts == 2 ? (wide ? split_kernel<NP, true, 2>() : split_kernel<NP, false, 2>())
+                                      : (wide ? split_kernel<NP, true, 1>() : split_kernel<NP, false, 1>());
+  if (kernel == nullptr) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
-  const cudaError_t e = launch_kernel(wide ? gemm_split_kernel<NP, true> : gemm_split_kernel<NP, false>, tiles * cfg.split, SPLIT_THREADS,
-                                      smem, stream, cfg.split, p);
+  const cudaError_t e = launch_kernel(kernel, tiles * cfg.split, SPLIT_THREADS, smem, stream, cfg.split, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
@@ -1204,7 +1217,7 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
       rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, true, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, true, stream); },
                     [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, true, stream); });
     } else if (c.kind == Choice::kSplit) {
-      const SplitConfig cfg{c.nt, c.split, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
+      const SplitConfig cfg{c.nt, c.split, 1, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
       rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
                     [&] { return launch_split<MAX_PROB>(g, cnt, cfg, stream); });
     } else {

@@ -2,8 +2,6 @@
 // dependency: a host-only test uses the same rules).
 #pragma once
 
-#include <math.h>
-
 #include <algorithm>
 
 namespace kvp {
@@ -24,51 +22,47 @@ constexpr int SPLIT_MAX_ROWS = 128;       // up to here always the split kernel
 struct SplitConfig {
   int nt;       // tokens per tile
   int split;    // CTAs of a cluster along K
+  int parts;    // accumulators of a CTA, each with half of its k-blocks where there are two
   int stages;
 };
 
-// Up to SPLIT_MAX_ROWS rows: tokens per tile and K split by an estimate of the time (us), whose constants were fitted to 1100
-// launches (15 weight shapes x 9 row counts, weights not in L2, each behind an element-wise kernel, replayed from a graph;
-// the choice it makes costs 0.5 % more than the best of all on average).  A CTA's k-blocks and the memory both count, as the
-// root of the sum of their squares; a cluster costs up to a microsecond, and clusters of eight do not all fit at once from
-// about seven tenths of the SMs on; more CTAs than SMs share them in twos, with half the ring.  The smallest split that gave
-// 128 CTAs, with all tokens in one tile, was 15 % slower on average (16 x 2048 x 2048 13.4 us -> 8.2, 16 x 2048 x 5504 15.4 ->
-// 9.7, 128 x 1024 x 1024 9.4 -> 6.7, 128 x 5504 x 2048 15.0 -> 11.4).
+// Up to SPLIT_MAX_ROWS rows.  K is cut into the smallest number of pieces that gives 128 CTAs, eight at most, each with an
+// accumulator of its own: by the columns and the depth alone, so that a row's bits do not depend on how many rows the call has.
+// Fewer pieces would be faster for many shapes, but the error of a tensor-core sum grows with its length: fp32 results of a
+// split chosen by time alone, often a half or a quarter of this one, lay 2.4 times as far from 64 bits on average, 7.7 times
+// at most, over the 442 of 720 shapes where it differed.
+// A cluster takes the pieces, a CTA each.  Where the launch would put a CTA on nearly every SM, not all clusters find room at
+// once (of eight CTAs from 13/16 of the SMs on, of four from 132 of 148): half as many CTAs with two accumulators take the
+// pieces then.  The tokens go into two or four tiles where all CTAs still fit.  Measured (us, one tile and one CTA a piece ->
+// this; weights not in L2, each launch behind an element-wise kernel, replayed from a graph): two accumulators, 16 x 2048 x
+// 2048 10.6 -> 7.8, 128 x 2048 x 2048 16.0 -> 11.2, 64 x 4608 x 4096 18.9 -> 15.4; more tiles, 128 x 256 x 256 7.3 -> 5.2, 128 x
+// 512 x 1024 7.9 -> 6.7.  On average over 15 weight shapes x 7 row counts 1.07 times as fast, over 31 other shapes 1.11, and 0.4 %
+// above the best cluster, tile and number of accumulators for these pieces on both.
 inline SplitConfig split_config(const GemmSize* probs, int n, int sms) {
-  int rows = 0, columns = 0, deepest = 0, shallowest = 1 << 30;
-  float weights = 0.f;
+  int rows = 0, columns = 0, kblocks = 1 << 30;
   for (int i = 0; i < n; ++i) {
-    const int kb = (probs[i].K + GEMM_BK - 1) / GEMM_BK;
     rows = std::max(rows, probs[i].M);
     columns += (probs[i].N + SPLIT_COLS - 1) / SPLIT_COLS;
-    deepest = std::max(deepest, kb);
-    shallowest = std::min(shallowest, kb);
-    weights += 2.f * probs[i].N * probs[i].K;
+    kblocks = std::min(kblocks, (probs[i].K + GEMM_BK - 1) / GEMM_BK);
   }
-  auto up = [](int x, int y) { return (x + y - 1) / y; };
-  SplitConfig best{0, 1, 0};
-  float best_us = 1e30f;
-  int ctas = 0;
-  for (int tok_tiles = 1; tok_tiles <= 4; tok_tiles *= 2) {
-    const int nt = up(up(rows, tok_tiles), 16) * 16, tiles = columns * tok_tiles;
-    if (up(rows, nt) != tok_tiles) continue;
-    for (int split = 1; split <= 8; split *= 2) {
-      if (split > 1 && 2 * split > shallowest) break;
-      if (tiles * split > (tok_tiles == 1 && split < 8 ? 2 * sms : sms) && (tok_tiles > 1 || split > 1)) break;
-      const float over = std::max(0.f, float(tiles * split) / sms - 1.f);   // CTAs that share an SM
-      const float main = up(deepest, split) * (0.144f + 0.017f * nt / 128.f) * (1.f + 3.7f * over), memory = weights / 7.2e6f;
-      const float cluster = split == 1 ? 0.f : split == 2 ? 0.6f : split == 4 ? 0.83f : 10 * tiles * split > 7 * sms ? 6.6f : 0.88f;
-      const float us = sqrtf(main * main + memory * memory) + 0.0277f * nt + cluster + 0.098f * nt * over;
-      if (us >= best_us) continue;
-      best_us = us;
-      best.nt = nt;
-      best.split = split;
-      ctas = tiles * split;
-    }
+  auto tile = [&](int tiles) { return ((rows + tiles - 1) / tiles + 15) / 16 * 16; };
+  SplitConfig c{tile(1), 1, 1, 0};
+  while (c.split < 8 && 2 * c.split <= kblocks && columns * c.split < 128) c.split *= 2;
+  int ctas = columns * c.split;
+  auto fit = [&] { return c.split == 8 ? 13 * sms / 16 : c.split == 4 ? sms - 16 : sms; };
+  if (ctas > fit() && ctas <= sms) {
+    c.split /= 2;
+    c.parts = 2;
+    ctas /= 2;
+  }
+  for (int tiles = 2; tiles <= 4 && columns * c.split * tiles <= fit(); tiles *= 2) {
+    if ((rows + tile(tiles) - 1) / tile(tiles) != tiles) break;
+    c.nt = tile(tiles);
+    ctas = columns * c.split * tiles;
   }
   const int ring_bytes = (ctas <= sms ? 220 : 110) * 1024;
-  best.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SPLIT_B_BYTES + best.nt * GEMM_BK * 2));
-  return best;
+  c.stages = std::min(SPLIT_MAX_STAGES, ring_bytes / (SPLIT_B_BYTES + c.nt * GEMM_BK * 2));
+  return c;
 }
 
 // ------------------------------------------------------------------------------------------------------------

@@ -12,9 +12,16 @@ SINGLE, PAIR, TALL, SPLIT = range(4)
 
 
 def compiled(folder):
-    """choose(list of (M, N, K)) -> (kernel, tokens per tile, K split)."""
+    """choose(list of (M, N, K)) -> (kernel, tokens per tile, K split); and, up to 128 rows, split_choice(the same) ->
+    (tokens per tile, CTAs of a cluster, accumulators of a CTA, stages)."""
     (folder / "c.cpp").write_text("""#include "kvp_gemm_choice.h"
 using namespace kvp;
+extern "C" void split_choice(const int* mnk, int n, int* out) {
+  GemmSize g[32];
+  for (int i = 0; i < n; ++i) g[i] = GemmSize{mnk[3 * i], mnk[3 * i + 1], mnk[3 * i + 2]};
+  const SplitConfig c = split_config(g, n, 148);
+  out[0] = c.nt, out[1] = c.split, out[2] = c.parts, out[3] = c.stages;
+}
 extern "C" void choose(const int* mnk, int n, int* out) {
   GemmSize g[32];
   int rows = 0;
@@ -36,16 +43,23 @@ extern "C" void choose(const int* mnk, int n, int* out) {
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, str(folder / "c.cpp"), "-o", str(folder / "c.so")], check=True)
     lib = C.CDLL(str(folder / "c.so"))
 
-    def choose(problems):
-        out, flat = (C.c_int * 3)(), [x for p in problems for x in p]
-        lib.choose((C.c_int * len(flat))(*flat), len(problems), out)
-        return tuple(out)
-    return choose
+    def caller(f, size):
+        def call(problems):
+            out, flat = (C.c_int * size)(), [x for p in problems for x in p]
+            f((C.c_int * len(flat))(*flat), len(problems), out)
+            return tuple(out)
+        return call
+    return caller(lib.choose, 3), caller(lib.split_choice, 4)
 
 
 @pytest.fixture(scope="module")
-def choose(tmp_path_factory):
+def choices(tmp_path_factory):
     return compiled(tmp_path_factory.mktemp("choice"))
+
+
+@pytest.fixture(scope="module")
+def choose(choices):
+    return choices[0]
 
 
 def some_lists(seed, n=3000):
@@ -76,3 +90,35 @@ def test_pair_tiles_go_in_steps_of_32_tokens(choose):
     assert seen > 300
     source = open(os.path.join(CSRC, "kvp_gemm.cu")).read()
     assert "unit = g.a_mn ? 128 : TALL_UNIT" in source
+
+
+def test_bounds_of_the_few_rows_kernel(choices):
+    """What its launch and its blocks rely on: tokens per tile an MMA can have, a ring of two stages or more, accumulators
+    that fit tensor memory and sums that fit shared memory, half of both where CTAs share an SM."""
+    seen = set()
+    for problems in some_lists(3, 6000):
+        problems = [((m - 1) % 128 + 1, n, k) for m, n, k in problems]
+        nt, split, parts, stages = choices[1](problems)
+        seen.add((split, parts))
+        rows = max(m for m, _, _ in problems)
+        ctas = sum((n + 127) // 128 * ((m + nt - 1) // nt) for m, n, _ in problems) * split
+        assert 16 <= nt <= 128 and nt % 16 == 0 and nt < rows + 16
+        assert split in (1, 2, 4, 8) and parts in (1, 2) and split * parts <= 8
+        assert split == 1 or ctas < 2 * SMS, problems
+        assert parts == 1 or split > 1 and ctas <= SMS
+        ring = (220 if ctas <= SMS else 110) * 1024
+        assert 2 <= stages <= 8 and stages * (16384 + nt * 128) <= ring and parts * nt * 512 <= ring, problems
+        assert parts * max(nt, 32) <= (512 if ctas <= SMS else 256)
+    assert seen == {(1, 1), (2, 1), (4, 1), (8, 1), (2, 2), (4, 2)}
+
+
+def test_pieces_of_k_go_by_columns_and_depth(choices):
+    """The smallest power of two that gives 128 tiles, two k-blocks in each: the same for any number of rows."""
+    for problems in some_lists(4):
+        columns, depth = sum((n + 127) // 128 for _, n, _ in problems), min((k + 63) // 64 for _, _, k in problems)
+        pieces = 1
+        while pieces < 8 and 2 * pieces <= depth and columns * pieces < 128:
+            pieces *= 2
+        for rows in (1, 16, 17, 64, 128):
+            _, split, parts, _ = choices[1]([(rows, n, k) for _, n, k in problems])
+            assert split * parts == pieces, (rows, problems)

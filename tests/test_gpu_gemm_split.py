@@ -102,7 +102,13 @@ def test_gradient_gemms(L, own, S, D, Hq, Hkv):
 @pytest.fixture(scope="module")
 def choose(tmp_path_factory):
     from test_gemm_choice_host import compiled
-    return compiled(tmp_path_factory.mktemp("choice"))
+    return compiled(tmp_path_factory.mktemp("choice"))[0]
+
+
+@pytest.fixture(scope="module")
+def split_choice(tmp_path_factory):
+    from test_gemm_choice_host import compiled
+    return compiled(tmp_path_factory.mktemp("split"))[1]
 
 
 # (kernel, tokens per tile, K split) that a launch is to take: a change of the rules that moves a case off the edge it is
@@ -123,15 +129,58 @@ def test_each_forward_kernel_at_its_edges(choose, M, N, K, kernel):
     test_few_rows(M, N, K)
 
 
-# tokens per tile and K split of the kernel of few rows, at both sides of the line from which a warp sums several tokens
-# (more than twelve per CTA of the cluster), with short last tiles of tokens, columns and k-blocks
-@pytest.mark.parametrize("M,N,K,nt,split", [
-    (16, 136, 1032, 16, 8), (16, 8200, 520, 16, 1), (30, 2056, 2056, 16, 4), (33, 136, 1032, 32, 8), (33, 1032, 1032, 32, 4),
-    (70, 5512, 2056, 80, 2), (97, 4104, 4104, 64, 2), (128, 2056, 2056, 32, 2),
+# tokens per tile, CTAs of a cluster and accumulators of a CTA in the kernel of few rows: short last tiles of tokens, columns
+# and k-blocks, both sides of the line from which a warp sums several tokens at a time (more than twelve per CTA of clusters
+# of one and two), the longest tile with every cluster, rings of three stages (more CTAs than SMs)
+@pytest.mark.parametrize("M,N,K,nt,split,parts", [
+    (16, 136, 1032, 16, 8, 1), (16, 8200, 520, 16, 2, 1), (33, 8200, 520, 48, 2, 1), (30, 2056, 2056, 32, 4, 2), (33, 136, 1032, 32, 8, 1),
+    (33, 1032, 1032, 48, 8, 1), (70, 5512, 2056, 80, 4, 1), (97, 4104, 4104, 112, 4, 1), (128, 2056, 2056, 128, 4, 2),
+    (128, 2048, 2056, 64, 4, 2), (113, 4616, 648, 64, 2, 2), (17, 4616, 4104, 16, 2, 2), (9, 4616, 200, 16, 2, 2),
+    (127, 8, 8, 32, 1, 1), (65, 264, 72, 48, 2, 1), (113, 520, 136, 32, 2, 1), (97, 648, 200, 32, 4, 1), (65, 520, 520, 48, 8, 1),
+    (128, 17416, 72, 128, 1, 1), (113, 19208, 200, 128, 1, 1), (115, 8200, 4104, 128, 2, 1), (128, 11016, 136, 128, 2, 1),
+    (128, 4104, 8200, 128, 4, 1), (113, 5512, 520, 128, 4, 1), (115, 1544, 648, 128, 8, 1), (113, 2824, 520, 128, 8, 1),
 ])
-def test_few_rows_sums(choose, M, N, K, nt, split):
-    assert choose([(M, N, K)]) == (3, nt, split)
+def test_few_rows_sums(split_choice, M, N, K, nt, split, parts):
+    assert split_choice([(M, N, K)])[:3] == (nt, split, parts)
     test_few_rows(M, N, K)
+
+
+@pytest.mark.parametrize("N,K", [(8, 72), (136, 1032), (520, 520), (1544, 648), (2056, 2056), (2824, 8200), (5512, 4104), (11016, 136), (19208, 200)])
+def test_a_row_does_not_depend_on_the_number_of_rows(N, K):
+    """Up to 128 rows the pieces of K, with an accumulator each, go by the columns and the depth: a row has the same bits
+    whichever tiles and clusters the call takes.  """
+    from paper_2608_15943_b200 import kvp
+    a, b = synth.normal((128, K), 35, 1, 1.0, "cuda"), synth.normal((N, K), 35, 2, 1.0, "cuda")
+    whole = kvp.gemm(a, b, torch.full((128, N), float("nan"), device="cuda"))
+    for M in (1, 16, 17, 33, 64, 65, 100, 127):
+        few = kvp.gemm(a[:M], b, torch.full((M, N), float("nan"), device="cuda"))
+        assert torch.equal(few, whole[:M]), M
+    assert kvp.device_status() == kvp.OK
+
+
+# three problems of one launch, and six, of more than 96 rows
+@pytest.mark.parametrize("owners,D,Hq,Hkv,nt,split,parts", [
+    (1, 576, 2, 1, 32, 8, 1), (1, 1536, 24, 4, 64, 4, 2), (1, 2048, 32, 8, 128, 8, 1), (2, 1536, 8, 4, 64, 4, 2), (2, 192, 24, 8, 128, 2, 1),
+    (2, 576, 48, 8, 128, 2, 1),
+])
+def test_many_rows_of_grouped_projections(split_choice, owners, D, Hq, Hkv, nt, split, parts):
+    from paper_2608_15943_b200 import kvp
+    B, dh = 113, 64
+    assert split_choice([(B, Hq * dh, D), (B, Hkv * dh, D), (B, Hkv * dh, D)] * owners)[:3] == (nt, split, parts)
+    sh = kvp.Shape(owners, B, 1, D, Hq, Hkv, dh)
+    x = [synth.normal((B, D), 36, synth.tid(0, l), 1.0, "cuda") for l in range(owners)]
+    w = {n: [synth.normal((h * dh, D), 36, synth.tid(i, l), 1.0, "cuda") for l in range(owners)]
+         for i, (n, h) in enumerate((("q", Hq), ("k", Hkv), ("v", Hkv)), 1)}
+    gd = Guarded()
+    out = {n: [gd.empty((B, 1, h, dh), torch.bfloat16, float("nan")) for _ in range(owners)] for n, h in (("q", Hq), ("k", Hkv), ("v", Hkv))}
+    kvp.proj_fwd(sh, list(range(owners)), x, w["q"], w["k"], w["v"], out["q"], out["k"], out["v"])
+    gd.check()
+    assert kvp.device_status() == kvp.OK
+    for l in range(owners):
+        for n in ("q", "k", "v"):
+            ref = x[l].double() @ w[n][l].double().T
+            bound = D * 2.0 ** -24 * (x[l].double().abs() @ w[n][l].double().abs().T)     # as test_few_rows
+            assert ((out[n][l].view(B, -1).double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all(), (n, l)
 
 
 @pytest.mark.parametrize("mode", [0, 2])
