@@ -474,9 +474,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
 // Measured (us, K x N at M tokens; 128 x 256 tiles -> this kernel; reading B at the copy rate): 4096 x 4096 at 16
 // tokens 28.7 -> 11.6 (5.2), 4096 x 11008 at 16 30.8 -> 20.6 (13.9), 11008 x 4096 at 16 65.5 -> 20.6 (13.9), 4096 x
 // 4096 at 128 28.9 -> 14.5 (5.5); a launch that does almost nothing takes 6.
-// Where a warp has more than two tokens to sum it takes four at a time with the parts of two CTAs: one token and part after
-// the other, each waiting for the other CTA's shared memory, took 4.5 of the 16 us of 347 x 4096 x 4096 (back to back 21.2 ->
-// 16.8; 347 x 4096 x 11008 40.8 -> 32.8).
+// In clusters of one and two, where a warp has more than two tokens to sum, it takes four at a time with two partials: one
+// token and partial after the other, each waiting for the other CTA's shared memory, took 4.5 of the 16 us of 347 x 4096 x 4096
+// (back to back 21.2 -> 16.8; 347 x 4096 x 11008 40.8 -> 32.8).  In larger clusters a warp has fewer tokens, and the longer code
+// takes more to fetch than it saves: 129 x 4096 x 4096, four CTAs, 13.7 -> 14.5, 128 x 1024 x 1024, eight, 8.0 -> 9.3.
 // ------------------------------------------------------------------------------------------------------------
 constexpr int SROWS = SPLIT_COLS;                // rows of B (output columns) per tile: the M of the MMA
 constexpr int SB_BYTES = SPLIT_B_BYTES;          // 16 KB
@@ -504,7 +505,7 @@ struct SplitParams {
   uint32_t idesc;
 };
 
-// WIDE: a warp has more than two tokens to sum.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.
+// WIDE: four tokens a warp at a time.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.
 template <int NP, bool WIDE, int PARTS>
 __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
   extern __shared__ uint8_t smem_raw[];
@@ -1074,7 +1075,7 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.parts * cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
-  const bool wide = cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
+  const bool wide = cfg.split <= 2 && cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
   auto* const kernel = cfg.parts == 2 ? (wide ? split_kernel<NP, true, 2>() : split_kernel<NP, false, 2>())
                                       : (wide ? split_kernel<NP, true, 1>() : split_kernel<NP, false, 1>());
   if (kernel == nullptr) return KVP_ERR_CUDA;
