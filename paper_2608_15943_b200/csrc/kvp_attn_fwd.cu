@@ -550,7 +550,7 @@ int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* con
                     const void* const* v, void* const* o, bool o_f32, float* const* lse, int n, cudaStream_t stream) {
   if (n < 1 || n > FWD_MAX_LAYERS) return KVP_ERR_INVALID_ARG;
   static thread_local FwdParams p;   // 3 KB of tensor maps: kept off the stack
-  const FwdSizes sizes{s->S, s->Hq / s->Hkv, causal != 0, (long long)n * s->B * s->Hkv, sm_count()};
+  const FwdSizes sizes{s->S, s->Hq / s->Hkv, s->dh, causal != 0, (long long)n * s->B * s->Hkv, sm_count()};
   p.pack = fwd_pack(sizes);
   for (int i = 0; i < n; ++i) {
     int rc = make_map_bshd(&p.map_q[i], q[i], s->B, s->S, s->Hq, s->dh, BQ >> p.pack, 1 << p.pack);

@@ -10,6 +10,7 @@ constexpr int FWD_MAX_PACK = 4;    // log2 of the heads that share a tile at mos
 
 struct FwdSizes {
   int S, G;                // tokens; query heads per KV head
+  int dh;
   bool causal;
   long long kv_heads;      // of the launch: layers x batch x KV heads
   int sms;
@@ -53,16 +54,21 @@ inline FwdTime fwd_time(const FwdSizes& z, int pack) {
 
 // Tiles of several heads waste less on the last, part-filled tile of a sequence and on the keys that a causal mask hides from
 // a tile's first rows; both matter for short sequences only, and where the launch has fewer items than SMs an item's own time
-// counts.  With a mask the two tiles of an item also walk the same number of key tiles, which gains where the estimate says
-// that nothing changes, if there are items enough.  Measured over 208 shapes (heads packed / not, geometric mean, extremes):
-// where this says so 0.947 (0.80, 1.004), elsewhere 1.04 (0.95, 1.39); 3 x 776 tokens, 16 heads of 64 on 4, three layers 35.7
-// -> 31.6 us.
+// counts.  With a mask the two tiles of an item also walk the same number of key tiles, which gains at heads of 64 where the
+// estimate says that nothing changes, if there are items enough.  At heads of 128 and without a mask the packed kernel itself
+// takes up to a tenth longer for the same key tiles (long launches, against the estimate: causal heads of 64 1.00, full
+// attention 1.05 to 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an eighth.
+// Measured on 1660 shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so): launches of up to
+// a millisecond 0.79, 2 % of them more than 3 % slower, 1.08 at most; longer ones 0.95, 1.04 at most; 3 x 776 tokens, 16 heads of
+// 64 on 4, three layers 35.7 -> 31.6 us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
+// average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 -> 2.78 ms).
 constexpr int FWD_PACK_TOKENS = 2048;
 inline int fwd_pack(const FwdSizes& z) {
   const int pack = fwd_most_pack(z.G);
   if (pack == 0 || z.S > FWD_PACK_TOKENS) return 0;
   const FwdTime heads = fwd_time(z, pack), head = fwd_time(z, 0);
-  const bool even = z.causal && heads.average > (z.S < 1024 ? 1.4f : 1.f) * heads.longest && heads.total() <= head.total();
+  if (!z.causal || z.dh > 64) return heads.total() < 0.88f * head.total() ? pack : 0;
+  const bool even = heads.average > (z.S < 1024 ? 1.4f : 1.f) * heads.longest && heads.total() <= head.total();
   return heads.total() < 0.97f * head.total() || even ? pack : 0;
 }
 

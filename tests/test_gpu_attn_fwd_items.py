@@ -1,12 +1,9 @@
 """Attention forward with more work items than CTAs: the roles of a CTA walk several items in a row."""
-import ctypes as C
-import subprocess
-
 import pytest
 import torch
 
 from oracle import attention as A
-from test_bwd_shape_host import CSRC
+from test_fwd_shape_host import compiled
 from test_gpu_parity import attn_inputs, close, f64l, lse_close
 
 pytestmark = pytest.mark.gpu
@@ -38,14 +35,7 @@ def test_items_of_an_odd_number_of_query_tiles(B, S, Hq, Hkv, dh, donor, causal)
 
 @pytest.fixture(scope="module")
 def pack_of(tmp_path_factory):
-    d = tmp_path_factory.mktemp("fwd")
-    (d / "r.cpp").write_text("""#include "kvp_fwd_shape.h"
-extern "C" int pack_of(int B, int S, int Hq, int Hkv, int L, int causal) {
-  return kvp::fwd_pack(kvp::FwdSizes{S, Hq / Hkv, causal != 0, (long long)L * B * Hkv, 148});
-}
-""")
-    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, str(d / "r.cpp"), "-o", str(d / "r.so")], check=True)
-    return C.CDLL(str(d / "r.so")).pack_of
+    return compiled(tmp_path_factory.mktemp("fwd"))
 
 
 # tiles of 1 << pack heads; the sequence ends in a tile's first token, its last, or between
@@ -53,17 +43,33 @@ extern "C" int pack_of(int B, int S, int Hq, int Hkv, int L, int causal) {
     (20, 257, 4, 2, 64, [0], True, 1),       # 64 tokens of two heads: five tiles, the last of one token
     (9, 161, 24, 4, 128, [0], True, 1),      # six heads to a KV head: three groups of two
     (6, 140, 16, 8, 64, [0, 0], False, 1),   # full attention
-    (9, 129, 8, 2, 128, [0, 1], True, 2),    # 32 tokens of four heads, the last tile of one token
+    (10, 129, 8, 2, 128, [0, 1], True, 2),    # 32 tokens of four heads, the last tile of one token
     (10, 264, 8, 2, 64, [0], True, 2),
+    (8, 145, 16, 2, 128, [0, 0], True, 3),   # 16 tokens of eight heads, the last tile of one token
+    (4, 272, 24, 3, 64, [0], True, 3),       # every tile full
+    (10, 264, 8, 1, 64, [0, 0], False, 3),   # the last tile half full
     (12, 33, 32, 2, 128, [0, 0], True, 4),   # eight tokens of sixteen heads, five tiles for one key tile
     (5, 264, 32, 2, 64, [0], False, 4),      # every tile full
 ])
 def test_tiles_of_several_heads(pack_of, B, S, Hq, Hkv, dh, donor, causal, pack):
-    assert pack_of(B, S, Hq, Hkv, len(donor), int(causal)) == pack
+    assert pack_of(B, S, Hq, Hkv, dh, len(donor), int(causal)) == pack
     test_items_of_an_odd_number_of_query_tiles(B, S, Hq, Hkv, dh, donor, causal)
 
 
-def test_heads_stay_by_themselves_where_nothing_is_gained(pack_of):
-    assert pack_of(1, 300, 16, 4, 1, 1) == 0      # 20 items instead of 32, and longer ones
-    assert pack_of(2, 512, 32, 8, 2, 1) == 0
-    assert pack_of(2, 8192, 32, 8, 8, 1) == 0 and pack_of(4, 347, 32, 32, 1, 1) == 0
+@pytest.mark.parametrize("B,S,Hq,Hkv,dh,pack", [(20, 257, 4, 2, 64, 1), (10, 257, 8, 2, 128, 2), (4, 272, 24, 3, 64, 3)])
+def test_fp32_interface_with_tiles_of_several_heads(pack_of, B, S, Hq, Hkv, dh, pack):
+    """fp32 tensors that hold bf16 values: the same bits as through the bf16 interface."""
+    from paper_2608_15943_b200 import kvp
+    assert pack_of(B, S, Hq, Hkv, dh, 1, 1) == pack
+    q, k, v, _ = attn_inputs(B, S, Hq, Hkv, dh, [0])
+    results = []
+    for dtype, code in ((torch.bfloat16, kvp.BF16), (torch.float32, kvp.F32)):
+        sh = kvp.Shape(1, B, S, 64, Hq, Hkv, dh, code)
+        ws = torch.empty(max(256, kvp.workspace_bytes(kvp.OP_ATTN_FWD, sh, [0])), dtype=torch.uint8, device="cuda")
+        o = torch.full(q[0].shape, float("nan"), dtype=dtype, device="cuda")
+        lse = torch.full((B, Hq, S), float("nan"), device="cuda")
+        kvp.attn_fwd(sh, [0], [q[0].to(dtype)], [k[0].to(dtype)], [v[0].to(dtype)], [o], [lse], ws=ws)
+        torch.cuda.synchronize()
+        assert kvp.device_status() == kvp.OK
+        results.append((o.float(), lse))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
