@@ -150,24 +150,35 @@ def test_a_long_sequence_among_short_ones(lens, Hkv, dh, page):
     ([700] * 33, [700] * 32 + [8000], 2, 64, 16),         # more lengths than a warp's lanes
 ])
 def test_lengths_written_by_the_kernel_ahead(first, second, Hkv, dh, page):
-    """The lengths are looked at before the kernel ahead has finished; what it writes counts.  It is the library's own add
-    (whose CTAs let the next kernel come up early) over the lengths' bits as bf16 numbers, plus zero."""
+    """The lengths are looked at before the kernel ahead has finished; what it writes counts.  It is the library's GEMM of one
+    row, whose blocks let the next kernel come up as soon as they are set up, and which then takes tens of microseconds on
+    eight SMs: its one-hot row picks a row of bf16 numbers whose bits are those of the lengths (from 128 on, all of them
+    normal), in turn those of one list and the other's."""
     from paper_2608_15943_b200 import kvp
     longest = [max(a, b) for a, b in zip(first, second)]
     kc, vc, bt = paged(longest, Hkv, dh, page, 74)
     q = synth.normal((len(first), 4 * Hkv, dh), 74, 3, 1.0, "cuda")
     want = [exact_on_gpu(q, kc, vc, bt, lens, page) for lens in (first, second)]
-    pad = -len(first) % 4                                 # 16-byte pieces
-    bits = [torch.tensor(lens + [0] * pad, dtype=torch.int32, device="cuda").view(torch.bfloat16) for lens in (first, second)]
-    lengths, zero = bits[1].clone(), torch.zeros_like(bits[0])
+    pad, K = -len(first) % 4, 1 << 17                      # 16-byte rows
+    bits = torch.tensor([lens + [0] * pad for lens in (first, second)], dtype=torch.int32, device="cuda").view(torch.bfloat16)
+    assert all(128 <= n < 32640 for n in first + second)
+    table_of = torch.zeros(bits.shape[1], K, dtype=torch.bfloat16, device="cuda")
+    table_of[:, 0], table_of[:, K - 1] = bits[0], bits[1]
+    pick = torch.zeros(2, 1, K, dtype=torch.bfloat16, device="cuda")
+    pick[0, 0, 0] = pick[1, 0, K - 1] = 1.0
+    lengths = bits[1:].clone()
     desc = kvp.DecodeDesc(1, len(first), 4 * Hkv, Hkv, dh, page, bt.shape[1], kc.shape[0])
     ws = torch.empty(kvp.decode_workspace_bytes(desc, [0]), dtype=torch.uint8, device="cuda")
     table = bt.cuda()
     out = [(torch.full_like(q, float("nan")), torch.full(q.shape[:2], float("nan"), device="cuda")) for _ in range(20)]
+    seen = [torch.empty_like(lengths) for _ in out]
+    torch.cuda.synchronize()
     for i, (o, lse) in enumerate(out):
-        kvp.add(bits[i % 2], zero, lengths)
-        kvp.decode(desc, [0], [q], [kc], [vc], table, lengths.view(torch.int32)[:len(first)], [o], [lse], ws)
+        kvp.gemm(pick[i % 2], table_of, lengths)
+        kvp.decode(desc, [0], [q], [kc], [vc], table, lengths.view(torch.int32).view(-1)[:len(first)], [o], [lse], ws)
+        seen[i].copy_(lengths)
     assert kvp.device_status() == kvp.OK
     for i, (o, lse) in enumerate(out):
+        assert torch.equal(seen[i].view(torch.int32), bits[i % 2:i % 2 + 1].view(torch.int32))
         ro, rl = want[i % 2]
         assert (o.double() - ro).norm() <= REL * ro.norm() and (lse.double() - rl).abs().max() <= 2e-6, i
