@@ -60,7 +60,8 @@ struct FwdSmem {
 constexpr int FWD_MAX_LAYERS = 8;   // layers per launch
 
 struct FwdParams {
-  // per layer: 4-D [B, S, H, dh] tensors, box {64, 1, 128, 1}; K and V are those of the layer's donor
+  // per layer: 4-D [B, S, H, dh] tensors; K and V are those of the layer's donor, in boxes of {64, 1, 128, 1}, Q in boxes of
+  // {64, h, 128 / h, 1} for the h heads that share a tile
   CUtensorMap map_q[FWD_MAX_LAYERS], map_k[FWD_MAX_LAYERS], map_v[FWD_MAX_LAYERS];
   void* o[FWD_MAX_LAYERS];           // [B, S, Hq, dh], bf16 or (o_f32) the bf16 values as fp32
   float* lse[FWD_MAX_LAYERS];        // [B, Hq, S]
@@ -498,7 +499,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) attn_fwd_kernel(const __grid_c
       ok = __all_sync(0xffffffffu, ok);
       if (ok && my_n > 0) {
         const float l_sum = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
-        if (q_row < p.S) p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq + x * w.dhq + (r & in_pack)) * p.S + q_row] = (m_used + log2f(l_sum)) * 0.6931471805599453f;
+        if (q_row < p.S)
+          p.lse[w.layer][(size_t(w.b) * p.Hq + w.hq + x * w.dhq + (r & in_pack)) * p.S + q_row] =
+              (m_used + log2f(l_sum)) * 0.6931471805599453f;
         ok = n_done == 0 || mbar_wait(&o_free[x], (n_done - 1) & 1, err);   // the epilogue warps have read the last item's
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         inv_sum[x * BQ + r] = 1.f / l_sum;

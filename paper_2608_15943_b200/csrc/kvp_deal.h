@@ -11,7 +11,7 @@
 
 namespace kvp {
 
-// (nearly all dividends fit 32 bits, where a division takes a fifth of the time)
+// (nearly all dividends fit 32 bits, and all divisors, where a division takes a fifth of the time)
 KVP_HD inline long long div_places(long long a, long long b) {
   return (a | b) >> 32 == 0 ? (long long)(unsigned(a) / unsigned(b)) : a / b;
 }

@@ -110,17 +110,14 @@ __device__ __forceinline__ int early_length(const DecParams& p) {
   return lane < p.B ? __ldcg(p.lengths + lane) : 0;
 }
 // The first T mod n of n shares of a list of T granules hold one more than the others.
-__device__ __forceinline__ uint32_t div_long(long long a, uint32_t b) {   // quotients here fit 32 bits; so do nearly all dividends
-  return a <= 0xffffffffll ? uint32_t(a) / b : uint32_t(a / b);
-}
 struct Dealt {
   uint32_t q, r;
-  __device__ __forceinline__ Dealt(long long total, uint32_t n) : q(div_long(total, n)), r(uint32_t(total - (long long)q * n)) {}
+  __device__ __forceinline__ Dealt(long long total, uint32_t n) : q(uint32_t(div_places(total, n))), r(uint32_t(total - (long long)q * n)) {}
   __device__ __forceinline__ long long begin(uint32_t i) const { return (long long)i * q + min(i, r); }
   __device__ __forceinline__ uint32_t size(uint32_t i) const { return q + (i < r ? 1u : 0u); }
   __device__ __forceinline__ int share_of(long long g) const {
     const long long longer = (long long)r * (q + 1);
-    return g < longer ? int(div_long(g, q + 1)) : int(r + div_long(g - longer, q));
+    return g < longer ? int(div_places(g, q + 1)) : int(r + div_places(g - longer, q));
   }
 };
 
@@ -224,7 +221,7 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
     long long at = dealt.begin(blockIdx.x);
     todo = int(dealt.size(blockIdx.x));
     c.id = 0;
-    c.grp = int(div_long(at, uint32_t(per_group)));
+    c.grp = int(div_places(at, per_group));
     at -= c.grp * per_group;                       // inside the group: find the sequence, 32 lengths at a time
     for (int b0 = 0;; b0 += 32) {
       const int len = b0 + lane < p.B ? clamp_length(p, b0 == 0 ? len0 : p.lengths[b0 + lane]) : 0;

@@ -3,8 +3,8 @@
 //
 // One persistent CTA per SM walks 128 x 256 output tiles.  Warp 0 issues TMA loads into a
 // 4-stage shared-memory ring, warp 1 issues tcgen05.mma into one of two 256-column TMEM
-// accumulators, warps 2-5 drain the other accumulator (tcgen05.ld -> registers -> global), so
-// the epilogue of tile i overlaps the main loop of tile i+1.  Either operand may be K-major or
+// accumulators, warps 2-5 drain the other accumulator (tcgen05.ld -> registers -> shared memory ->
+// TMA stores), so the epilogue of tile i overlaps the main loop of tile i+1.  Either operand may be K-major or
 // MN-major in memory; that only changes the TMA box and the shared-memory descriptor.
 // The K extent may be split over up to three operand pairs ("segments") that accumulate into the
 // same tile, which is how dX = dQ Wq + dK Wk + dV Wv is produced with one output pass.
@@ -438,8 +438,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
       bool ok = mbar_wait(&acc_full[acc], acc_ph, err, p.wait_limit_ns);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
-      store_rows(&p.map_c[pi], tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN, tm * PBM + int(rank) * PHALF + quarter * 32, pr.M, tn * BN, pr.N,
-                 pr.out_f32, epi + quarter * 8192, pieces, [&]() {
+      store_rows(&p.map_c[pi], tmem_base + (uint32_t(quarter * 32) << 16) + acc * BN, tm * PBM + int(rank) * PHALF + quarter * 32,
+                 pr.M, tn * BN, pr.N, pr.out_f32, epi + quarter * 8192, pieces, [&]() {
                    tc_fence_before_sync();
                    __syncwarp();
                    if (lane == 0) mbar_arrive_cluster(cluster_addr_of(&acc_empty[acc], 0));
@@ -975,7 +975,7 @@ int encode_operand(CUtensorMap* map, const void* base, int64_t ld, int rows, int
 int launch_group(const GemmProblem* probs, int n, cudaStream_t stream, int withhold_at, unsigned long long wait_limit_ns,
                  bool pair) {
   const int bm = pair ? PBM : BM;
-  static thread_local GemmParams p;   // 15 KB: kept off the stack
+  static thread_local GemmParams p;   // 19 KB: kept off the stack
   p.nprob = n;
   p.withhold_at = withhold_at;
   p.wait_limit_ns = wait_limit_ns != 0 ? wait_limit_ns : kWaitLimitNs;

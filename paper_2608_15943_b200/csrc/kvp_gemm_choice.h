@@ -68,8 +68,10 @@ inline SplitConfig split_config(const GemmSize* probs, int n, int sms) {
 // ------------------------------------------------------------------------------------------------------------
 // Which kernel a forward GEMM of more than 128 rows runs on.  The times (us) of each are estimated from a model with the
 // terms that bound it -- launches and tiles at fixed cost, an SM's share of L2 bandwidth, the tensor pipe, memory -- whose
-// constants were fitted to 3400 measurements (11 weight shapes x 28 row counts, weights not in L2).  The choice it makes
-// costs 0.7 % more than the best of all choices on average, CTA pairs always 50 %.  From PAIR_ROUNDS rounds of pair tiles on
+// constants were fitted to 3400 measurements (11 weight shapes x 28 row counts, weights not in L2) before the split kernel's
+// sum and the tile kernels' stores were shortened.  On the kernels as they are the choice costs 0.6 % more than the best of all
+// choices on average over 15 weight shapes x 14 row counts (11 % at most; CTA pairs always 38 %), 1.2 % over 31 shapes that
+// the fit never saw (10 %; 52 %).  From PAIR_ROUNDS rounds of pair tiles on
 // and above 4096 rows the pairs' order of tiles (an A slab stays in L2) counts, and they stand: 3000 rows x 32000 x 4096 508
 // us on them, 597 in tiles of one size.
 // ------------------------------------------------------------------------------------------------------------
@@ -122,7 +124,7 @@ inline Choice choose_forward(const GemmSize* probs, int n, int sms) {
     const int most = (split == 4 ? sms - 16 : sms) / (split * cols128);   // token tiles that fit
     if (most < 1) break;
     const int nt = std::max(48, up(up(M, most), 16) * 16);
-    if (nt > 224) continue;   // (longer tiles draw more from L2 than the model says: 900 x 4096 x 11008 76 us for 65)
+    if (nt > 224) continue;   // (longer tiles draw more from L2 than the model says: 1000 x 4096 x 11008 82 us for 74)
     consider(Choice::kSplit, nt, split, 4.7f + std::max(float(kb) / split * 0.11f * (1.f + nt / 128.f), (weights + rows) / 9.6e6f) +
                                                    0.027f * nt + (split > 1 ? 0.75f : 0.f));
   }

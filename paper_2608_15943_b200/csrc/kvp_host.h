@@ -105,7 +105,8 @@ struct SameType { using type = T; };   // keeps the argument types of launch_ker
 
 // Every kernel of the library is launched through this: programmatic stream serialisation lets its CTAs come up (barriers,
 // tensor-memory allocation, descriptor fetches) while the kernel before it on the stream drains.  The kernel must
-// execute grid_dep_wait() before it touches global memory, and grid_dep_launch() so that the next kernel may do the same:
+// execute grid_dep_wait() before it relies on or changes global memory (decode and its merge look at the lengths ahead of it,
+// and again behind it), and grid_dep_launch() so that the next kernel may do the same:
 // the long ones when their last loads are out, the short ones (split GEMM, cache append, merge of decode pieces) as soon as
 // a CTA is set up.  (Any thread's grid_dep_launch() counts for its CTA.  Given at set-up by the long ones too, it parked
 // the next kernel's CTAs on the SMs for the whole of each, and the 46 ms training step of 2 x 8192 tokens took 1.2 ms

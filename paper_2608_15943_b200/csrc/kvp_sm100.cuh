@@ -25,9 +25,10 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // Programmatic dependent launch.  Between the two calls a kernel may only set up its own CTA (shared memory, barriers,
-// tensor memory, kernel parameters, prefetches, or work that it checks against memory again behind the wait): after grid_dep_wait() everything the kernels before it on the stream
-// wrote is visible, and everything they read may be overwritten.  EVERY thread block executes grid_dep_wait(), so that
-// the completion of a kernel implies the completion of all kernels before it.  So a kernel's inputs change while it lives:
+// tensor memory, kernel parameters, prefetches, or work that it checks against memory again behind the wait): after
+// grid_dep_wait() everything the kernels before it on the stream wrote is visible, and everything they read may be
+// overwritten.  EVERY thread block executes grid_dep_wait(), so that the completion of a kernel implies the completion of all
+// kernels before it.  So a kernel's inputs change while it lives:
 // no pointer to them is qualified __restrict__, which would let the compiler take them for constant and load them early,
 // through the read-only path or across the wait.  (Outputs may also be inputs: the element-wise operators work in place.)
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
