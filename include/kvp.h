@@ -87,8 +87,8 @@ int kvp_set_timing_events(int kernel, void** starts, void** stops, int n);
 int kvp_timing_events_used(int kernel);
 /* Measurement switch of the GEMM's tile shape.  1 (the default): forward GEMMs (K-major operands) run on CTA pairs
  * (256 x 256 tiles, one per pair of SMs), or up to 4096 rows and sixteen rounds of such tiles on whichever of the
- * library's kernels an estimate of their times prefers; the gradient GEMMs on pairs that own 256 columns, large launches (more than 0.5 TFLOP) on single-CTA
- * 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: 256 x 256 tiles on CTA pairs for every launch whose problems all
+ * library's kernels an estimate of their times prefers; the gradient GEMMs on pairs that own 256 columns, large launches
+ * (more than 0.5 TFLOP) on single-CTA 128 x 256 tiles.  0: single-CTA tiles everywhere; 2: 256 x 256 tiles on CTA pairs for every launch whose problems all
  * have more than 128 rows.  (K-major problems of at most 128 rows have a kernel of their own in every mode.)  The tile
  * kernels sum the same products in the same order along K in every mode; up to 4096 rows K may be split over a cluster of
  * CTAs, whose partial sums are added in a fixed order.  Not thread-safe. */
@@ -245,7 +245,8 @@ int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal, float sca
  * (C = A B^T in storage terms), else stored [K,N].  out_f32: C fp32, else bf16.  Leading dimensions
  * in elements, multiples of 8; K a multiple of 8.  The paper's 2mkn matrix-multiplication rule.
  * The kernel, and whether K is summed in parts, follow from the sizes of the whole launch (K-major operands, up to 4096
- * rows): a row's last bits can differ between calls with different numbers of rows, never between equal calls.  The
+ * rows).  Up to 128 rows the parts go by the columns and depths of the launch alone, and a row has the same bits in calls of
+ * 1 to 128 rows; beyond, its last bits can differ between calls with different numbers of rows, never between equal calls.  The
  * projections (kvp_proj_fwd, kvp_out_proj_fwd) run on the same kernels. */
 int kvp_gemm(int M, int N, int K, const void* a, int64_t lda, int a_mn, const void* b, int64_t ldb, int b_mn,
              void* c, int64_t ldc, int out_f32, kvp_stream_t stream);

@@ -60,7 +60,7 @@ inline FwdTime fwd_time(const FwdSizes& z, int pack) {
 // attention 1.05 to 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an eighth.
 // Measured on 1660 shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so): launches of up to
 // a millisecond 0.79, 2 % of them more than 3 % slower, 1.08 at most; longer ones 0.95, 1.04 at most; 3 x 776 tokens, 16 heads of
-// 64 on 4, three layers 35.7 -> 31.6 us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
+// 64 on 4, three layers 35.2 -> 31.3 us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
 // average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 -> 2.78 ms).
 constexpr int FWD_PACK_TOKENS = 2048;
 inline int fwd_pack(const FwdSizes& z) {
