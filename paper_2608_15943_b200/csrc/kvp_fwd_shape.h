@@ -28,48 +28,62 @@ inline bool fwd_odd_by_heads(const FwdSizes& z, int pack) {
   return pack == 0 && z.G % 2 == 0 && z.kv_heads * z.G * ((tiles + 1) / 2) > z.sms;
 }
 
-// A launch's time in units of a key tile of a work item (two query tiles): the average over the SMs, but no less than the
-// longest item.  An item costs one unit besides its key tiles, and an item of one query tile 0.6 of a unit for each.
-struct FwdTime {
-  float average, longest;
-  float total() const { return std::max(average, longest); }
-};
-inline FwdTime fwd_time(const FwdSizes& z, int pack) {
+// A launch's time in units of a key tile of a work item (two query tiles).  An item costs one unit besides its key tiles, and
+// an item of one query tile 0.6 of a unit for each.  Up to FWD_ROUNDS rounds of items the list is dealt out as the kernel does it
+// (longest first, rounds in alternating direction, one CTA per SM), and the fullest CTA counts; beyond, the average.
+constexpr int FWD_ROUNDS = 6;
+inline float fwd_time(const FwdSizes& z, int pack) {
   const int rows = FWD_ROWS >> pack, tiles = (z.S + rows - 1) / rows;
+  const long long groups = z.kv_heads * (z.G >> pack);
+  const bool by_heads = fwd_odd_by_heads(z, pack);
+  // the list: the last of an odd number of tiles, then the pairs of tiles from the end of the sequence on
+  const long long n_odd = tiles & 1 ? (by_heads ? groups / 2 : groups) : 0, n = n_odd + groups * (tiles / 2);
   auto key_tiles = [&](int t) { return ((z.causal ? std::min(z.S, (t + 1) * rows) : z.S) + FWD_ROWS - 1) / FWD_ROWS; };
-  float sum = 0.f, longest = 0.f;
-  for (int t = 0; t + 1 < tiles; t += 2) {
-    const float cost = 1.f + 0.5f * (key_tiles(t) + key_tiles(t + 1));
-    sum += cost;
-    longest = std::max(longest, cost);
+  const float odd = n_odd > 0 ? 1.f + (by_heads ? 1.f : 0.6f) * key_tiles(tiles - 1) : 0.f;
+  auto pair = [&](int k) { return 1.f + 0.5f * (key_tiles((tiles & ~1) - 2 - 2 * k) + key_tiles((tiles & ~1) - 1 - 2 * k)); };
+  const int pairs = tiles / 2;
+  const float longest = std::max(odd, pairs > 0 ? pair(0) : 0.f);
+  if (n <= z.sms) return longest;
+  const int sms = z.sms;
+  if (n > (long long)FWD_ROUNDS * sms) {
+    float sum = float(n_odd) * odd;
+    for (int k = 0; k < pairs; ++k) sum += float(groups) * pair(k);
+    return std::max(sum / float(sms), longest);
   }
-  if (tiles & 1) {
-    const bool by_heads = fwd_odd_by_heads(z, pack);
-    const float cost = 1.f + (by_heads ? 1.f : 0.6f) * key_tiles(tiles - 1);
-    sum += by_heads ? 0.5f * cost : cost;
-    longest = std::max(longest, cost);
+  const int items = int(n), first = int(n_odd), per = int(groups);
+  auto cost = [&](int i) { return i < first ? odd : pair((i - first) / per); };
+  auto load = [&](int cta) {
+    float sum = 0.f;
+    for (int r = 0, at = 0; at < items; ++r, at += sms) {
+      const int i = at + (r & 1 ? sms - 1 - cta : cta);
+      if (i < items) sum += cost(i);
+    }
+    return sum;
+  };
+  // neighbouring CTAs differ only where the cost changes along the list, or the list ends
+  float most = std::max(load(0), load(sms - 1));
+  auto look = [&](int i) { most = std::max(most, load((i / sms) & 1 ? sms - 1 - i % sms : i % sms)); };
+  for (int at = first; at <= items; at += per) {
+    if (at > 0) look(at - 1);
+    look(at);
   }
-  return FwdTime{sum * float(z.kv_heads * (z.G >> pack)) / z.sms, longest};
+  return most;
 }
 
 // Tiles of several heads waste less on the last, part-filled tile of a sequence and on the keys that a causal mask hides from
-// a tile's first rows; both matter for short sequences only, and where the launch has fewer items than SMs an item's own time
-// counts.  With a mask the two tiles of an item also walk the same number of key tiles, which gains at heads of 64 where the
-// estimate says that nothing changes, if there are items enough.  At heads of 128 and without a mask the packed kernel itself
-// takes up to a tenth longer for the same key tiles (long launches, against the estimate: causal heads of 64 1.00, full
-// attention 1.05 to 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an eighth.
-// Measured on 1660 shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so): launches of up to
-// a millisecond 0.79, 2 % of them more than 3 % slower, 1.08 at most; longer ones 0.95, 1.04 at most; 3 x 776 tokens, 16 heads of
-// 64 on 4, three layers 35.2 -> 31.3 us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
-// average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 -> 2.78 ms).
+// a tile's first rows; both matter for short sequences only.  At heads of 128 and without a mask the packed kernel itself takes up
+// to a tenth longer for the same key tiles (long launches, against the estimate: causal heads of 64 1.00, full attention 1.05 to
+// 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an eighth.  Measured on 1660
+// shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so): launches of up to a
+// millisecond 0.76, 1.03 at most, longer ones 0.93, 0.99 at most, on 428 packed ones drawn afterwards 0.77, 1.03; 3 x 776 tokens, 16 heads of 64 on 4, three layers 35.2 -> 31.3
+// us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
+// average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 -> 2.78 ms); with the average over the SMs in the
+// place of the fullest CTA, launches of one or two rounds lost up to 12 % (2 x 203 tokens, 64 heads of 128 on 8, two layers).
 constexpr int FWD_PACK_TOKENS = 2048;
 inline int fwd_pack(const FwdSizes& z) {
   const int pack = fwd_most_pack(z.G);
   if (pack == 0 || z.S > FWD_PACK_TOKENS) return 0;
-  const FwdTime heads = fwd_time(z, pack), head = fwd_time(z, 0);
-  if (!z.causal || z.dh > 64) return heads.total() < 0.88f * head.total() ? pack : 0;
-  const bool even = heads.average > (z.S < 1024 ? 1.4f : 1.f) * heads.longest && heads.total() <= head.total();
-  return heads.total() < 0.97f * head.total() || even ? pack : 0;
+  return fwd_time(z, pack) < (z.causal && z.dh == 64 ? 0.97f : 0.88f) * fwd_time(z, 0) ? pack : 0;
 }
 
 }  // namespace kvp

@@ -36,6 +36,8 @@ def test_heads_stay_by_themselves_where_nothing_is_gained(pack_of):
     (10, 1948, 128, 8, 128, 3, False, False),   # 7.49, 8.25
     (2, 1606, 16, 1, 64, 4, False, False),      # 135 us, 146
     (14, 117, 64, 8, 128, 4, True, False),      # 57, 63
+    (2, 203, 64, 8, 128, 2, True, False),       # 13.9, 15.6: the fullest SM has one packed item more
+    (6, 115, 64, 8, 64, 4, True, False),        # 22.7, 24.8
     (6, 1158, 128, 8, 64, 6, True, True),       # 2.01 ms, 1.67
     (3, 776, 16, 4, 64, 3, True, True),
     (10, 264, 16, 4, 128, 4, True, True),

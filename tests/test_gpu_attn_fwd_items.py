@@ -42,14 +42,14 @@ def pack_of(tmp_path_factory):
 @pytest.mark.parametrize("B,S,Hq,Hkv,dh,donor,causal,pack", [
     (20, 257, 4, 2, 64, [0], True, 1),       # 64 tokens of two heads: five tiles, the last of one token
     (9, 161, 24, 4, 128, [0], True, 1),      # six heads to a KV head: three groups of two
-    (6, 140, 16, 8, 64, [0, 0], False, 1),   # full attention
+    (14, 140, 16, 8, 64, [0, 0], False, 1),  # full attention
     (10, 129, 8, 2, 128, [0, 1], True, 2),    # 32 tokens of four heads, the last tile of one token
     (10, 264, 8, 2, 64, [0], True, 2),
     (8, 145, 16, 2, 128, [0, 0], True, 3),   # 16 tokens of eight heads, the last tile of one token
     (4, 272, 24, 3, 64, [0], True, 3),       # every tile full
-    (10, 264, 8, 1, 64, [0, 0], False, 3),   # the last tile half full
+    (19, 136, 8, 1, 64, [0], False, 3),      # full attention, the last tile half full
     (12, 33, 32, 2, 128, [0, 0], True, 4),   # eight tokens of sixteen heads, five tiles for one key tile
-    (5, 264, 32, 2, 64, [0], False, 4),      # every tile full
+    (5, 136, 32, 2, 64, [0], False, 4),      # every tile full
 ])
 def test_tiles_of_several_heads(pack_of, B, S, Hq, Hkv, dh, donor, causal, pack):
     assert pack_of(B, S, Hq, Hkv, dh, len(donor), int(causal)) == pack
