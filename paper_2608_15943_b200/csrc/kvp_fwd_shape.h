@@ -70,15 +70,16 @@ inline float fwd_time(const FwdSizes& z, int pack) {
   return most;
 }
 
-// Tiles of several heads waste less on the last, part-filled tile of a sequence and on the keys that a causal mask hides from
-// a tile's first rows; both matter for short sequences only.  At heads of 128 and without a mask the packed kernel itself takes up
-// to a tenth longer for the same key tiles (long launches, against the estimate: causal heads of 64 1.00, full attention 1.05 to
-// 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an eighth.  Measured on 1660
-// shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so): launches of up to a
-// millisecond 0.76, 1.03 at most, longer ones 0.93, 0.99 at most, on 428 packed ones drawn afterwards 0.77, 1.03; 3 x 776 tokens, 16 heads of 64 on 4, three layers 35.2 -> 31.3
-// us.  One line at 0.97 for all of them slowed long launches at heads of 128 by 6 % on
-// average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 -> 2.78 ms); with the average over the SMs in the
-// place of the fullest CTA, launches of one or two rounds lost up to 12 % (2 x 203 tokens, 64 heads of 128 on 8, two layers).
+// Tiles of several heads waste less on the last, part-filled tile of a sequence and on the keys that a causal mask hides
+// from a tile's first rows; both matter for short sequences only.  At heads of 128 and without a mask the packed kernel
+// itself takes up to a tenth longer for the same key tiles (long launches, against the estimate: causal heads of 64 1.00,
+// full attention 1.05 to 1.08, heads of 128 1.02 to 1.05 up to 1200 tokens and 1.09 beyond), so that there it has to save an
+// eighth.  Measured on 1660 shapes of 8 to 3000 tokens (heads packed / not, geometric mean of those where this says so):
+// launches of up to a millisecond 0.76, 1.03 at most, longer ones 0.93, 0.99 at most, on 428 packed ones drawn afterwards
+// 0.77, 1.03; 3 x 776 tokens, 16 heads of 64 on 4, three layers 35.2 -> 31.3 us.  One line at 0.97 for all of them slowed
+// long launches at heads of 128 by 6 % on average and 19 % at most (9 x 2032 tokens, 64 heads on 8, four layers, 2.33 ->
+// 2.78 ms); with the average over the SMs in the place of the fullest CTA, launches of one or two rounds lost up to 12 % (2
+// x 203 tokens, 64 heads of 128 on 8, two layers).
 constexpr int FWD_PACK_TOKENS = 2048;
 inline int fwd_pack(const FwdSizes& z) {
   const int pack = fwd_most_pack(z.G);
