@@ -21,7 +21,7 @@
 //  dq_convert_kernel  scales the fp32 dQ accumulators and writes dQ as bf16 [B,S,Hq,dh].
 //
 // Delta = rowsum(dO * O) comes from a small pre-pass.  The dQ accumulators live in the caller's
-// workspace in a blocked layout ([b][hq][64-query tile][32-column quarter][64][32] fp32) so that every
+// workspace in a blocked layout ([b][hq][64-query tile][32-column quarter][16][32 columns][4 queries] fp32) so that every
 // reduction is one contiguous 8 KB run; they, and the dK / dV sums, are cleared by the pre-pass of each launch.  The
 // order in which partials reach an accumulator is not fixed, so dQ, dK and dV are reproducible only up to fp32 rounding
 // order (bit for bit up to 128 tokens, where no element has more than two terms).
@@ -122,7 +122,7 @@ __device__ __forceinline__ uint4 split3_bf16(float v) {
   return out;
 }
 
-// Floats of one layer's dQ accumulator: [B][Hq][ceil(S/64)][DH/32][64][32].
+// Floats of one layer's dQ accumulator: [B][Hq][ceil(S/64)][DH/32][16][32][4].
 __host__ __device__ inline size_t dq_acc_floats(int B, int S, int Hq, int dh) {
   return size_t(B) * Hq * ((S + BQ2 - 1) / BQ2) * BQ2 * dh;
 }
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   uint64_t* dp_free = st_full + 1;                // dP^T of the step is in registers (256 arrivals)
   uint64_t* pds_ready = dp_free + 1;              // [2] P^T, dS^T written (TMEM and shared memory), next statistics staged
   uint64_t* dq_full = pds_ready + 2;              // dQ^T of the step is in TMEM; its dS^T tile may be overwritten
-  uint64_t* dq_free = dq_full + 1;                // dQ^T of the step is in registers, statistics of step +3 staged (128 arrivals)
+  uint64_t* dq_free = dq_full + 1;                // dQ^T of the step is in registers, statistics of step +3 staged before (128 arrivals)
   uint64_t* stat0 = dq_free + 1;                  // statistics of the first steps staged (128 arrivals)
   uint64_t* acc_done = stat0 + 1;                 // all MMAs have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_done + 1);
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   // Statistics.  The drain warpgroup also prepares the per-query operand tiles the tensor core adds to the scores:
   // thread t < 64 handles -LSE/scale of query column t, thread 64 + t handles -Delta of column t, as the
   // three-term bf16 split.  The raw fp32 values come in through cp.async into a small ring in shared memory,
-  // requested eight steps before the step that uses them and staged as an operand tile three steps before: no
+  // requested eight steps before the step that uses them and staged as an operand tile four steps before: no
   // register ever waits on global memory, and the compute warpgroups never touch the statistics.
   const int stat_tid = int(threadIdx.x) - 10 * 32;   // (used by the drain warpgroup only)
   const int stat_kind = stat_tid >> 6;   // 0 lse, 1 delta
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     cf.row = row_of(cf.li, cf.g);
     cp = cf;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) vbits |= uint32_t(request()) << i;
+    for (int i = 0; i < 4; ++i) vbits |= uint32_t(request()) << i;
   }
   // constant operand tiles: ones in the first three columns; statistics tiles and the shared zero half start as zeros
   for (int i = threadIdx.x; i < (L::OFF_RAW - L::OFF_ONES) / 16; i += blockDim.x) {
@@ -547,24 +547,27 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   } else {
     // ------------------------------ dQ drain warpgroup ------------------------------
     // TMEM lane == column of dQ (dh index): this warp owns dh columns [32*quarter, 32*quarter + 32) of the
-    // step's 64 queries, lays them out as [64 queries x 32 columns] fp32 in shared memory and adds them to the
-    // accumulator with one 8 KB bulk reduction, which has a whole step to read the buffer before it is rewritten.
+    // step's 64 queries, lays them out as [16 groups of four queries][32 columns][4] fp32 in shared memory, a lane's four
+    // queries with one store, and adds them to the accumulator with one 8 KB bulk reduction.
+    // The chain of a step is short on purpose: dQ^T to registers, dq_free, the copy, and the statistics last.  Stored a
+    // float at a time, and with the statistics ahead of dq_free, this warpgroup was busy for 1650 of a step's 1830 cycles
+    // at DH 64 (1720 of 2020 at 128) and the step waited for it.
     const int quarter = warp & 3;
     const uint32_t lane_sel = uint32_t(quarter * 32) << 16;
     const bool active = quarter * 32 < DH;  // with DH == 64 the upper lanes hold nothing
-    float* stg = reinterpret_cast<float*>(smem + L::OFF_DQ + (warp - 10) * DQ_STAGE_BYTES);
-    const uint32_t stg_s = smem_u32(stg);
-    // the statistics of steps 0, 1, 2 were requested above
+    // the reduction of the step before (with the idle warps' space at DH 64, of the step before that) has a step to read its buffer
+    constexpr int BUFS = DH == 64 ? 2 : 1;
+    uint8_t* const stg = smem + L::OFF_DQ + quarter * BUFS * DQ_STAGE_BYTES;
+    // the statistics of steps 0 to 3 were requested above
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    stage(0, vbits & 1u);
-    stage(1, vbits & 2u);
-    stage(2, vbits & 4u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) stage(i, vbits >> i & 1u);
     fence_proxy_async_smem();
     mbar_arrive(stat0);
-    // Five more requests stay in flight (vbits: their validity, oldest in bit 0); from here on a ring slot is requested
+    // Four more requests stay in flight (vbits: their validity, oldest in bit 0); from here on a ring slot is requested
     // again only after its value has been staged.
     vbits = 0;
-    for (int i = 0; i < 5; ++i) vbits |= uint32_t(request()) << i;
+    for (int i = 0; i < 4; ++i) vbits |= uint32_t(request()) << i;
     for (int i = 0; i < kStatAhead + 8; ++i) look_ahead();
     int li = stream0 / G, g = stream0 % G, qi = 0;
     bool ok = true;
@@ -572,38 +575,41 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       ok = mbar_wait(dq_full, it & 1, err);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after_sync();
-      uint32_t a[32], c[32];
-      tmem_ld_x32(tm_dq + lane_sel, a);
-      tmem_ld_x32(tm_dq + lane_sel + 32, c);
-      tmem_ld_wait();
-      // The operand tile of step it+3 (last read by the scores of step it-1, which completed before this step's
-      // dQ^T did) and the request for step it+8.  The arrival below publishes the tile: the issuing warp waits for
-      // it before the next step's dQ^T, a whole step before the scores of step it+3 are issued.
-      look_ahead();
-      vbits |= uint32_t(request()) << 5;
-      asm volatile("cp.async.wait_group 5;" ::: "memory");
-      stage(it + 3, vbits & 1u);
-      vbits >>= 1;
-      fence_proxy_async_smem();
+      uint32_t a[64];
+      if (active) {
+        tmem_ld_x32(tm_dq + lane_sel, *reinterpret_cast<uint32_t(*)[32]>(&a[0]));
+        tmem_ld_x32(tm_dq + lane_sel + 32, *reinterpret_cast<uint32_t(*)[32]>(&a[32]));
+        tmem_ld_wait();
+      }
       tc_fence_before_sync();
-      mbar_arrive(dq_free);
+      mbar_arrive(dq_free);   // (and the statistics staged behind the step before)
       if (active) {
         const size_t tile = ((size_t(b) * p.Hq + hk * G + g) * n_qt + (qt_first + qi)) * (DH / 32) + quarter;
         float* dst = p.dq_acc[slot0 + li] + tile * (BQ2 * 32);
-        // the previous step's reduction has read the buffer
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        uint8_t* const buf = stg + (it & (BUFS - 1)) * DQ_STAGE_BYTES;
+        // the reduction that last used the buffer has read it
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BUFS - 1) : "memory");
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < BQ2; ++q) stg[q * 32 + lane] = __uint_as_float(q < 32 ? a[q & 31] : c[q & 31]);
+        for (int q = 0; q < BQ2; q += 4) *reinterpret_cast<uint4*>(buf + q * 128 + lane * 16) = make_uint4(a[q], a[q + 1], a[q + 2], a[q + 3]);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst), "r"(stg_s),
+          asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(buf)),
                        "n"(DQ_STAGE_BYTES)
                        : "memory");
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
       }
+      // The operand tile of step it+4 (last read by the scores of step it, which completed before this step's dQ^T did) and
+      // the request for step it+8.  The arrival of step it+1 publishes the tile: the issuing warp waits for it ahead of the
+      // dQ^T of step it+2, and issues the scores of step it+4 behind that.
+      look_ahead();
+      vbits |= uint32_t(request()) << 4;
+      asm volatile("cp.async.wait_group 4;" ::: "memory");
+      stage(it + 4, vbits & 1u);
+      vbits >>= 1;
+      fence_proxy_async_smem();
       if (++qi == per_stream) {
         qi = 0;
         if (++g == G) {
@@ -644,45 +650,57 @@ struct AuxParams {
   float scale;
 };
 
-// After: dq[b,s,hq,:] = bf16(scale * accumulator), from the blocked fp32 layout [b][hq][tile][quarter][64][32].
-// One thread per 8 consecutive columns of one query row: two 16-byte loads, one 16-byte store.  Bound: HBM.
+// After: dq[b,s,hq,:] = bf16(scale * accumulator), from the blocked fp32 layout [b][hq][tile][quarter][16][32 columns][4 queries].
+// A warp takes 16 queries x 32 columns at a time: a lane loads its column's queries, four of them with each of four 16-byte
+// loads, and three exchanges (lanes 1, 2 and 4 apart) leave it with eight consecutive columns of two queries.  Bound: HBM.
 template <int DH>
 __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
-  constexpr int TPR = DH / 8;  // threads per query row
   grid_dep_wait();
-  const float* acc = p.dq_acc[blockIdx.y];
-  const int S = p.S, Hq = p.Hq;
+  const float4* acc = reinterpret_cast<const float4*>(p.dq_acc[blockIdx.y]);
+  const int S = p.S, Hq = p.Hq, lane = threadIdx.x & 31;
   const float scale = p.scale;
   const int n_qt = (S + BQ2 - 1) / BQ2;
-  const size_t rows = size_t(p.B) * Hq * n_qt * BQ2;
-  const size_t stride = size_t(gridDim.x) * blockDim.x / TPR;
-  const int j = threadIdx.x % TPR;
-  const int quarter = j / 4, d0 = (j % 4) * 8;
-  for (size_t row = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) / TPR; row < rows; row += stride) {
-    if (row + stride >= rows) grid_dep_launch();
-    const int q = int(row % BQ2);
-    const size_t tile = row / BQ2;  // (b * Hq + hq) * n_qt + qt
-    const int qt = int(tile % n_qt);
+  const size_t units = size_t(p.B) * Hq * n_qt * (DH / 32) * (BQ2 / 16);
+  const size_t stride = size_t(gridDim.x) * blockDim.x / 32;
+  const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
+  const int own = (b0 ? 4 : 0) + (b1 ? 2 : 0) + (b2 ? 1 : 0);   // of eight queries, the one this lane stores
+  for (size_t u = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32; u < units; u += stride) {
+    if (u + stride >= units) grid_dep_launch();
+    const size_t block = u / (BQ2 / 16);                        // tile * (DH / 32) + quarter
+    const size_t tile = block / (DH / 32);                      // (b * Hq + hq) * n_qt + qt
     const size_t bh = tile / n_qt;
-    const int s = qt * BQ2 + q;
-    if (s >= S) continue;
-    const float* src = acc + ((tile * (DH / 32) + quarter) * BQ2 + q) * 32 + d0;
-    const float4 lo = *reinterpret_cast<const float4*>(src);
-    const float4 hi = *reinterpret_cast<const float4*>(src + 4);
-    uint4 v;
-    v.x = pack_bf16(lo.x * scale, lo.y * scale);
-    v.y = pack_bf16(lo.z * scale, lo.w * scale);
-    v.z = pack_bf16(hi.x * scale, hi.y * scale);
-    v.w = pack_bf16(hi.z * scale, hi.w * scale);
-    const int hq = int(bh % Hq);
-    const int bb = int(bh / Hq);
-    const size_t at = ((size_t(bb) * S + s) * Hq + hq) * DH + quarter * 32 + d0;
-    if (p.dq_f32) {
-      float* out = reinterpret_cast<float*>(p.dq[blockIdx.y]) + at;
-      *reinterpret_cast<uint4*>(out) = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
-      *reinterpret_cast<uint4*>(out + 4) = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
-    } else {
-      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dq[blockIdx.y]) + at) = v;
+    const int s0 = int(tile % n_qt) * BQ2 + int(u % (BQ2 / 16)) * 16;
+    if (s0 >= S) continue;
+    float4 f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = acc[u * 128 + i * 32 + lane];
+    const int hq = int(bh % Hq), bb = int(bh / Hq);
+    const int col = int(block % (DH / 32)) * 32 + (lane & 24);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 x = f[2 * h], y = f[2 * h + 1];
+      const uint32_t w[4] = {pack_bf16(x.x * scale, x.y * scale), pack_bf16(x.z * scale, x.w * scale),   // queries 0 1, 2 3,
+                             pack_bf16(y.x * scale, y.y * scale), pack_bf16(y.z * scale, y.w * scale)};  // 4 5, 6 7
+      const uint32_t e0 = __shfl_xor_sync(0xffffffffu, b0 ? w[0] : w[2], 1), e1 = __shfl_xor_sync(0xffffffffu, b0 ? w[1] : w[3], 1);
+      const uint32_t lo0 = b0 ? e0 : w[0], lo1 = b0 ? e1 : w[1], hi0 = b0 ? w[2] : e0, hi1 = b0 ? w[3] : e1;
+      // two columns of four queries
+      const uint32_t t0 = __byte_perm(lo0, hi0, 0x5410), t1 = __byte_perm(lo0, hi0, 0x7632);
+      const uint32_t t2 = __byte_perm(lo1, hi1, 0x5410), t3 = __byte_perm(lo1, hi1, 0x7632);
+      const uint32_t g0 = __shfl_xor_sync(0xffffffffu, b1 ? t0 : t2, 2), g1 = __shfl_xor_sync(0xffffffffu, b1 ? t1 : t3, 2);
+      // four columns of two queries: (x0, y0) and (x1, y1)
+      const uint32_t x0 = b1 ? g0 : t0, y0 = b1 ? t2 : g0, x1 = b1 ? g1 : t1, y1 = b1 ? t3 : g1;
+      const uint32_t k0 = __shfl_xor_sync(0xffffffffu, b2 ? x0 : x1, 4), k1 = __shfl_xor_sync(0xffffffffu, b2 ? y0 : y1, 4);
+      const uint4 v = b2 ? make_uint4(k0, k1, x1, y1) : make_uint4(x0, y0, k0, k1);
+      const int s = s0 + h * 8 + own;
+      if (s >= S) continue;
+      const size_t at = ((size_t(bb) * S + s) * Hq + hq) * DH + col;
+      if (p.dq_f32) {
+        float* out = reinterpret_cast<float*>(p.dq[blockIdx.y]) + at;
+        *reinterpret_cast<uint4*>(out) = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
+        *reinterpret_cast<uint4*>(out + 4) = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
+      } else {
+        *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dq[blockIdx.y]) + at) = v;
+      }
     }
   }
 }
@@ -949,11 +967,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     ax.acc_v4 = dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;
     ax.kv_v4 = size_t(s->B) * s->S * s->Hkv * dh / 4;
     ax.scale = sc;
-    // enough blocks for every slot to fill the device, no more than its 8-element pieces (convert) give work to
-    const int aux_blocks = int(min(size_t(sm_count()) * 16, (dq_acc_floats(s->B, s->S, s->Hq, dh) / 8 + 255) / 256));
-    const dim3 aux_grid(aux_blocks, slots);
+    // enough blocks for every slot to fill the device, no more than its pieces of 8 (16: convert) accumulators give work to
+    const size_t acc_floats = dq_acc_floats(s->B, s->S, s->Hq, dh);
+    auto aux_grid = [&](size_t per_thread) { return dim3(unsigned(min(size_t(sm_count()) * 16, (acc_floats / per_thread + 255) / 256)), slots); };
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128> : bwd_prepare_kernel<64>, aux_grid, 256, 0, stream, 1, ax);
+    cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128> : bwd_prepare_kernel<64>, aux_grid(8), 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     dim3 grid(p.cta_begin[ng]);
@@ -963,7 +981,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     timing_after(KVP_KERNEL_ATTN_BWD, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid, 256, 0, stream, 1, ax);
+    e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid(16), 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
   }

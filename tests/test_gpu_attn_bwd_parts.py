@@ -43,3 +43,14 @@ def test_backward_in_parts(B, S, Hq, Hkv, dh, donor, causal):
         again = backward(kvp, B, S, Hq, Hkv, dh, donor, causal, inputs)
         for a, b in zip(dq + dk + dv, again[0] + again[1] + again[2]):
             assert (a is None and b is None) or torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("S", [9, 47, 79, 321])   # ends inside an eight, a sixteen and a tile of queries; more steps than any ring holds
+def test_dq_of_ragged_tiles(S, dh):
+    from paper_2608_15943_b200 import kvp
+    inputs = attn_inputs(2, S, 6, 2, dh, [0, 0])
+    dq = backward(kvp, 2, S, 6, 2, dh, [0, 0], True, inputs)[0]
+    rq = A.attn_bwd(*(f64l(x) for x in inputs), [0, 0], causal=True)[0]
+    for l in range(2):
+        close(f"dq[{l}]", dq[l], rq[l])
