@@ -7,7 +7,7 @@
 //               query tiles the causal mask lets see the keys.  dK and dV of the donor are therefore summed
 //               on chip across layers and heads and added to the fp32 sums in HBM once per CTA; where a key
 //               tile has several (windows, and parts of the streams in small calls), in no fixed order.  Per step, transposed so that TMEM
-//               lane == key row:  S^T = K Q^T, dP^T = V dO^T (tcgen05, operands in shared memory), each
+//               lane == key row:  S^T = K Q^T, dP^T = V dO^T (tcgen05; K and V from TMEM at DH 64), each
 //               followed by one rank-3 MMA that subtracts the query's LSE/scale resp. Delta (a bf16
 //               three-term split against a tile of ones), so the accumulators already hold the
 //               exponent and dP - Delta; P^T = exp2(c acc), dS^T = P^T acc' are written back as bf16
@@ -52,25 +52,33 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 two compute warpgroups, warps 10-13 dQ drain
-constexpr int BWD_THREADS = 448;
-constexpr int BWD_STAGES = 3;        // ring of (Q, dO) 64-row tiles
+// warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 two compute warpgroups, warps 10-13 dQ drain, warps 14 and 15 statistics
+// Bound at DH 128: the shared-memory port (1760 of about 1850 cycles a step).  At DH 64 a step has half the MMA work and the
+// same exponentials, and the serial part of a compute warpgroup's step counts: there the warpgroups take every other step,
+// which their own buffers of dP^T, dS^T and staged dQ allow.  Measured (us, whole attn_bwd call, as DH 128 -> so): 2 layers of 4 x
+// 2048, 16 heads on 8, 325 -> 275; 8192, 32 heads on 8, 1020 -> 860; three layers of 3 x 776, 16 heads on 4, 89 -> 75.
+constexpr int BWD_THREADS = 512;
+constexpr int STAT_BYTES = 2 * BQ2 * 16;      // the statistics of 64 queries: [lse, delta][64][8] bf16
 constexpr int DQ_STAGE_BYTES = BQ2 * 32 * 4;  // one drain warp's share of a step: [64 queries x 32 columns] fp32
 template <int DH>
 struct BwdSmem {
+  static constexpr bool SMALL = DH == 64;   // TMEM and shared memory have room for more
+  static constexpr int STAGES = SMALL ? 5 : 3;            // ring of (Q, dO) 64-row tiles
+  static constexpr int DS_BUFS = SMALL ? 2 : 1;
+  static constexpr int STEP_THREADS = SMALL ? 128 : 256;  // compute threads that work on a step
+  static constexpr int DQ_BUFS = SMALL ? 2 : 1;           // staging buffers of a drain warp (two of the four have work at DH 64)
   static constexpr int KV_TILE = BT * DH * 2;
   static constexpr int Q_TILE = BQ2 * DH * 2;
   static constexpr int STAGE = 2 * Q_TILE;  // Q then dO
   static constexpr int OFF_K = 0;
   static constexpr int OFF_V = OFF_K + KV_TILE;
   static constexpr int OFF_RING = OFF_V + KV_TILE;
-  static constexpr int OFF_DS = OFF_RING + BWD_STAGES * STAGE;     // dS^T [128 keys x 64 queries] bf16, 128-B swizzle
-  static constexpr int OFF_DQ = OFF_DS + BT * BQ2 * 2;             // [4 drain warps][64 x 32] fp32
+  static constexpr int OFF_DS = OFF_RING + STAGES * STAGE;         // dS^T [128 keys x 64 queries] bf16, 128-B swizzle
+  static constexpr int OFF_DQ = OFF_DS + DS_BUFS * BT * BQ2 * 2;   // [4 drain warps][64 x 32] fp32
   static constexpr int OFF_ONES = OFF_DQ + 4 * DQ_STAGE_BYTES;     // [128 x 8] bf16: columns 0-7 of the tile of ones
-  static constexpr int OFF_STAT = OFF_ONES + 2048;                 // [4 steps][lse, delta][64 x 8] bf16: columns 0-7
-  static constexpr int OFF_ZERO = OFF_STAT + 8 * 1024;             // [128 x 8] zeros: columns 8-15 of all of the above
-  static constexpr int OFF_RAW = OFF_ZERO + 2048;                  // [8 steps][lse, delta][64] fp32 as loaded
-  static constexpr int OFF_BAR = OFF_RAW + 4096;
+  static constexpr int OFF_STAT = OFF_ONES + 2048;                 // [STAGES][lse, delta][64 x 8] bf16: columns 0-7
+  static constexpr int OFF_ZERO = OFF_STAT + STAGES * STAT_BYTES;  // [128 x 8] zeros: columns 8-15 of all of the above
+  static constexpr int OFF_BAR = OFF_ZERO + 2048;
   static constexpr int TOTAL = OFF_BAR + 256 + 1024;
 };
 
@@ -127,8 +135,9 @@ __host__ __device__ inline size_t dq_acc_floats(int B, int S, int Hq, int dh) {
   return size_t(B) * Hq * ((S + BQ2 - 1) / BQ2) * BQ2 * dh;
 }
 
-// TMEM columns: S^T of step parity i at [i*64, i*64+64) (P^T and dS^T overwrite it as bf16), dP^T at
-// [128, 192), the step's dQ^T at [192, 256), dK at [256, 256+DH), dV above it.
+// TMEM columns: S^T of step parity i at [i*64, i*64+64) (P^T and dS^T overwrite it as bf16), then dP^T, the step's dQ^T (64),
+// dK and dV (DH each).  At DH 64 dP^T too has a buffer for each parity, and K and V follow as bf16 A operands of S^T and dP^T:
+// an MMA whose A comes from TMEM reads 2 KB of shared memory instead of 6, 32 cycles instead of 48.
 //
 // The per-query statistics are applied BY THE TENSOR CORE: one extra K-step multiplies a [128 x 16] tile
 // of ones (first three columns) with a [64 x 16] tile holding -LSE/scale (resp. -Delta) of each query
@@ -146,16 +155,16 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
   uint64_t* kv_full = bars + 0;
-  uint64_t* q_full = bars + 1;                    // [STAGES]
-  uint64_t* q_empty = q_full + BWD_STAGES;        // [STAGES]
-  uint64_t* st_full = q_empty + BWD_STAGES;       // S^T and dP^T of the step are in TMEM
-  uint64_t* dp_free = st_full + 1;                // dP^T of the step is in registers (256 arrivals)
-  uint64_t* pds_ready = dp_free + 1;              // [2] P^T, dS^T written (TMEM and shared memory), next statistics staged
-  uint64_t* dq_full = pds_ready + 2;              // dQ^T of the step is in TMEM; its dS^T tile may be overwritten
-  uint64_t* dq_free = dq_full + 1;                // dQ^T of the step is in registers, statistics of step +3 staged before (128 arrivals)
-  uint64_t* stat0 = dq_free + 1;                  // statistics of the first steps staged (128 arrivals)
-  uint64_t* acc_done = stat0 + 1;                 // all MMAs have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_done + 1);
+  uint64_t* q_full = bars + 1;                    // [STAGES] Q and dO loaded, statistics staged (64 arrivals)
+  uint64_t* q_empty = q_full + L::STAGES;         // [STAGES]
+  uint64_t* st_full = q_empty + L::STAGES;        // [2] S^T and dP^T of the step are in TMEM
+  uint64_t* dp_free = st_full + 2;                // [2] dP^T of the step is in registers (STEP_THREADS arrivals)
+  uint64_t* pds_ready = dp_free + 2;              // [2] P^T, dS^T written (TMEM and shared memory; STEP_THREADS arrivals)
+  uint64_t* dq_full = pds_ready + 2;              // [2] dQ^T of the step is in TMEM; its dS^T tile may be overwritten
+  uint64_t* dq_free = dq_full + 2;                // dQ^T of the step is in registers (128 arrivals)
+  uint64_t* acc_done = dq_free + 1;               // all MMAs have completed
+  uint64_t* a_ready = acc_done + 1;               // DH 64: K and V are in TMEM (256 arrivals)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(a_ready + 1);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -221,7 +230,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   auto load_step = [&](int it, uint32_t leader) {
     int li, hq, q0;
     decode_iter(it, li, hq, q0);
-    const int s = it % BWD_STAGES;
+    const int s = it % L::STAGES;
     mbar_expect_tx_e(&q_full[s], L::STAGE, leader);
     uint8_t* dst = smem + L::OFF_RING + s * L::STAGE;
 #pragma unroll
@@ -231,85 +240,25 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     }
   };
 
-  // Statistics.  The drain warpgroup also prepares the per-query operand tiles the tensor core adds to the scores:
-  // thread t < 64 handles -LSE/scale of query column t, thread 64 + t handles -Delta of column t, as the
-  // three-term bf16 split.  The raw fp32 values come in through cp.async into a small ring in shared memory,
-  // requested eight steps before the step that uses them and staged as an operand tile four steps before: no
-  // register ever waits on global memory, and the compute warpgroups never touch the statistics.
-  const int stat_tid = int(threadIdx.x) - 10 * 32;   // (used by the drain warpgroup only)
-  const int stat_kind = stat_tid >> 6;   // 0 lse, 1 delta
-  const int stat_col = stat_tid & 63;
-  uint8_t* stat_row = smem + L::OFF_STAT + stat_kind * 1024 + stat_col * 16;
-  float* raw = reinterpret_cast<float*>(smem + L::OFF_RAW) + stat_tid;   // ring slot s at raw[s * 128]
-  const float stat_mul = stat_kind == 0 ? -1.f / p.scale : -1.f;
-  const float stat_pad = stat_kind == 0 ? -30000.f : 0.f;  // a query beyond the sequence: exp2 underflows to zero
-  // Two cursors walk the steps in order (incremental decode of step -> layer, head, query tile): one for the
-  // step whose statistics are requested next, one kStatAhead steps further that only pulls the line into L2.
-  // `row` is the statistic row of the cursor's (layer, head): it is looked up (an indexed read of the kernel
-  // parameters) only when the stream changes, never on the per-step path.
-  constexpr int kStatAhead = 12;
-  struct Cursor {
-    int it = 0, qi = 0, g = 0, li = 0;
-    const float* row = nullptr;
-  };
-  auto row_of = [&](int li, int g) {
-    const int slot = slot0 + (li < n_layers ? li : 0);
-    const float* src = stat_kind == 0 ? p.lse[slot] : p.delta[slot];
-    return src + (size_t(b) * p.Hq + hk * G + g) * p.S;
-  };
-  auto advance = [&](Cursor& c) {
-    ++c.it;
-    if (++c.qi == per_stream) {
-      c.qi = 0;
-      if (++c.g == G) {
-        c.g = 0;
-        ++c.li;
-      }
-      c.row = row_of(c.li, c.g);
-    }
-  };
-  auto locate = [&](const Cursor& c, bool& valid) {  // address of this thread's statistic of step c (clamped, always valid)
-    const int qc = (qt_first + c.qi) * BQ2 + stat_col;
-    valid = c.it < n_iter && qc < p.S;
-    return c.row + (valid ? qc : p.S - 1);
-  };
-  Cursor cf, cp;
-  auto request = [&]() -> bool {  // cp.async of the next step's value into its ring slot; returns its validity
-    bool valid;
-    const float* ptr = locate(cf, valid);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(raw + (cf.it & 7) * 128)), "l"(ptr) : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    advance(cf);
-    return valid;
-  };
-  auto look_ahead = [&]() {  // the line of the step kStatAhead further on, into L2
-    bool valid;
-    const float* ahead = locate(cp, valid);
-    if ((stat_col & 31) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead));
-    advance(cp);
-  };
-  auto stage = [&](int step, bool valid) {  // the value of `step` has landed: split it into the step's operand tile
-    *reinterpret_cast<uint4*>(stat_row + (step & 3) * 2048) = split3_bf16(valid ? raw[(step & 7) * 128] * stat_mul : stat_pad);
-  };
-  uint32_t vbits = 0;
-
   // The loads that everything waits for go out before the block has set itself up: the TMA warp initialises the barriers
-  // and fills the ring, the drain warpgroup requests the first statistics, then the block meets.
+  // and fills the ring, then the block meets.
   if (warp == 0) {
     const uint32_t leader = elect_one();
     if (leader) {
       mbar_init(kv_full, 1);
-      for (int s = 0; s < BWD_STAGES; ++s) {
-        mbar_init(&q_full[s], 1);
+      for (int s = 0; s < L::STAGES; ++s) {
+        mbar_init(&q_full[s], 1 + 64);
         mbar_init(&q_empty[s], 1);
       }
-      mbar_init(st_full, 1);
-      mbar_init(dp_free, 256);
-      for (int i = 0; i < 2; ++i) mbar_init(&pds_ready[i], 256);
-      mbar_init(dq_full, 1);
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(&st_full[i], 1);
+        mbar_init(&dp_free[i], L::STEP_THREADS);
+        mbar_init(&pds_ready[i], L::STEP_THREADS);
+      }
+      for (int i = 0; i < 2; ++i) mbar_init(&dq_full[i], 1);
       mbar_init(dq_free, 128);
-      mbar_init(stat0, 128);
       mbar_init(acc_done, 1);
+      mbar_init(a_ready, 256);
       mbar_fence_init();
       fence_proxy_async_smem();
     }
@@ -321,22 +270,13 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       tma_load_4d_e(smem + L::OFF_K + h * HALF_BYTES, &p.map_k[grp], kv_full, h * 64, hk, kv0, b, leader);
       tma_load_4d_e(smem + L::OFF_V + h * HALF_BYTES, &p.map_v[grp], kv_full, h * 64, hk, kv0, b, leader);
     }
-    for (int it = 0; it < min(n_iter, BWD_STAGES); ++it) load_step(it, leader);
+    for (int it = 0; it < min(n_iter, L::STAGES); ++it) load_step(it, leader);
   }
-  if (warp >= 10) {
-    grid_dep_wait();
-    cf.li = stream0 / G;
-    cf.g = stream0 % G;
-    cf.row = row_of(cf.li, cf.g);
-    cp = cf;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) vbits |= uint32_t(request()) << i;
-  }
-  // constant operand tiles: ones in the first three columns; statistics tiles and the shared zero half start as zeros
-  for (int i = threadIdx.x; i < (L::OFF_RAW - L::OFF_ONES) / 16; i += blockDim.x) {
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (i < 128) v = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);  // row i, columns 0-7 = 1,1,1,0,0,0,0,0
-    *reinterpret_cast<uint4*>(smem + L::OFF_ONES + i * 16) = v;
+  // constant operand tiles: ones in the first three columns, and the zeros
+  if (threadIdx.x < 256) {
+    const bool ones = threadIdx.x < 128;   // row i, columns 0-7 = 1,1,1,0,0,0,0,0
+    *reinterpret_cast<uint4*>(smem + (ones ? L::OFF_ONES : L::OFF_ZERO) + (threadIdx.x & 127) * 16) =
+        make_uint4(ones ? 0x3F803F80u : 0u, ones ? 0x00003F80u : 0u, 0u, 0u);
   }
   fence_proxy_async_smem();
   if (warp == 1) {
@@ -348,16 +288,17 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   grid_dep_wait();
-  const uint32_t tm_dp = tmem_base + 128;
-  const uint32_t tm_dq = tmem_base + 192;
-  const uint32_t tm_dk = tmem_base + 256;
-  const uint32_t tm_dv = tmem_base + 256 + DH;
+  const uint32_t tm_dp = tmem_base + 128;                                   // [2] at DH 64
+  const uint32_t tm_dq = tmem_base + (L::SMALL ? 256 : 192);
+  const uint32_t tm_dk = tm_dq + 64;
+  const uint32_t tm_dv = tm_dk + DH;
+  const uint32_t tm_k = tmem_base + 448, tm_v = tmem_base + 480;            // DH 64
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     const uint32_t leader = elect_one();  // the whole warp runs the loop; one lane issues
-    for (int it = BWD_STAGES; it < n_iter; ++it) {
-      if (!mbar_wait(&q_empty[it % BWD_STAGES], ((it / BWD_STAGES) & 1) ^ 1, err)) break;
+    for (int it = L::STAGES; it < n_iter; ++it) {
+      if (!mbar_wait(&q_empty[it % L::STAGES], ((it / L::STAGES) & 1) ^ 1, err)) break;
       load_step(it, leader);
     }
     grid_dep_launch();   // all loads are out
@@ -384,46 +325,68 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       const uint32_t stat_base = smem_u32(smem + L::OFF_STAT);
       const uint32_t ring = smem_u32(smem + L::OFF_RING);
       bool ok = mbar_wait(kv_full, 0, err);
-      if (ok) ok = mbar_wait(stat0, 0, err);
+      if (L::SMALL && ok) ok = mbar_wait(a_ready, 0, err);
+      // One score product and the statistics of its queries: S^T - LSE / scale, dP^T - Delta.
+      auto product = [&](uint32_t d, uint32_t a_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t stat_addr) {
+#pragma unroll
+        for (int ks = 0; ks < KSTEPS_DH; ++ks) {
+          const uint32_t b = desc_lo_add(b_lo, (ks / 4) * QHALF_BYTES + (ks % 4) * 32);
+          if constexpr (L::SMALL) umma_ts_w(d, a_tmem + ks * 8, b, hi, idesc_st, ks != 0, leader);
+          else umma_ss_w(d, desc_lo_add(a_lo, (ks / 4) * HALF_BYTES + (ks % 4) * 32), b, hi, idesc_st, ks != 0, leader);
+        }
+        umma_ss_w(d, ones_lo, desc_lo_plain(stat_addr, zero_addr - stat_addr), hi_plain, idesc_st, 1, leader);
+      };
+      auto issue_s = [&](int it) {
+        const int s = it % L::STAGES;
+        product(tmem_base + (it & 1) * 64, tm_k, k_lo, desc_lo_sw128(ring + s * L::STAGE, 0), stat_base + s * STAT_BYTES);
+      };
+      auto issue_dp = [&](int it) {
+        const int s = it % L::STAGES;
+        product(tm_dp + (L::SMALL ? (it & 1) * 64 : 0), tm_v, v_lo, desc_lo_sw128(ring + s * L::STAGE + L::Q_TILE, 0),
+                stat_base + s * STAT_BYTES + BQ2 * 16);
+      };
+      auto stage_full = [&](int it) -> bool {
+        const bool w = mbar_wait(&q_full[it % L::STAGES], (it / L::STAGES) & 1, err);
+        tc_fence_after_sync();
+        return w;
+      };
+      // DH 128.  The single dP^T buffer takes the next step once the compute warps hold the previous one in registers.
       auto issue_scores = [&](int it) -> bool {
-        const int s = it % BWD_STAGES;
-        if (!mbar_wait(&q_full[s], (it / BWD_STAGES) & 1, err)) return false;
+        if (!stage_full(it)) return false;
+        issue_s(it);
+        if (it > 0 && !mbar_wait(&dp_free[(it - 1) & 1], ((it - 1) >> 1) & 1, err)) return false;
         tc_fence_after_sync();
-        const uint32_t q_lo = desc_lo_sw128(ring + s * L::STAGE, 0);
-        const uint32_t do_lo = desc_lo_sw128(ring + s * L::STAGE + L::Q_TILE, 0);
-        const uint32_t tm = tmem_base + (it & 1) * 64;
-        const uint32_t lse_addr = stat_base + (it & 3) * 2048;
-        const uint32_t stat_lo = desc_lo_plain(lse_addr, zero_addr - lse_addr);
-        const uint32_t delta_lo = desc_lo_plain(lse_addr + 1024, zero_addr - lse_addr - 1024);
-#pragma unroll
-        for (int ks = 0; ks < KSTEPS_DH; ++ks) {
-          const uint32_t offa = (ks / 4) * HALF_BYTES + (ks % 4) * 32;
-          const uint32_t offb = (ks / 4) * QHALF_BYTES + (ks % 4) * 32;
-          umma_ss_w(tm, desc_lo_add(k_lo, offa), desc_lo_add(q_lo, offb), hi, idesc_st, ks != 0, leader);
-        }
-        umma_ss_w(tm, ones_lo, stat_lo, hi_plain, idesc_st, 1, leader);                          // S^T -= LSE / scale
-        // the single dP^T buffer takes the next step once the compute warps hold the previous one in registers
-        if (it > 0 && !mbar_wait(dp_free, (it - 1) & 1, err)) return false;
-        tc_fence_after_sync();
-#pragma unroll
-        for (int ks = 0; ks < KSTEPS_DH; ++ks) {
-          const uint32_t offa = (ks / 4) * HALF_BYTES + (ks % 4) * 32;
-          const uint32_t offb = (ks / 4) * QHALF_BYTES + (ks % 4) * 32;
-          umma_ss_w(tm_dp, desc_lo_add(v_lo, offa), desc_lo_add(do_lo, offb), hi, idesc_st, ks != 0, leader);
-        }
-        umma_ss_w(tm_dp, ones_lo, delta_lo, hi_plain, idesc_st, 1, leader);                      // dP^T -= Delta
-        umma_commit(st_full, leader);
+        issue_dp(it);
+        umma_commit(&st_full[it & 1], leader);
         return true;
       };
-      if (ok && n_iter > 0) ok = issue_scores(0);
+      if constexpr (L::SMALL) {
+        for (int it = 0; it < min(n_iter, 2) && ok; ++it) {
+          ok = stage_full(it);
+          if (!ok) break;
+          issue_s(it);
+          issue_dp(it);
+          umma_commit(&st_full[it], leader);
+        }
+      } else {
+        if (ok && n_iter > 0) ok = issue_scores(0);
+      }
       for (int it = 0; it < n_iter && ok; ++it) {
-        // S^T of the next step goes to the other score buffer; its previous readers (the accumulate MMAs
-        // of step it-1) precede this in the in-order tensor pipe, and its statistics tile was staged
-        // before pds_ready(it-1)
-        if (it + 1 < n_iter && !issue_scores(it + 1)) { ok = false; break; }
+        // DH 128: S^T of the next step goes to the other score buffer; its previous readers (the accumulate MMAs
+        // of step it-1) precede this in the in-order tensor pipe
+        if constexpr (L::SMALL) {
+          // dP^T of the step after the next, over the buffer that this step's warps have read
+          if (it + 2 < n_iter) {
+            if (!stage_full(it + 2) || !mbar_wait(&dp_free[it & 1], (it >> 1) & 1, err)) { ok = false; break; }
+            tc_fence_after_sync();
+            issue_dp(it + 2);
+          }
+        } else {
+          if (it + 1 < n_iter && !issue_scores(it + 1)) { ok = false; break; }
+        }
         if (!mbar_wait(&pds_ready[it & 1], (it >> 1) & 1, err)) { ok = false; break; }
         tc_fence_after_sync();
-        const int s = it % BWD_STAGES;
+        const int s = it % L::STAGES;
         const uint32_t qmn_lo = desc_lo_sw128(ring + s * L::STAGE, QHALF_BYTES);                 // Q  as MN-major B
         const uint32_t domn_lo = desc_lo_sw128(ring + s * L::STAGE + L::Q_TILE, QHALF_BYTES);    // dO as MN-major B
         const uint32_t tm = tmem_base + (it & 1) * 64;
@@ -435,12 +398,18 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
         for (int ks = 0; ks < KSTEPS_Q; ++ks)  // dK += dS^T Q
           umma_ts_w(tm_dk, tm + (ks / 2) * 32 + 16 + (ks % 2) * 8, desc_lo_add(qmn_lo, ks * 2048), hi, idesc_acc, (it | ks) != 0, leader);
         umma_commit(&q_empty[s], leader);  // the ring stage is free as soon as dV and dK have read it
+        // DH 64: S^T of the step after the next, over the score buffer that dV and dK have just read, goes ahead of dQ^T, whose
+        // dS^T tile has a twin
+        if (L::SMALL && it + 2 < n_iter) {
+          issue_s(it + 2);
+          umma_commit(&st_full[it & 1], leader);
+        }
         if (it > 0 && !mbar_wait(dq_free, (it - 1) & 1, err)) { ok = false; break; }
         tc_fence_after_sync();
 #pragma unroll
         for (int ks = 0; ks < KSTEPS_KV; ++ks)  // dQ^T = K^T dS^T
-          umma_ss_w(tm_dq, desc_lo_add(kmn_lo, ks * 2048), desc_lo_add(ds_lo, ks * 2048), hi, idesc_dq, ks != 0, leader);
-        umma_commit(dq_full, leader);
+          umma_ss_w(tm_dq, desc_lo_add(kmn_lo, ks * 2048), desc_lo_add(ds_lo, (it & (L::DS_BUFS - 1)) * (BT * BQ2 * 2) + ks * 2048), hi, idesc_dq, ks != 0, leader);
+        umma_commit(&dq_full[it & 1], leader);
       }
       if (ok) umma_commit(acc_done, leader);
     }
@@ -452,58 +421,88 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     const uint32_t lane_sel = uint32_t(quarter * 32) << 16;
     const int kv_row = kv0 + r;
     const uint64_t c2 = pack_f2(p.scale_log2, p.scale_log2);
-    // P^T and dS^T (bf16 pairs) overwrite the warpgroup's OWN score columns, which the other warpgroup never
-    // reads: P^T in 32-bit columns [wg*32, wg*32+16), dS^T in [wg*32+16, wg*32+32)
-    const uint32_t col = wg * 32;
     uint8_t* ds_smem = smem + L::OFF_DS;
-    int qi = 0;  // query tile index of the current step inside its stream
+    if constexpr (L::SMALL) {   // K (warpgroup 0) and V (warpgroup 1) as A operands in TMEM, key row by key row
+      bool w = mbar_wait(kv_full, 0, err);
+      if (__all_sync(0xffffffffu, w)) {
+        uint32_t row[32];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint4 v = *reinterpret_cast<const uint4*>(smem + (wg == 0 ? L::OFF_K : L::OFF_V) + sw128_offset(r, j));
+          row[4 * j] = v.x;
+          row[4 * j + 1] = v.y;
+          row[4 * j + 2] = v.z;
+          row[4 * j + 3] = v.w;
+        }
+        tmem_st_x32((wg == 0 ? tm_k : tm_v) + lane_sel, row);
+        tmem_st_wait();
+        tc_fence_before_sync();
+        mbar_arrive(a_ready);
+      }
+    }
+    // DH 128: the warpgroups take half of the queries of every step each.  DH 64, where a step has half the MMA time and the
+    // same exponentials: every other step each, so that the loads, stores and waits of one fall into the exponentials of the
+    // other.
+    constexpr int STRIDE = L::SMALL ? 2 : 1, PARTS = L::SMALL ? 2 : 1;
+    int qi = L::SMALL ? wg % per_stream : 0;  // query tile index of the current step inside its stream
     bool ok = true;
-    for (int it = 0; it < n_iter; ++it) {
+    for (int it = L::SMALL ? wg : 0; it < n_iter; it += STRIDE) {
       const int set = it & 1;
-      const uint32_t tm = tmem_base + set * 64;
-      ok = mbar_wait(st_full, it & 1, err);
+      ok = mbar_wait(&st_full[set], (it >> 1) & 1, err);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after_sync();
-      uint32_t st[32], dp[32];
-      tmem_ld_x32(tm + lane_sel + col, st);
-      tmem_ld_x32(tm_dp + lane_sel + col, dp);
-      const int q_col0 = (qt_first + qi) * BQ2 + wg * 32;           // query of this warpgroup's first column
-      const bool diag = p.causal && q_col0 - wg * 32 < kv0 + BT;    // the query tile straddles the diagonal
-      const int first_visible = diag ? kv_row - q_col0 : 0;         // own columns below this are masked for this key row
-      uint32_t pk[16], dk[16];
-      tmem_ld_wait();
-      tc_fence_before_sync();
-      mbar_arrive(dp_free);
+      const int q0 = (qt_first + qi) * BQ2;
+      const bool diag = p.causal && q0 < kv0 + BT;                    // the query tile straddles the diagonal
+      uint8_t* const ds_tile = ds_smem + (it & (L::DS_BUFS - 1)) * (BT * BQ2 * 2);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const uint64_t x = fmul2(pack_f2(__uint_as_float(st[2 * i]), __uint_as_float(st[2 * i + 1])), c2);
-        float e0 = fast_exp2(f2_lo(x)), e1 = fast_exp2(f2_hi(x));
-        if (diag) {
-          e0 = 2 * i < first_visible ? 0.f : e0;
-          e1 = 2 * i + 1 < first_visible ? 0.f : e1;
+      for (int part = 0; part < PARTS; ++part) {
+        // P^T and dS^T (bf16 pairs) overwrite the 32 score columns they come from, which no other thread reads: P^T the
+        // first 16, dS^T the others
+        const int half = L::SMALL ? part : wg;                        // queries [32 half, 32 half + 32)
+        const uint32_t col = tmem_base + set * 64 + half * 32 + lane_sel;
+        uint32_t st[32], dp[32];
+        tmem_ld_x32(col, st);
+        tmem_ld_x32(tm_dp + (L::SMALL ? set * 64 : 0) + half * 32 + lane_sel, dp);
+        const int first_visible = diag ? kv_row - q0 - half * 32 : 0; // columns below this are masked for this key row
+        uint32_t pk[16], dk[16];
+        tmem_ld_wait();
+        if (part == PARTS - 1) {
+          tc_fence_before_sync();
+          mbar_arrive(&dp_free[set]);
         }
-        pk[i] = pack_bf16(e0, e1);
-        const uint64_t d = fmul2(pack_f2(e0, e1), pack_f2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])));
-        dk[i] = pack_bf16(f2_lo(d), f2_hi(d));
-      }
-      // keys beyond the sequence contribute nothing (their K/V rows are zero-filled; dK/dV rows are not stored)
-      tmem_st_x16(tm + lane_sel + col, pk);
-      tmem_st_x16(tm + lane_sel + col + 16, dk);
-      // dS^T also goes to shared memory as the B operand of dQ^T = K^T dS^T; the previous step's product
-      // must have finished reading the tile
-      if (it > 0) {
-        ok = mbar_wait(dq_full, (it - 1) & 1, err);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      }
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        *reinterpret_cast<uint4*>(ds_smem + sw128_offset(r, wg * 4 + j)) =
-            make_uint4(dk[4 * j], dk[4 * j + 1], dk[4 * j + 2], dk[4 * j + 3]);
+        for (int i = 0; i < 16; ++i) {
+          const uint64_t x = fmul2(pack_f2(__uint_as_float(st[2 * i]), __uint_as_float(st[2 * i + 1])), c2);
+          float e0 = fast_exp2(f2_lo(x)), e1 = fast_exp2(f2_hi(x));
+          if (diag) {
+            e0 = 2 * i < first_visible ? 0.f : e0;
+            e1 = 2 * i + 1 < first_visible ? 0.f : e1;
+          }
+          pk[i] = pack_bf16(e0, e1);
+          const uint64_t d = fmul2(pack_f2(e0, e1), pack_f2(__uint_as_float(dp[2 * i]), __uint_as_float(dp[2 * i + 1])));
+          dk[i] = pack_bf16(f2_lo(d), f2_hi(d));
+        }
+        // keys beyond the sequence contribute nothing (their K/V rows are zero-filled; dK/dV rows are not stored)
+        tmem_st_x16(col, pk);
+        tmem_st_x16(col + 16, dk);
+        // dS^T also goes to shared memory as the B operand of dQ^T = K^T dS^T; the product of the step that last used the
+        // tile must have finished reading it
+        if (part == 0 && it >= L::DS_BUFS) {
+          ok = mbar_wait(&dq_full[(it - L::DS_BUFS) & 1], ((it - L::DS_BUFS) >> 1) & 1, err);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<uint4*>(ds_tile + sw128_offset(r, half * 4 + j)) =
+              make_uint4(dk[4 * j], dk[4 * j + 1], dk[4 * j + 2], dk[4 * j + 3]);
+      }
+      if (!ok) break;
       tmem_st_wait();
       fence_proxy_async_smem();  // dS^T is read by the tensor core's proxy
       tc_fence_before_sync();
       mbar_arrive(&pds_ready[set]);
-      if (++qi == per_stream) qi = 0;
+      qi += STRIDE;
+      while (qi >= per_stream) qi -= per_stream;
     }
     ok = __all_sync(0xffffffffu, ok);
     if (ok) {
@@ -544,35 +543,73 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
         __syncwarp();
       }
     }
+  } else if (warp >= 14) {
+    // ------------------------------ statistics ------------------------------
+    // Thread t forms the two operand rows of query column t, -LSE / scale and -Delta in three bf16 terms each, in the ring slot
+    // of the step, from values that it asked for two steps before.  (As a side job of the drain warpgroup they took 500 to 600
+    // of its 1800 cycles a step.)
+    const int t = int(threadIdx.x) - 14 * 32;
+    const float lse_mul = -1.f / p.scale;
+    uint8_t* const row = smem + L::OFF_STAT + t * 16;
+    int li = stream0 / G, g = stream0 % G, qi = 0, asked = 0;
+    auto ask = [&](float& lse, float& delta) {   // of the next step; a query beyond the sequence: exp2 underflows to zero
+      const int q = (qt_first + qi) * BQ2 + t;
+      lse = 30000.f * p.scale;
+      delta = 0.f;
+      if (asked < n_iter && q < p.S) {
+        const size_t at = (size_t(b) * p.Hq + hk * G + g) * p.S + q;
+        lse = p.lse[slot0 + li][at];
+        delta = p.delta[slot0 + li][at];
+      }
+      ++asked;
+      if (++qi == per_stream) {
+        qi = 0;
+        if (++g == G) {
+          g = 0;
+          ++li;
+        }
+      }
+    };
+    float l0, d0, l1, d1, l2, d2;
+    ask(l0, d0);
+    ask(l1, d1);
+    int s = 0;
+    uint32_t ph = 1;
+    for (int it = 0; it < n_iter; ++it) {
+      ask(l2, d2);
+      const bool ok = mbar_wait(&q_empty[s], ph, err);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      *reinterpret_cast<uint4*>(row + s * STAT_BYTES) = split3_bf16(l0 * lse_mul);
+      *reinterpret_cast<uint4*>(row + s * STAT_BYTES + BQ2 * 16) = split3_bf16(-d0);
+      fence_proxy_async_smem();
+      mbar_arrive(&q_full[s]);
+      l0 = l1;
+      d0 = d1;
+      l1 = l2;
+      d1 = d2;
+      if (++s == L::STAGES) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
   } else {
     // ------------------------------ dQ drain warpgroup ------------------------------
     // TMEM lane == column of dQ (dh index): this warp owns dh columns [32*quarter, 32*quarter + 32) of the
     // step's 64 queries, lays them out as [16 groups of four queries][32 columns][4] fp32 in shared memory, a lane's four
     // queries with one store, and adds them to the accumulator with one 8 KB bulk reduction.
-    // The chain of a step is short on purpose: dQ^T to registers, dq_free, the copy, and the statistics last.  Stored a
-    // float at a time, and with the statistics ahead of dq_free, this warpgroup was busy for 1650 of a step's 1830 cycles
-    // at DH 64 (1720 of 2020 at 128) and the step waited for it.
+    // The chain of a step is short on purpose: dQ^T to registers, dq_free, the copy.  Stored a float at a time, and with the
+    // operand tiles of the statistics formed here too, ahead of dq_free, this warpgroup was busy for 1650 of a step's 1830
+    // cycles at DH 64 (1720 of 2020 at 128) and the step waited for it.
     const int quarter = warp & 3;
     const uint32_t lane_sel = uint32_t(quarter * 32) << 16;
     const bool active = quarter * 32 < DH;  // with DH == 64 the upper lanes hold nothing
     // the reduction of the step before (with the idle warps' space at DH 64, of the step before that) has a step to read its buffer
-    constexpr int BUFS = DH == 64 ? 2 : 1;
+    constexpr int BUFS = L::DQ_BUFS;
     uint8_t* const stg = smem + L::OFF_DQ + quarter * BUFS * DQ_STAGE_BYTES;
-    // the statistics of steps 0 to 3 were requested above
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 4; ++i) stage(i, vbits >> i & 1u);
-    fence_proxy_async_smem();
-    mbar_arrive(stat0);
-    // Four more requests stay in flight (vbits: their validity, oldest in bit 0); from here on a ring slot is requested
-    // again only after its value has been staged.
-    vbits = 0;
-    for (int i = 0; i < 4; ++i) vbits |= uint32_t(request()) << i;
-    for (int i = 0; i < kStatAhead + 8; ++i) look_ahead();
     int li = stream0 / G, g = stream0 % G, qi = 0;
     bool ok = true;
     for (int it = 0; it < n_iter; ++it) {
-      ok = mbar_wait(dq_full, it & 1, err);
+      ok = mbar_wait(&dq_full[it & 1], (it >> 1) & 1, err);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after_sync();
       uint32_t a[64];
@@ -582,7 +619,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
         tmem_ld_wait();
       }
       tc_fence_before_sync();
-      mbar_arrive(dq_free);   // (and the statistics staged behind the step before)
+      mbar_arrive(dq_free);
       if (active) {
         const size_t tile = ((size_t(b) * p.Hq + hk * G + g) * n_qt + (qt_first + qi)) * (DH / 32) + quarter;
         float* dst = p.dq_acc[slot0 + li] + tile * (BQ2 * 32);
@@ -601,15 +638,6 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
       }
-      // The operand tile of step it+4 (last read by the scores of step it, which completed before this step's dQ^T did) and
-      // the request for step it+8.  The arrival of step it+1 publishes the tile: the issuing warp waits for it ahead of the
-      // dQ^T of step it+2, and issues the scores of step it+4 behind that.
-      look_ahead();
-      vbits |= uint32_t(request()) << 4;
-      asm volatile("cp.async.wait_group 4;" ::: "memory");
-      stage(it + 4, vbits & 1u);
-      vbits >>= 1;
-      fence_proxy_async_smem();
       if (++qi == per_stream) {
         qi = 0;
         if (++g == G) {
@@ -706,9 +734,10 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
 }
 
 // Before: clears the slot's dQ accumulator and the slot's share of the dK / dV sums (stores, nothing waits for them),
-// and forms Delta[b,hq,s] = sum_c dO[b,s,hq,c] * O[b,s,hq,c].  A row of DH bf16 is DH/8 16-byte pieces: each warp takes
-// 256/DH rows at a time (one piece per lane, every lane busy), two such groups per iteration so that four
-// loads per lane are in flight, and reduces inside the DH/8-lane segments.  Bound: HBM.
+// and forms Delta[b,hq,s] = sum_c dO[b,s,hq,c] * O[b,s,hq,c].
+// A row of DH bf16 is DH/8 16-byte pieces, and a load of a warp takes 256/DH rows (every lane busy): of consecutive tokens of one
+// head, whose results lie side by side, with the other heads of these tokens in the warps beside it.  Two such loads of
+// O and of dO are in flight, reduced inside the DH/8-lane segments.  Bound: HBM.
 template <int DH>
 __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
   constexpr int LANES = DH / 8;          // lanes per row
@@ -727,13 +756,13 @@ __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
   }
   const __nv_bfloat16* o = p.o[slot];
   const __nv_bfloat16* d_o = p.d_o[slot];
-  float* delta = p.delta[slot];
+  float* const delta = p.delta[slot];
   const int S = p.S, Hq = p.Hq;
-  const size_t rows = size_t(p.B) * S * Hq;
+  constexpr int TOKS = 2 * ROWS;         // of a unit
+  const int per_seq = (S + TOKS - 1) / TOKS;
+  const size_t units = size_t(p.B) * per_seq * Hq;
   const int lane = threadIdx.x & 31;
   const int sub = lane / LANES, piece = lane % LANES;
-  const size_t warp_global = first >> 5;
-  const size_t n_warps = stride >> 5;
   auto dot8 = [](const uint4& a, const uint4& g) {
     const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
     const __nv_bfloat162* pg = reinterpret_cast<const __nv_bfloat162*>(&g);
@@ -745,33 +774,26 @@ __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
     }
     return acc;
   };
-  for (size_t base = warp_global * (2 * ROWS); base < rows; base += n_warps * (2 * ROWS)) {
-    if (base + n_warps * (2 * ROWS) >= rows) grid_dep_launch();
-    const size_t r0 = base + sub, r1 = base + ROWS + sub;
+  for (size_t u = first >> 5; u < units; u += stride >> 5) {
+    if (u + (stride >> 5) >= units) grid_dep_launch();
+    const int hq = int(u % Hq);
+    const size_t group = u / Hq, b = group / per_seq;
+    const int s0 = int(group % per_seq) * TOKS + sub, s1 = s0 + ROWS;
+    const size_t at = ((b * S + s0) * Hq + hq) * DH + piece * 8, next = size_t(ROWS) * Hq * DH;
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    const uint4 a0 = r0 < rows ? *reinterpret_cast<const uint4*>(o + r0 * DH + piece * 8) : z;
-    const uint4 g0 = r0 < rows ? *reinterpret_cast<const uint4*>(d_o + r0 * DH + piece * 8) : z;
-    const uint4 a1 = r1 < rows ? *reinterpret_cast<const uint4*>(o + r1 * DH + piece * 8) : z;
-    const uint4 g1 = r1 < rows ? *reinterpret_cast<const uint4*>(d_o + r1 * DH + piece * 8) : z;
+    const uint4 a0 = s0 < S ? *reinterpret_cast<const uint4*>(o + at) : z;
+    const uint4 g0 = s0 < S ? *reinterpret_cast<const uint4*>(d_o + at) : z;
+    const uint4 a1 = s1 < S ? *reinterpret_cast<const uint4*>(o + at + next) : z;
+    const uint4 g1 = s1 < S ? *reinterpret_cast<const uint4*>(d_o + at + next) : z;
     float acc0 = dot8(a0, g0), acc1 = dot8(a1, g1);
 #pragma unroll
     for (int sft = LANES / 2; sft > 0; sft >>= 1) {
       acc0 += __shfl_xor_sync(0xffffffffu, acc0, sft);
       acc1 += __shfl_xor_sync(0xffffffffu, acc1, sft);
     }
-    if (piece == 0) {
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const size_t row = u == 0 ? r0 : r1;
-        if (row < rows) {
-          const int hq = int(row % Hq);
-          const size_t tok = row / Hq;
-          const int sx = int(tok % S);
-          const int bx = int(tok / S);
-          delta[(size_t(bx) * Hq + hq) * S + sx] = u == 0 ? acc0 : acc1;
-        }
-      }
-    }
+    // a lane each for the rows of the two loads
+    const int s = piece == 0 ? s0 : s1;
+    if (piece < 2 && s < S) delta[(b * Hq + hq) * S + s] = piece == 0 ? acc0 : acc1;
   }
 }
 
@@ -904,12 +926,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         if (rc == KVP_OK) rc = make_map_bshd(&p.map_do[slots], d_o[l], s->B, s->S, s->Hq, dh, BQ2);
         if (rc != KVP_OK) return rc;
         p.lse[slots] = lse[l];
-        p.delta[slots] = reinterpret_cast<const float*>(wsb + size_t(l) * delta_bytes);
+        p.delta[slots] = ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
         ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
         ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
         ax.dq[slots] = dq[l];
-        ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
         ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
       }

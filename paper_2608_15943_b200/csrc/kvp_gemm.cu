@@ -1070,9 +1070,9 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   p.idesc = umma_idesc_bf16(SROWS, cfg.nt, 0, 0);
   // Tensor memory is shared out in proportion to shared memory, so that CTAs of this kernel that fit on an SM by the latter
   // never wait for the former: a CTA that waits holds up the peers of its cluster.  40 KB keep it off the SMs of the GEMM
-  // kernels that take all 512 columns, which have peers too, and of the attention kernels at head size 128.  Those at head
-  // size 64 (114 and 149 KB) can share an SM with it, and one of the two then waits in its allocation until the other
-  // ends; it does end, for a CTA of the attention waits for no other CTA.
+  // kernels that take all 512 columns, which have peers too, and of the attention backward and the forward at head size 128.
+  // The forward at head size 64 (114 KB) can share an SM with it, and one of the two then waits in its allocation until the
+  // other ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.parts * cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
   const bool wide = cfg.split <= 2 && cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
