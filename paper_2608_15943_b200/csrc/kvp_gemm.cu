@@ -485,6 +485,11 @@ constexpr int SPLIT_THREADS = 192;
 // k-blocks of B a CTA asks into L2 before the kernels ahead of it have finished (a token step's 56 kernels: 601 us
 // without, 595 with 8, 613 with 32)
 constexpr int SPLIT_PREFETCH = 8;
+// From this much of B on, a quarter of L2, and with one tile of tokens, B is read with the policy evict_first: nothing finds it in
+// L2 again, and what the launches beside it ask into L2 stays (token steps with d 4096 of 1, 8, 16 and 32 sequences, us: 199 -> 195, 396
+// -> 389, 548 -> 541, 425 -> 417).  Smaller ones may be there still at the next step, and loads with a policy of any kind slow
+// tiles that share B (1155 x 1024 x 2816 11.1 -> 12.2).
+constexpr double SPLIT_STREAM_BYTES = 32 * 1024 * 1024;
 
 struct SplitProblem {
   int M, N;
@@ -505,8 +510,9 @@ struct SplitParams {
   uint32_t idesc;
 };
 
-// WIDE: four tokens a warp at a time.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.
-template <int NP, bool WIDE, int PARTS>
+// WIDE: four tokens a warp at a time.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.  STREAM: B,
+// which one CTA reads once, is marked first to go in L2.
+template <int NP, bool WIDE, int PARTS, bool STREAM>
 __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -557,13 +563,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
 
   if (warp == 0) {
     const uint32_t leader = elect_one();
+    const uint64_t policy = STREAM ? l2_evict_first() : 0;
     int s = 0;
     uint32_t ph = 1;
     for (int kb = kb0; kb < kb1; ++kb) {
       if (!mbar_wait(&empty[s], ph, err)) break;
       uint8_t* sb = smem + s * stage_bytes;
       mbar_expect_tx_e(&full[s], stage_bytes, leader);
-      tma_load_2d_e(sb, &p.map_b[pi], &full[s], kb * BK, n0, leader);
+      if constexpr (STREAM) tma_load_2d_e(sb, &p.map_b[pi], &full[s], kb * BK, n0, policy, leader);
+      else tma_load_2d_e(sb, &p.map_b[pi], &full[s], kb * BK, n0, leader);
       tma_load_2d_e(sb + SB_BYTES, &p.map_a[pi], &full[s], kb * BK, m0, leader);
       if (++s == stages) {
         s = 0;
@@ -1038,14 +1046,17 @@ bool k_major(const GemmProblem* probs, int n) {
 }
 
 template <int NP, bool WIDE, int PARTS>
-auto split_kernel() -> decltype(&gemm_split_kernel<NP, WIDE, PARTS>) {
-  return allow_smem<gemm_split_kernel<NP, WIDE, PARTS>>(226 * 1024) == cudaSuccess ? &gemm_split_kernel<NP, WIDE, PARTS> : nullptr;
+auto split_kernel(bool stream_b) -> decltype(&gemm_split_kernel<NP, WIDE, PARTS, true>) {
+  if (stream_b) return allow_smem<gemm_split_kernel<NP, WIDE, PARTS, true>>(226 * 1024) == cudaSuccess ? &gemm_split_kernel<NP, WIDE, PARTS, true> : nullptr;
+  return allow_smem<gemm_split_kernel<NP, WIDE, PARTS, false>>(226 * 1024) == cudaSuccess ? &gemm_split_kernel<NP, WIDE, PARTS, false> : nullptr;
 }
 
 template <int NP>
 int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaStream_t stream) {
   SplitParams<NP> p;
   int tiles = 0;
+  bool once = true;      // one tile of tokens: no element of B is read by a second CTA
+  double b_bytes = 0;
   for (int i = 0; i < n; ++i) {
     const GemmProblem& g = probs[i];
     SplitProblem& q = p.prob[i];
@@ -1053,6 +1064,8 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
     q.N = g.N;
     q.tok_tiles = (g.M + cfg.nt - 1) / cfg.nt;
     tiles += q.tok_tiles * ((g.N + SROWS - 1) / SROWS);
+    once = once && q.tok_tiles == 1;
+    b_bytes += 2. * g.N * g.segs[0].K;
     q.tile_end = tiles;
     q.kblocks = (g.segs[0].K + BK - 1) / BK;
     q.out_f32 = g.out_f32;
@@ -1075,9 +1088,10 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // other ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.parts * cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
+  const bool stream_b = once && b_bytes >= SPLIT_STREAM_BYTES;
   const bool wide = cfg.split <= 2 && cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
-  auto* const kernel = cfg.parts == 2 ? (wide ? split_kernel<NP, true, 2>() : split_kernel<NP, false, 2>())
-                                      : (wide ? split_kernel<NP, true, 1>() : split_kernel<NP, false, 1>());
+  auto* const kernel = cfg.parts == 2 ? (wide ? split_kernel<NP, true, 2>(stream_b) : split_kernel<NP, false, 2>(stream_b))
+                                      : (wide ? split_kernel<NP, true, 1>(stream_b) : split_kernel<NP, false, 1>(stream_b));
   if (kernel == nullptr) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e = launch_kernel(kernel, tiles * cfg.split, SPLIT_THREADS, smem, stream, cfg.split, p);

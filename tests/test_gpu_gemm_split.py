@@ -42,6 +42,12 @@ def test_few_rows(M, N, K):
     assert ((c16.double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all()
 
 
+@pytest.mark.parametrize("M,N,K", [(5, 4104, 4104), (128, 11016, 1608), (33, 18440, 920), (70, 1032, 16400)])
+def test_few_rows_streamed_b(M, N, K):
+    """B just above a quarter of L2, read with a cache policy: two accumulators, one, no split, eight pieces of K."""
+    test_few_rows(M, N, K)
+
+
 def test_few_rows_grouped_projections():
     """Q, K and V projections of twelve layers with one token per sequence: 20 problems in one launch, two widths."""
     from paper_2608_15943_b200 import kvp
