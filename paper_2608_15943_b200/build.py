@@ -16,6 +16,7 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
+HEADER = os.path.join(os.path.dirname(HERE), "include", "kvp.h")
 LIB = os.path.join(HERE, "libkvp.so")
 PACK = os.path.join(HERE, "_pack.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -28,7 +29,7 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std
 
 def _newest_header() -> float:
     hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
-    hs.append(os.path.join(os.path.dirname(HERE), "include", "kvp.h"))
+    hs.append(HEADER)
     return max(os.path.getmtime(h) for h in hs)
 
 
@@ -56,7 +57,7 @@ def _build_pack(force: bool) -> None:
     src = os.path.join(CSRC, "kvp_pack.cpp")
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
     key, key_file = _pack_key(torch_dir), os.path.join(OBJ, "_pack.key")
-    if not force and os.path.exists(PACK) and os.path.getmtime(PACK) > os.path.getmtime(src) and os.path.exists(key_file):
+    if not force and os.path.exists(PACK) and os.path.getmtime(PACK) > max(os.path.getmtime(src), os.path.getmtime(HEADER)) and os.path.exists(key_file):
         with open(key_file) as fh:
             if fh.read() == key:
                 return

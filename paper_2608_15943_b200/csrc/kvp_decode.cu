@@ -49,7 +49,7 @@ constexpr int DEC_CTAS_PER_SM = DH == 128 ? 2 : 4;   // as many as shared memory
 // granules a warp, 2.12e-3 so, 0.6 % slower.  Against the largest of each granule by itself: 1.94e-3, 1.2 % slower.)
 constexpr int REFERENCE_GRANULES = 16;
 constexpr float REFERENCE_DROP = 8.f;
-constexpr int MAX_DEC_GROUPS = 64;
+constexpr int MAX_DEC_GROUPS = 64, FEW_DEC_GROUPS = 8;   // a launch of few groups has a parameter block of 1 KB, not 8: 0.6 us less to launch
 constexpr int MAX_MEMBERS = 4;     // layers of a donor group served by one pass (rows = members * G <= 16)
 
 __device__ int g_dec_status;
@@ -64,8 +64,7 @@ struct DecGroup {
   int pad;
 };
 
-struct DecParams {
-  DecGroup grp[MAX_DEC_GROUPS];
+struct DecSizes {
   const int32_t* block_table;  // [B, max_pages]
   const int32_t* lengths;      // [B]
   float* part_o;               // [pieces][rows][DH]
@@ -79,14 +78,18 @@ struct DecParams {
   int io_f32;                  // queries are read and outputs written as fp32 (rounded to bf16 on load / widened on store)
   float scale_log2;
 };
+template <int NG>
+struct DecParams : DecSizes {
+  DecGroup grp[NG];
+};
 
-__device__ __forceinline__ int clamp_length(const DecParams& p, int len) { return min(max(len, 1), p.max_pages * p.page_size); }
-__device__ __forceinline__ int clamped_length(const DecParams& p, int b) { return clamp_length(p, p.lengths[b]); }
+__device__ __forceinline__ int clamp_length(const DecSizes& p, int len) { return min(max(len, 1), p.max_pages * p.page_size); }
+__device__ __forceinline__ int clamped_length(const DecSizes& p, int b) { return clamp_length(p, p.lengths[b]); }
 __device__ __forceinline__ int granules_of(int len) { return (len + GRAN - 1) / GRAN; }
 
 // Over the batch, formed by one warp: granules (of one KV head) of the sequences before b_before, of all, and of the longest.
 // len0: the length (unclamped) of the lane's sequence among the first 32.
-__device__ __forceinline__ void sum_granules(const DecParams& p, int len0, int b_before, int& before, int& all, int& longest) {
+__device__ __forceinline__ void sum_granules(const DecSizes& p, int len0, int b_before, int& before, int& all, int& longest) {
   const int lane = threadIdx.x & 31;
   int sum = 0, most = 0, first = 0;
   for (int b = lane; b < p.B; b += 32) {
@@ -105,7 +108,7 @@ __device__ __forceinline__ void sum_granules(const DecParams& p, int len0, int b
 // only look behind it.  (From the wait to a block's first data went 4.2 to 6 us, most of it this arithmetic out of a cold
 // instruction cache.  Append, decode and merge, us: 8 sequences of 8K-16K in four layers 133.4 -> 130.0, 15 of 2K-4K in six
 // 40.5 -> 37.0, 8 of 12K in five 67.3 -> 63.3, 28 of 1000 in three 30.4 -> 28.3.)
-__device__ __forceinline__ int early_length(const DecParams& p) {
+__device__ __forceinline__ int early_length(const DecSizes& p) {
   const int lane = threadIdx.x & 31;
   return lane < p.B ? __ldcg(p.lengths + lane) : 0;
 }
@@ -169,8 +172,8 @@ __device__ __forceinline__ uint32_t ring_off(int row, int chunk) {
   return uint32_t(row) * (DH * 2) + (uint32_t(chunk ^ (row & 7)) << 4);
 }
 
-template <int DH>
-__global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kernel(const __grid_constant__ DecParams p) {
+template <int DH, int NG>
+__global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kernel(const __grid_constant__ DecParams<NG> p) {
   constexpr int ROW_BYTES = DH * 2;
   constexpr int CHUNKS = ROW_BYTES / 16;           // 16-byte chunks per row
   constexpr int TILE_BYTES = GRAN * ROW_BYTES;     // K (or V) part of a stage
@@ -616,8 +619,8 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM<DH>) decode_kerne
 // `wpr` of them share a row of a unit (one where a unit has few pieces, eight where it has many), each lane four
 // columns.  Bound: latency; the pieces are in L2.
 constexpr int COMBINE_THREADS = 256;
-template <int DH>
-__global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const __grid_constant__ DecParams p, int wpr) {
+template <int DH, int NG>
+__global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const __grid_constant__ DecParams<NG> p, int wpr) {
   constexpr int LANES = DH / 4;               // lanes per piece and row
   constexpr int PER_WARP = 32 / LANES;        // pieces a warp takes at a time
   __shared__ float s_m[COMBINE_THREADS / 32], s_l[COMBINE_THREADS / 32];
@@ -738,18 +741,23 @@ __global__ void __launch_bounds__(COMBINE_THREADS) decode_combine_kernel(const _
 }
 
 // Owners write the new token's K and V rows into their pages.
-struct AppendParams {
-  const void* k_new[MAX_DEC_GROUPS];   // [B,Hkv,dh] bf16, or fp32 when new_f32 (rounded to bf16 as it is stored)
-  const void* v_new[MAX_DEC_GROUPS];
-  __nv_bfloat16* k_cache[MAX_DEC_GROUPS];
-  __nv_bfloat16* v_cache[MAX_DEC_GROUPS];
+struct AppendLayer {
+  const void *k_new, *v_new;           // [B,Hkv,dh] bf16, or fp32 when new_f32 (rounded to bf16 as it is stored)
+  __nv_bfloat16 *k_cache, *v_cache;
+};
+struct AppendSizes {
   const int32_t* block_table;
   const int32_t* lengths;
   int B, Hkv, dh, page_size, max_pages, n_pages;
   int new_f32;
 };
+template <int NG>
+struct AppendParams : AppendSizes {
+  AppendLayer at[NG];
+};
 
-__global__ void append_kernel(const __grid_constant__ AppendParams p) {
+template <int NG>
+__global__ void append_kernel(const __grid_constant__ AppendParams<NG> p) {
   const int layer = blockIdx.y;
   const int b = blockIdx.x;
   grid_dep_launch();
@@ -768,8 +776,8 @@ __global__ void append_kernel(const __grid_constant__ AppendParams p) {
   const int n = p.Hkv * row_chunks;
   uint4 k = make_uint4(0u, 0u, 0u, 0u), v = k;
   if (threadIdx.x < n) {
-    k = eight(p.k_new[layer], threadIdx.x);
-    v = eight(p.v_new[layer], threadIdx.x);
+    k = eight(p.at[layer].k_new, threadIdx.x);
+    v = eight(p.at[layer].v_new, threadIdx.x);
   }
   const int len = p.lengths[b];
   const int cap = p.max_pages * p.page_size;
@@ -780,14 +788,22 @@ __global__ void append_kernel(const __grid_constant__ AppendParams p) {
   for (int idx = threadIdx.x; idx < n;) {
     const int hk = idx / row_chunks, c = idx % row_chunks;
     const size_t dst = ((size_t(page) * p.Hkv + hk) * p.page_size + pos % p.page_size) * p.dh + c * 8;
-    *reinterpret_cast<uint4*>(p.k_cache[layer] + dst) = k;
-    *reinterpret_cast<uint4*>(p.v_cache[layer] + dst) = v;
+    *reinterpret_cast<uint4*>(p.at[layer].k_cache + dst) = k;
+    *reinterpret_cast<uint4*>(p.at[layer].v_cache + dst) = v;
     idx += blockDim.x;
     if (idx < n) {
-      k = eight(p.k_new[layer], idx);
-      v = eight(p.v_new[layer], idx);
+      k = eight(p.at[layer].k_new, idx);
+      v = eight(p.at[layer].v_new, idx);
     }
   }
+}
+
+template <int NG>
+cudaError_t launch_append(const AppendParams<MAX_DEC_GROUPS>& all, int n, cudaStream_t stream) {
+  AppendParams<NG> p;
+  static_cast<AppendSizes&>(p) = all;
+  std::copy(all.at, all.at + n, p.at);
+  return launch_kernel(append_kernel<NG>, dim3(all.B, n), 128, 0, stream, 1, p);
 }
 
 int check_desc(const kvp_decode_desc* d) {
@@ -909,7 +925,7 @@ extern "C" int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, 
   for (int l = 0; l < d->L; ++l)
     if (donor[l] < 0 || donor[l] > l || donor[donor[l]] != donor[l]) return KVP_ERR_BAD_DONOR;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  AppendParams p;
+  AppendParams<MAX_DEC_GROUPS> p;
   p.block_table = block_table;
   p.lengths = lengths;
   p.B = d->B;
@@ -925,14 +941,10 @@ extern "C" int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, 
     if (owner) {
       if (k_new[l] == nullptr || v_new[l] == nullptr || k_cache[l] == nullptr || v_cache[l] == nullptr)
         return KVP_ERR_INVALID_ARG;
-      p.k_new[n] = k_new[l];
-      p.v_new[n] = v_new[l];
-      p.k_cache[n] = reinterpret_cast<__nv_bfloat16*>(k_cache[l]);
-      p.v_cache[n] = reinterpret_cast<__nv_bfloat16*>(v_cache[l]);
-      ++n;
+      p.at[n++] = AppendLayer{k_new[l], v_new[l], reinterpret_cast<__nv_bfloat16*>(k_cache[l]), reinterpret_cast<__nv_bfloat16*>(v_cache[l])};
     }
     if (n == MAX_DEC_GROUPS || (l == d->L && n > 0)) {
-      if (launch_kernel(append_kernel, dim3(d->B, n), 128, 0, stream, 1, p) != cudaSuccess) return KVP_ERR_CUDA;
+      if ((n <= FEW_DEC_GROUPS ? launch_append<FEW_DEC_GROUPS>(p, n, stream) : launch_append<MAX_DEC_GROUPS>(p, n, stream)) != cudaSuccess) return KVP_ERR_CUDA;
       n = 0;
     }
   }
@@ -941,6 +953,22 @@ extern "C" int kvp_cache_append(const kvp_decode_desc* d, const int32_t* donor, 
 
 namespace kvp {
 namespace {
+
+template <int DH, int NG>
+cudaError_t launch_decode(const DecParams<MAX_DEC_GROUPS>& all, dim3 grid, dim3 combine_grid, int wpr, cudaStream_t stream) {
+  constexpr int smem = DEC_WARPS * DEC_STAGES * 2 * GRAN * DH * 2;
+  cudaError_t e = allow_smem<decode_kernel<DH, NG>>(smem);
+  if (e != cudaSuccess) return e;
+  DecParams<NG> p;
+  static_cast<DecSizes&>(p) = all;
+  std::copy(all.grp, all.grp + all.n_groups, p.grp);
+  timing_before(KVP_KERNEL_DECODE, stream);
+  e = launch_kernel(decode_kernel<DH, NG>, grid, DEC_THREADS, smem, stream, 1, p);
+  timing_after(KVP_KERNEL_DECODE, stream);
+  if (e == cudaSuccess && (p.num_splits > 0 || p.by_units == 0))   // whole units leave no pieces
+    e = launch_kernel(decode_combine_kernel<DH, NG>, combine_grid, COMBINE_THREADS, 0, stream, 1, p, wpr);
+  return e;
+}
 
 int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, const void* const* q, const void* const* k_cache,
                 const void* const* v_cache, const int32_t* block_table, const int32_t* lengths, void* const* o,
@@ -961,7 +989,7 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
   if (ws == nullptr || ws_bytes < sc_plan.bytes || !aligned16(ws)) return KVP_ERR_WORKSPACE;
   const size_t po_bytes = align256(sc_plan.pieces * sc_plan.rows * d->dh * 4);
 
-  DecParams p;
+  DecParams<MAX_DEC_GROUPS> p;
   p.block_table = block_table;
   p.lengths = lengths;
   p.part_o = reinterpret_cast<float*>(ws);
@@ -979,9 +1007,6 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
   p.io_f32 = d->dtype == KVP_F32;
   const float sc = scale == 0.f ? 1.f / sqrtf(float(d->dh)) : scale;
   p.scale_log2 = sc * 1.4426950408889634f;
-
-  const int smem = DEC_WARPS * DEC_STAGES * 2 * GRAN * d->dh * 2;
-  if ((d->dh == 128 ? allow_smem<decode_kernel<128>>(smem) : allow_smem<decode_kernel<64>>(smem)) != cudaSuccess) return KVP_ERR_CUDA;
 
   for (int s0 = 0; s0 < n_sub; s0 += MAX_DEC_GROUPS) {
     const int n = n_sub - s0 < MAX_DEC_GROUPS ? n_sub - s0 : MAX_DEC_GROUPS;
@@ -1017,11 +1042,9 @@ int decode_impl(const kvp_decode_desc* d, const int32_t* donor, float scale, con
     const int rows_per_block = COMBINE_THREADS / 32 / wpr;
     const dim3 grid(static_cast<unsigned>(blocks));
     const dim3 cgrid(unsigned(units), (rows + rows_per_block - 1) / rows_per_block);
-    timing_before(KVP_KERNEL_DECODE, stream);
-    cudaError_t e = launch_kernel(d->dh == 128 ? decode_kernel<128> : decode_kernel<64>, grid, DEC_THREADS, smem, stream, 1, p);
-    timing_after(KVP_KERNEL_DECODE, stream);
-    if (e == cudaSuccess && (d->num_splits > 0 || p.by_units == 0))   // whole units leave no pieces
-      e = launch_kernel(d->dh == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, cgrid, COMBINE_THREADS, 0, stream, 1, p, wpr);
+    const bool few = n <= FEW_DEC_GROUPS;
+    const cudaError_t e = d->dh == 128 ? (few ? launch_decode<128, FEW_DEC_GROUPS>(p, grid, cgrid, wpr, stream) : launch_decode<128, MAX_DEC_GROUPS>(p, grid, cgrid, wpr, stream))
+                                       : (few ? launch_decode<64, FEW_DEC_GROUPS>(p, grid, cgrid, wpr, stream) : launch_decode<64, MAX_DEC_GROUPS>(p, grid, cgrid, wpr, stream));
     if (e != cudaSuccess) return KVP_ERR_CUDA;
   }
   return KVP_OK;

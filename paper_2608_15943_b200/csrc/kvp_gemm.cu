@@ -1174,8 +1174,9 @@ int gemm_pair_mode() { return g_pair_mode; }
 
 namespace {
 
-template <typename F1, typename F4, typename F32>
-int by_count(int n, F1 one, F4 four, F32 many) { return n == 1 ? one() : n <= 4 ? four() : many(); }
+// parameter blocks of three sizes: each 8 KB of them take 0.6 us to launch
+template <typename F1, typename F8, typename F32>
+int by_count(int n, F1 one, F8 eight, F32 many) { return n == 1 ? one() : n <= 8 ? eight() : many(); }
 
 // The gradient GEMMs of a launch (pair mode 1) run on gemm_tall_kernel, in tiles of 256 rows; of 128 where those would
 // leave half of the pairs idle.  Measured (us, all weight and input gradients of a backward pass: gemm_kernel / tiles of
@@ -1198,7 +1199,7 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
   if (flop > GRADIENT_MAX_FLOP) return launch_group(probs, n, stream, 0, 0, false);
   const int nt = 4 * tiles <= sm_count() ? 128 : 256;
   if (segs == 1) return launch_tall<1, 1>(probs, n, nt, false, stream);
-  if (segs <= 4) return launch_tall<4, 4>(probs, n, nt, false, stream);
+  if (n <= 8 && segs <= 12) return launch_tall<8, 12>(probs, n, nt, false, stream);
   return launch_tall<MAX_PROB, MAX_MAPS / 2>(probs, n, nt, false, stream);
 }
 
@@ -1216,7 +1217,7 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
       const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
       const GemmProblem* g = probs + begin;
       const SplitConfig cfg = split_config(sizes_of(g, cnt), cnt, sm_count());
-      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
+      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream); },
                               [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream); });
       if (rc != KVP_OK) return rc;
     }
@@ -1229,11 +1230,11 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
     const Choice c = choose_forward(sizes_of(g, cnt), cnt, sm_count());
     int rc;
     if (c.kind == Choice::kTall) {
-      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, true, stream); }, [&] { return launch_tall<4, 4>(g, cnt, c.nt, true, stream); },
+      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, true, stream); }, [&] { return launch_tall<8, 8>(g, cnt, c.nt, true, stream); },
                     [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, true, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, 1, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
-      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<4>(g, cnt, cfg, stream); },
+      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream); },
                     [&] { return launch_split<MAX_PROB>(g, cnt, cfg, stream); });
     } else {
       rc = launch_group(g, cnt, stream, 0, 0, c.kind == Choice::kPair);

@@ -105,6 +105,10 @@ lib.kvp_gemm.argtypes = [C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int64, C.c_i
 def gemm(a: torch.Tensor, b: torch.Tensor, c: torch.Tensor, a_mn: bool = False, b_mn: bool = False) -> torch.Tensor:
     """c[M,N] = A B.  a is stored [M,K] (a_mn False) or [K,M]; b is stored [N,K] (b_mn False) or
     [K,N]; c is bf16 or fp32, row-major."""
+    status = _pack.gemm(a, b, c, a_mn, b_mn, _stream())
+    if status is not NotImplemented:
+        _check(status, "kvp_gemm")
+        return c
     M, N = c.shape
     K = a.shape[0] if a_mn else a.shape[1]
     _check(lib.kvp_gemm(M, N, K, a.data_ptr(), a.stride(0), int(a_mn), b.data_ptr(), b.stride(0), int(b_mn),
@@ -127,6 +131,10 @@ lib.kvp_add.argtypes = [C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_
 
 def rmsnorm(x: torch.Tensor, w: torch.Tensor, eps: float, y: torch.Tensor) -> torch.Tensor:
     """kvp_rmsnorm: y[T,D] = x / sqrt(mean(x^2) + eps) * w (bf16)."""
+    status = _pack.rmsnorm(x, w, eps, y, _stream())
+    if status is not NotImplemented:
+        _check(status, "kvp_rmsnorm")
+        return y
     T, D = x.shape
     _check(lib.kvp_rmsnorm(T, D, x.data_ptr(), w.data_ptr(), float(eps), y.data_ptr(), _stream()), "kvp_rmsnorm")
     return y
@@ -134,6 +142,10 @@ def rmsnorm(x: torch.Tensor, w: torch.Tensor, eps: float, y: torch.Tensor) -> to
 
 def rope(x: torch.Tensor, theta: float = 10000.0, pos0: int = 0) -> torch.Tensor:
     """kvp_rope: in place on x [B,S,H,dh] (bf16)."""
+    status = _pack.rope(x, theta, pos0, _stream())
+    if status is not NotImplemented:
+        _check(status, "kvp_rope")
+        return x
     B, S, H, dh = x.shape
     _check(lib.kvp_rope(B, S, H, dh, float(theta), int(pos0), x.data_ptr(), _stream()), "kvp_rope")
     return x
@@ -141,12 +153,20 @@ def rope(x: torch.Tensor, theta: float = 10000.0, pos0: int = 0) -> torch.Tensor
 
 def swiglu(gate: torch.Tensor, up: torch.Tensor, out: torch.Tensor) -> torch.Tensor:
     """kvp_swiglu: out = silu(gate) * up (bf16, same shapes)."""
+    status = _pack.swiglu(gate, up, out, _stream())
+    if status is not NotImplemented:
+        _check(status, "kvp_swiglu")
+        return out
     _check(lib.kvp_swiglu(gate.numel(), gate.data_ptr(), up.data_ptr(), out.data_ptr(), _stream()), "kvp_swiglu")
     return out
 
 
 def add(a: torch.Tensor, b: torch.Tensor, out: torch.Tensor) -> torch.Tensor:
     """kvp_add: out = a + b (bf16, same shapes)."""
+    status = _pack.add(a, b, out, _stream())
+    if status is not NotImplemented:
+        _check(status, "kvp_add")
+        return out
     _check(lib.kvp_add(a.numel(), a.data_ptr(), b.data_ptr(), out.data_ptr(), _stream()), "kvp_add")
     return out
 
@@ -268,6 +288,9 @@ def _ws(ws: Optional[torch.Tensor]):
 
 
 def proj_fwd(shape, donor, x, wq, wk, wv, q, k, v, ws=None):
+    status = _pack.proj_fwd(shape, donor, x, wq, wk, wv, q, k, v, ws, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_proj_fwd")
     p, n = _ws(ws)
     _check(lib.kvp_proj_fwd(C.byref(shape), _donors(donor), _ptr_array(x), _ptr_array(wq), _ptr_array(wk),
                             _ptr_array(wv), _ptr_array(q), _ptr_array(k), _ptr_array(v), p, n, _stream()),
@@ -276,6 +299,10 @@ def proj_fwd(shape, donor, x, wq, wk, wv, q, k, v, ws=None):
 
 def proj_bwd(shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx, ws, layer_begin=None, layer_end=None):
     """kvp_proj_bwd, or kvp_proj_bwd_range when a layer range is given."""
+    if layer_begin is None and layer_end is None:
+        status = _pack.proj_bwd(shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx, ws, _stream())
+        if status is not NotImplemented:
+            return _check(status, "kvp_proj_bwd")
     p, n = _ws(ws)
     args = (C.byref(shape), _donors(donor), _ptr_array(x), _ptr_array(wq), _ptr_array(wk), _ptr_array(wv),
             _ptr_array(dq), _ptr_array(dk_sum), _ptr_array(dv_sum), _ptr_array(dwq), _ptr_array(dwk), _ptr_array(dwv),
@@ -288,16 +315,25 @@ def proj_bwd(shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx,
 
 
 def out_proj_fwd(shape, o, wo, y):
+    status = _pack.out_proj_fwd(shape, o, wo, y, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_out_proj_fwd")
     _check(lib.kvp_out_proj_fwd(C.byref(shape), _ptr_array(o), _ptr_array(wo), _ptr_array(y), _stream()),
            "kvp_out_proj_fwd")
 
 
 def out_proj_bwd(shape, o, wo, dy, d_o, dwo):
+    status = _pack.out_proj_bwd(shape, o, wo, dy, d_o, dwo, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_out_proj_bwd")
     _check(lib.kvp_out_proj_bwd(C.byref(shape), _ptr_array(o), _ptr_array(wo), _ptr_array(dy), _ptr_array(d_o),
                                 _ptr_array(dwo), _stream()), "kvp_out_proj_bwd")
 
 
 def attn_fwd(shape, donor, q, k, v, o, lse, causal=True, scale=0.0, ws=None):
+    status = _pack.attn_fwd(shape, donor, causal, scale, q, k, v, o, lse, ws, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_attn_fwd")
     p, n = _ws(ws)
     _check(lib.kvp_attn_fwd(C.byref(shape), _donors(donor), int(causal), float(scale), _ptr_array(q),
                             _ptr_array(k), _ptr_array(v), _ptr_array(o), _ptr_array(lse), p, n, _stream()),
@@ -305,6 +341,9 @@ def attn_fwd(shape, donor, q, k, v, o, lse, causal=True, scale=0.0, ws=None):
 
 
 def attn_bwd(shape, donor, q, k, v, o, d_o, lse, dq, dk_sum, dv_sum, ws, causal=True, scale=0.0):
+    status = _pack.attn_bwd(shape, donor, causal, scale, q, k, v, o, d_o, lse, dq, dk_sum, dv_sum, ws, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_attn_bwd")
     p, n = _ws(ws)
     _check(lib.kvp_attn_bwd(C.byref(shape), _donors(donor), int(causal), float(scale), _ptr_array(q),
                             _ptr_array(k), _ptr_array(v), _ptr_array(o), _ptr_array(d_o), _ptr_array(lse),
@@ -333,11 +372,20 @@ lib.kvp_decode.argtypes = [C.POINTER(DecodeDesc), C.c_void_p, C.c_float] + [_PP]
     [C.c_void_p, C.c_void_p] + [_PP] * 2 + [C.c_int, C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]
 
 
+# The calls above and below go through _pack where their arguments are plain tensors, lists and numbers, through ctypes otherwise.
+_pack.bind([C.cast(getattr(lib, "kvp_" + n), C.c_void_p).value for n in (
+    "gemm", "rmsnorm", "rope", "swiglu", "add", "proj_fwd", "proj_bwd", "out_proj_fwd", "out_proj_bwd", "attn_fwd", "attn_bwd",
+    "cache_append", "decode")], Shape, DecodeDesc)
+
+
 def decode_workspace_bytes(desc: DecodeDesc, donor) -> int:
     return int(lib.kvp_decode_workspace_bytes(C.byref(desc), _donors(donor)))
 
 
 def cache_append(desc, donor, k_new, v_new, k_cache, v_cache, block_table, lengths):
+    status = _pack.cache_append(desc, donor, k_new, v_new, k_cache, v_cache, block_table, lengths, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_cache_append")
     _check(lib.kvp_cache_append(C.byref(desc), _donors(donor), _ptr_array(k_new), _ptr_array(v_new),
                                 _ptr_array(k_cache), _ptr_array(v_cache), block_table.data_ptr(),
                                 lengths.data_ptr(), _stream()), "kvp_cache_append")
@@ -345,6 +393,9 @@ def cache_append(desc, donor, k_new, v_new, k_cache, v_cache, block_table, lengt
 
 def decode(desc, donor, q, k_cache, v_cache, block_table, lengths, o, lse, ws, scale=0.0, layer_begin=0,
            layer_end=None):
+    status = _pack.decode(desc, donor, scale, q, k_cache, v_cache, block_table, lengths, o, lse, layer_begin, layer_end, ws, _stream())
+    if status is not NotImplemented:
+        return _check(status, "kvp_decode")
     p, n = _ws(ws)
     _check(lib.kvp_decode(C.byref(desc), _donors(donor), float(scale), _ptr_array(q), _ptr_array(k_cache),
                           _ptr_array(v_cache), block_table.data_ptr(), lengths.data_ptr(), _ptr_array(o),

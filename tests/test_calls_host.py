@@ -1,0 +1,134 @@
+"""The native calls of the binding hand the library what its ctypes path does, and leave everything unusual to that path."""
+import ctypes as C
+import types
+
+import pytest
+import torch
+
+NAMES = ("gemm", "rmsnorm", "rope", "swiglu", "add", "proj_fwd", "proj_bwd", "out_proj_fwd", "out_proj_bwd", "attn_fwd", "attn_bwd",
+         "cache_append", "decode")
+# arguments of the entry points: i integer, l 64-bit integer, f float, p pointer, S structure, D donor map, A array of pointers
+FORMS = {"gemm": "iiiplipliplip", "rmsnorm": "iippfpp", "rope": "iiiifipp", "swiglu": "lpppp", "add": "lpppp",
+         "proj_fwd": "SDAAAAAAAplp", "proj_bwd": "SDAAAAAAAAAAAplp", "out_proj_fwd": "SAAAp", "out_proj_bwd": "SAAAAAp",
+         "attn_fwd": "SDifAAAAAplp", "attn_bwd": "SDifAAAAAAAAAplp", "cache_append": "SDAAAAppp", "decode": "SDfAAAppAAiiplp"}
+TYPES = dict(i=C.c_int, l=C.c_int64, f=C.c_float, p=C.c_void_p, S=C.c_void_p, D=C.c_void_p, A=C.c_void_p)
+
+
+@pytest.fixture
+def record(monkeypatch):
+    """What reaches the library, by either path: (name, arguments with the arrays read out)."""
+    from paper_2608_15943_b200 import kvp
+    seen, keep = [], []
+
+    def make(name):
+        form = FORMS[name]
+        size = C.sizeof(kvp.DecodeDesc if name in ("cache_append", "decode") else kvp.Shape)
+
+        def called(*args):
+            layers = C.cast(args[0], C.POINTER(C.c_int32))[0] if form[0] == "S" else 0
+            read = {"S": lambda v: C.string_at(v, size), "D": lambda v: C.string_at(v, 4 * layers), "A": lambda v: C.string_at(v, 8 * layers)}
+            seen.append((name, [read.get(k, lambda v: v)(v) for k, v in zip(form, args)]))
+            return 0
+        return C.CFUNCTYPE(C.c_int, *[TYPES[k] for k in form])(called)
+    for name in NAMES:
+        cb = make(name)
+        keep.append(cb)
+        monkeypatch.setattr(kvp.lib, "kvp_" + name, cb)
+    real = kvp._pack
+    original = [C.cast(getattr(C.CDLL(kvp.LIB_PATH), "kvp_" + n), C.c_void_p).value for n in NAMES]
+    real.bind([C.cast(cb, C.c_void_p).value for cb in keep], kvp.Shape, kvp.DecodeDesc)
+    monkeypatch.setattr(kvp, "_stream", lambda: 0x7f0000001238)
+    none = types.SimpleNamespace(**{n: lambda *a: NotImplemented for n in NAMES})
+
+    def both(call):
+        """The arguments that `call` hands over through ctypes, and whether the native path took it (with the same ones)."""
+        del seen[:]
+        monkeypatch.setattr(kvp, "_pack", none)
+        call()
+        taken = []
+        spy = types.SimpleNamespace(**{n: (lambda n: lambda *a: taken.append(getattr(real, n)(*a)) or taken[-1])(n) for n in NAMES})
+        monkeypatch.setattr(kvp, "_pack", spy)
+        call()
+        monkeypatch.setattr(kvp, "_pack", real)
+        assert len(seen) == 2 and seen[0] == seen[1]
+        return taken == [0]
+    yield kvp, both
+    real.bind(original, kvp.Shape, kvp.DecodeDesc)
+
+
+def bf(*shape):
+    return torch.zeros(*shape, dtype=torch.bfloat16)
+
+
+class Sub(torch.Tensor):
+    pass
+
+
+def test_single_operators(record):
+    kvp, both = record
+    a, b, c = bf(6, 16), bf(24, 16), bf(6, 24)
+    for form in ((a, b, c), (a, b, c.float()), (bf(6, 40)[:, 8:24], bf(24, 32)[:, :16], bf(6, 64)[:, 8:32]), (bf(16, 6), b, c, True), (a, bf(16, 24), c, False, True),
+                 (bf(16, 6), bf(16, 24), c, True, True), (a.t(), b, c)):
+        assert both(lambda: kvp.gemm(*form))
+    x, w, y = bf(5, 32), torch.nn.Parameter(bf(32)), bf(5, 32)
+    assert both(lambda: kvp.rmsnorm(x, w, 1e-5, y))
+    for t in (bf(2, 3, 4, 64), bf(2, 3, 8, 64)[:, 1:, :4]):
+        assert both(lambda: kvp.rope(t)) and both(lambda: kvp.rope(t, 500000.0, 77))
+    for f in (kvp.add, kvp.swiglu):
+        for t in (bf(3, 8), bf(24), bf(0), bf(2, 3, 4)[1], torch.zeros(())):
+            assert both(lambda: f(t, t, t))
+    # left to ctypes: subclasses, other kinds of numbers
+    s, flat, small = bf(6, 16).as_subclass(Sub), bf(384), bf(1, 1, 1, 8)
+    assert not both(lambda: kvp.gemm(s, b, c)) and not both(lambda: kvp.gemm(a, b, c, 0, 0)) and not both(lambda: kvp.gemm(a, flat, c))
+    assert not both(lambda: kvp.rmsnorm(x, w, 1, x)) and not both(lambda: kvp.rope(small, 10000, 2)) and not both(lambda: kvp.add(s, s, s))
+
+
+def test_layer_calls(record):
+    kvp, both = record
+    L = 3
+    sh, de = kvp.Shape(L, 2, 5, 64, 4, 2, 64, kvp.F32), kvp.DecodeDesc(L, 2, 4, 2, 64, 16, 3, 7)
+    donor, t, ws = [0, 1, 1], lambda: [bf(2), None, bf(3, 4)[1:]], bf(100)
+    kinds = (lambda x: x, tuple)
+    for kind in kinds:
+        arr = [kind(t()) for _ in range(11)]
+        dm = kind(donor)
+        assert both(lambda: kvp.proj_fwd(sh, dm, *arr[:7])) and both(lambda: kvp.proj_fwd(sh, dm, *arr[:7], ws))
+        assert both(lambda: kvp.proj_bwd(sh, dm, *arr, ws))
+        assert both(lambda: kvp.out_proj_fwd(sh, *arr[:3])) and both(lambda: kvp.out_proj_bwd(sh, *arr[:5]))
+        for more in ({}, dict(causal=False, scale=0.5, ws=ws)):
+            assert both(lambda: kvp.attn_fwd(sh, dm, *arr[:5], **more))
+        for more in ({}, dict(causal=False, scale=0.25)):
+            assert both(lambda: kvp.attn_bwd(sh, dm, *arr[:9], ws, **more))
+        table, lengths = torch.zeros(2, 3, dtype=torch.int32), torch.ones(2, dtype=torch.int32)
+        assert both(lambda: kvp.cache_append(de, dm, *arr[:4], table, lengths))
+        for more in ({}, dict(scale=0.125, layer_begin=1), dict(layer_end=2), dict(layer_begin=1, layer_end=3)):
+            assert both(lambda: kvp.decode(de, dm, *arr[:3], table, lengths, *arr[3:5], ws, **more))
+    arr = [t() for _ in range(11)]
+    odd = [t()[:2] + [bf(4).as_subclass(Sub)]] + arr[1:]
+    assert not both(lambda: kvp.proj_fwd(sh, donor, *odd[:7])) and not both(lambda: kvp.attn_fwd(sh, donor, *odd[:5]))
+    assert not both(lambda: kvp.proj_fwd(sh, torch.tensor(donor), *arr[:7])) and not both(lambda: kvp.attn_fwd(sh, [0, True, 1], *arr[:5], causal=1, scale=0))
+    assert not both(lambda: kvp.decode(de, donor, *arr[:3], table, lengths, *arr[3:5], ws, scale=0))
+
+
+def test_many_layers(record):
+    """More entries than the native path has room for."""
+    kvp, both = record
+    for L, native in ((60, True), (256, False), (300, False)):
+        sh, ws = kvp.Shape(L, 1, 1, 64, 1, 1, 64), bf(1)
+        arr = [[ws] * L] * 11
+        assert both(lambda: kvp.proj_bwd(sh, [0] * L, *arr, ws)) == native
+
+
+def test_refused_as_before():
+    """What ctypes refuses, and how, with the library itself."""
+    from paper_2608_15943_b200 import kvp
+    x = bf(4, 8)
+    for call, err in ((lambda: kvp.add(x, x, None), AttributeError), (lambda: kvp.gemm(x, x, bf(4)), ValueError), (lambda: kvp.rope(x), ValueError),
+                      (lambda: kvp.attn_fwd(kvp.Shape(1, 1, 1, 64, 1, 1, 64), [2**31], *[[x]] * 5), OverflowError),
+                      (lambda: kvp.attn_fwd(kvp.DecodeDesc(1, 1, 1, 1, 64, 16, 1, 1), [0], *[[x]] * 5), C.ArgumentError),
+                      (lambda: kvp.rmsnorm(x, x, "x", x), ValueError)):
+        with pytest.raises(err):
+            call()
+    with pytest.raises(kvp.KvpError) as e:
+        kvp.add(bf(3), bf(3), bf(3))
+    assert e.value.status == kvp.ERR_UNSUPPORTED and "kvp_add" in str(e.value)
