@@ -18,7 +18,8 @@
 //               accumulator in global memory with bulk reductions (cp.reduce.async.bulk .add.f32, 8 KB
 //               each), so S and dP are computed once for all three gradients.
 //
-//  dq_convert_kernel  scales the fp32 dQ accumulators and writes dQ as bf16 [B,S,Hq,dh].
+//  dq_convert_kernel  scales the fp32 dQ accumulators and writes dQ as bf16 [B,S,Hq,dh].  (Up to 128 tokens a dQ tile has one
+//               partial, which bwd_kernel writes as dQ itself.)
 //
 // Delta = rowsum(dO * O) comes from a small pre-pass.  The dQ accumulators live in the caller's
 // workspace in a blocked layout ([b][hq][64-query tile][32-column quarter][16][32 columns][4 queries] fp32) so that every
@@ -92,6 +93,8 @@ struct BwdParams {
   const float* lse[MAX_GROUP];    // [B,Hq,S]
   const float* delta[MAX_GROUP];  // [B,Hq,S]
   float* dq_acc[MAX_GROUP];       // blocked fp32 accumulators, see dq_acc_floats()
+  void* dq[MAX_GROUP];            // one key tile: dQ itself, [B,S,Hq,dh], bf16 or (dq_f32) the bf16 values as fp32
+  int dq_f32;
   CUtensorMap map_dk[MAX_GROUP], map_dv[MAX_GROUP]; // per group: the fp32 sums [B,S,Hkv,dh], box 32 rows x 32 columns
   int first_slot[MAX_GROUP + 1];
   int cta_begin[MAX_GROUP + 1];
@@ -128,6 +131,17 @@ __device__ __forceinline__ uint4 split3_bf16(float v) {
   out.z = 0u;
   out.w = 0u;
   return out;
+}
+
+// Eight columns from element `at` of dQ on: bf16, or the bf16 values as fp32.
+__device__ __forceinline__ void store_dq(void* dq, int f32, size_t at, const uint4& v) {
+  if (f32) {
+    float* out = reinterpret_cast<float*>(dq) + at;
+    *reinterpret_cast<uint4*>(out) = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
+    *reinterpret_cast<uint4*>(out + 4) = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
+  } else {
+    *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(dq) + at) = v;
+  }
 }
 
 // Floats of one layer's dQ accumulator: [B][Hq][ceil(S/64)][DH/32][16][32][4].
@@ -620,7 +634,32 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       }
       tc_fence_before_sync();
       mbar_arrive(dq_free);
-      if (active) {
+      if (active && n_jt == 1) {
+        // One key tile: the partial is the whole sum, and goes out as dQ: rounded, a lane's eight queries a row of 16 bytes of an
+        // 8x8 matrix in shared memory, back transposed as eight columns of one query, 16 bytes a store.  (Exchanged between lanes
+        // instead it took 1900 cycles a step, more than the rest of the step.)
+        const int q0 = (qt_first + qi) * BQ2 + lane / 4;
+        const size_t at = ((size_t(b) * p.S + q0) * p.Hq + hk * G + g) * DH + quarter * 32 + lane % 4 * 8, step = size_t(8) * p.Hq * DH;
+        void* const dq = p.dq[slot0 + li];
+        // column c of an eight of queries at place (c ^ 2 (c / 8)), which keeps both the stores and the matrices' rows clear of
+        // bank conflicts; row i of matrix m: column 8 (i / 2) + 2 m + i % 2, so that a lane's four registers are adjacent columns
+        auto place = [](int c) { return uint32_t(c ^ (c >> 3 << 1)) * 16; };
+        uint8_t* const put = stg + place(lane);
+        const uint32_t get = smem_u32(stg) + place((lane & 6) * 4 + (lane >> 3) * 2 + (lane & 1));
+        __syncwarp();   // (the reads of the step before)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          auto pair = [&](int i) { return pack_bf16(__uint_as_float(a[8 * e + i]) * p.scale, __uint_as_float(a[8 * e + i + 1]) * p.scale); };
+          *reinterpret_cast<uint4*>(put + e * 512) = make_uint4(pair(0), pair(2), pair(4), pair(6));
+        }
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          uint4 v;
+          ldsm_x4_t(get + e * 512, v.x, v.y, v.z, v.w);
+          if (q0 + 8 * e < p.S) store_dq(dq, p.dq_f32, at + e * step, v);
+        }
+      } else if (active) {
         const size_t tile = ((size_t(b) * p.Hq + hk * G + g) * n_qt + (qt_first + qi)) * (DH / 32) + quarter;
         float* dst = p.dq_acc[slot0 + li] + tile * (BQ2 * 32);
         uint8_t* const buf = stg + (it & (BUFS - 1)) * DQ_STAGE_BYTES;
@@ -722,13 +761,7 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
       const int s = s0 + h * 8 + own;
       if (s >= S) continue;
       const size_t at = ((size_t(bb) * S + s) * Hq + hq) * DH + col;
-      if (p.dq_f32) {
-        float* out = reinterpret_cast<float*>(p.dq[blockIdx.y]) + at;
-        *reinterpret_cast<uint4*>(out) = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
-        *reinterpret_cast<uint4*>(out + 4) = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
-      } else {
-        *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dq[blockIdx.y]) + at) = v;
-      }
+      store_dq(p.dq[blockIdx.y], p.dq_f32, at, v);
     }
   }
 }
@@ -930,7 +963,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
         ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
         ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
-        ax.dq[slots] = dq[l];
+        p.dq[slots] = ax.dq[slots] = dq[l];
         ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
       }
@@ -957,6 +990,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
       p.lse[i] = p.lse[0];
       p.delta[i] = p.delta[0];
       p.dq_acc[i] = p.dq_acc[0];
+      p.dq[i] = p.dq[0];
     }
     for (int i = ng; i < MAX_GROUP; ++i) {
       p.map_k[i] = p.map_k[0];
@@ -981,11 +1015,11 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     p.scale = sc;
     p.scale_log2 = sc * 1.4426950408889634f;
     ax.n_groups = ng;
-    ax.dq_f32 = dq_f32;
+    p.dq_f32 = ax.dq_f32 = dq_f32;
     ax.B = s->B;
     ax.S = s->S;
     ax.Hq = s->Hq;
-    ax.acc_v4 = dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;
+    ax.acc_v4 = n_jt == 1 ? 0 : dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;   // one key tile: bwd_kernel writes dQ
     ax.kv_v4 = size_t(s->B) * s->S * s->Hkv * dh / 4;
     ax.scale = sc;
     // enough blocks for every slot to fill the device, no more than its pieces of 8 (16: convert) accumulators give work to
@@ -1001,6 +1035,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
                   : launch_kernel(bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream, 1, p);
     timing_after(KVP_KERNEL_ATTN_BWD, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
+    if (n_jt == 1) continue;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
     e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid(16), 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
