@@ -704,8 +704,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
 // N, split between the CTAs' loads).  256 x 256 tiles of gemm_pair_kernel pad 347 tokens to 512; here the tokens are cut
 // into tiles of up to 256, in steps of 32.  Forward they are all of one size, walked column by column, so that the columns'
 // weights come from memory once.  Gradients have whole tiles and one of the remainder (in steps of 128 where A is MN-major:
-// its TMA boxes hold 64 rows and each CTA loads half of the tile); the whole tiles go before all remainders, pairs taking
-// turns in alternating direction, so that the short ones fill the pairs that have no second long one.  A lane of the
+// its TMA boxes hold 64 rows and each CTA loads half of the tile), dealt out by cost (kvp_gemm_choice.h).  A lane of the
 // epilogue holds a column, so a warp stores rows of 64
 // consecutive bytes, two at a time (128 in fp32), where a lane of gemm_pair_kernel's holds a row.  Roles, segments and
 // barriers are those of gemm_pair_kernel, the ring has as many stages as tiles of the launch's size leave room for;
@@ -719,7 +718,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
 // ------------------------------------------------------------------------------------------------------------
 constexpr int TCOLS = 256;                        // columns of C per pair
 constexpr int TMAX_STAGES = 10;                   // a stage holds, per CTA, 128 rows of B and half of a tile's rows of A
-constexpr int TALL_EPI_WARPS = 16;                // four for every quarter of the TMEM lanes, taking 32 tokens each in turn
+// Four for every quarter of the TMEM lanes, taking 32 tokens each in turn: all on every tile, or (launches in which pairs have
+// several tiles of few k-blocks) eight on every other one, so that the stores of one tile run while the other eight wait for the
+// next and read it out.  With all sixteen on each the stores of a tile of fp32 results went out at 6.7 TB/s, and nothing for as
+// long again.  Measured (us, sixteen -> eight): 264 tokens, 7 layers of d 1024 74 -> 69; 128 tokens, 8 layers of d 4096 232 -> 216; but
+// 2328 tokens, 3 layers of d 1024 36 -> 39, where the last tiles count.
+constexpr int TALL_EPI_WARPS = 16, TALL_ALTERNATE_ROUNDS = 6, TALL_SHORT_KBLOCKS = 12;
 constexpr int TALL_THREADS = (2 + TALL_EPI_WARPS) * 32;
 constexpr int TALL_RING = 224 * 1024;             // the ring takes as many stages as fit
 constexpr int TALL_SMEM = 1024 + TALL_RING + 256;
@@ -728,6 +732,7 @@ struct TallList {                                 // the tiles of one problem th
   int prob;
   int nt;                                         // tokens (rows of C) per tile, a multiple of 32; of 128 if A is MN-major
   int m_first, n_tok;                             // first token, tiles along the tokens
+  float inv_n_tok;
   int tile_end;                                   // one past the list's last tile in the launch's tile order
   uint32_t idesc;
   short map_a[MAX_SEG];                           // per segment; the box holds half of a tile's tokens
@@ -739,13 +744,24 @@ struct TallProblem {
   long long ldc;
   void* c;
 };
+template <bool MANY>
+struct TallDeal {                                 // gradients: the pairs' tiles, class by class (0 classes: pairs take tiles in turn)
+  int n_classes;
+  uint16_t first[DEAL_CLASSES][DEAL_PAIRS + 1];
+};
+template <>
+struct TallDeal<false> {
+  static constexpr int n_classes = 0;
+};
 template <int NP, int NSEG>                       // problems, and segments of all of them, that the parameter block holds
 struct TallParams {
+  TallDeal<(NP > 1)> deal;
   CUtensorMap map_b[NSEG], map_a[2 * NSEG];
   TallProblem prob[NP];
   TallList list[2 * NP];
   int total_tiles;
   int stages, stage_bytes;
+  int alternate;                                  // eight epilogue warps a tile
 };
 
 template <int NP, int NSEG>
@@ -775,7 +791,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 2 * TALL_EPI_WARPS);
+      mbar_init(&acc_empty[a], 2 * TALL_EPI_WARPS >> p.alternate);
     }
     mbar_fence_init();
   }
@@ -792,19 +808,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
 
   struct Tile {
     int li, prob, nt, m0, n0;
+    int turn, t;   // next tile: round (tiles in turn) or class, and its number there
   };
-  // tile of a round: rounds of n_pairs tiles, dealt forwards and backwards in turn; li only grows
-  auto tile_of = [&](int round, Tile& w) -> bool {
-    const int t = round * n_pairs + ((round & 1) ? n_pairs - 1 - pair : pair);
-    if (t >= total_tiles) return false;
+  // The pair's next tile; li only grows.  In turn: rounds of n_pairs tiles, dealt forwards and backwards.
+  auto next_tile = [&](Tile& w) -> bool {
+    int t;
+    bool dealt = false;
+    if constexpr (NP > 1) {
+      dealt = p.deal.n_classes > 0;
+      if (dealt) {
+        while (w.t >= p.deal.first[w.turn][pair + 1]) {
+          if (++w.turn == p.deal.n_classes) return false;
+          w.t = p.deal.first[w.turn][pair];
+        }
+        t = w.t++;
+      }
+    }
+    if (!dealt) {
+      do {
+        if (w.turn * n_pairs >= total_tiles) return false;
+        t = w.turn * n_pairs + ((w.turn & 1) ? n_pairs - 1 - pair : pair);
+        ++w.turn;
+      } while (t >= total_tiles);   // only the last round can be short
+    }
     while (t >= p.list[w.li].tile_end) ++w.li;
     const TallList& l = p.list[w.li];
     const int within = t - (w.li ? p.list[w.li - 1].tile_end : 0);
     w.prob = l.prob;
     w.nt = l.nt;
-    w.m0 = l.m_first + (within % l.n_tok) * l.nt;
-    w.n0 = (within / l.n_tok) * TCOLS;
+    int column = int(float(within) * l.inv_n_tok), tok = within - column * l.n_tok;   // (right to within one, for up to 2^24 tiles)
+    if (tok < 0) {
+      --column;
+      tok += l.n_tok;
+    } else if (tok >= l.n_tok) {
+      ++column;
+      tok -= l.n_tok;
+    }
+    w.m0 = l.m_first + tok * l.nt;
+    w.n0 = column * TCOLS;
     return true;
+  };
+  auto first_tile = [&]() {
+    Tile w{};
+    if constexpr (NP > 1)
+      if (p.deal.n_classes > 0) w.t = p.deal.first[0][pair];
+    return w;
   };
 
   if (warp == 0) {
@@ -813,9 +861,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
     int s = 0;
     uint32_t ph = 1;
     bool ok = true;
-    Tile w{};
-    for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
-      if (!tile_of(round, w)) continue;   // only the last round can be short
+    Tile w = first_tile();
+    while (ok && next_tile(w)) {
       const TallProblem& pr = p.prob[w.prob];
       const int half = w.nt / 2, a_mn = pr.a_mn, b_mn = pr.b_mn;
       const uint32_t bytes = 2u * uint32_t(PA_BYTES + half * (BK * 2));   // of both CTAs
@@ -856,9 +903,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
       int s = 0;
       uint32_t ph = 0, tile_i = 0;
       bool ok = true;
-      Tile w{};
-      for (int round = 0; round * n_pairs < total_tiles && ok; ++round) {
-        if (!tile_of(round, w)) continue;
+      Tile w = first_tile();
+      while (ok && next_tile(w)) {
         const uint32_t idesc = p.list[w.li].idesc;
         const TallProblem& pr = p.prob[w.prob];
         const int nkb = pr.total_kb;
@@ -893,30 +939,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
   } else {
     // ------------------------------ epilogue (warps 2.. of both CTAs): lane = column of C ------------------------------
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
+    const bool alternate = p.alternate;
+    const int group = alternate ? (warp - 2) >> 3 : 0, step = alternate ? 64 : 128;
+    const int first = 32 * ((warp - 2) >> 2) & (step - 1);
     uint32_t tile_i = 0;
-    Tile w{};
-    for (int round = 0; round * n_pairs < total_tiles; ++round) {
-      if (!tile_of(round, w)) continue;
-      const TallProblem& pr = p.prob[w.prob];
+    Tile w = first_tile();
+    for (; next_tile(w); ++tile_i) {
       const int acc = tile_i & 1;
+      if (alternate && acc != group) continue;
+      const TallProblem& pr = p.prob[w.prob];
       const bool ok = mbar_wait(&acc_full[acc], (tile_i >> 1) & 1, err);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
       const int col = w.n0 + int(rank) * 128 + quarter * 32 + lane;
       const int n_tok = min(w.nt, pr.M - w.m0);
       const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + acc * 256;
+      // 32 tokens at a time.  The accumulator is given back ahead of the last stores, by an arrival that does not wait for any.
 #pragma unroll 1
-      for (int c0 = 32 * ((warp - 2) >> 2); c0 < n_tok; c0 += 8 * TALL_EPI_WARPS) {   // the quarter's warps take turns
+      for (int c0 = first;; c0 += step) {
         uint32_t r[32];
-        tmem_ld_x32(taddr + c0, r);
+        const bool last = c0 + step >= n_tok;
+        if (c0 < n_tok) tmem_ld_x32(taddr + c0, r);
         tmem_ld_wait();
+        if (last) {
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster_relaxed(cluster_addr_of(&acc_empty[acc], 0));
+        }
         const int left = col < pr.N ? n_tok - c0 : 0;
         if (pr.out_f32) {
+          if (pr.out_f32 == OUT_F32_OF_BF16)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) r[i] = bf16_bits_f32(__uint_as_float(r[i]));
           float* dst = reinterpret_cast<float*>(pr.c) + size_t(w.m0 + c0) * pr.ldc + col;
 #pragma unroll
           for (int i = 0; i < 32; ++i, dst += pr.ldc)
-            if (i < left) *dst = __uint_as_float(pr.out_f32 == OUT_F32_OF_BF16 ? bf16_bits_f32(__uint_as_float(r[i])) : r[i]);
-        } else {
+            if (i < left) *dst = __uint_as_float(r[i]);
+        } else if (c0 < n_tok) {
           // two tokens at a time: even lanes end up with two columns of the first, odd lanes with two of the second
           const int odd = lane & 1;
           __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(pr.c) + size_t(w.m0 + c0 + odd) * pr.ldc + (col - odd);
@@ -927,11 +986,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
             if (i + odd < left) *reinterpret_cast<uint32_t*>(dst) = pack_bf16(lo, hi);
           }
         }
+        if (last) break;
       }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(cluster_addr_of(&acc_empty[acc], 0));
-      ++tile_i;
     }
   }
 
@@ -1124,33 +1180,66 @@ int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t
       if (rc != KVP_OK) return rc;
     }
   }
-  // the whole tiles of all problems first, then the remainders
-  for (int part = 0; part < 2; ++part)
-    for (int i = 0; i < n; ++i) {
-      const GemmProblem& g = probs[i];
-      const int whole = even ? (g.M + nt - 1) / nt : g.M / nt, rest = std::max(0, g.M - whole * nt), unit = g.a_mn ? 128 : TALL_UNIT;
-      TallList l{};
-      l.prob = i;
-      l.nt = part == 0 ? nt : (rest + unit - 1) / unit * unit;
-      l.m_first = part == 0 ? 0 : whole * nt;
-      l.n_tok = part == 0 ? whole : (rest > 0 ? 1 : 0);
-      if (l.n_tok == 0) continue;
-      tiles += l.n_tok * ((g.N + TCOLS - 1) / TCOLS);
-      l.tile_end = tiles;
-      l.idesc = umma_idesc_bf16(256, l.nt, g.b_mn, g.a_mn);
-      for (int e = 0; e < g.nseg; ++e) {
-        l.map_a[e] = short(maps_a);
-        const int rc = encode_operand(&p.map_a[maps_a++], g.segs[e].a, g.segs[e].lda, g.M, g.segs[e].K, g.a_mn, uint32_t(l.nt / 2));
-        if (rc != KVP_OK) return rc;
-      }
-      p.list[lists++] = l;
+  // Lists: forward the tiles of each problem, all of one size.  Gradients: whole tiles and one of the remainder, input gradients
+  // (K-major A) of up to two tiles in equal ones; the costliest lists first.
+  struct Part {
+    int prob, nt, m_first, n_tok;
+    float us;
+  } parts[2 * NP];
+  int n_parts = 0;
+  for (int i = 0; i < n; ++i) {
+    const GemmProblem& g = probs[i];
+    const int unit = g.a_mn ? 128 : TALL_UNIT, most = (g.M + nt - 1) / nt;
+    const bool equal = even || (!g.a_mn && most == 2);   // (a few rows more than one tile: both tiles read all of B)
+    const int size = even ? nt : equal ? ((g.M + most - 1) / most + unit - 1) / unit * unit : nt;
+    const int whole = equal ? (g.M + size - 1) / size : g.M / size, rest = std::max(0, g.M - whole * size);
+    auto add = [&](int t, int first, int cnt) {
+      if (cnt > 0) parts[n_parts++] = Part{i, t, first, cnt, even ? 0.f : gradient_tile_us(p.prob[i].total_kb, t, g.out_f32 != 0)};
+    };
+    add(size, 0, whole);
+    add((rest + unit - 1) / unit * unit, whole * size, rest > 0 ? 1 : 0);
+  }
+  if (!even) std::stable_sort(parts, parts + n_parts, [](const Part& a, const Part& b) { return a.us > b.us; });
+  int classes = 0, in_class[DEAL_CLASSES], short_tiles = 0;
+  float class_us[DEAL_CLASSES];
+  for (int i = 0; i < n_parts; ++i) {
+    const Part& q = parts[i];
+    const GemmProblem& g = probs[q.prob];
+    TallList l{};
+    l.prob = q.prob;
+    l.nt = q.nt;
+    l.m_first = q.m_first;
+    l.n_tok = q.n_tok;
+    l.inv_n_tok = 1.f / q.n_tok;
+    const int here = q.n_tok * ((g.N + TCOLS - 1) / TCOLS);
+    tiles += here;
+    l.tile_end = tiles;
+    l.idesc = umma_idesc_bf16(256, l.nt, g.b_mn, g.a_mn);
+    for (int e = 0; e < g.nseg; ++e) {
+      l.map_a[e] = short(maps_a);
+      const int rc = encode_operand(&p.map_a[maps_a++], g.segs[e].a, g.segs[e].lda, g.M, g.segs[e].K, g.a_mn, uint32_t(l.nt / 2));
+      if (rc != KVP_OK) return rc;
     }
+    p.list[lists++] = l;
+    if (classes == 0 || (q.us < class_us[classes - 1] && classes < DEAL_CLASSES)) {
+      class_us[classes] = q.us;
+      in_class[classes++] = 0;
+    }
+    in_class[classes - 1] += here;
+    if (p.prob[q.prob].total_kb <= TALL_SHORT_KBLOCKS) short_tiles += here;
+  }
+  const int pairs = std::min(tiles, sm_count() / 2);
+  if constexpr (NP > 1) {
+    p.deal.n_classes = !even && classes > 1 && in_class[0] < pairs && pairs <= DEAL_PAIRS && tiles <= 0xffff ? classes : 0;
+    if (p.deal.n_classes > 0) deal_tiles(class_us, in_class, classes, pairs, p.deal.first);
+  }
   p.total_tiles = tiles;
   p.stage_bytes = PA_BYTES + nt / 2 * (BK * 2);
   p.stages = std::min(TMAX_STAGES, TALL_RING / p.stage_bytes);
+  p.alternate = short_tiles >= TALL_ALTERNATE_ROUNDS * pairs;
   if (allow_smem<gemm_tall_kernel<NP, NSEG>>(TALL_SMEM) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
-  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * std::min(tiles, sm_count() / 2), TALL_THREADS, TALL_SMEM, stream, 1, p);
+  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * pairs, TALL_THREADS, TALL_SMEM, stream, 1, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
@@ -1182,6 +1271,9 @@ int by_count(int n, F1 one, F8 eight, F32 many) { return n == 1 ? one() : n <= 8
 // leave half of the pairs idle.  Measured (us, all weight and input gradients of a backward pass: gemm_kernel / tiles of
 // 128 / 256): 256 tokens x 256, four layers 14.4 / 7.0 / 9.0; 400 x 4096, two layers 32.1 / 28.9 / 23.2; 1984 x 1024, six
 // layers 70.6 / 72.8 / 59.3; 1664 x 4096, five layers 140 / 147 / 120; 4096 x 4096, one layer 303 / 352 / 282.
+// With the costliest tiles first, two equal tiles where 256 rows leave a few, and accumulators given back without waiting for
+// stores (an arrival with release semantics at cluster scope waits until all the thread's stores have reached L2): 264 tokens, 7
+// layers of d 1024 102 -> 69; 288, 8 of 2048 79 -> 65; 128, 8 of 4096 250 -> 216; 264 with output projection, 2 of 4096 200 -> 140.
 // Launches of more than GRADIENT_MAX_FLOP (about 0.3 ms) stay on gemm_kernel, although by themselves they too are a little
 // faster on pairs (4096 x 4096, four layers, 0.8 TFLOP: 1140 / - / 1030): they belong to steps of many milliseconds, which
 // the board's power limit bounds, and there the rest of the step slows by more than the pairs gain (training step of eight

@@ -354,6 +354,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
+// The same for a thread that hands over nothing but tensor memory it has read (tcgen05.wait::ld): a release would wait until
+// every store the thread has under way has reached L2.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t bar_cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+}
 // TMA load into this CTA's shared memory whose bytes are counted on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_2d_pair_e(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int x, int y,
                                                    uint32_t leader) {

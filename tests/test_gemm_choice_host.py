@@ -122,3 +122,46 @@ def test_pieces_of_k_go_by_columns_and_depth(choices):
         for rows in (1, 16, 17, 64, 128):
             _, split, parts, _ = choices[1]([(rows, n, k) for _, n, k in problems])
             assert split * parts == pieces, (rows, problems)
+
+
+@pytest.fixture(scope="module")
+def deal(tmp_path_factory):
+    folder = tmp_path_factory.mktemp("deal")
+    (folder / "d.cpp").write_text("""#include "kvp_gemm_choice.h"
+using namespace kvp;
+extern "C" float tile_us(int kb, int nt, int f32) { return gradient_tile_us(kb, nt, f32 != 0); }
+extern "C" void deal(const float* cost, const int* tiles, int n, int pairs, unsigned short* out) {
+  static uint16_t first[DEAL_CLASSES][DEAL_PAIRS + 1];
+  deal_tiles(cost, tiles, n, pairs, first);
+  for (int c = 0; c < n; ++c)
+    for (int p = 0; p <= pairs; ++p) out[c * (pairs + 1) + p] = first[c][p];
+}
+""")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I" + CSRC, str(folder / "d.cpp"), "-o", str(folder / "d.so")], check=True)
+    lib = C.CDLL(str(folder / "d.so"))
+    lib.tile_us.restype = C.c_float
+
+    def call(cost, tiles, pairs):
+        n, out = len(cost), (C.c_ushort * (len(cost) * (pairs + 1)))()
+        lib.deal((C.c_float * n)(*cost), (C.c_int * n)(*tiles), n, pairs, out)
+        return [list(out[c * (pairs + 1):(c + 1) * (pairs + 1)]) for c in range(n)]
+    return call, lib.tile_us
+
+
+def test_gradient_tiles_are_dealt_out(deal):
+    """Every tile to one pair, in order; no pair fuller than the average plus one tile of the costliest class it could lack."""
+    call, tile_us = deal
+    rng = random.Random(5)
+    for _ in range(300):
+        n, pairs = rng.randint(1, 6), rng.choice((1, 2, 7, 66, 74, 96))
+        cost = sorted((tile_us(rng.randint(1, 200), rng.choice((32, 128, 160, 256)), rng.randint(0, 1)) for _ in range(n)), reverse=True)
+        tiles = [rng.choice((1, 3, 28, 74, 75, 672, 9000)) for _ in range(n)]
+        first, load, at = call(cost, tiles, pairs), [0.0] * pairs, 0
+        for c in range(n):
+            assert first[c][0] == at and first[c] == sorted(first[c])
+            at += tiles[c]
+            assert first[c][pairs] == at
+            before = max(load)
+            for p in range(pairs):
+                load[p] += cost[c] * (first[c][p + 1] - first[c][p])
+            assert max(load) <= max(before, sum(load) / pairs + cost[c]) * 1.001 + 1e-3

@@ -74,6 +74,8 @@ def test_few_rows_grouped_projections():
     (5, 2, 392, 1088, 6, 3),      # tiles of 256 rows, one and three K segments
     (20, 8, 104, 576, 4, 1),       # more problems than one launch holds
     (1, 1, 7048, 4096, 64, 16),   # above the line to single-CTA tiles
+    (6, 5, 264, 1088, 66, 6),     # tiles dealt out by cost, two equal ones along the tokens; eight epilogue warps a tile
+    (2, 1, 296, 2112, 20, 2),     # dealt out, all epilogue warps on every tile
 ])
 def test_gradient_gemms(L, own, S, D, Hq, Hkv):
     from paper_2608_15943_b200 import kvp
