@@ -80,7 +80,7 @@ int kvp_selftest_bounded_wait_pair(void* scratch, size_t scratch_bytes, kvp_stre
 /* Benchmark bookkeeping.  kvp_launch_count: kernels launched by this library since it was loaded.
  * kvp_set_timing_events: record the caller's CUDA events (HOST arrays of n cudaEvent_t, created by
  * the caller) immediately before and after each of the next n launches of one kernel
- * (0 GEMM, 1 attention forward, 2 attention backward, 3 decode, 4 the backward's helper passes: Delta, accumulator clear, dQ conversion, one pair per group of launches); n == 0 switches it off.
+ * (0 GEMM, 1 attention forward, 2 attention backward, 3 decode, 4 the backward's helper passes: Delta, accumulator clear, dQ conversion, one pair per group of launches, the first alone up to 128 tokens); n == 0 switches it off.
  * kvp_timing_events_used: how many pairs have been recorded since.  Not thread-safe. */
 unsigned long long kvp_launch_count(void);
 int kvp_set_timing_events(int kernel, void** starts, void** stops, int n);

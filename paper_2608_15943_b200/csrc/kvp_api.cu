@@ -12,7 +12,7 @@ int attn_fwd_max_layers();
 size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor);
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, bool dq_f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 const float* const* lse, void* const* dq, const BwdF32* f32, float* const* dk_sum, float* const* dv_sum, void* ws,
                  cudaStream_t stream);
 
 namespace {
@@ -74,6 +74,8 @@ class Shadows {
       if (arr[l] != nullptr) inputs_.push_back(CastItem{src[l], arr[l], t.elems});
     return reinterpret_cast<const void* const*>(arr.data());
   }
+  // room for the bf16 copies alone
+  const void* const* space(const TensorSet& t) { return reinterpret_cast<const void* const*>(reserve(t).data()); }
   const std::vector<CastItem>& inputs() const { return inputs_; }
   int round_inputs() { return cast_tensors(inputs_.data(), int(inputs_.size()), stream_); }
 
@@ -417,13 +419,12 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* q16 = sh.in(q, z.q);
     const void* const* k16 = sh.in(k, z.kv);
     const void* const* v16 = sh.in(v, z.kv);
-    const void* const* o16 = sh.in(o, z.q);
-    const void* const* do16 = sh.in(d_o, z.q);
-    rc = sh.round_inputs();
-    if (rc != KVP_OK) return rc;
-    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, true, dk_sum, dv_sum, ws,
+    const void* const* o16 = sh.space(z.q);
+    const void* const* do16 = sh.space(z.q);
+    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size())};
+    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, dk_sum, dv_sum, ws,
                         reinterpret_cast<cudaStream_t>(stream_));
   }
-  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, false, dk_sum, dv_sum, ws,
+  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, nullptr, dk_sum, dv_sum, ws,
                       reinterpret_cast<cudaStream_t>(stream_));
 }

@@ -32,8 +32,7 @@
 #include <vector>
 
 #include "kvp_bwd_shape.h"
-#include "kvp_host.h"
-#include "kvp_sm100.cuh"
+#include "kvp_cast.cuh"
 
 namespace kvp {
 namespace {
@@ -766,17 +765,33 @@ __global__ void dq_convert_kernel(const __grid_constant__ AuxParams p) {
   }
 }
 
+// fp32 interface: the pre-pass reads the caller's O and dO, stores dO as bf16 (to d_o), and beside the slots rounds a list of
+// other tensors; a launch of its own for that took 3 us of the smallest steps' 42.
+template <bool F32>
+struct PrepareParams : AuxParams {};
+template <>
+struct PrepareParams<true> : AuxParams {
+  const float *o32[MAX_GROUP], *do32[MAX_GROUP];
+  int slots;                  // blockIdx.y beyond: the casts
+  CastParams casts;
+};
+
 // Before: clears the slot's dQ accumulator and the slot's share of the dK / dV sums (stores, nothing waits for them),
 // and forms Delta[b,hq,s] = sum_c dO[b,s,hq,c] * O[b,s,hq,c].
 // A row of DH bf16 is DH/8 16-byte pieces, and a load of a warp takes 256/DH rows (every lane busy): of consecutive tokens of one
 // head, whose results lie side by side, with the other heads of these tokens in the warps beside it.  Two such loads of
 // O and of dO are in flight, reduced inside the DH/8-lane segments.  Bound: HBM.
-template <int DH>
-__global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
+template <int DH, bool F32>
+__global__ void bwd_prepare_kernel(const __grid_constant__ PrepareParams<F32> p) {
   constexpr int LANES = DH / 8;          // lanes per row
   constexpr int ROWS = 32 / LANES;       // rows per warp and load
   grid_dep_wait();
   const int slot = blockIdx.y;
+  if constexpr (F32)
+    if (slot == p.slots) {
+      cast_chunks(p.casts, blockIdx.x, gridDim.x);
+      return;
+    }
   const size_t first = size_t(blockIdx.x) * blockDim.x + threadIdx.x, stride = size_t(gridDim.x) * blockDim.x;
   auto clear = [&](float* dst, size_t n) {
     float4* d = reinterpret_cast<float4*>(dst);
@@ -814,10 +829,33 @@ __global__ void bwd_prepare_kernel(const __grid_constant__ AuxParams p) {
     const int s0 = int(group % per_seq) * TOKS + sub, s1 = s0 + ROWS;
     const size_t at = ((b * S + s0) * Hq + hq) * DH + piece * 8, next = size_t(ROWS) * Hq * DH;
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    const uint4 a0 = s0 < S ? *reinterpret_cast<const uint4*>(o + at) : z;
-    const uint4 g0 = s0 < S ? *reinterpret_cast<const uint4*>(d_o + at) : z;
-    const uint4 a1 = s1 < S ? *reinterpret_cast<const uint4*>(o + at + next) : z;
-    const uint4 g1 = s1 < S ? *reinterpret_cast<const uint4*>(d_o + at + next) : z;
+    uint4 a0 = z, g0 = z, a1 = z, g1 = z;
+    if constexpr (F32) {
+      auto rounded = [](const float* src) {
+        const float4 x = *reinterpret_cast<const float4*>(src), y = *reinterpret_cast<const float4*>(src + 4);
+        return make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
+      };
+      __nv_bfloat16* const out = const_cast<__nv_bfloat16*>(d_o);
+      if (s0 < S) {
+        a0 = rounded(p.o32[slot] + at);
+        g0 = rounded(p.do32[slot] + at);
+        *reinterpret_cast<uint4*>(out + at) = g0;
+      }
+      if (s1 < S) {
+        a1 = rounded(p.o32[slot] + at + next);
+        g1 = rounded(p.do32[slot] + at + next);
+        *reinterpret_cast<uint4*>(out + at + next) = g1;
+      }
+    } else {
+      if (s0 < S) {
+        a0 = *reinterpret_cast<const uint4*>(o + at);
+        g0 = *reinterpret_cast<const uint4*>(d_o + at);
+      }
+      if (s1 < S) {
+        a1 = *reinterpret_cast<const uint4*>(o + at + next);
+        g1 = *reinterpret_cast<const uint4*>(d_o + at + next);
+      }
+    }
     float acc0 = dot8(a0, g0), acc1 = dot8(a1, g1);
 #pragma unroll
     for (int sft = LANES / 2; sft > 0; sft >>= 1) {
@@ -904,7 +942,7 @@ size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor) {
 
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, bool dq_f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 const float* const* lse, void* const* dq, const BwdF32* f32, float* const* dk_sum, float* const* dv_sum, void* ws,
                  cudaStream_t stream) {
   const int dh = s->dh;
   const float sc = scale == 0.f ? 1.f / sqrtf(float(dh)) : scale;
@@ -941,9 +979,15 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   const BwdSizes sizes{n_jt, n_qt, n_pairs, G, causal != 0, sm_count()};
   const double steps_per_sm = bwd_steps_per_sm(sizes, s->L);
   const int target = bwd_target_steps(steps_per_sm);
+  bool first_launch = true;
   size_t gi = 0;
+  if (f32 != nullptr && f32->n_casts > MAX_CAST) {   // more than the pre-pass has room for
+    const int rc = cast_tensors(f32->casts, f32->n_casts, stream);
+    if (rc != KVP_OK) return rc;
+  }
   while (gi < groups.size()) {
     BwdParams p;
+    const float *o32[MAX_GROUP] = {}, *do32[MAX_GROUP] = {};
     AuxParams ax = {};
     int slots = 0, ng = 0;
     p.cta_begin[0] = 0;
@@ -961,8 +1005,12 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         p.lse[slots] = lse[l];
         p.delta[slots] = ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
-        ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
+        ax.o[slots] = f32 != nullptr ? nullptr : reinterpret_cast<const __nv_bfloat16*>(o[l]);
         ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
+        if (f32 != nullptr) {
+          o32[slots] = f32->o[l];
+          do32[slots] = f32->d_o[l];
+        }
         p.dq[slots] = ax.dq[slots] = dq[l];
         ax.dq_acc[slots] = p.dq_acc[slots];
         ++slots;
@@ -1015,7 +1063,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     p.scale = sc;
     p.scale_log2 = sc * 1.4426950408889634f;
     ax.n_groups = ng;
-    p.dq_f32 = ax.dq_f32 = dq_f32;
+    p.dq_f32 = ax.dq_f32 = f32 != nullptr;
     ax.B = s->B;
     ax.S = s->S;
     ax.Hq = s->Hq;
@@ -1026,7 +1074,26 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     const size_t acc_floats = dq_acc_floats(s->B, s->S, s->Hq, dh);
     auto aux_grid = [&](size_t per_thread) { return dim3(unsigned(min(size_t(sm_count()) * 16, (acc_floats / per_thread + 255) / 256)), slots); };
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128> : bwd_prepare_kernel<64>, aux_grid(8), 256, 0, stream, 1, ax);
+    cudaError_t e;
+    if (f32 != nullptr) {
+      PrepareParams<true> pre;
+      static_cast<AuxParams&>(pre) = ax;
+      std::copy(o32, o32 + MAX_GROUP, pre.o32);
+      std::copy(do32, do32 + MAX_GROUP, pre.do32);
+      pre.slots = slots;
+      pre.casts.chunks = 0;
+      dim3 grid = aux_grid(8);
+      if (first_launch && f32->n_casts <= MAX_CAST) {
+        if (fill_casts(pre.casts, f32->casts, f32->n_casts) != f32->n_casts) return KVP_ERR_UNSUPPORTED;
+        ++grid.y;
+      }
+      e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, true> : bwd_prepare_kernel<64, true>, grid, 256, 0, stream, 1, pre);
+    } else {
+      PrepareParams<false> pre;
+      static_cast<AuxParams&>(pre) = ax;
+      e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, false> : bwd_prepare_kernel<64, false>, aux_grid(8), 256, 0, stream, 1, pre);
+    }
+    first_launch = false;
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     dim3 grid(p.cta_begin[ng]);

@@ -65,6 +65,13 @@ struct CastItem {
 };
 int cast_tensors(const CastItem* items, int n, cudaStream_t stream);
 
+// The attention backward of the fp32 interface: O and dO as the caller has them, per layer, and what else is to be rounded.
+struct BwdF32 {
+  const float *const *o, *const *d_o;
+  const CastItem* casts;
+  int n_casts;
+};
+
 void gemm_set_pair_mode(int mode);   // 0: single-CTA tiles only, 1: pairs where the caller prefers them, 2: pairs everywhere
 int gemm_pair_mode();
 int gemm_read_status();
