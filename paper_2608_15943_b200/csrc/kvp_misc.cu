@@ -3,7 +3,8 @@
 //
 // One launch converts a whole list of tensors: a call of the fp32 interface has 3 to 5 of them per layer, each of a few
 // hundred KB at the sizes that interface is for, where a launch costs more than the copy.  A four-layer training step of
-// 2 x 128 tokens had 64 conversion launches of 1.6 us each, outputs included; it has 4 (device time of the step 124 -> 78
+// 2 x 128 tokens had 64 conversion launches of 1.6 us each, outputs included; it has 3, and the backward's pre-pass converts
+// beside its own work (kvp_cast.cuh; device time of the step 124 -> 78
 // us with a launch per list, 55 -> 52 with the outputs widened where they are produced).  Bound: HBM for large tensors,
 // launch latency for small.
 #include <algorithm>

@@ -1,4 +1,5 @@
-"""ctypes binding of the C-ABI library (``include/kvp.h``): argument marshalling only.
+"""Binding of the C-ABI library (``include/kvp.h``): argument marshalling only, in ctypes and (the per-step calls) in the native
+module ``_pack``.
 
 Every function takes torch tensors (device memory, streams) and passes raw pointers and sizes to
 the entry point of the same name; all computation happens in the library's CUDA kernels.  Importing
@@ -80,8 +81,7 @@ def _ptr(t: Optional[torch.Tensor]) -> int:
 
 
 # Host arrays of the entry points are passed as packed bytes.  Packed natively: four pointers 0.1 us instead of 0.7, a
-# donor map of four layers 0.1 instead of 1.0; the smallest training step, four calls with 36 arrays, is bound by the
-# host and went from 64 to 47 us (the device takes 45), the smallest decode step, two calls, from 16.7 to 11.
+# donor map of four layers 0.1 instead of 1.0.  (The per-step calls pack theirs in _pack's own functions.)
 _ptr_array = _pack.pointers    # tensors (None: a null pointer), one per layer
 _donors = _pack.donors
 
