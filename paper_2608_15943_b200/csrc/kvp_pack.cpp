@@ -10,18 +10,28 @@
 #define PY_SSIZE_T_CLEAN
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <algorithm>
+
 #include "../../include/kvp.h"
 
 namespace {
 
-// [tensor or None, ...] -> their data pointers (0 for None) as 64-bit integers
-PyObject* pointers(PyObject*, PyObject* seq) {
+// An entry point reads an array of L entries (owner layers of some, kvp.h).  What a list does not have is a null pointer to it, and
+// refused where it would be read.
+
+// [tensor or None, ...] -> their data pointers (0 for None) as 64-bit integers; at least `entries` of them where that is given, or
+// (negative) so many more than the list has
+PyObject* pointers(PyObject*, PyObject* args) {
+  PyObject* seq;
+  Py_ssize_t entries = 0;
+  if (!PyArg_ParseTuple(args, "O|n", &seq, &entries)) return nullptr;
   PyObject* fast = PySequence_Fast(seq, "expected a sequence of tensors");
   if (fast == nullptr) return nullptr;
-  const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast);
-  PyObject* out = PyBytes_FromStringAndSize(nullptr, n * Py_ssize_t(sizeof(uint64_t)));
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast), all = entries < 0 ? n - entries : std::max(n, entries);
+  PyObject* out = PyBytes_FromStringAndSize(nullptr, all * Py_ssize_t(sizeof(uint64_t)));
   uint64_t* dst = out == nullptr ? nullptr : reinterpret_cast<uint64_t*>(PyBytes_AS_STRING(out));
   bool ok = out != nullptr;
+  if (ok) std::fill(dst + n, dst + all, uint64_t(0));
   for (Py_ssize_t i = 0; i < n && ok; ++i) {
     PyObject* o = PySequence_Fast_GET_ITEM(fast, i);
     if (o == Py_None) {
@@ -112,6 +122,8 @@ struct Reader {
   PyObject* const* a;
   Py_ssize_t left;
   bool ok;
+  int layers = 0;            // L
+  Py_ssize_t entries = 0;    // of the arrays, at least
   Reader(PyObject* const* args, Py_ssize_t n, Py_ssize_t want) : a(args), left(n), ok(n == want && lib.add != nullptr) {}
   PyObject* next() { return left-- > 0 ? *a++ : Py_None; }
   const at::Tensor* tensor(int dims) {   // dims < 0: any number
@@ -169,12 +181,13 @@ struct Reader {
     ok = view.len == Py_ssize_t(sizeof(T));
     const T* p = static_cast<const T*>(view.buf);
     PyBuffer_Release(&view);
+    if (ok) layers = p->L;
     return p;
   }
   // host arrays
   static constexpr int kRoom = 768;
   void* room[kRoom];
-  int32_t numbers[256];
+  int32_t numbers[257];
   int used = 0;
   PyObject** items(PyObject* o, Py_ssize_t& n) {
     ok = ok && (PyList_CheckExact(o) || PyTuple_CheckExact(o));
@@ -183,17 +196,19 @@ struct Reader {
     return PySequence_Fast_ITEMS(o);
   }
   template <typename T>
-  T* pointers() {
+  T* pointers(int more = 0) {   // more: entries behind the list (without a donor map, whose length bounds L)
     Py_ssize_t n = 0;
     PyObject** it = items(next(), n);
-    ok = ok && used + n <= kRoom;
+    const Py_ssize_t all = std::max(n + more, entries);
+    ok = ok && used + all <= kRoom;
     if (!ok) return nullptr;
     void** const dst = room + used;
+    std::fill(dst + n, dst + all, nullptr);
     for (Py_ssize_t i = 0; i < n && ok; ++i) {
       ok = it[i] == Py_None || THPVariable_CheckExact(it[i]);
       if (ok) dst[i] = it[i] == Py_None ? nullptr : THPVariable_Unpack(it[i]).data_ptr();
     }
-    used += int(n);
+    used += int(all);
     return reinterpret_cast<T*>(dst);
   }
   const int32_t* donor_map() {
@@ -208,6 +223,9 @@ struct Reader {
       ok = over == 0 && v >= INT32_MIN && v <= INT32_MAX;
       numbers[i] = int32_t(v);
     }
+    if (!ok) return nullptr;
+    if (n < layers) numbers[n] = -1;   // no donor: the map is refused before anything else is read
+    else entries = layers;
     return numbers;
   }
   struct Space {
@@ -330,8 +348,8 @@ ENTRY(proj_bwd) {   // shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk
 ENTRY(out_proj_fwd) {   // shape, o, wo, y, stream
   return run(args, n, 5, [](Reader& r) {
     auto* s = r.structure<kvp_shape>(shape_type);
-    In o = r.pointers<const void* const>(), wo = r.pointers<const void* const>();
-    Out y = r.pointers<void* const>();
+    In o = r.pointers<const void* const>(1), wo = r.pointers<const void* const>(1);
+    Out y = r.pointers<void* const>(1);
     const kvp_stream_t stream = r.stream();
     return [=] { return lib.out_proj_fwd(s, o, wo, y, stream); };
   });
@@ -339,9 +357,9 @@ ENTRY(out_proj_fwd) {   // shape, o, wo, y, stream
 ENTRY(out_proj_bwd) {   // shape, o, wo, dy, d_o, dwo, stream
   return run(args, n, 7, [](Reader& r) {
     auto* s = r.structure<kvp_shape>(shape_type);
-    In o = r.pointers<const void* const>(), wo = r.pointers<const void* const>(), dy = r.pointers<const void* const>();
-    Out d_o = r.pointers<void* const>();
-    OutF dwo = r.pointers<float* const>();
+    In o = r.pointers<const void* const>(1), wo = r.pointers<const void* const>(1), dy = r.pointers<const void* const>(1);
+    Out d_o = r.pointers<void* const>(1);
+    OutF dwo = r.pointers<float* const>(1);
     const kvp_stream_t stream = r.stream();
     return [=] { return lib.out_proj_bwd(s, o, wo, dy, d_o, dwo, stream); };
   });
@@ -409,7 +427,7 @@ ENTRY(decode) {   // desc, donor, scale, q, k_cache, v_cache, block_table, lengt
 }
 #define METHOD(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(fn)), METH_FASTCALL, nullptr}
 
-PyMethodDef methods[] = {{"pointers", pointers, METH_O, nullptr}, {"donors", donors, METH_O, nullptr}, {"bind", bind, METH_VARARGS, nullptr},
+PyMethodDef methods[] = {{"pointers", pointers, METH_VARARGS, nullptr}, {"donors", donors, METH_O, nullptr}, {"bind", bind, METH_VARARGS, nullptr},
                          METHOD("gemm", gemm), METHOD("rmsnorm", rmsnorm), METHOD("rope", rope), METHOD("swiglu", zip<false>), METHOD("add", zip<true>),
                          METHOD("proj_fwd", proj_fwd), METHOD("proj_bwd", proj_bwd), METHOD("out_proj_fwd", out_proj_fwd), METHOD("out_proj_bwd", out_proj_bwd),
                          METHOD("attn_fwd", attn_fwd), METHOD("attn_bwd", attn_bwd), METHOD("cache_append", cache_append), METHOD("decode", decode),

@@ -82,8 +82,15 @@ def _ptr(t: Optional[torch.Tensor]) -> int:
 
 # Host arrays of the entry points are passed as packed bytes.  Packed natively: four pointers 0.1 us instead of 0.7, a
 # donor map of four layers 0.1 instead of 1.0.  (The per-step calls pack theirs in _pack's own functions.)
-_ptr_array = _pack.pointers    # tensors (None: a null pointer), one per layer
+_ptr_array = _pack.pointers    # tensors (None: a null pointer), one per layer; what a list lacks of so many entries is a null pointer
 _donors = _pack.donors
+
+
+def _map(sizes, donor):
+    """Donor map of a call, and how many entries its lists need.  One that is too short goes on with a layer without a donor, which
+    the entry points refuse before they read a list."""
+    d, layers = _donors(donor), max(getattr(sizes, "L", 0), 0)
+    return (d, layers) if len(d) >= 4 * layers else (d + b"\xff" * 4, 0)
 
 
 def _i32_array(xs: Sequence[int]):
@@ -280,7 +287,7 @@ lib.kvp_attn_bwd.argtypes = [C.POINTER(Shape), C.c_void_p, C.c_int, C.c_float] +
 
 
 def workspace_bytes(op: int, shape: Shape, donor) -> int:
-    return int(lib.kvp_workspace_bytes(op, C.byref(shape), _donors(donor)))
+    return int(lib.kvp_workspace_bytes(op, C.byref(shape), _map(shape, donor)[0]))
 
 
 def _ws(ws: Optional[torch.Tensor]):
@@ -291,9 +298,10 @@ def proj_fwd(shape, donor, x, wq, wk, wv, q, k, v, ws=None):
     status = _pack.proj_fwd(shape, donor, x, wq, wk, wv, q, k, v, ws, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_proj_fwd")
-    p, n = _ws(ws)
-    _check(lib.kvp_proj_fwd(C.byref(shape), _donors(donor), _ptr_array(x), _ptr_array(wq), _ptr_array(wk),
-                            _ptr_array(wv), _ptr_array(q), _ptr_array(k), _ptr_array(v), p, n, _stream()),
+    d, n = _map(shape, donor)
+    p, size = _ws(ws)
+    _check(lib.kvp_proj_fwd(C.byref(shape), d, _ptr_array(x, n), _ptr_array(wq, n), _ptr_array(wk, n),
+                            _ptr_array(wv, n), _ptr_array(q, n), _ptr_array(k, n), _ptr_array(v, n), p, size, _stream()),
            "kvp_proj_fwd")
 
 
@@ -303,14 +311,15 @@ def proj_bwd(shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx,
         status = _pack.proj_bwd(shape, donor, x, wq, wk, wv, dq, dk_sum, dv_sum, dwq, dwk, dwv, dx, ws, _stream())
         if status is not NotImplemented:
             return _check(status, "kvp_proj_bwd")
-    p, n = _ws(ws)
-    args = (C.byref(shape), _donors(donor), _ptr_array(x), _ptr_array(wq), _ptr_array(wk), _ptr_array(wv),
-            _ptr_array(dq), _ptr_array(dk_sum), _ptr_array(dv_sum), _ptr_array(dwq), _ptr_array(dwk), _ptr_array(dwv),
-            _ptr_array(dx))
+    d, n = _map(shape, donor)
+    p, size = _ws(ws)
+    args = (C.byref(shape), d, _ptr_array(x, n), _ptr_array(wq, n), _ptr_array(wk, n), _ptr_array(wv, n),
+            _ptr_array(dq, n), _ptr_array(dk_sum, n), _ptr_array(dv_sum, n), _ptr_array(dwq, n), _ptr_array(dwk, n), _ptr_array(dwv, n),
+            _ptr_array(dx, n))
     if layer_begin is None and layer_end is None:
-        _check(lib.kvp_proj_bwd(*args, p, n, _stream()), "kvp_proj_bwd")
+        _check(lib.kvp_proj_bwd(*args, p, size, _stream()), "kvp_proj_bwd")
     else:
-        _check(lib.kvp_proj_bwd_range(*args, int(layer_begin or 0), shape.L if layer_end is None else int(layer_end), p, n,
+        _check(lib.kvp_proj_bwd_range(*args, int(layer_begin or 0), shape.L if layer_end is None else int(layer_end), p, size,
                                       _stream()), "kvp_proj_bwd_range")
 
 
@@ -318,7 +327,7 @@ def out_proj_fwd(shape, o, wo, y):
     status = _pack.out_proj_fwd(shape, o, wo, y, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_out_proj_fwd")
-    _check(lib.kvp_out_proj_fwd(C.byref(shape), _ptr_array(o), _ptr_array(wo), _ptr_array(y), _stream()),
+    _check(lib.kvp_out_proj_fwd(C.byref(shape), _ptr_array(o, -1), _ptr_array(wo, -1), _ptr_array(y, -1), _stream()),
            "kvp_out_proj_fwd")
 
 
@@ -326,17 +335,18 @@ def out_proj_bwd(shape, o, wo, dy, d_o, dwo):
     status = _pack.out_proj_bwd(shape, o, wo, dy, d_o, dwo, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_out_proj_bwd")
-    _check(lib.kvp_out_proj_bwd(C.byref(shape), _ptr_array(o), _ptr_array(wo), _ptr_array(dy), _ptr_array(d_o),
-                                _ptr_array(dwo), _stream()), "kvp_out_proj_bwd")
+    _check(lib.kvp_out_proj_bwd(C.byref(shape), _ptr_array(o, -1), _ptr_array(wo, -1), _ptr_array(dy, -1), _ptr_array(d_o, -1),
+                                _ptr_array(dwo, -1), _stream()), "kvp_out_proj_bwd")
 
 
 def attn_fwd(shape, donor, q, k, v, o, lse, causal=True, scale=0.0, ws=None):
     status = _pack.attn_fwd(shape, donor, causal, scale, q, k, v, o, lse, ws, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_attn_fwd")
-    p, n = _ws(ws)
-    _check(lib.kvp_attn_fwd(C.byref(shape), _donors(donor), int(causal), float(scale), _ptr_array(q),
-                            _ptr_array(k), _ptr_array(v), _ptr_array(o), _ptr_array(lse), p, n, _stream()),
+    d, n = _map(shape, donor)
+    p, size = _ws(ws)
+    _check(lib.kvp_attn_fwd(C.byref(shape), d, int(causal), float(scale), _ptr_array(q, n),
+                            _ptr_array(k, n), _ptr_array(v, n), _ptr_array(o, n), _ptr_array(lse, n), p, size, _stream()),
            "kvp_attn_fwd")
 
 
@@ -344,10 +354,11 @@ def attn_bwd(shape, donor, q, k, v, o, d_o, lse, dq, dk_sum, dv_sum, ws, causal=
     status = _pack.attn_bwd(shape, donor, causal, scale, q, k, v, o, d_o, lse, dq, dk_sum, dv_sum, ws, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_attn_bwd")
-    p, n = _ws(ws)
-    _check(lib.kvp_attn_bwd(C.byref(shape), _donors(donor), int(causal), float(scale), _ptr_array(q),
-                            _ptr_array(k), _ptr_array(v), _ptr_array(o), _ptr_array(d_o), _ptr_array(lse),
-                            _ptr_array(dq), _ptr_array(dk_sum), _ptr_array(dv_sum), p, n, _stream()), "kvp_attn_bwd")
+    d, n = _map(shape, donor)
+    p, size = _ws(ws)
+    _check(lib.kvp_attn_bwd(C.byref(shape), d, int(causal), float(scale), _ptr_array(q, n),
+                            _ptr_array(k, n), _ptr_array(v, n), _ptr_array(o, n), _ptr_array(d_o, n), _ptr_array(lse, n),
+                            _ptr_array(dq, n), _ptr_array(dk_sum, n), _ptr_array(dv_sum, n), p, size, _stream()), "kvp_attn_bwd")
 
 
 # ------------------------------------------------------------------------------------------
@@ -379,15 +390,17 @@ _pack.bind([C.cast(getattr(lib, "kvp_" + n), C.c_void_p).value for n in (
 
 
 def decode_workspace_bytes(desc: DecodeDesc, donor) -> int:
-    return int(lib.kvp_decode_workspace_bytes(C.byref(desc), _donors(donor)))
+    d, entries = _map(desc, donor)
+    return int(lib.kvp_decode_workspace_bytes(C.byref(desc), d)) if entries else 0
 
 
 def cache_append(desc, donor, k_new, v_new, k_cache, v_cache, block_table, lengths):
     status = _pack.cache_append(desc, donor, k_new, v_new, k_cache, v_cache, block_table, lengths, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_cache_append")
-    _check(lib.kvp_cache_append(C.byref(desc), _donors(donor), _ptr_array(k_new), _ptr_array(v_new),
-                                _ptr_array(k_cache), _ptr_array(v_cache), block_table.data_ptr(),
+    d, n = _map(desc, donor)
+    _check(lib.kvp_cache_append(C.byref(desc), d, _ptr_array(k_new, n), _ptr_array(v_new, n),
+                                _ptr_array(k_cache, n), _ptr_array(v_cache, n), block_table.data_ptr(),
                                 lengths.data_ptr(), _stream()), "kvp_cache_append")
 
 
@@ -396,10 +409,11 @@ def decode(desc, donor, q, k_cache, v_cache, block_table, lengths, o, lse, ws, s
     status = _pack.decode(desc, donor, scale, q, k_cache, v_cache, block_table, lengths, o, lse, layer_begin, layer_end, ws, _stream())
     if status is not NotImplemented:
         return _check(status, "kvp_decode")
-    p, n = _ws(ws)
-    _check(lib.kvp_decode(C.byref(desc), _donors(donor), float(scale), _ptr_array(q), _ptr_array(k_cache),
-                          _ptr_array(v_cache), block_table.data_ptr(), lengths.data_ptr(), _ptr_array(o),
-                          _ptr_array(lse), layer_begin, desc.L if layer_end is None else layer_end, p, n, _stream()),
+    d, n = _map(desc, donor)
+    p, size = _ws(ws)
+    _check(lib.kvp_decode(C.byref(desc), d, float(scale), _ptr_array(q, n), _ptr_array(k_cache, n),
+                          _ptr_array(v_cache, n), block_table.data_ptr(), lengths.data_ptr(), _ptr_array(o, n),
+                          _ptr_array(lse, n), layer_begin, desc.L if layer_end is None else layer_end, p, size, _stream()),
            "kvp_decode")
 
 
@@ -492,7 +506,8 @@ def decode_static(desc, donor, q, k_cache, v_cache, block_table, lengths, o, lse
     (no workspace tensor is passed and the library allocates nothing).  Raises KvpError with
     ERR_STATIC_SCRATCH when the request does not fit the built-in DECODE_STATIC_SCRATCH_BYTES array.
     Calls share that array, so do not let two of them overlap on the GPU."""
-    _check(lib.kvp_decode_static(C.byref(desc), _donors(donor), float(scale), _ptr_array(q), _ptr_array(k_cache),
-                                 _ptr_array(v_cache), block_table.data_ptr(), lengths.data_ptr(), _ptr_array(o),
-                                 _ptr_array(lse), layer_begin, desc.L if layer_end is None else layer_end, _stream()),
+    d, n = _map(desc, donor)
+    _check(lib.kvp_decode_static(C.byref(desc), d, float(scale), _ptr_array(q, n), _ptr_array(k_cache, n),
+                                 _ptr_array(v_cache, n), block_table.data_ptr(), lengths.data_ptr(), _ptr_array(o, n),
+                                 _ptr_array(lse, n), layer_begin, desc.L if layer_end is None else layer_end, _stream()),
            "kvp_decode_static")

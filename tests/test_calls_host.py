@@ -52,6 +52,7 @@ def record(monkeypatch):
         monkeypatch.setattr(kvp, "_pack", real)
         assert len(seen) == 2 and seen[0] == seen[1]
         return taken == [0]
+    both.seen = seen
     yield kvp, both
     real.bind(original, kvp.Shape, kvp.DecodeDesc)
 
@@ -108,6 +109,77 @@ def test_layer_calls(record):
     assert not both(lambda: kvp.proj_fwd(sh, donor, *odd[:7])) and not both(lambda: kvp.attn_fwd(sh, donor, *odd[:5]))
     assert not both(lambda: kvp.proj_fwd(sh, torch.tensor(donor), *arr[:7])) and not both(lambda: kvp.attn_fwd(sh, [0, True, 1], *arr[:5], causal=1, scale=0))
     assert not both(lambda: kvp.decode(de, donor, *arr[:3], table, lengths, *arr[3:5], ws, scale=0))
+
+
+def test_short_lists(record):
+    """What a list lacks of its L entries reaches the library as null pointers, never as entries of the next list."""
+    kvp, both = record
+    L = 4
+    sh, de, ws = kvp.Shape(L, 2, 5, 64, 4, 2, 64), kvp.DecodeDesc(L, 2, 4, 2, 64, 16, 3, 7), bf(100)
+    donor, table = [0, 1, 1, 1], torch.zeros(2, 3, dtype=torch.int32)
+
+    def arrays(short, n):
+        a = [[bf(2) for _ in range(L)] for _ in range(11)]
+        a[short] = a[short][:n]
+        return a
+
+    def passed(call, at, entries):
+        """`call` hands over, as its array number `at`, the tensors of `entries` and nulls behind them."""
+        want = b"".join(t.data_ptr().to_bytes(8, "little") for t in entries)
+        assert both(call)
+        name, args = both.seen[0]
+        got = [v for kind, v in zip(FORMS[name], args) if kind == "A"][at]
+        assert got == want + bytes(8 * L - len(want))
+    for n in (0, 1, 3):
+        for i in range(11):
+            a = arrays(i, n)
+            passed(lambda: kvp.proj_bwd(sh, donor, *a, ws), i, a[i])
+            if i < 9:
+                passed(lambda: kvp.attn_bwd(sh, donor, *a[:9], ws), i, a[i])
+            if i < 7:
+                passed(lambda: kvp.proj_fwd(sh, donor, *a[:7]), i, a[i])
+            if i < 5:
+                passed(lambda: kvp.attn_fwd(sh, donor, *a[:5]), i, a[i])
+                passed(lambda: kvp.decode(de, donor, *a[:3], table, table, *a[3:5], ws), i, a[i])
+            if i < 4:
+                passed(lambda: kvp.cache_append(de, donor, *a[:4], table, table), i, a[i])
+    sh, a = kvp.Shape(2, 1, 8, 64, 1, 1, 64), [[bf(2) for _ in range(2)] for _ in range(5)]
+    for i in range(5):                           # without a donor map: one null, at which the entry points stop
+        b = a[:i] + [a[i][:1]] + a[i + 1:]
+        for call, lists in ((kvp.out_proj_fwd, 3), (kvp.out_proj_bwd, 5)):
+            if i < lists:
+                assert both(lambda: call(sh, *b[:lists]))
+                assert both.seen[0][1][1 + i] == b[i][0].data_ptr().to_bytes(8, "little") + bytes(8)
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_short_lists_refused(native, monkeypatch):
+    """By the library itself, before it launches anything."""
+    from paper_2608_15943_b200 import kvp
+    if not native:
+        monkeypatch.setattr(kvp, "_pack", types.SimpleNamespace(**{n: lambda *a: NotImplemented for n in NAMES}))
+    x, table = bf(64, 64), torch.zeros(2, 3, dtype=torch.int32)
+    sh, de = kvp.Shape(2, 1, 64, 64, 1, 1, 64), kvp.DecodeDesc(2, 2, 1, 1, 64, 16, 3, 7)
+    full, one, ws = [x, x], [x], bf(1 << 23)
+
+    def refused(call, status):
+        with pytest.raises(kvp.KvpError) as e:
+            call()
+        assert e.value.status == status
+    calls = ((lambda d, *a: kvp.proj_fwd(sh, d, *a, ws), 7), (lambda d, *a: kvp.proj_bwd(sh, d, *a, ws), 11), (lambda d, *a: kvp.proj_bwd(sh, d, *a, ws, 0, 1), 11),
+             (lambda d, *a: kvp.attn_fwd(sh, d, *a, ws=ws), 5), (lambda d, *a: kvp.attn_bwd(sh, d, *a, ws), 9),
+             (lambda d, *a: kvp.cache_append(de, d, *a, table, table), 4), (lambda d, *a: kvp.decode(de, d, *a[:3], table, table, *a[3:], ws), 5),
+             (lambda d, *a: kvp.decode_static(de, d, *a[:3], table, table, *a[3:]), 5))
+    for call, lists in calls:
+        refused(lambda: call([0], *[full] * lists), kvp.ERR_BAD_DONOR)
+        if call is calls[-1][0]:
+            continue      # (looks for its scratch on the device first)
+        for i in range(lists):
+            refused(lambda: call([0, 1], *[one if j == i else full for j in range(lists)]), kvp.ERR_INVALID_ARG)
+    for call, lists in ((kvp.out_proj_fwd, 3), (kvp.out_proj_bwd, 5)):
+        for i in range(lists):
+            refused(lambda: call(sh, *[one if j == i else full for j in range(lists)]), kvp.ERR_INVALID_ARG)
+    assert kvp.workspace_bytes(kvp.OP_ATTN_BWD, sh, [0]) == 0 and kvp.decode_workspace_bytes(de, [0]) == 0
 
 
 def test_many_layers(record):
