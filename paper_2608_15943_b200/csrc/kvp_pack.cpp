@@ -11,6 +11,9 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
+#include <new>
+#include <optional>
+#include <string>
 
 #include "../../include/kvp.h"
 
@@ -243,23 +246,39 @@ struct Reader {
 };
 
 // Reads the arguments with `read`, which returns the call; what a tensor throws (no storage, symbolic sizes) sends the call to
-// kvp.py's own path.
+// kvp.py's own path.  The call itself is made once: what a library function throws becomes an exception of Python's, with the
+// interpreter's lock held again.
 template <typename F>
 PyObject* run(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, F read) {
+  Reader r(args, n, want);
+  std::optional<decltype(read(r))> call;
   try {
-    Reader r(args, n, want);
-    auto call = read(r);
-    if (r.ok) {
-      int status;
-      Py_BEGIN_ALLOW_THREADS
-      status = call();
-      Py_END_ALLOW_THREADS
-      return PyLong_FromLong(status);
-    }
+    call.emplace(read(r));
   } catch (const std::exception&) {
+    r.ok = false;
   }
-  if (PyErr_Occurred()) PyErr_Clear();
-  Py_RETURN_NOTIMPLEMENTED;
+  if (!r.ok) {
+    if (PyErr_Occurred()) PyErr_Clear();
+    Py_RETURN_NOTIMPLEMENTED;
+  }
+  int status = 0;
+  PyObject* thrown = nullptr;   // its kind
+  std::string what;
+  Py_BEGIN_ALLOW_THREADS
+  try {
+    status = (*call)();
+  } catch (const std::bad_alloc&) {
+    thrown = PyExc_MemoryError;
+  } catch (const std::exception& e) {
+    thrown = PyExc_RuntimeError;
+    what = e.what();
+  }
+  Py_END_ALLOW_THREADS
+  if (thrown != nullptr) {
+    PyErr_SetString(thrown, what.c_str());
+    return nullptr;
+  }
+  return PyLong_FromLong(status);
 }
 #define ENTRY(name) PyObject* name(PyObject*, PyObject* const* args, Py_ssize_t n)
 

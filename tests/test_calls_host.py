@@ -1,10 +1,14 @@
 """The native calls of the binding hand the library what its ctypes path does, and leave everything unusual to that path."""
 import ctypes as C
+import os
+import subprocess
+import sys
 import types
 
 import pytest
 import torch
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 NAMES = ("gemm", "rmsnorm", "rope", "swiglu", "add", "proj_fwd", "proj_bwd", "out_proj_fwd", "out_proj_bwd", "attn_fwd", "attn_bwd",
          "cache_append", "decode")
 # arguments of the entry points: i integer, l 64-bit integer, f float, p pointer, S structure, D donor map, A array of pointers
@@ -204,3 +208,38 @@ def test_refused_as_before():
     with pytest.raises(kvp.KvpError) as e:
         kvp.add(bf(3), bf(3), bf(3))
     assert e.value.status == kvp.ERR_UNSUPPORTED and "kvp_add" in str(e.value)
+
+
+THROWS = """
+#include <new>
+#include <stdexcept>
+int calls = 0;
+extern "C" int count() { return calls; }
+extern "C" int no_memory(long, void*, void*, void*, void*) { ++calls; throw std::bad_alloc(); }
+extern "C" int error(long, void*, void*, void*, void*) { ++calls; throw std::runtime_error("of the library"); }
+"""
+CATCHES = """
+import ctypes as C, sys, threading, torch
+from paper_2608_15943_b200 import kvp
+lib, x = C.CDLL(sys.argv[1]), torch.zeros(8, dtype=torch.bfloat16)
+for n, (name, kind) in enumerate((("no_memory", MemoryError), ("error", RuntimeError))):
+    kvp._pack.bind([C.cast(getattr(lib, name), C.c_void_p).value] * 13, kvp.Shape, kvp.DecodeDesc)
+    try:
+        kvp.add(x, x, x)
+    except kind as e:
+        assert name == "no_memory" or "of the library" in str(e)
+    else:
+        raise AssertionError(name)
+    assert lib.count() == n + 1
+    t = threading.Thread(target=lambda: sum(range(1000)))   # the interpreter's lock is held, and can be handed on
+    t.start()
+    t.join()
+"""
+
+
+def test_exceptions_of_the_library(tmp_path):
+    """An exception out of an entry point reaches Python; the entry point is not called again."""
+    (tmp_path / "throws.cpp").write_text(THROWS)
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(tmp_path / "throws.so"), str(tmp_path / "throws.cpp")], check=True)
+    done = subprocess.run([sys.executable, "-c", CATCHES, str(tmp_path / "throws.so")], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr
