@@ -233,7 +233,8 @@ int kvp_attn_fwd(const kvp_shape* s, const int32_t* donor, int causal, float sca
  * tile pair for all three gradients; partial sums that different thread blocks own (dq over key tiles, dk_sum /
  * dv_sum over windows of query tiles) are combined by fp32 reductions in global memory, so these outputs are
  * reproducible up to fp32 summation order, not bit for bit.  dk_sum / dv_sum are overwritten (cleared first),
- * never accumulated into.  At most 8 layers may share one donor.
+ * never accumulated into.  At most 8 layers may share one donor.  KVP_F32: gradients may lie in the memory of q, k, v, o and
+ * d_o, of any layer (all inputs are read first then, by a launch of their own).
  * Workspace: kvp_workspace_bytes(KVP_OP_ATTN_BWD): Delta per layer plus fp32 dq accumulators for up to 8 layers. */
 int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,

@@ -4,6 +4,7 @@
 #include <vector>
 
 #include "kvp_host.h"
+#include "kvp_overlap.h"
 
 namespace kvp {
 int attn_fwd_layers(const kvp_shape* s, int causal, float scale, const void* const* q, const void* const* k,
@@ -421,7 +422,13 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* v16 = sh.in(v, z.kv);
     const void* const* o16 = sh.space(z.q);
     const void* const* do16 = sh.space(z.q);
-    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size())};
+    // Gradients in place of inputs: everything is read before anything is written.
+    const Tensors ins[] = {{q, z.q.elems * 4, nullptr}, {k, z.kv.elems * 4, donor}, {v, z.kv.elems * 4, donor}, {o, z.q.elems * 4, nullptr}, {d_o, z.q.elems * 4, nullptr}};
+    const Tensors outs[] = {{dq, z.q.elems * 4, nullptr}, {reinterpret_cast<const void* const*>(dk_sum), z.kv.elems * 4, donor}, {reinterpret_cast<const void* const*>(dv_sum), z.kv.elems * 4, donor}};
+    bool shared = false;
+    for (const Tensors& out : outs)
+      for (const Tensors& in : ins) shared = shared || share_memory(s->L, out, in);
+    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()), shared};
     return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, dk_sum, dv_sum, ws,
                         reinterpret_cast<cudaStream_t>(stream_));
   }

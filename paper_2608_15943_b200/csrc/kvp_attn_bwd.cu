@@ -979,10 +979,44 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
   const BwdSizes sizes{n_jt, n_qt, n_pairs, G, causal != 0, sm_count()};
   const double steps_per_sm = bwd_steps_per_sm(sizes, s->L);
   const int target = bwd_target_steps(steps_per_sm);
-  bool first_launch = true;
   size_t gi = 0;
   if (f32 != nullptr && f32->n_casts > MAX_CAST) {   // more than the pre-pass has room for
     const int rc = cast_tensors(f32->casts, f32->n_casts, stream);
+    if (rc != KVP_OK) return rc;
+  }
+  // enough blocks for every slot to fill the device, no more than its pieces of 8 (16: convert) accumulators give work to
+  const size_t acc_floats = dq_acc_floats(s->B, s->S, s->Hq, dh);
+  auto aux_grid = [&](size_t per_thread, int slots) { return dim3(unsigned(min(size_t(sm_count()) * 16, (acc_floats / per_thread + 255) / 256)), slots); };
+  // The pre-pass of the fp32 interface; the first of a call rounds the other tensors too.
+  bool first_launch = true;
+  auto prepare_f32 = [&](const AuxParams& ax, int slots, const float* const* o32, const float* const* do32) {
+    PrepareParams<true> pre;
+    static_cast<AuxParams&>(pre) = ax;
+    std::copy(o32, o32 + slots, pre.o32);
+    std::copy(do32, do32 + slots, pre.do32);
+    pre.slots = slots;
+    pre.casts.chunks = 0;
+    dim3 grid = aux_grid(8, slots);
+    if (first_launch && f32->n_casts <= MAX_CAST) {
+      if (fill_casts(pre.casts, f32->casts, f32->n_casts) != f32->n_casts) return int(KVP_ERR_UNSUPPORTED);
+      ++grid.y;
+    }
+    first_launch = false;
+    const cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, true> : bwd_prepare_kernel<64, true>, grid, 256, 0, stream, 1, pre);
+    return int(e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA);
+  };
+  const bool read_first = f32 != nullptr && f32->read_first;
+  for (int l0 = 0; read_first && l0 < s->L; l0 += MAX_GROUP) {   // the pre-passes of all layers, which clear nothing
+    const int n = std::min(MAX_GROUP, s->L - l0);
+    AuxParams ax = {};
+    for (int i = 0; i < n; ++i) {
+      ax.d_o[i] = reinterpret_cast<const __nv_bfloat16*>(d_o[l0 + i]);
+      ax.delta[i] = reinterpret_cast<float*>(wsb + size_t(l0 + i) * delta_bytes);
+    }
+    ax.B = s->B;
+    ax.S = s->S;
+    ax.Hq = s->Hq;
+    const int rc = prepare_f32(ax, n, f32->o + l0, f32->d_o + l0);
     if (rc != KVP_OK) return rc;
   }
   while (gi < groups.size()) {
@@ -1070,30 +1104,17 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     ax.acc_v4 = n_jt == 1 ? 0 : dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;   // one key tile: bwd_kernel writes dQ
     ax.kv_v4 = size_t(s->B) * s->S * s->Hkv * dh / 4;
     ax.scale = sc;
-    // enough blocks for every slot to fill the device, no more than its pieces of 8 (16: convert) accumulators give work to
-    const size_t acc_floats = dq_acc_floats(s->B, s->S, s->Hq, dh);
-    auto aux_grid = [&](size_t per_thread) { return dim3(unsigned(min(size_t(sm_count()) * 16, (acc_floats / per_thread + 255) / 256)), slots); };
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    cudaError_t e;
-    if (f32 != nullptr) {
-      PrepareParams<true> pre;
-      static_cast<AuxParams&>(pre) = ax;
-      std::copy(o32, o32 + MAX_GROUP, pre.o32);
-      std::copy(do32, do32 + MAX_GROUP, pre.do32);
-      pre.slots = slots;
-      pre.casts.chunks = 0;
-      dim3 grid = aux_grid(8);
-      if (first_launch && f32->n_casts <= MAX_CAST) {
-        if (fill_casts(pre.casts, f32->casts, f32->n_casts) != f32->n_casts) return KVP_ERR_UNSUPPORTED;
-        ++grid.y;
-      }
-      e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, true> : bwd_prepare_kernel<64, true>, grid, 256, 0, stream, 1, pre);
+    cudaError_t e = cudaSuccess;
+    if (f32 != nullptr && !read_first) {
+      const int rc = prepare_f32(ax, slots, o32, do32);
+      if (rc != KVP_OK) return rc;
     } else {
       PrepareParams<false> pre;
       static_cast<AuxParams&>(pre) = ax;
-      e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, false> : bwd_prepare_kernel<64, false>, aux_grid(8), 256, 0, stream, 1, pre);
+      if (read_first) pre.B = 0;   // no rows: it only clears
+      e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, false> : bwd_prepare_kernel<64, false>, aux_grid(8, slots), 256, 0, stream, 1, pre);
     }
-    first_launch = false;
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     dim3 grid(p.cta_begin[ng]);
@@ -1104,7 +1125,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     if (e != cudaSuccess) return KVP_ERR_CUDA;
     if (n_jt == 1) continue;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
-    e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid(16), 256, 0, stream, 1, ax);
+    e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid(16, slots), 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
   }

@@ -70,6 +70,7 @@ struct BwdF32 {
   const float *const *o, *const *d_o;
   const CastItem* casts;
   int n_casts;
+  bool read_first;   // all inputs are read before any output is written
 };
 
 void gemm_set_pair_mode(int mode);   // 0: single-CTA tiles only, 1: pairs where the caller prefers them, 2: pairs everywhere
