@@ -234,7 +234,8 @@ int kvp_attn_fwd(const kvp_shape* s, const int32_t* donor, int causal, float sca
  * dv_sum over windows of query tiles) are combined by fp32 reductions in global memory, so these outputs are
  * reproducible up to fp32 summation order, not bit for bit.  dk_sum / dv_sum are overwritten (cleared first),
  * never accumulated into.  At most 8 layers may share one donor.  KVP_F32: gradients may lie in the memory of q, k, v, o and
- * d_o, of any layer (all inputs are read first then, by a launch of their own).
+ * d_o, of any layer (all inputs are read first then, by a launch of their own).  KVP_BF16: dq[l] may lie in that of q[l], o[l]
+ * or d_o[l]; up to eight layers also in that of any of their q, k, v, o and d_o.
  * Workspace: kvp_workspace_bytes(KVP_OP_ATTN_BWD): Delta per layer plus fp32 dq accumulators for up to 8 layers. */
 int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,

@@ -1,8 +1,10 @@
 // C-ABI entry points of the training / prefill path: argument validation and the sequence of
 // kernel launches per layer.  No allocation, no synchronisation.
 #include <algorithm>
+#include <initializer_list>
 #include <vector>
 
+#include "kvp_bwd_shape.h"
 #include "kvp_host.h"
 #include "kvp_overlap.h"
 
@@ -13,7 +15,7 @@ int attn_fwd_max_layers();
 size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor);
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, const BwdF32* f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 const float* const* lse, void* const* dq, const BwdF32* f32, bool dq_last, float* const* dk_sum, float* const* dv_sum, void* ws,
                  cudaStream_t stream);
 
 namespace {
@@ -414,24 +416,35 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
   if (scale < 0.f) return KVP_ERR_INVALID_ARG;
   const size_t need = kvp_workspace_bytes(KVP_OP_ATTN_BWD, s, donor);
   if (need > 0 && (ws == nullptr || ws_bytes < need || !aligned16(ws))) return KVP_ERR_WORKSPACE;
-  if (s->dtype == KVP_F32) {
-    const Sizes z = sizes_of(s);
+  // Gradients in the memory of inputs.  fp32: everything is read before anything is written.  bf16: dQ is the last to be written, not
+  // by the kernel that still reads the inputs, unless it takes the place of that layer's q or d_o, which that kernel has read when
+  // it writes there.
+  const Sizes z = sizes_of(s);
+  const bool f32_io = s->dtype == KVP_F32;
+  const size_t e = f32_io ? 4 : 2;
+  const Tensors in_q{q, z.q.elems * e, nullptr}, in_k{k, z.kv.elems * e, donor}, in_v{v, z.kv.elems * e, donor}, in_o{o, z.q.elems * e, nullptr},
+      in_do{d_o, z.q.elems * e, nullptr}, in_lse{reinterpret_cast<const void* const*>(lse), size_t(s->B) * s->S * s->Hq * 4, nullptr};
+  const Tensors out_q{dq, z.q.elems * e, nullptr}, out_k{reinterpret_cast<const void* const*>(dk_sum), z.kv.elems * 4, donor},
+      out_v{reinterpret_cast<const void* const*>(dv_sum), z.kv.elems * 4, donor};
+  auto shared = [&](const Tensors& out, std::initializer_list<const Tensors*> ins) {
+    for (const Tensors* in : ins)
+      if (share_memory(s->L, out, *in)) return true;
+    return false;
+  };
+  if (f32_io) {
     Shadows sh(s, donor, ws, align256(op_scratch_bytes(KVP_OP_ATTN_BWD, s, donor)), reinterpret_cast<cudaStream_t>(stream_));
     const void* const* q16 = sh.in(q, z.q);
     const void* const* k16 = sh.in(k, z.kv);
     const void* const* v16 = sh.in(v, z.kv);
     const void* const* o16 = sh.space(z.q);
     const void* const* do16 = sh.space(z.q);
-    // Gradients in place of inputs: everything is read before anything is written.
-    const Tensors ins[] = {{q, z.q.elems * 4, nullptr}, {k, z.kv.elems * 4, donor}, {v, z.kv.elems * 4, donor}, {o, z.q.elems * 4, nullptr}, {d_o, z.q.elems * 4, nullptr}};
-    const Tensors outs[] = {{dq, z.q.elems * 4, nullptr}, {reinterpret_cast<const void* const*>(dk_sum), z.kv.elems * 4, donor}, {reinterpret_cast<const void* const*>(dv_sum), z.kv.elems * 4, donor}};
-    bool shared = false;
-    for (const Tensors& out : outs)
-      for (const Tensors& in : ins) shared = shared || share_memory(s->L, out, in);
-    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()), shared};
-    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, dk_sum, dv_sum, ws,
+    const auto inputs = {&in_q, &in_k, &in_v, &in_o, &in_do};
+    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()),
+                     shared(out_q, inputs) || shared(out_k, inputs) || shared(out_v, inputs)};
+    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, shared(out_q, {&in_lse}), dk_sum, dv_sum, ws,
                         reinterpret_cast<cudaStream_t>(stream_));
   }
-  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, nullptr, dk_sum, dv_sum, ws,
+  const bool dq_last = s->S <= BWD_KEYS && (shared(out_q, {&in_k, &in_v, &in_lse}) || share_memory(s->L, out_q, in_q, true) || share_memory(s->L, out_q, in_do, true));
+  return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, nullptr, dq_last, dk_sum, dv_sum, ws,
                       reinterpret_cast<cudaStream_t>(stream_));
 }

@@ -92,8 +92,9 @@ struct BwdParams {
   const float* lse[MAX_GROUP];    // [B,Hq,S]
   const float* delta[MAX_GROUP];  // [B,Hq,S]
   float* dq_acc[MAX_GROUP];       // blocked fp32 accumulators, see dq_acc_floats()
-  void* dq[MAX_GROUP];            // one key tile: dQ itself, [B,S,Hq,dh], bf16 or (dq_f32) the bf16 values as fp32
+  void* dq[MAX_GROUP];            // dQ itself, [B,S,Hq,dh], bf16 or (dq_f32) the bf16 values as fp32
   int dq_f32;
+  int dq_direct;                  // a dQ tile has one partial, and this kernel writes it (one key tile)
   CUtensorMap map_dk[MAX_GROUP], map_dv[MAX_GROUP]; // per group: the fp32 sums [B,S,Hkv,dh], box 32 rows x 32 columns
   int first_slot[MAX_GROUP + 1];
   int cta_begin[MAX_GROUP + 1];
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
       }
       tc_fence_before_sync();
       mbar_arrive(dq_free);
-      if (active && n_jt == 1) {
+      if (active && p.dq_direct) {
         // One key tile: the partial is the whole sum, and goes out as dQ: rounded, a lane's eight queries a row of 16 bytes of an
         // 8x8 matrix in shared memory, back transposed as eight columns of one query, 16 bytes a store.  (Exchanged between lanes
         // instead it took 1900 cycles a step, more than the rest of the step.)
@@ -942,7 +943,7 @@ size_t attn_bwd_workspace(const kvp_shape* s, const int32_t* donor) {
 
 int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float scale, const void* const* q,
                  const void* const* k, const void* const* v, const void* const* o, const void* const* d_o,
-                 const float* const* lse, void* const* dq, const BwdF32* f32, float* const* dk_sum, float* const* dv_sum, void* ws,
+                 const float* const* lse, void* const* dq, const BwdF32* f32, bool dq_last, float* const* dk_sum, float* const* dv_sum, void* ws,
                  cudaStream_t stream) {
   const int dh = s->dh;
   const float sc = scale == 0.f ? 1.f / sqrtf(float(dh)) : scale;
@@ -1005,6 +1006,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     const cudaError_t e = launch_kernel(dh == 128 ? bwd_prepare_kernel<128, true> : bwd_prepare_kernel<64, true>, grid, 256, 0, stream, 1, pre);
     return int(e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA);
   };
+  const bool direct = n_jt == 1 && !dq_last;   // bwd_kernel writes dQ
   const bool read_first = f32 != nullptr && f32->read_first;
   for (int l0 = 0; read_first && l0 < s->L; l0 += MAX_GROUP) {   // the pre-passes of all layers, which clear nothing
     const int n = std::min(MAX_GROUP, s->L - l0);
@@ -1101,7 +1103,8 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     ax.B = s->B;
     ax.S = s->S;
     ax.Hq = s->Hq;
-    ax.acc_v4 = n_jt == 1 ? 0 : dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;   // one key tile: bwd_kernel writes dQ
+    p.dq_direct = direct;
+    ax.acc_v4 = direct ? 0 : dq_acc_floats(s->B, s->S, s->Hq, dh) / 4;
     ax.kv_v4 = size_t(s->B) * s->S * s->Hkv * dh / 4;
     ax.scale = sc;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
@@ -1123,7 +1126,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
                   : launch_kernel(bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::TOTAL, stream, 1, p);
     timing_after(KVP_KERNEL_ATTN_BWD, stream);
     if (e != cudaSuccess) return KVP_ERR_CUDA;
-    if (n_jt == 1) continue;
+    if (direct) continue;
     timing_before(KVP_KERNEL_ATTN_BWD_AUX, stream);
     e = launch_kernel(dh == 128 ? dq_convert_kernel<128> : dq_convert_kernel<64>, aux_grid(16, slots), 256, 0, stream, 1, ax);
     timing_after(KVP_KERNEL_ATTN_BWD_AUX, stream);

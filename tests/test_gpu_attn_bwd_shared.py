@@ -61,3 +61,22 @@ def test_fp32_gradients_in_place_of_inputs(case, B, S, H, dh, L):
     ins, sh, ws = inputs(B, S, H, H, dh, donor, torch.float32)
     want = backward(ins, sh, ws, donor, lambda n, l, t: None)
     same(want, backward(ins, sh, ws, donor, IN_PLACE[case]), S)
+
+
+DQ_OVER = {   # up to 128 tokens the kernel that reads q, k, v and d_o writes dQ too, where it has read what lies there
+    "q": lambda l, t: t["q"][l],
+    "d_o": lambda l, t: t["d_o"][l],
+    "o": lambda l, t: t["o"][l],
+    "k or v": lambda l, t: t["kv"[l % 2]][l],
+    "q of another layer": lambda l, t: t["q"][-1 - l],
+    "d_o of another layer": lambda l, t: t["d_o"][l - 1],
+}
+
+
+@pytest.mark.parametrize("over", DQ_OVER)
+@pytest.mark.parametrize("B,S,H,dh,L", [(2, 128, 4, 64, 4), (3, 41, 2, 128, 3), (1, 65, 8, 128, 8), (1, 200, 2, 64, 2)])
+def test_dq_in_place_of_inputs(over, B, S, H, dh, L):
+    donor = list(range(L))
+    ins, sh, ws = inputs(B, S, H, H, dh, donor, torch.bfloat16)
+    want = backward(ins, sh, ws, donor, lambda n, l, t: None)
+    same(want, backward(ins, sh, ws, donor, lambda n, l, t: DQ_OVER[over](l, t) if n == "dq" else None), S)

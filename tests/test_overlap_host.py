@@ -13,17 +13,17 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 def shares(tmp_path_factory):
     d = tmp_path_factory.mktemp("overlap")
     (d / "r.cpp").write_text("""#include "kvp_overlap.h"
-extern "C" int shares(int L, const void* const* a, size_t na, const int32_t* da, const void* const* b, size_t nb, const int32_t* db) {
-  return kvp::share_memory(L, kvp::Tensors{a, na, da}, kvp::Tensors{b, nb, db});
+extern "C" int shares(int L, const void* const* a, size_t na, const int32_t* da, const void* const* b, size_t nb, const int32_t* db, int same_layer) {
+  return kvp::share_memory(L, kvp::Tensors{a, na, da}, kvp::Tensors{b, nb, db}, same_layer != 0);
 }
 """)
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, str(d / "r.cpp"), "-o", str(d / "r.so")], check=True)
     lib = C.CDLL(str(d / "r.so"))
 
-    def call(a, na, da, b, nb, db):
+    def call(a, na, da, b, nb, db, same_layer=False):
         arr = lambda xs: (C.c_void_p * len(xs))(*xs)
         ints = lambda xs: None if xs is None else (C.c_int32 * len(xs))(*xs)
-        return bool(lib.shares(len(a), arr(a), C.c_size_t(na), ints(da), arr(b), C.c_size_t(nb), ints(db)))
+        return bool(lib.shares(len(a), arr(a), C.c_size_t(na), ints(da), arr(b), C.c_size_t(nb), ints(db), int(same_layer)))
     return call
 
 
@@ -33,6 +33,9 @@ def test_edges(shares):
     a, b = [100, 0], [400, 0]                       # the consumers' entries are no tensors, null or not
     assert not shares(a, 10, [0, 0], b, 10, [0, 0]) and not shares([100, 400], 10, [0, 0], [400, 100], 10, [0, 0])
     assert shares([100, 400], 10, None, [400, 100], 10, [0, 0]) and not shares([100, 0], 10, [0, 0], [0, 300], 10, None)
+
+    assert not shares([100, 200], 10, None, [100, 200], 10, None, True) and shares([100, 200], 10, None, [100, 205], 10, None, True)
+    assert shares([100, 200], 10, None, [200, 100], 10, None, True)
 
 
 def test_any(shares):
