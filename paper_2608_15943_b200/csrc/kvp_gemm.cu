@@ -485,11 +485,6 @@ constexpr int SPLIT_THREADS = 192;
 // k-blocks of B a CTA asks into L2 before the kernels ahead of it have finished (a token step's 56 kernels: 601 us
 // without, 595 with 8, 613 with 32)
 constexpr int SPLIT_PREFETCH = 8;
-// From this much of B on, a quarter of L2, and with one tile of tokens, B is read with the policy evict_first: nothing finds it in
-// L2 again, and what the launches beside it ask into L2 stays (token steps with d 4096 of 1, 8, 16 and 32 sequences, us: 199 -> 195, 396
-// -> 389, 548 -> 541, 425 -> 417).  Smaller ones may be there still at the next step, and loads with a policy of any kind slow
-// tiles that share B (1155 x 1024 x 2816 11.1 -> 12.2).
-constexpr double SPLIT_STREAM_BYTES = 32 * 1024 * 1024;
 
 struct SplitProblem {
   int M, N;
@@ -511,7 +506,7 @@ struct SplitParams {
 };
 
 // WIDE: four tokens a warp at a time.  PARTS: accumulators of a CTA (one or two), each with a run of its k-blocks.  STREAM: B,
-// which one CTA reads once, is marked first to go in L2.
+// which one CTA reads once, is marked first to go in L2 (stream_weights, kvp_gemm_choice.h).
 template <int NP, bool WIDE, int PARTS, bool STREAM>
 __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __grid_constant__ SplitParams<NP> p) {
   extern __shared__ uint8_t smem_raw[];
@@ -1108,11 +1103,9 @@ auto split_kernel(bool stream_b) -> decltype(&gemm_split_kernel<NP, WIDE, PARTS,
 }
 
 template <int NP>
-int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaStream_t stream) {
+int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, bool stream_b, cudaStream_t stream) {
   SplitParams<NP> p;
   int tiles = 0;
-  bool once = true;      // one tile of tokens: no element of B is read by a second CTA
-  double b_bytes = 0;
   for (int i = 0; i < n; ++i) {
     const GemmProblem& g = probs[i];
     SplitProblem& q = p.prob[i];
@@ -1120,8 +1113,6 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
     q.N = g.N;
     q.tok_tiles = (g.M + cfg.nt - 1) / cfg.nt;
     tiles += q.tok_tiles * ((g.N + SROWS - 1) / SROWS);
-    once = once && q.tok_tiles == 1;
-    b_bytes += 2. * g.N * g.segs[0].K;
     q.tile_end = tiles;
     q.kblocks = (g.segs[0].K + BK - 1) / BK;
     q.out_f32 = g.out_f32;
@@ -1144,7 +1135,6 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, cudaSt
   // other ends; it does end, for a CTA of the attention waits for no other CTA.
   const int ring = cfg.stages * (SB_BYTES + cfg.nt * BK * 2), part = cfg.parts * cfg.nt * SROWS * 4;
   const int smem = 1024 + std::max(std::max(ring, part), std::max(40 * 1024, p.tmem_cols * 440));
-  const bool stream_b = once && b_bytes >= SPLIT_STREAM_BYTES;
   const bool wide = cfg.split <= 2 && cfg.nt > 2 * cfg.split * (SPLIT_THREADS / 32);
   auto* const kernel = cfg.parts == 2 ? (wide ? split_kernel<NP, true, 2>(stream_b) : split_kernel<NP, false, 2>(stream_b))
                                       : (wide ? split_kernel<NP, true, 1>(stream_b) : split_kernel<NP, false, 1>(stream_b));
@@ -1296,7 +1286,7 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
 }
 
 // A forward GEMM (K-major operands, one segment): -1 when the tile kernels take it
-int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
+int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t stream) {
   int rows = 0;
   for (int i = 0; i < n; ++i) rows = std::max(rows, probs[i].M);
   GemmSize sizes[MAX_PROB];
@@ -1309,8 +1299,9 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
       const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
       const GemmProblem* g = probs + begin;
       const SplitConfig cfg = split_config(sizes_of(g, cnt), cnt, sm_count());
-      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream); },
-                              [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream); });
+      const bool stream_b = read_once && stream_weights(sizes, cnt, cfg.nt);
+      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream_b, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream_b, stream); },
+                              [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream_b, stream); });
       if (rc != KVP_OK) return rc;
     }
     return KVP_OK;
@@ -1326,8 +1317,8 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
                     [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, true, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, 1, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
-      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream); },
-                    [&] { return launch_split<MAX_PROB>(g, cnt, cfg, stream); });
+      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, false, stream); }, [&] { return launch_split<8>(g, cnt, cfg, false, stream); },
+                    [&] { return launch_split<MAX_PROB>(g, cnt, cfg, false, stream); });
     } else {
       rc = launch_group(g, cnt, stream, 0, 0, c.kind == Choice::kPair);
     }
@@ -1338,7 +1329,7 @@ int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
 
 }  // namespace
 
-int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream) {
+int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool read_once) {
   if (n < 0 || (n > 0 && probs == nullptr)) return KVP_ERR_INVALID_ARG;
   for (int i = 0; i < n; ++i) {
     const int rc = check_problem(probs[i]);
@@ -1346,7 +1337,7 @@ int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream) {
   }
   const bool forward = k_major(probs, n);
   if (forward) {
-    const int rc = gemm_forward(probs, n, stream);
+    const int rc = gemm_forward(probs, n, read_once, stream);
     if (rc >= 0) return rc;
   }
   // as many problems per launch as the parameter block holds
@@ -1376,7 +1367,7 @@ int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, v
   g.c = c;
   g.ldc = ldc;
   g.out_f32 = out_f32;
-  if (withhold_at == 0) return gemm_grouped(&g, 1, stream);
+  if (withhold_at == 0) return gemm_grouped(&g, 1, stream, true);
   const int rc = check_problem(g);
   return rc == KVP_OK ? launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1)) : rc;
 }

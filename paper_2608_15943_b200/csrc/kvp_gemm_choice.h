@@ -134,6 +134,28 @@ inline Choice choose_forward(const GemmSize* probs, int n, int sms) {
 }
 
 // ------------------------------------------------------------------------------------------------------------
+// Up to 128 rows: are the weights read with the policy evict_first?  From 32 MB on, with one tile of tokens, and where the call says
+// that they are not read again in this pass (a token step's projections, kvp_gemm): a pass streams far more than L2 holds then, and
+// so some of it is there still at the next.  Measured (us, without -> with): token steps of two layers of d 4096, 1, 8 and 64
+// sequences 182.6 -> 173.3, 190.3 -> 184.0, 253.2 -> 250.2, of four layers, 16 sequences 531.1 -> 529.3 (the latter of the size of
+// the noise); a head of 64 MB behind a layer of d 1024 61.8 -> 58.0.  Not in training steps, whose backward reads the weights again:
+// with the policy four layers of 128 tokens, d 2048 72.3 -> 75.1, two of d 4096 68.8 -> 72.9.  What it costs where less than L2
+// holds passes between two uses of the same weights: 4096 x 11008 again and again at 1 and 32 rows 11.3 -> 12.3 to 13.2, 12.1 -> 12.7
+// to 13.6, three of 4096 x 4096 in turn 23.1 -> 24.0; one or two of them nothing, and 11008 x 4096 and four or more of 4096 x 4096
+// gain (18.1 -> 16.1 at 32 rows, 34.4 -> 31.9).  At 160 rows it gains nothing (eight of 11008 x 4096 168.4 -> 168.4), and loads with
+// a policy of any kind slow tiles that share B (1155 x 1024 x 2816 11.1 -> 12.2).
+// ------------------------------------------------------------------------------------------------------------
+constexpr double SPLIT_STREAM_BYTES = 32 * 1024 * 1024;
+inline bool stream_weights(const GemmSize* probs, int n, int nt) {
+  double bytes = 0;
+  for (int i = 0; i < n; ++i) {
+    if (probs[i].M > std::min(nt, SPLIT_MAX_ROWS)) return false;
+    bytes += 2. * probs[i].N * probs[i].K;
+  }
+  return bytes >= SPLIT_STREAM_BYTES;
+}
+
+// ------------------------------------------------------------------------------------------------------------
 // The tiles of a launch of gradient GEMMs, dealt out to CTA pairs.  They come in classes of equal cost, the costliest first:
 // input gradients run over all columns of the weights (96 k-blocks and more), weight gradients over the tokens (a few).  Each
 // class goes to the pairs so that the fullest of them is as empty as can be, a run of consecutive tiles to each.  Only where the

@@ -22,6 +22,11 @@ extern "C" void split_choice(const int* mnk, int n, int* out) {
   const SplitConfig c = split_config(g, n, 148);
   out[0] = c.nt, out[1] = c.split, out[2] = c.parts, out[3] = c.stages;
 }
+extern "C" int streams(const int* mnk, int n) {
+  GemmSize g[32];
+  for (int i = 0; i < n; ++i) g[i] = GemmSize{mnk[3 * i], mnk[3 * i + 1], mnk[3 * i + 2]};
+  return stream_weights(g, n, split_config(g, n, 148).nt);
+}
 extern "C" void choose(const int* mnk, int n, int* out) {
   GemmSize g[32];
   int rows = 0;
@@ -49,7 +54,10 @@ extern "C" void choose(const int* mnk, int n, int* out) {
             f((C.c_int * len(flat))(*flat), len(problems), out)
             return tuple(out)
         return call
-    return caller(lib.choose, 3), caller(lib.split_choice, 4)
+    def streams(problems):
+        flat = [x for p in problems for x in p]
+        return bool(lib.streams((C.c_int * len(flat))(*flat), len(problems)))
+    return caller(lib.choose, 3), caller(lib.split_choice, 4), streams
 
 
 @pytest.fixture(scope="module")
@@ -60,6 +68,15 @@ def choices(tmp_path_factory):
 @pytest.fixture(scope="module")
 def choose(choices):
     return choices[0]
+
+
+@pytest.mark.parametrize("problems,streamed", [
+    ([(1, 4096, 4096)], True), ([(128, 4096, 4096)], True), ([(16, 4096, 4088)], False),    # 32 MB and a little less
+    ([(8, 4096, 2048), (8, 1024, 2048), (8, 1024, 2048)], False), ([(8, 4096, 4096), (8, 1024, 4096), (8, 1024, 4096)], True),
+    ([(8, 4096, 4096), (160, 4096, 4096)], False), ([(129, 11008, 4096)], False),           # more rows than one tile, than 128
+])
+def test_streamed_weights(choices, problems, streamed):
+    assert choices[2](problems) == streamed
 
 
 def some_lists(seed, n=3000):
