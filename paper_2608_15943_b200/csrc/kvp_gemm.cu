@@ -713,11 +713,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4) gemm_split_kernel(const __gr
 // ------------------------------------------------------------------------------------------------------------
 constexpr int TCOLS = 256;                        // columns of C per pair
 constexpr int TMAX_STAGES = 10;                   // a stage holds, per CTA, 128 rows of B and half of a tile's rows of A
-// Four for every quarter of the TMEM lanes, taking 32 tokens each in turn: all on every tile, or (launches in which pairs have
-// several tiles of few k-blocks) eight on every other one, so that the stores of one tile run while the other eight wait for the
+// Four for every quarter of the TMEM lanes, taking 32 tokens each in turn: all on every tile, or (gradient launches in which pairs
+// have several tiles of few k-blocks) eight on every other one, so that the stores of one tile run while the other eight wait for the
 // next and read it out.  With all sixteen on each the stores of a tile of fp32 results went out at 6.7 TB/s, and nothing for as
 // long again.  Measured (us, sixteen -> eight): 264 tokens, 7 layers of d 1024 74 -> 69; 128 tokens, 8 layers of d 4096 232 -> 216; but
-// 2328 tokens, 3 layers of d 1024 36 -> 39, where the last tiles count.
+// 2328 tokens, 3 layers of d 1024 36 -> 39, where the last tiles count.  Forward, with bf16 results and K up to 768, it makes no
+// difference (four of 2048 x 4096 x 512 44.6 -> 44.8, three of 3000 x 4096 x 768 70.6 -> 69.0, runs 2 apart).
 constexpr int TALL_EPI_WARPS = 16, TALL_ALTERNATE_ROUNDS = 6, TALL_SHORT_KBLOCKS = 12;
 constexpr int TALL_THREADS = (2 + TALL_EPI_WARPS) * 32;
 constexpr int TALL_RING = 224 * 1024;             // the ring takes as many stages as fit
@@ -1226,7 +1227,7 @@ int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t
   p.total_tiles = tiles;
   p.stage_bytes = PA_BYTES + nt / 2 * (BK * 2);
   p.stages = std::min(TMAX_STAGES, TALL_RING / p.stage_bytes);
-  p.alternate = short_tiles >= TALL_ALTERNATE_ROUNDS * pairs;
+  p.alternate = !even && short_tiles >= TALL_ALTERNATE_ROUNDS * pairs;
   if (allow_smem<gemm_tall_kernel<NP, NSEG>>(TALL_SMEM) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
   const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * pairs, TALL_THREADS, TALL_SMEM, stream, 1, p);
