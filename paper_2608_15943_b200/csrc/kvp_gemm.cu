@@ -12,6 +12,7 @@
 // types): the Q, K and V projections of every layer are one launch, so are all weight and input gradients of a
 // backward pass, and the SMs idle only behind the last tile of the list instead of behind each GEMM's last wave.
 #include <algorithm>
+#include <type_traits>
 
 #include "kvp_gemm_choice.h"
 #include "kvp_host.h"
@@ -740,7 +741,7 @@ struct TallProblem {
   long long ldc;
   void* c;
 };
-template <bool MANY>
+template <bool DEAL>
 struct TallDeal {                                 // gradients: the pairs' tiles, class by class (0 classes: pairs take tiles in turn)
   int n_classes;
   uint16_t first[DEAL_CLASSES][DEAL_PAIRS + 1];
@@ -749,9 +750,9 @@ template <>
 struct TallDeal<false> {
   static constexpr int n_classes = 0;
 };
-template <int NP, int NSEG>                       // problems, and segments of all of them, that the parameter block holds
+template <int NP, int NSEG, bool DEAL>            // problems, and segments of all of them, that the parameter block holds
 struct TallParams {
-  TallDeal<(NP > 1)> deal;
+  TallDeal<DEAL> deal;
   CUtensorMap map_b[NSEG], map_a[2 * NSEG];
   TallProblem prob[NP];
   TallList list[2 * NP];
@@ -760,9 +761,9 @@ struct TallParams {
   int alternate;                                  // eight epilogue warps a tile
 };
 
-template <int NP, int NSEG>
+template <int NP, int NSEG, bool DEAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
-    gemm_tall_kernel(const __grid_constant__ TallParams<NP, NSEG> p) {
+    gemm_tall_kernel(const __grid_constant__ TallParams<NP, NSEG, DEAL> p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + TALL_RING);
@@ -810,7 +811,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
   auto next_tile = [&](Tile& w) -> bool {
     int t;
     bool dealt = false;
-    if constexpr (NP > 1) {
+    if constexpr (DEAL) {
       dealt = p.deal.n_classes > 0;
       if (dealt) {
         while (w.t >= p.deal.first[w.turn][pair + 1]) {
@@ -846,7 +847,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TALL_THREADS, 1)
   };
   auto first_tile = [&]() {
     Tile w{};
-    if constexpr (NP > 1)
+    if constexpr (DEAL)
       if (p.deal.n_classes > 0) w.t = p.deal.first[0][pair];
     return w;
   };
@@ -1146,9 +1147,9 @@ int launch_split(const GemmProblem* probs, int n, const SplitConfig& cfg, bool s
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
 
-template <int NP, int NSEG>
+template <int NP, int NSEG, bool DEAL>
 int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t stream) {
-  TallParams<NP, NSEG> p;
+  TallParams<NP, NSEG, DEAL> p;
   int lists = 0, tiles = 0, maps_a = 0, maps_b = 0;
   for (int i = 0; i < n; ++i) {
     const GemmProblem& g = probs[i];
@@ -1220,7 +1221,7 @@ int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t
     if (p.prob[q.prob].total_kb <= TALL_SHORT_KBLOCKS) short_tiles += here;
   }
   const int pairs = std::min(tiles, sm_count() / 2);
-  if constexpr (NP > 1) {
+  if constexpr (DEAL) {
     p.deal.n_classes = !even && classes > 1 && in_class[0] < pairs && pairs <= DEAL_PAIRS && tiles <= 0xffff ? classes : 0;
     if (p.deal.n_classes > 0) deal_tiles(class_us, in_class, classes, pairs, p.deal.first);
   }
@@ -1228,9 +1229,9 @@ int launch_tall(const GemmProblem* probs, int n, int nt, bool even, cudaStream_t
   p.stage_bytes = PA_BYTES + nt / 2 * (BK * 2);
   p.stages = std::min(TMAX_STAGES, TALL_RING / p.stage_bytes);
   p.alternate = !even && short_tiles >= TALL_ALTERNATE_ROUNDS * pairs;
-  if (allow_smem<gemm_tall_kernel<NP, NSEG>>(TALL_SMEM) != cudaSuccess) return KVP_ERR_CUDA;
+  if (allow_smem<gemm_tall_kernel<NP, NSEG, DEAL>>(TALL_SMEM) != cudaSuccess) return KVP_ERR_CUDA;
   timing_before(KVP_KERNEL_GEMM, stream);
-  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG>, 2 * pairs, TALL_THREADS, TALL_SMEM, stream, 1, p);
+  const cudaError_t e = launch_kernel(gemm_tall_kernel<NP, NSEG, DEAL>, 2 * pairs, TALL_THREADS, TALL_SMEM, stream, 1, p);
   timing_after(KVP_KERNEL_GEMM, stream);
   return e == cudaSuccess ? KVP_OK : KVP_ERR_CUDA;
 }
@@ -1254,9 +1255,14 @@ int gemm_pair_mode() { return g_pair_mode; }
 
 namespace {
 
-// parameter blocks of three sizes: each 8 KB of them take 0.6 us to launch
-template <typename F1, typename F8, typename F32>
-int by_count(int n, F1 one, F8 eight, F32 many) { return n == 1 ? one() : n <= 8 ? eight() : many(); }
+// Parameter blocks of four sizes: each 8 KB of them take 0.6 us to launch.  f is given the size.
+template <typename F>
+int by_count(int n, F f) {
+  if (n == 1) return f(std::integral_constant<int, 1>());
+  if (n <= 4) return f(std::integral_constant<int, 4>());
+  if (n <= 8) return f(std::integral_constant<int, 8>());
+  return f(std::integral_constant<int, MAX_PROB>());
+}
 
 // The gradient GEMMs of a launch (pair mode 1) run on gemm_tall_kernel, in tiles of 256 rows; of 128 where those would
 // leave half of the pairs idle.  Measured (us, all weight and input gradients of a backward pass: gemm_kernel / tiles of
@@ -1281,9 +1287,10 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
   }
   if (flop > GRADIENT_MAX_FLOP) return launch_group(probs, n, stream, 0, 0, false);
   const int nt = 4 * tiles <= sm_count() ? 128 : 256;
-  if (segs == 1) return launch_tall<1, 1>(probs, n, nt, false, stream);
-  if (n <= 8 && segs <= 12) return launch_tall<8, 12>(probs, n, nt, false, stream);
-  return launch_tall<MAX_PROB, MAX_MAPS / 2>(probs, n, nt, false, stream);
+  if (segs == 1) return launch_tall<1, 1, false>(probs, n, nt, false, stream);
+  if (segs <= 4) return launch_tall<4, 4, true>(probs, n, nt, false, stream);
+  if (n <= 8 && segs <= 12) return launch_tall<8, 12, true>(probs, n, nt, false, stream);
+  return launch_tall<MAX_PROB, MAX_MAPS / 2, true>(probs, n, nt, false, stream);
 }
 
 // A forward GEMM (K-major operands, one segment): -1 when the tile kernels take it
@@ -1301,8 +1308,7 @@ int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t s
       const GemmProblem* g = probs + begin;
       const SplitConfig cfg = split_config(sizes_of(g, cnt), cnt, sm_count());
       const bool stream_b = read_once && stream_weights(sizes, cnt, cfg.nt);
-      const int rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, stream_b, stream); }, [&] { return launch_split<8>(g, cnt, cfg, stream_b, stream); },
-                              [&] { return launch_split<SPLIT_MAX_PROB>(g, cnt, cfg, stream_b, stream); });
+      const int rc = by_count(cnt, [&](auto np) { return launch_split<np>(g, cnt, cfg, stream_b, stream); });
       if (rc != KVP_OK) return rc;
     }
     return KVP_OK;
@@ -1314,12 +1320,10 @@ int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t s
     const Choice c = choose_forward(sizes_of(g, cnt), cnt, sm_count());
     int rc;
     if (c.kind == Choice::kTall) {
-      rc = by_count(cnt, [&] { return launch_tall<1, 1>(g, cnt, c.nt, true, stream); }, [&] { return launch_tall<8, 8>(g, cnt, c.nt, true, stream); },
-                    [&] { return launch_tall<MAX_PROB, MAX_MAPS / 2>(g, cnt, c.nt, true, stream); });
+      rc = by_count(cnt, [&](auto np) { return launch_tall<np, np, false>(g, cnt, c.nt, true, stream); });
     } else if (c.kind == Choice::kSplit) {
       const SplitConfig cfg{c.nt, c.split, 1, std::min(SPLIT_MAX_STAGES, 220 * 1024 / (SB_BYTES + c.nt * BK * 2))};
-      rc = by_count(cnt, [&] { return launch_split<1>(g, cnt, cfg, false, stream); }, [&] { return launch_split<8>(g, cnt, cfg, false, stream); },
-                    [&] { return launch_split<MAX_PROB>(g, cnt, cfg, false, stream); });
+      rc = by_count(cnt, [&](auto np) { return launch_split<np>(g, cnt, cfg, false, stream); });
     } else {
       rc = launch_group(g, cnt, stream, 0, 0, c.kind == Choice::kPair);
     }

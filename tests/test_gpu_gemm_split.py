@@ -43,8 +43,9 @@ def test_few_rows(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(5, 4104, 4104), (128, 11016, 1608), (33, 18440, 920), (70, 1032, 16400)])
-def test_few_rows_streamed_b(M, N, K):
+def test_few_rows_streamed_b(streams, M, N, K):
     """B just above a quarter of L2, read with a cache policy: two accumulators, one, no split, eight pieces of K."""
+    assert streams([(M, N, K)])
     test_few_rows(M, N, K)
 
 
@@ -107,10 +108,39 @@ def test_gradient_gemms(L, own, S, D, Hq, Hkv):
         assert ((dx[l].double() - ref).abs() <= bound + 2.0 ** -8 * ref.abs()).all(), l
 
 
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 5, 8, 9])      # L problems forward, 2 L backward: parameter blocks of 1, 4, 8 and 32
+@pytest.mark.parametrize("T,kind", [(40, "split"), (200, "tall")])
+def test_parameter_blocks_of_each_size(choose, L, T, kind):
+    from paper_2608_15943_b200 import kvp
+    D, Hq, dh = 1024, 1, 64
+    N = Hq * dh
+    assert ("single", "pair", "tall", "split")[choose([(T, D, N)] * L)[0]] == kind
+    sh = kvp.Shape(L, 1, T, D, Hq, 1, dh)
+    o, wo, dy = ([synth.normal(s, 37, synth.tid(i, l), 1.0, "cuda") for l in range(L)] for i, s in enumerate(((T, N), (D, N), (T, D))))
+    gd = Guarded()
+    y, d_o = ([gd.empty(s, torch.bfloat16, float("nan")) for _ in range(L)] for s in ((T, D), (T, N)))
+    dwo = [gd.empty((D, N), torch.float32, float("nan")) for _ in range(L)]
+    kvp.out_proj_fwd(sh, o, wo, y)
+    kvp.out_proj_bwd(sh, o, wo, dy, d_o, dwo)
+    gd.check()
+    assert kvp.device_status() == kvp.OK
+    for l in range(L):
+        for got, a, b in ((y[l], o[l], wo[l].T), (d_o[l], dy[l], wo[l]), (dwo[l], dy[l].T, o[l])):
+            a, b = a.double(), b.double()
+            half_ulp = 2.0 ** -8 * (a @ b).abs() if got.dtype == torch.bfloat16 else 0.0      # bounds as test_few_rows
+            assert ((got.double() - a @ b).abs() <= a.shape[1] * 2.0 ** -24 * (a.abs() @ b.abs()) + half_ulp + 1e-30).all()
+
+
 @pytest.fixture(scope="module")
 def choose(tmp_path_factory):
     from test_gemm_choice_host import compiled
     return compiled(tmp_path_factory.mktemp("choice"))[0]
+
+
+@pytest.fixture(scope="module")
+def streams(tmp_path_factory):
+    from test_gemm_choice_host import compiled
+    return compiled(tmp_path_factory.mktemp("streams"))[2]
 
 
 @pytest.fixture(scope="module")
