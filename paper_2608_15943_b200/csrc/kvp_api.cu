@@ -1,7 +1,6 @@
 // C-ABI entry points of the training / prefill path: argument validation and the sequence of
 // kernel launches per layer.  No allocation, no synchronisation.
 #include <algorithm>
-#include <initializer_list>
 #include <vector>
 
 #include "kvp_bwd_shape.h"
@@ -426,11 +425,6 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
       in_do{d_o, z.q.elems * e, nullptr}, in_lse{reinterpret_cast<const void* const*>(lse), size_t(s->B) * s->S * s->Hq * 4, nullptr};
   const Tensors out_q{dq, z.q.elems * e, nullptr}, out_k{reinterpret_cast<const void* const*>(dk_sum), z.kv.elems * 4, donor},
       out_v{reinterpret_cast<const void* const*>(dv_sum), z.kv.elems * 4, donor};
-  auto shared = [&](const Tensors& out, std::initializer_list<const Tensors*> ins) {
-    for (const Tensors* in : ins)
-      if (share_memory(s->L, out, *in)) return true;
-    return false;
-  };
   if (f32_io) {
     Shadows sh(s, donor, ws, align256(op_scratch_bytes(KVP_OP_ATTN_BWD, s, donor)), reinterpret_cast<cudaStream_t>(stream_));
     const void* const* q16 = sh.in(q, z.q);
@@ -438,13 +432,17 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* v16 = sh.in(v, z.kv);
     const void* const* o16 = sh.space(z.q);
     const void* const* do16 = sh.space(z.q);
-    const auto inputs = {&in_q, &in_k, &in_v, &in_o, &in_do};
-    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()),
-                     shared(out_q, inputs) || shared(out_k, inputs) || shared(out_v, inputs)};
-    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, shared(out_q, {&in_lse}), dk_sum, dv_sum, ws,
+    Outputs outs(s->L, {out_q, out_k, out_v});
+    const bool read_first = outs.meet(in_q) || outs.meet(in_k) || outs.meet(in_v) || outs.meet(in_o) || outs.meet(in_do);
+    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()), read_first};
+    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, outs.meet(in_lse), dk_sum, dv_sum, ws,
                         reinterpret_cast<cudaStream_t>(stream_));
   }
-  const bool dq_last = s->S <= BWD_KEYS && (shared(out_q, {&in_k, &in_v, &in_lse}) || share_memory(s->L, out_q, in_q, true) || share_memory(s->L, out_q, in_do, true));
+  bool dq_last = false;
+  if (s->S <= BWD_KEYS) {
+    Outputs outs(s->L, {out_q});
+    dq_last = outs.meet(in_q, &out_q) || outs.meet(in_k) || outs.meet(in_v) || outs.meet(in_do, &out_q) || outs.meet(in_lse);
+  }
   return attn_bwd_all(s, donor, causal, scale, q, k, v, o, d_o, lse, dq, nullptr, dq_last, dk_sum, dv_sum, ws,
                       reinterpret_cast<cudaStream_t>(stream_));
 }

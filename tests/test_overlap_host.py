@@ -1,4 +1,4 @@
-"""Whether per-layer arrays of a call share memory, compiled for the host."""
+"""Whether outputs of a call share memory with its inputs, compiled for the host."""
 import ctypes as C
 import os
 import random
@@ -14,7 +14,8 @@ def shares(tmp_path_factory):
     d = tmp_path_factory.mktemp("overlap")
     (d / "r.cpp").write_text("""#include "kvp_overlap.h"
 extern "C" int shares(int L, const void* const* a, size_t na, const int32_t* da, const void* const* b, size_t nb, const int32_t* db, int same_layer) {
-  return kvp::share_memory(L, kvp::Tensors{a, na, da}, kvp::Tensors{b, nb, db}, same_layer != 0);
+  const kvp::Tensors out{a, na, da};
+  return kvp::Outputs(L, {out}).meet(kvp::Tensors{b, nb, db}, same_layer ? &out : nullptr);
 }
 """)
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, str(d / "r.cpp"), "-o", str(d / "r.so")], check=True)
@@ -34,7 +35,7 @@ def test_edges(shares):
     assert not shares(a, 10, [0, 0], b, 10, [0, 0]) and not shares([100, 400], 10, [0, 0], [400, 100], 10, [0, 0])
     assert shares([100, 400], 10, None, [400, 100], 10, [0, 0]) and not shares([100, 0], 10, [0, 0], [0, 300], 10, None)
 
-    assert not shares([100, 200], 10, None, [100, 200], 10, None, True) and shares([100, 200], 10, None, [100, 205], 10, None, True)
+    assert not shares([100, 200], 10, None, [100, 200], 10, None, True) and shares([100, 200], 10, None, [100, 206], 10, None, True)
     assert shares([100, 200], 10, None, [200, 100], 10, None, True)
 
 
@@ -43,8 +44,8 @@ def test_any(shares):
     found = 0
     for _ in range(400):
         L = rng.randint(1, 6)
-        a, b = ([rng.randrange(1000, 1400) for _ in range(L)] for _ in range(2))
         na, nb = rng.randint(1, 30), rng.randint(1, 30)
+        a, b = [x * na for x in rng.sample(range(40, 40 + 400 // na), L)], [rng.randrange(40 * na, 40 * na + 400) for _ in range(L)]   # outputs apart
         da, db = (rng.choice((None, [rng.choice((l, 0)) for l in range(L)])) for _ in range(2))
         tensors = lambda xs, d: [x for l, x in enumerate(xs) if d is None or d[l] == l]
         want = any(set(range(x, x + na)) & set(range(y, y + nb)) for x in tensors(a, da) for y in tensors(b, db))
