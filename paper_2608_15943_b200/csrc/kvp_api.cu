@@ -158,8 +158,8 @@ size_t op_shadow_bytes(int op, const kvp_shape* s, const int32_t* donor) {
       return shadow_bytes(s, donor, sets, 3);
     }
     case KVP_OP_ATTN_BWD: {
-      const TensorSet sets[] = {z.q, z.kv, z.kv, z.q, z.q};      // q, k, v, o, dO
-      return shadow_bytes(s, donor, sets, 5);
+      const TensorSet sets[] = {z.q, z.kv, z.kv, z.q};           // q, k, v, dO
+      return shadow_bytes(s, donor, sets, 4);
     }
     default:
       return 0;
@@ -430,12 +430,11 @@ extern "C" int kvp_attn_bwd(const kvp_shape* s, const int32_t* donor, int causal
     const void* const* q16 = sh.in(q, z.q);
     const void* const* k16 = sh.in(k, z.kv);
     const void* const* v16 = sh.in(v, z.kv);
-    const void* const* o16 = sh.space(z.q);
     const void* const* do16 = sh.space(z.q);
     Outputs outs(s->L, {out_q, out_k, out_v});
     const bool read_first = outs.meet(in_q) || outs.meet(in_k) || outs.meet(in_v) || outs.meet(in_o) || outs.meet(in_do);
-    const BwdF32 f32{reinterpret_cast<const float* const*>(o), reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()), read_first};
-    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o16, do16, lse, dq, &f32, outs.meet(in_lse), dk_sum, dv_sum, ws,
+    const BwdF32 f32{reinterpret_cast<const float* const*>(d_o), sh.inputs().data(), int(sh.inputs().size()), read_first};
+    return attn_bwd_all(s, donor, causal, scale, q16, k16, v16, o, do16, lse, dq, &f32, outs.meet(in_lse), dk_sum, dv_sum, ws,
                         reinterpret_cast<cudaStream_t>(stream_));
   }
   bool dq_last = false;

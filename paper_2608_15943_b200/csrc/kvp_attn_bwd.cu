@@ -1023,7 +1023,7 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
     ax.B = s->B;
     ax.S = s->S;
     ax.Hq = s->Hq;
-    const int rc = prepare_f32(ax, n, f32->o + l0, f32->d_o + l0);
+    const int rc = prepare_f32(ax, n, reinterpret_cast<const float* const*>(o) + l0, f32->d_o + l0);
     if (rc != KVP_OK) return rc;
   }
   while (gi < groups.size()) {
@@ -1046,11 +1046,12 @@ int attn_bwd_all(const kvp_shape* s, const int32_t* donor, int causal, float sca
         p.lse[slots] = lse[l];
         p.delta[slots] = ax.delta[slots] = reinterpret_cast<float*>(wsb + size_t(l) * delta_bytes);
         p.dq_acc[slots] = reinterpret_cast<float*>(acc_base + size_t(slots) * acc_bytes);
-        ax.o[slots] = f32 != nullptr ? nullptr : reinterpret_cast<const __nv_bfloat16*>(o[l]);
         ax.d_o[slots] = reinterpret_cast<const __nv_bfloat16*>(d_o[l]);
         if (f32 != nullptr) {
-          o32[slots] = f32->o[l];
+          o32[slots] = reinterpret_cast<const float*>(o[l]);
           do32[slots] = f32->d_o[l];
+        } else {
+          ax.o[slots] = reinterpret_cast<const __nv_bfloat16*>(o[l]);
         }
         p.dq[slots] = ax.dq[slots] = dq[l];
         ax.dq_acc[slots] = p.dq_acc[slots];

@@ -66,9 +66,9 @@ struct CastItem {
 };
 int cast_tensors(const CastItem* items, int n, cudaStream_t stream);
 
-// The attention backward of the fp32 interface: O and dO as the caller has them, per layer, and what else is to be rounded.
+// The attention backward of the fp32 interface: dO as the caller has it (O is in either interface), and what else is to be rounded.
 struct BwdF32 {
-  const float *const *o, *const *d_o;
+  const float* const* d_o;
   const CastItem* casts;
   int n_casts;
   bool read_first;   // all inputs are read before any output is written

@@ -63,6 +63,15 @@ def test_workspace_queries_and_argument_validation_without_gpu(kvp):
     assert kvp.decode_workspace_bytes(kvp.DecodeDesc(4, 2, 8, 2, 128, 100, 10, 20), [0, 0, 2, 2]) == 0
 
 
+def test_workspace_of_the_fp32_backward(kvp):
+    """The bf16 form's, and bf16 copies of q and dO of every layer and of k and v of the owners; O is read in place."""
+    donor = [0, 0, 2, 2, 2]
+    for B, S, Hq, Hkv, dh in ((2, 776, 16, 4, 64), (1, 1, 3, 1, 64), (3, 128, 8, 8, 128)):
+        bf, f = (kvp.workspace_bytes(kvp.OP_ATTN_BWD, kvp.Shape(5, B, S, 64, Hq, Hkv, dh, dt), donor) for dt in (kvp.BF16, kvp.F32))
+        align = lambda n: (n + 255) // 256 * 256
+        assert f == align(bf) + 10 * align(2 * B * S * Hq * dh) + 4 * align(2 * B * S * Hkv * dh)
+
+
 def test_self_tests_and_tile_mode_switch_validate_before_touching_the_device(kvp):
     # both bounded-wait self-tests refuse a missing or too small scratch buffer before any launch
     for fn, need in ((kvp.lib.kvp_selftest_bounded_wait, 512 * 1024), (kvp.lib.kvp_selftest_bounded_wait_pair, 768 * 1024)):
