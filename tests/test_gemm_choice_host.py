@@ -74,6 +74,7 @@ def choose(choices):
     ([(1, 4096, 4096)], True), ([(128, 4096, 4096)], True), ([(16, 4096, 4088)], False),    # 32 MB and a little less
     ([(8, 4096, 2048), (8, 1024, 2048), (8, 1024, 2048)], False), ([(8, 4096, 4096), (8, 1024, 4096), (8, 1024, 4096)], True),
     ([(8, 4096, 4096), (160, 4096, 4096)], False), ([(129, 11008, 4096)], False),           # more rows than one tile, than 128
+    ([(5, 4104, 4104)], True), ([(128, 11016, 1608)], True), ([(33, 18440, 920)], True), ([(70, 1032, 16400)], True),   # (those of the GPU's test)
 ])
 def test_streamed_weights(choices, problems, streamed):
     assert choices[2](problems) == streamed

