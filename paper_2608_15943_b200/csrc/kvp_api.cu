@@ -186,7 +186,7 @@ int proj_fwd_bf16(const kvp_shape* s, const int32_t* donor, const void* const* x
     probs.push_back(problem(T, Nkv, {x[l], wk[l], D, D, D}, 0, 0, k[l], Nkv, out));
     probs.push_back(problem(T, Nkv, {x[l], wv[l], D, D, D}, 0, 0, v[l], Nkv, out));
   }
-  return gemm_grouped(probs.data(), int(probs.size()), stream, s->S == 1);   // (one token per sequence: no training step)
+  return gemm_grouped(probs.data(), int(probs.size()), stream);
 }
 
 // before: conversions that the same launch as those of the first chunk's sums performs
@@ -352,7 +352,7 @@ extern "C" int kvp_out_proj_fwd(const kvp_shape* s, const void* const* o, const 
     if (o[l] == nullptr || wo[l] == nullptr || y[l] == nullptr) return KVP_ERR_INVALID_ARG;
     probs.push_back(problem(T, D, {o[l], wo[l], Nq, Nq, Nq}, 0, 0, y[l], D, 0));
   }
-  return gemm_grouped(probs.data(), int(probs.size()), stream, s->S == 1);
+  return gemm_grouped(probs.data(), int(probs.size()), stream);
 }
 
 extern "C" int kvp_out_proj_bwd(const kvp_shape* s, const void* const* o, const void* const* wo,

@@ -1294,7 +1294,7 @@ int gemm_gradient(const GemmProblem* probs, int n, cudaStream_t stream) {
 }
 
 // A forward GEMM (K-major operands, one segment): -1 when the tile kernels take it
-int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t stream) {
+int gemm_forward(const GemmProblem* probs, int n, cudaStream_t stream) {
   int rows = 0;
   for (int i = 0; i < n; ++i) rows = std::max(rows, probs[i].M);
   GemmSize sizes[MAX_PROB];
@@ -1307,7 +1307,7 @@ int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t s
       const int cnt = std::min(SPLIT_MAX_PROB, n - begin);
       const GemmProblem* g = probs + begin;
       const SplitConfig cfg = split_config(sizes_of(g, cnt), cnt, sm_count());
-      const bool stream_b = read_once && stream_weights(sizes, cnt, cfg.nt);
+      const bool stream_b = stream_weights(sizes, cnt, cfg.nt);
       const int rc = by_count(cnt, [&](auto np) { return launch_split<np>(g, cnt, cfg, stream_b, stream); });
       if (rc != KVP_OK) return rc;
     }
@@ -1334,7 +1334,7 @@ int gemm_forward(const GemmProblem* probs, int n, bool read_once, cudaStream_t s
 
 }  // namespace
 
-int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool read_once) {
+int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream) {
   if (n < 0 || (n > 0 && probs == nullptr)) return KVP_ERR_INVALID_ARG;
   for (int i = 0; i < n; ++i) {
     const int rc = check_problem(probs[i]);
@@ -1342,7 +1342,7 @@ int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool read
   }
   const bool forward = k_major(probs, n);
   if (forward) {
-    const int rc = gemm_forward(probs, n, read_once, stream);
+    const int rc = gemm_forward(probs, n, stream);
     if (rc >= 0) return rc;
   }
   // as many problems per launch as the parameter block holds
@@ -1372,7 +1372,7 @@ int gemm_bf16(int M, int N, const GemmSeg* segs, int nseg, int a_mn, int b_mn, v
   g.c = c;
   g.ldc = ldc;
   g.out_f32 = out_f32;
-  if (withhold_at == 0) return gemm_grouped(&g, 1, stream, true);
+  if (withhold_at == 0) return gemm_grouped(&g, 1, stream);
   const int rc = check_problem(g);
   return rc == KVP_OK ? launch_group(&g, 1, stream, withhold_at, wait_limit_ns, use_pair(&g, 1)) : rc;
 }

@@ -134,16 +134,20 @@ inline Choice choose_forward(const GemmSize* probs, int n, int sms) {
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Up to 128 rows: are the weights read with the policy evict_first?  From 32 MB on, with one tile of tokens, and where the call says
-// that they are not read again in this pass (a token step's projections, kvp_gemm): a pass streams far more than L2 holds then, and
-// so some of it is there still at the next.  Measured (us, without -> with): token steps of two layers of d 4096, 1, 8 and 64
-// sequences 182.6 -> 173.3, 190.3 -> 184.0, 253.2 -> 250.2, of four layers, 16 sequences 531.1 -> 529.3 (the latter of the size of
-// the noise); a head of 64 MB behind a layer of d 1024 61.8 -> 58.0.  Not in training steps, whose backward reads the weights again:
-// with the policy four layers of 128 tokens, d 2048 72.3 -> 75.1, two of d 4096 68.8 -> 72.9.  What it costs where less than L2
-// holds passes between two uses of the same weights: 4096 x 11008 again and again at 1 and 32 rows 11.3 -> 12.3 to 13.2, 12.1 -> 12.7
-// to 13.6, three of 4096 x 4096 in turn 23.1 -> 24.0; one or two of them nothing, and 11008 x 4096 and four or more of 4096 x 4096
-// gain (18.1 -> 16.1 at 32 rows, 34.4 -> 31.9).  At 160 rows it gains nothing (eight of 11008 x 4096 168.4 -> 168.4), and loads with
-// a policy of any kind slow tiles that share B (1155 x 1024 x 2816 11.1 -> 12.2).
+// Up to 128 rows: are the weights read with the policy evict_first?  From 32 MB on, with one tile of tokens.  Where more passes
+// between two uses of the same weights than L2 keeps, lines that leave first leave some of the others in place.  Measured (us,
+// without -> with): token steps of two layers of d 4096, 1, 8 and 64 sequences 182.6 -> 173.3, 190.3 -> 184.0, 253.2 -> 250.2, of four
+// layers, 16 sequences 531.1 -> 529.3 (the latter of the size of the noise); a head of 64 MB behind a layer of d 1024 61.8 ->
+// 58.0.  Prefill of layers of d 4096, three sets of weights in turn (one set): one layer, 96 tokens 22.0 -> 20.4 (18.4 -> 18.6), three,
+// 104 tokens 37.4 -> 35.9 (38.0 -> 35.2), five with few heads 30.5 -> 27.5 (29.5 -> 26.0); six of 128 tokens 72.9 -> 75.7, but 102 -> 89
+// on new weights, when L2 is full of what wrote them.
+// A training step of as few tokens reads its weights again in the backward, out of L2 where they are few: one layer of 96 tokens
+// 74.2 -> 76.2, two of 72 102.6 -> 107.4, but three of 104 149.8 -> 144.7, four of 64 166.7 -> 164.1; with output projections 0.98 to
+// 1.02 of the time.  A launch cannot tell one from the other, and prefill gains more.  Where the same weights come again at once:
+// 4096 x 11008 at 1 and 32 rows 11.3 -> 12.3 to 14.1, 12.1 -> 12.7 to 14.9, three of 4096 x 4096 in turn 7.7 -> 8.0 each; one or two of
+// them nothing, and 11008 x 4096 and four or more of 4096 x 4096 gain (18.1 -> 16.1 at 32 rows, 34.4 -> 31.9).
+// At 160 rows it gains nothing (eight of 11008 x 4096 168.4 -> 168.4), and loads with a policy of any kind slow tiles that share
+// B (1155 x 1024 x 2816 11.1 -> 12.2).
 // ------------------------------------------------------------------------------------------------------------
 constexpr double SPLIT_STREAM_BYTES = 32 * 1024 * 1024;
 inline bool stream_weights(const GemmSize* probs, int n, int nt) {

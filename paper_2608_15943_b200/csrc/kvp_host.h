@@ -53,9 +53,8 @@ struct GemmProblem {
 
 // All problems in as few launches as the kernel's parameter block allows (32 problems and 48 segments per launch);
 // the tiles are walked in the order of the list, so the problems with the longest tiles should come first.
-// Which kernel a launch takes follows from its sizes and operand modes (kvp_gemm.cu).  read_once: as far as the call can tell, B is
-// not read again before the next pass.
-int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream, bool read_once = false);
+// Which kernel a launch takes follows from its sizes and operand modes (kvp_gemm.cu).
+int gemm_grouped(const GemmProblem* probs, int n, cudaStream_t stream);
 
 // fp32 -> bf16 (round-to-nearest-even) of a list of tensors in as few launches as the parameter block allows.  elems:
 // multiples of 4.
