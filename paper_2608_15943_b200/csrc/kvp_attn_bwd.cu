@@ -19,7 +19,7 @@
 //               each), so S and dP are computed once for all three gradients.
 //
 //  dq_convert_kernel  scales the fp32 dQ accumulators and writes dQ as bf16 [B,S,Hq,dh].  (Up to 128 tokens a dQ tile has one
-//               partial, which bwd_kernel writes as dQ itself.)
+//               partial, which bwd_kernel writes as dQ itself, unless dQ lies over inputs that other CTAs may still read.)
 //
 // Delta = rowsum(dO * O) comes from a small pre-pass.  The dQ accumulators live in the caller's
 // workspace in a blocked layout ([b][hq][64-query tile][32-column quarter][16][32 columns][4 queries] fp32) so that every
@@ -53,7 +53,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 // warp 0 TMA, warp 1 MMA, warps 2-5 and 6-9 two compute warpgroups, warps 10-13 dQ drain, warps 14 and 15 statistics
-// Bound at DH 128: the shared-memory port (1760 of about 1850 cycles a step).  At DH 64 a step has half the MMA work and the
+// Bound at DH 128: the shared-memory port (1760 of about 1900 cycles a step).  At DH 64 a step has half the MMA work and the
 // same exponentials, and the serial part of a compute warpgroup's step counts: there the warpgroups take every other step,
 // which their own buffers of dP^T, dS^T and staged dQ allow.  Measured (us, whole attn_bwd call, as DH 128 -> so): 2 layers of 4 x
 // 2048, 16 heads on 8, 325 -> 275; 8192, 32 heads on 8, 1020 -> 860; three layers of 3 x 776, 16 heads on 4, 89 -> 75.
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_kernel(const __grid_consta
     }
   } else if (warp < 10) {
     // ------------------------------ compute warpgroups ------------------------------
-    const int wg = (warp - 2) >> 2;     // query columns [wg*32, wg*32+32) of every step
+    const int wg = (warp - 2) >> 2;     // DH 128: query columns [wg*32, wg*32+32) of every step; 64: all of every other step
     const int quarter = warp & 3;       // TMEM lane quarter of this warp
     const int r = quarter * 32 + lane;  // key row inside the tile == TMEM lane
     const uint32_t lane_sel = uint32_t(quarter * 32) << 16;
@@ -889,7 +889,8 @@ int make_map_sum(CUtensorMap* m, const void* base, int B, int S, int H, int dh) 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Orders the CTAs of a launch by their number of steps, longest first; 0 when there are more classes than the parameter
-// block holds.  Three layers of 3 x 776 tokens, dh 64, cut as now: 95 us in index order, 79 longest first.
+// block holds.  Three layers of 3 x 776 tokens, dh 64, cut as now, before heads of 64 had a pipeline of their own: 95 us in index
+// order, 79 longest first.
 int longest_first(BwdParams& p, int n_groups, int n_pairs, int n_jt, int n_qt, int G, int causal) {
   struct Class {
     int steps, ctas;

@@ -16,7 +16,8 @@ constexpr int kStepsPerCta = 256;
 constexpr int kMinWindow = 16;
 // A CTA costs about seven steps besides its steps (prologue, dK / dV reduction, gap between two CTAs), and the last CTAs of
 // a launch leave the device idle for some part of their length: with n steps per SM in all, n * 7 / t + 0.3 t is least at
-// t = sqrt(24 n), and there is nothing to gain from fewer CTAs than one for every SM (1.5 n).
+// t = sqrt(24 n), and there is nothing to gain from fewer CTAs than one for every SM (1.5 n).  Fitted, like the order below, when a
+// step took 1830 cycles at either head size; at heads of 64, where it now takes about a quarter less, a CTA's cost is more steps.
 // Measured (bwd_kernel, us; always 256 steps -> this, in the order below): B3 S776 H16/4 dh64, 3 layers 120 -> 79; B4 S632
 // H8/2 dh128, 8 layers 128 -> 107; B1 S2048 H8/8 dh128, 1 layer 51 -> 42; B1 S4096 H32/8 dh128, 1 layer 458 -> 351.  From
 // about 2700 steps per SM on the 256 stand.
