@@ -718,8 +718,9 @@ constexpr int TMAX_STAGES = 10;                   // a stage holds, per CTA, 128
 // have several tiles of few k-blocks) eight on every other one, so that the stores of one tile run while the other eight wait for the
 // next and read it out.  With all sixteen on each the stores of a tile of fp32 results went out at 6.7 TB/s, and nothing for as
 // long again.  Measured (us, sixteen -> eight): 264 tokens, 7 layers of d 1024 74 -> 69; 128 tokens, 8 layers of d 4096 232 -> 216; but
-// 2328 tokens, 3 layers of d 1024 36 -> 39, where the last tiles count.  Forward, with bf16 results and K up to 768, it makes no
-// difference (four of 2048 x 4096 x 512 44.6 -> 44.8, three of 3000 x 4096 x 768 70.6 -> 69.0, runs 2 apart).
+// 2328 tokens, 3 layers of d 1024 36 -> 39, where the last tiles count.  Forward, with K up to 768, it makes no
+// difference (four of 2048 x 4096 x 512 44.6 -> 44.8, three of 3000 x 4096 x 768 70.6 -> 69.0, runs 2 apart) or one either way (fp32
+// results, eight layers of d 512, 700 tokens 78.3 -> 76.8, of d 256, 500 tokens, heads of 64 28.5 -> 30.3).
 constexpr int TALL_EPI_WARPS = 16, TALL_ALTERNATE_ROUNDS = 6, TALL_SHORT_KBLOCKS = 12;
 constexpr int TALL_THREADS = (2 + TALL_EPI_WARPS) * 32;
 constexpr int TALL_RING = 224 * 1024;             // the ring takes as many stages as fit
